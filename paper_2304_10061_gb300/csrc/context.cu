@@ -92,7 +92,7 @@ struct Cap {
 struct Caps {
   Cap pos, types, species, row_ptr, col_ptr, count, cell_of, wrap, sorted, atom_struct, Eatom, F, Wat, pos4, pw, wraps;
   Cap ej, ei, eS, ed, col_edge, Ee, g;
-  Cap cc, cs, ccur;
+  Cap cc, cs, colc;
   Cap offs, cells, pbc, nimg, Eout, Wout;
 };
 
@@ -163,6 +163,7 @@ struct allegro_ctx {
   int* d_species = nullptr;
   int* d_row_ptr = nullptr;
   int* d_col_ptr = nullptr;
+  int* d_col_count = nullptr;              // zero between neighbour builds
   int* d_count = nullptr;
   int* d_cell_of = nullptr;
   int* d_wrap = nullptr;
@@ -183,9 +184,8 @@ struct allegro_ctx {
   float* d_Ee = nullptr;
   float* d_g = nullptr;
   // cells
-  int* d_cell_count = nullptr;
+  int* d_cell_count = nullptr;             // zero between neighbour builds
   int* d_cell_start = nullptr;
-  int* d_cell_cursor = nullptr;
   int64_t cell_cap = 0;
   // structures
   int64_t* d_offs = nullptr;
@@ -316,6 +316,13 @@ cudaError_t regrow(T*& p, int64_t& cap, int64_t need, double headroom = 1.05) {
 template <typename T>
 cudaError_t grow(T*& p, Cap& cap, int64_t need) {
   return regrow(p, cap.v, need);
+}
+
+// counters that every scan leaves at zero: cleared when they are allocated
+cudaError_t grow_zeroed(int*& p, Cap& cap, int64_t need, cudaStream_t st) {
+  if (need <= cap.v && p) return cudaSuccess;
+  const cudaError_t e = regrow(p, cap.v, need);
+  return e != cudaSuccess ? e : cudaMemsetAsync(p, 0, (size_t)cap.v * sizeof(int), st);
 }
 
 inline Caps& caps_of(allegro_ctx* c) { return c->caps; }
@@ -751,6 +758,7 @@ allegro_status stage_atoms(allegro_ctx* c, int64_t n, const double* pos, const i
   CUDA_TRY(c, grow(c->d_row_ptr, k.row_ptr, need + 1));
   CUDA_TRY(c, grow(c->d_col_ptr, k.col_ptr, need + 1));
   CUDA_TRY(c, grow(c->d_count, k.count, need + 1));
+  CUDA_TRY(c, grow_zeroed(c->d_col_count, k.colc, need + 1, c->stream));
   CUDA_TRY(c, grow(c->d_cell_of, k.cell_of, need));
   CUDA_TRY(c, grow(c->d_wrap, k.wrap, 3 * need));
   CUDA_TRY(c, grow(c->d_sorted, k.sorted, need));
@@ -820,17 +828,26 @@ allegro_status read_err(allegro_ctx* c, int* out) {
   return ALLEGRO_OK;
 }
 
-// CSC index and host row_ptr copy, shared by both neighbour paths.
-allegro_status finish_neighbors(allegro_ctx* c, int n, int64_t E) {
+// Each edge's arrival order in its column, from the fill pass to finish_neighbors: held in the
+// edge-energy array, which the next evaluation writes first.
+int* col_rank(allegro_ctx* c) { return reinterpret_cast<int*>(c->d_Ee); }
+
+// CSC index (from the fill pass's column counts and ranks) and host row_ptr copy, shared by all
+// neighbour paths.
+allegro_status finish_neighbors(allegro_ctx* c, int n, int64_t E, bool ranked = true) {
   cudaStream_t st = c->stream;
-  CUDA_TRY(c, cudaMemsetAsync(c->d_count, 0, (size_t)(n + 1) * 4, st));
   {
-    ProfScope ps(c, "nb_csc", 0.0, (double)E * 16 + (double)n * 16, 6);
-    nb_columns(c->d_ej, (int)E, n, c->d_count, st);
-    exclusive_scan_i32(c->d_count, c->d_col_ptr, n, nullptr, c->d_scan_tmp, c->scan_tmp_cap, st);
-    CUDA_TRY(c, cudaMemsetAsync(c->d_count, 0, (size_t)(n + 1) * 4, st));
-    nb_fill_columns(c->d_ej, (int)E, c->d_col_ptr, c->d_count, c->d_col_edge, st);
-    nb_sort_columns(c->d_col_ptr, n, c->d_col_edge, st);
+    ProfScope ps(c, "nb_csc", 0.0, (double)E * 16 + (double)n * 16, 0);
+    if (!ranked) {
+      nb_col_rank(c->d_ej, (int)E, c->d_col_count, col_rank(c), st);
+      ++c->launches;
+    }
+    c->launches += exclusive_scan_i32(c->d_col_count, c->d_col_ptr, n, c->d_scan_tmp, true, st);
+    if (E > 0) {
+      nb_place(c->d_ej, col_rank(c), (int)E, c->d_col_ptr, c->d_col_edge, st);
+      nb_sort_columns(c->d_col_ptr, n, c->d_col_edge, st);
+      c->launches += 2;
+    }
   }
   CUDA_TRY(c, cudaGetLastError());
   c->h_row_ptr.resize((size_t)n + 1);
@@ -1811,9 +1828,10 @@ allegro_status allegro_create(const void* weights_blob, size_t blob_bytes, const
       cudaMemcpy(c->d_map, c->species_map.data(), c->nmap * 4, cudaMemcpyHostToDevice) != cudaSuccess)
     return bail(fail(c, ALLEGRO_E_OOM, "species map upload failed"));
   if (cudaMalloc(&c->d_err, 16) != cudaSuccess || cudaMalloc(&c->d_total, 16) != cudaSuccess ||
-      cudaMalloc(&c->d_minmax, 12 * 8) != cudaSuccess || cudaMalloc(&c->d_red_scratch, 12 * 1024 * 8) != cudaSuccess)
+      cudaMalloc(&c->d_minmax, 12 * 8) != cudaSuccess || cudaMalloc(&c->d_red_scratch, kStructScratch * sizeof(double)) != cudaSuccess)
     return bail(fail(c, ALLEGRO_E_OOM, "scratch allocation failed"));
   cudaMemset(c->d_err, 0, 16);
+  cudaMemset(c->d_red_scratch, 0, kStructScratch * sizeof(double));
   *out = c;
   return ALLEGRO_OK;
 }
@@ -2004,9 +2022,8 @@ static allegro_status build_single(allegro_ctx* c, int64_t n_atoms, const double
     ncell = (int64_t)g.n[0] * g.n[1] * g.n[2];
   }
   Caps& k = caps_of(c);
-  CUDA_TRY(c, grow(c->d_cell_count, k.cc, ncell + 1));
+  CUDA_TRY(c, grow_zeroed(c->d_cell_count, k.cc, ncell + 1, st));
   CUDA_TRY(c, grow(c->d_cell_start, k.cs, ncell + 1));
-  CUDA_TRY(c, grow(c->d_cell_cursor, k.ccur, ncell + 1));
   size_t need_tmp = scan_tmp_bytes((int)std::max<int64_t>(ncell, n)) + 4096;
   if (need_tmp > c->scan_tmp_cap) {
     if (c->d_scan_tmp) cudaFree(c->d_scan_tmp);
@@ -2014,15 +2031,13 @@ static allegro_status build_single(allegro_ctx* c, int64_t n_atoms, const double
     CUDA_TRY(c, cudaMalloc(&c->d_scan_tmp, need_tmp * 2));
     c->scan_tmp_cap = need_tmp * 2;
   }
-  CUDA_TRY(c, cudaMemsetAsync(c->d_cell_count, 0, (size_t)(ncell + 1) * 4, st));
   {
-    ProfScope ps(c, "nb_bin_sort", 0.0, (double)n * 80 + (double)ncell * 16, 7);
-    nb_bin(c->d_pos, n, g, c->d_cell_of, c->d_wrap, c->d_cell_count, st);
-    exclusive_scan_i32(c->d_cell_count, c->d_cell_start, (int)ncell, nullptr, c->d_scan_tmp, c->scan_tmp_cap, st);
-    CUDA_TRY(c, cudaMemsetAsync(c->d_cell_cursor, 0, (size_t)(ncell + 1) * 4, st));
-    nb_place(c->d_cell_of, n, c->d_cell_start, c->d_cell_cursor, c->d_sorted, st);
-    nb_sort_cells(c->d_cell_start, (int)ncell, c->d_sorted, st);
-    nb_pos4(c->d_pos, c->d_species, n, g, c->d_wrap, c->d_sorted, c->d_pos4, c->d_pw, c->d_wraps, st);
+    ProfScope ps(c, "nb_bin_sort", 0.0, (double)n * 80 + (double)ncell * 16, 3);
+    nb_bin(c->d_pos, n, g, c->d_cell_of, c->d_wrap, c->d_cell_count, c->d_count, st);
+    c->launches += exclusive_scan_i32(c->d_cell_count, c->d_cell_start, (int)ncell, c->d_scan_tmp, true, st);
+    nb_place(c->d_cell_of, c->d_count, n, c->d_cell_start, c->d_sorted, st);
+    nb_sort_cells(c->d_pos, c->d_species, g, (int)ncell, c->d_cell_start, c->d_wrap, c->d_sorted, c->d_pos4, c->d_pw,
+                  c->d_wraps, st);
   }
   // Error band of the float32 prefilter: bound X on |wrapped coordinate| and
   // |image offset|, per-component error <= 8 ulp(X), squared-distance error
@@ -2045,11 +2060,11 @@ static allegro_status build_single(allegro_ctx* c, int64_t n_atoms, const double
   }
   const double rc2 = rc * rc;
   {
-    ProfScope ps(c, "nb_search_count", 0.0, (double)n * 64, 4);
+    ProfScope ps(c, "nb_search_count", 0.0, (double)n * 64);
     nb_search(false, c->d_pos, n, g, c->d_cell_of, c->d_wraps, c->d_cell_start, c->d_sorted, c->d_pos4, c->d_pw, rc2,
               band, pair_rc2, c->arch.ns, c->d_count,
-              nullptr, nullptr, nullptr, nullptr, nullptr, c->d_err, st);
-    exclusive_scan_i32(c->d_count, c->d_row_ptr, n, nullptr, c->d_scan_tmp, c->scan_tmp_cap, st);
+              nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, c->d_err, st);
+    c->launches += exclusive_scan_i32(c->d_count, c->d_row_ptr, n, c->d_scan_tmp, false, st);
   }
   int hE = 0;
   CUDA_TRY(c, cudaMemcpyAsync(&hE, c->d_row_ptr + n, 4, cudaMemcpyDeviceToHost, st));
@@ -2057,13 +2072,14 @@ static allegro_status build_single(allegro_ctx* c, int64_t n_atoms, const double
   CUDA_TRY(c, cudaGetLastError());
   if (hE < 0) return fail(c, ALLEGRO_E_CAPACITY, "edge count overflows int32");
   if ((s = ensure_edges(c, hE)) != ALLEGRO_OK) return s;
+  bool ranked = true;
   {
     ProfScope ps(c, "nb_search_fill", 0.0, (double)hE * 44 + (double)n * 64);
-    nb_search(true, c->d_pos, n, g, c->d_cell_of, c->d_wraps, c->d_cell_start, c->d_sorted, c->d_pos4, c->d_pw, rc2,
+    ranked = nb_search(true, c->d_pos, n, g, c->d_cell_of, c->d_wraps, c->d_cell_start, c->d_sorted, c->d_pos4, c->d_pw, rc2,
               band, pair_rc2, c->arch.ns, nullptr,
-              c->d_row_ptr, c->d_ej, c->d_ei, c->d_eS, c->d_ed, c->d_err, st);
+              c->d_row_ptr, c->d_ej, c->d_ei, c->d_eS, c->d_ed, c->d_col_count, col_rank(c), c->d_err, st);
   }
-  if ((s = finish_neighbors(c, n, hE)) != ALLEGRO_OK) return s;
+  if ((s = finish_neighbors(c, n, hE, ranked)) != ALLEGRO_OK) return s;
   c->n_centres = g.n_centres;
   if (n_edges_out) *n_edges_out = hE;
   return ALLEGRO_OK;
@@ -2152,15 +2168,16 @@ allegro_status allegro_neighbors_batched(allegro_ctx* c, int32_t n_struct, const
   atom_struct_kernel<<<n_struct, 128, 0, st>>>(c->d_offs, n_struct, c->d_atom_struct);
   const double rc2 = rc * rc;
   nb_bruteforce_batched(false, c->d_pos, c->d_offs, n_struct, cells ? c->d_cells : nullptr, c->d_pbc, c->d_nimg, rc2,
-                        c->d_species, c->arch.pair_rc2, c->arch.ns, c->d_atom_struct, n, c->d_count, nullptr, nullptr, nullptr, nullptr, nullptr, c->d_err, st);
-  exclusive_scan_i32(c->d_count, c->d_row_ptr, n, nullptr, c->d_scan_tmp, c->scan_tmp_cap, st);
+                        c->d_species, c->arch.pair_rc2, c->arch.ns, c->d_atom_struct, n, c->d_count, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
+                        c->d_err, st);
+  c->launches += exclusive_scan_i32(c->d_count, c->d_row_ptr, n, c->d_scan_tmp, false, st);
   int hE = 0;
   CUDA_TRY(c, cudaMemcpyAsync(&hE, c->d_row_ptr + n, 4, cudaMemcpyDeviceToHost, st));
   CUDA_TRY(c, cudaStreamSynchronize(st));
   CUDA_TRY(c, cudaGetLastError());
   if ((s = ensure_edges(c, hE)) != ALLEGRO_OK) return s;
   nb_bruteforce_batched(true, c->d_pos, c->d_offs, n_struct, cells ? c->d_cells : nullptr, c->d_pbc, c->d_nimg, rc2,
-                        c->d_species, c->arch.pair_rc2, c->arch.ns, c->d_atom_struct, n, nullptr, c->d_row_ptr, c->d_ej, c->d_ei, c->d_eS, c->d_ed, c->d_err, st);
+                        c->d_species, c->arch.pair_rc2, c->arch.ns, c->d_atom_struct, n, nullptr, c->d_row_ptr, c->d_ej, c->d_ei, c->d_eS, c->d_ed, c->d_col_count, col_rank(c), c->d_err, st);
   if ((s = finish_neighbors(c, n, hE)) != ALLEGRO_OK) return s;
   c->nstruct = n_struct;
   c->batched = true;
@@ -2276,11 +2293,11 @@ allegro_status allegro_md_verlet(allegro_ctx* c, int64_t n_atoms, double* pos, d
     }
     c->have_nb = false;
     {
-      ProfScope ps(c, "nb_skin_filter", 0.0, (double)n * 64, 2);
+      ProfScope ps(c, "nb_skin_filter", 0.0, (double)n * 64);
       nb_skin_filter(false, c->d_pos, n, c->d_cell9, c->d_sk_row, c->d_sk_j, c->d_sk_S, c->arch.rc * c->arch.rc,
                      c->arch.pair_rc2, c->d_species, c->arch.ns, c->d_count, nullptr, nullptr, nullptr, nullptr,
-                     nullptr, st);
-      exclusive_scan_i32(c->d_count, c->d_row_ptr, n, nullptr, c->d_scan_tmp, c->scan_tmp_cap, st);
+                     nullptr, nullptr, nullptr, st);
+      c->launches += exclusive_scan_i32(c->d_count, c->d_row_ptr, n, c->d_scan_tmp, false, st);
     }
     int hE = 0;
     CUDA_TRY(c, cudaMemcpyAsync(&hE, c->d_row_ptr + n, 4, cudaMemcpyDeviceToHost, st));
@@ -2290,7 +2307,7 @@ allegro_status allegro_md_verlet(allegro_ctx* c, int64_t n_atoms, double* pos, d
       ProfScope ps(c, "nb_skin_filter", 0.0, (double)hE * 44 + (double)n * 64);
       nb_skin_filter(true, c->d_pos, n, c->d_cell9, c->d_sk_row, c->d_sk_j, c->d_sk_S, c->arch.rc * c->arch.rc,
                      c->arch.pair_rc2, c->d_species, c->arch.ns, nullptr, c->d_row_ptr, c->d_ej, c->d_ei, c->d_eS,
-                     c->d_ed, st);
+                     c->d_ed, c->d_col_count, col_rank(c), st);
     }
     CUDA_TRY(c, cudaGetLastError());
     return finish_neighbors(c, n, hE);
@@ -2465,7 +2482,7 @@ void allegro_destroy(allegro_ctx* c) {
   void* bufs[] = {c->d_map, c->d_pos, c->d_types, c->d_species, c->d_row_ptr, c->d_col_ptr, c->d_count,
                   c->d_cell_of, c->d_wrap, c->d_sorted, c->d_pos4, c->d_pw, c->d_atom_struct, c->d_Eatom, c->d_F, c->d_Wat,
                   c->d_ej, c->d_ei, c->d_eS, c->d_ed, c->d_col_edge, c->d_Ee, c->d_g, c->d_cell_count,
-                  c->d_cell_start, c->d_cell_cursor, c->d_offs, c->d_cells, c->d_pbc, c->d_nimg, c->d_Eout,
+                  c->d_cell_start, c->d_col_count, c->d_offs, c->d_cells, c->d_pbc, c->d_nimg, c->d_Eout,
                   c->d_Wout, c->d_scan_tmp, c->d_err, c->d_total, c->d_minmax, c->d_red_scratch, c->ws,
                   c->d_md_pos, c->d_md_vel, c->d_md_invm, c->d_md_types, c->d_md_masses, c->d_md_E, c->d_md_K,
                   c->d_md_part, c->d_pair_basis, c->d_pair_rc2, c->d_zbl, c->d_sk_row, c->d_sk_j,

@@ -665,98 +665,186 @@ __global__ void atom_reduce_kernel(int n, int n_centres, const int* __restrict__
   }
 }
 
+// The same sums with 16 lanes per atom, for systems too small to fill the GPU with a thread per
+// atom.  The lanes fetch 16 edges at a time (one each, the ZBL term included) into shared memory,
+// then lane q accumulates one of the atom's 14 sums over them in edge order: the float64 operations
+// of each sum are those of the kernel above, in the same order, so both give the same bits.
+constexpr int kReduceAtoms = 8;   // atoms per block (16 lanes each)
+
+__global__ void __launch_bounds__(16 * kReduceAtoms) atom_reduce_group_kernel(
+    int n, int n_centres, const int* __restrict__ row_ptr, const int* __restrict__ col_ptr,
+    const int* __restrict__ col_edge, const float* __restrict__ Ee, const float* __restrict__ g,
+    const double* __restrict__ ed, const int* __restrict__ species, const double* __restrict__ sigma,
+    const double* __restrict__ mu, bool want_forces, double* __restrict__ E_atom, double* __restrict__ F,
+    double* __restrict__ Wat, const int* __restrict__ ei, const int* __restrict__ ej, const float2* __restrict__ zbl,
+    BasisConst bc) {
+  // per edge: -d (3), 1, g (3), E, E_ZBL
+  __shared__ double sh[kReduceAtoms][16][9];
+  const int q = threadIdx.x & 15, w = threadIdx.x >> 4;
+  const unsigned mask = 0xffffu << (threadIdx.x & 16);
+  const int i = blockIdx.x * kReduceAtoms + w;
+  if (i >= n) return;
+  const int z = species[i];
+  // lane q's factors: W[3 a + b] -= d_a g_b (q < 9), f_b += g_b (9..11), E (12), E_ZBL (13)
+  const int ka = q < 9 ? q / 3 : 3, kb = q < 9 ? 4 + q % 3 : (q < 12 ? 4 + q - 9 : (q == 12 ? 7 : 8));
+  double acc = 0.0;
+  const int b = row_ptr[i], e1 = row_ptr[i + 1];
+  for (int e0 = b; e0 < e1; e0 += 16) {
+    const int m = min(16, e1 - e0);
+    if (q < m) {
+      const size_t e = (size_t)e0 + q;
+      double gx = 0.0, gy = 0.0, gz = 0.0, ezd = 0.0;
+      if (want_forces) {
+        gx = g[3 * e]; gy = g[3 * e + 1]; gz = g[3 * e + 2];
+      }
+      const double d0 = ed[3 * e], d1 = ed[3 * e + 1], d2 = ed[3 * e + 2];
+      if (zbl) {
+        const int zj = species[ej[e]];
+        const float r = (float)sqrt(d0 * d0 + d1 * d1 + d2 * d2);
+        float ez, dedr;
+        zbl_edge(r, zbl[z * bc.ns + zj], pair_basis(bc, z, zj).x, bc, ez, dedr);
+        ezd = (double)ez;
+        const double s = (double)(dedr / r);
+        gx += s * d0; gy += s * d1; gz += s * d2;
+      }
+      double* o = sh[w][q];
+      o[0] = -d0; o[1] = -d1; o[2] = -d2; o[3] = 1.0;
+      o[4] = gx; o[5] = gy; o[6] = gz; o[7] = (double)Ee[e]; o[8] = ezd;
+    }
+    __syncwarp(mask);
+    if (q < 14 && (want_forces || q >= 12))
+      for (int k = 0; k < m; ++k) acc = fma(sh[w][k][ka], sh[w][k][kb], acc);
+    __syncwarp(mask);
+  }
+  const double Ei = __shfl_sync(mask, acc, 12, 16), Ez = __shfl_sync(mask, acc, 13, 16);
+  if (q == 0) E_atom[i] = (i < n_centres) ? sigma[z] * Ei + mu[z] + Ez : 0.0;
+  if (!want_forces) return;
+  if (q < 9) Wat[9 * (size_t)i + q] = acc;
+  const int c0 = col_ptr[i], c1 = col_ptr[i + 1];
+  for (int k0 = c0; k0 < c1; k0 += 16) {
+    const int m = min(16, c1 - k0);
+    if (q < m) {
+      const size_t e = (size_t)col_edge[k0 + q];
+      double gx = g[3 * e], gy = g[3 * e + 1], gz = g[3 * e + 2];
+      if (zbl) {   // the ZBL part of this edge's dE/dd (edge (k -> i): centre species first)
+        const double d0 = ed[3 * e], d1 = ed[3 * e + 1], d2 = ed[3 * e + 2];
+        const int zc = species[ei[e]];
+        const float r = (float)sqrt(d0 * d0 + d1 * d1 + d2 * d2);
+        float ez, dedr;
+        zbl_edge(r, zbl[zc * bc.ns + z], pair_basis(bc, zc, z).x, bc, ez, dedr);
+        const double s = (double)(dedr / r);
+        gx += s * d0; gy += s * d1; gz += s * d2;
+      }
+      double* o = sh[w][q];
+      o[4] = gx; o[5] = gy; o[6] = gz;
+    }
+    __syncwarp(mask);
+    if (q >= 9 && q < 12)
+      for (int k = 0; k < m; ++k) acc -= sh[w][k][kb];
+    __syncwarp(mask);
+  }
+  if (q >= 9 && q < 12) F[3 * (size_t)i + q - 9] = acc;
+}
+
+// Up to this many atoms 16 lanes per atom (a thread's chain of dependent float64 additions takes 31 to
+// 41 us at any size; float64 issue makes the lanes' idle slots cost more above): us, group / thread, with
+// forces 64 atoms 10 / 31, 3,072 atoms 14 / 41, 16,384 atoms 45 / 43, with the ZBL term 16,411 atoms 53 / 92;
+// energies alone 12,345 atoms 25 / 10.
+constexpr int kReduceGroupAtoms = 12000, kReduceGroupAtomsZbl = 24000, kReduceGroupAtomsEnergy = 3000;
+
 void atom_reduce(int n, int n_centres, const int* row_ptr, const int* col_ptr, const int* col_edge, const float* Ee,
                  const float* g, const double* ed, const int* species, const double* sigma, const double* mu,
                  bool want_forces, double* E_atom, double* F, double* Wat, const int* ei, const int* ej,
                  const Arch& a, cudaStream_t st) {
   if (n <= 0) return;
-  atom_reduce_kernel<<<(n + 127) / 128, 128, 0, st>>>(n, n_centres, row_ptr, col_ptr, col_edge, Ee, g, ed, species, sigma,
-                                                      mu, want_forces, E_atom, F, Wat, ei, ej,
-                                                      reinterpret_cast<const float2*>(a.zbl), make_basis(a));
+  const float2* zbl = reinterpret_cast<const float2*>(a.zbl);
+  if (n <= (zbl ? kReduceGroupAtomsZbl : (want_forces ? kReduceGroupAtoms : kReduceGroupAtomsEnergy)))
+    atom_reduce_group_kernel<<<(n + kReduceAtoms - 1) / kReduceAtoms, 16 * kReduceAtoms, 0, st>>>(
+        n, n_centres, row_ptr, col_ptr, col_edge, Ee, g, ed, species, sigma, mu, want_forces, E_atom, F, Wat, ei, ej,
+        zbl, make_basis(a));
+  else
+    atom_reduce_kernel<<<(n + 127) / 128, 128, 0, st>>>(n, n_centres, row_ptr, col_ptr, col_edge, Ee, g, ed, species,
+                                                        sigma, mu, want_forces, E_atom, F, Wat, ei, ej, zbl,
+                                                        make_basis(a));
 }
 
-// One block per structure: E_b = sum of its atoms' Etilde_i, W_b = sum of W_i
-// (fixed-order tree reduction, so results are bitwise reproducible).  Also
-// flags non-finite per-atom energies or forces.
-__global__ void struct_reduce_kernel(const int64_t* __restrict__ offs, const double* __restrict__ E_atom,
-                                     const double* __restrict__ Wat, const double* __restrict__ F, bool want_w,
-                                     double* __restrict__ E_out, double* __restrict__ W_out,
-                                     int* __restrict__ d_err) {
-  const int b = blockIdx.x;
-  const long long a0 = offs[b], a1 = offs[b + 1];
-  __shared__ double sh[10][256];
-  double acc[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+// Per structure: E_b = sum of its atoms' Etilde_i, W_b = sum of W_i, in a fixed
+// order (bitwise reproducible); flags non-finite per-atom energies or forces.
+// Ten warps per block, warp q one of the ten sums: float64 is the slow unit
+// here, and a tree over ten sums per thread costs five times the additions.
+// A large single structure is cut into `parts` ranges, one block each; the
+// block that finishes last (a ticket counter that it resets) sums the partials
+// in order, so the whole reduction is one launch.
+constexpr int kStructThreads = 320;
+constexpr int kStructParts = 1024;   // most ranges of one structure
+constexpr int kStructAtoms = 256;    // atoms per range below that
+
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+__global__ void __launch_bounds__(kStructThreads) struct_reduce_kernel(
+    const int64_t* __restrict__ offs, const double* __restrict__ E_atom, const double* __restrict__ Wat,
+    const double* __restrict__ F, bool want_w, int parts, double* __restrict__ part, unsigned* __restrict__ ticket,
+    double* __restrict__ E_out, double* __restrict__ W_out, int* __restrict__ d_err) {
+  const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+  long long a0, a1;
+  if (parts > 1) {
+    const long long n = offs[1];
+    a0 = n * blockIdx.x / parts;
+    a1 = n * (blockIdx.x + 1) / parts;
+  } else {
+    a0 = offs[blockIdx.x];
+    a1 = offs[blockIdx.x + 1];
+  }
+  const bool on = q == 0 || want_w;
+  double acc = 0.0;
   bool bad = false;
-  for (long long i = a0 + threadIdx.x; i < a1; i += blockDim.x) {
-    double e = E_atom[i];
-    acc[0] += e;
-    bad |= !isfinite(e);
-    if (want_w) {
-      for (int q = 0; q < 9; ++q) acc[1 + q] += Wat[9 * i + q];
-      bad |= !(isfinite(F[3 * i]) && isfinite(F[3 * i + 1]) && isfinite(F[3 * i + 2]));
+  if (on) {
+    const double* src = q == 0 ? E_atom : Wat + (q - 1);
+    const int ld = q == 0 ? 1 : 9;
+    for (long long i = a0 + lane; i < a1; i += 32) {
+      const double x = src[ld * i];
+      acc += x;
+      if (q == 0) bad |= !isfinite(x);
+      if (want_w && q >= 1 && q <= 3) bad |= !isfinite(F[3 * i + q - 1]);
     }
+    acc = warp_sum(acc);
   }
   if (bad) atomicOr(d_err, kErrNonFinite);
-  for (int q = 0; q < 10; ++q) sh[q][threadIdx.x] = acc[q];
+  if (parts == 1) {
+    if (on && lane == 0) (q == 0 ? E_out[blockIdx.x] : W_out[9 * (size_t)blockIdx.x + q - 1]) = acc;
+    return;
+  }
+  __shared__ bool last;
+  if (on && lane == 0) part[(size_t)q * kStructParts + blockIdx.x] = acc;
+  __threadfence();
   __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s)
-      for (int q = 0; q < 10; ++q) sh[q][threadIdx.x] += sh[q][threadIdx.x + s];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    E_out[b] = sh[0][0];
-    if (want_w)
-      for (int q = 0; q < 9; ++q) W_out[9 * b + q] = sh[1 + q][0];
-  }
-}
-
-// Large single structures: first a fixed grid of blocks reduces contiguous
-// atom ranges into partials (offsets describe the ranges), then one block
-// reduces the partials; both in fixed order.
-__global__ void partial_offsets_kernel(const int64_t* __restrict__ offs, int parts, int64_t* __restrict__ po) {
-  const long long n = offs[1];
-  for (int p = threadIdx.x; p <= parts; p += blockDim.x) po[p] = (n * p) / parts;
-}
-
-__global__ void sum_partials_kernel(const double* __restrict__ partE, const double* __restrict__ partW, int parts,
-                                    bool want_w, double* __restrict__ E_out, double* __restrict__ W_out) {
-  __shared__ double sh[10][256];
-  double acc[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-  for (int p = threadIdx.x; p < parts; p += blockDim.x) {
-    acc[0] += partE[p];
-    if (want_w)
-      for (int q = 0; q < 9; ++q) acc[1 + q] += partW[9 * (size_t)p + q];
-  }
-  for (int q = 0; q < 10; ++q) sh[q][threadIdx.x] = acc[q];
+  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == (unsigned)parts - 1;
   __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s)
-      for (int q = 0; q < 10; ++q) sh[q][threadIdx.x] += sh[q][threadIdx.x + s];
-    __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (on) {
+    acc = 0.0;
+    for (int p = lane; p < parts; p += 32) acc += __ldcg(part + (size_t)q * kStructParts + p);
+    acc = warp_sum(acc);
+    if (lane == 0) (q == 0 ? E_out[0] : W_out[q - 1]) = acc;
   }
-  if (threadIdx.x == 0) {
-    E_out[0] = sh[0][0];
-    if (want_w)
-      for (int q = 0; q < 9; ++q) W_out[q] = sh[1 + q][0];
-  }
+  if (threadIdx.x == 0) *ticket = 0;
 }
 
+// scratch: kStructScratch doubles, zero before the first call
 void struct_reduce(int nstruct, const int64_t* offs, const double* E_atom, const double* Wat, const double* F,
                    bool want_w, double* E_out, double* W_out, int* d_err, double* scratch, int64_t n_atoms,
                    cudaStream_t st) {
   if (nstruct <= 0) return;
-  const int parts = 1024;
-  if (nstruct == 1 && n_atoms > 16 * parts && scratch) {
-    int64_t* po = reinterpret_cast<int64_t*>(scratch);
-    double* pE = scratch + (parts + 2);
-    double* pW = pE + parts;
-    partial_offsets_kernel<<<1, 256, 0, st>>>(offs, parts, po);
-    struct_reduce_kernel<<<parts, 256, 0, st>>>(po, E_atom, Wat, F, want_w, pE, pW, d_err);
-    sum_partials_kernel<<<1, 256, 0, st>>>(pE, pW, parts, want_w, E_out, W_out);
-    return;
-  }
-  struct_reduce_kernel<<<nstruct, 256, 0, st>>>(offs, E_atom, Wat, F, want_w, E_out, W_out, d_err);
+  static_assert(kStructScratch > 10 * kStructParts, "partials and the ticket");
+  const int parts = nstruct == 1 ? (int)std::min<int64_t>(kStructParts, (n_atoms + kStructAtoms - 1) / kStructAtoms) : 1;
+  struct_reduce_kernel<<<parts > 1 ? parts : nstruct, kStructThreads, 0, st>>>(
+      offs, E_atom, Wat, F, want_w, std::max(parts, 1), scratch, reinterpret_cast<unsigned*>(scratch + 10 * kStructParts),
+      E_out, W_out, d_err);
 }
 
 }  // namespace alg

@@ -162,8 +162,9 @@ void fp8_quantize(const float* src, int rows, int cols, int lds, uint8_t* dst, i
                   cudaStream_t st);
 
 // scan / utilities
-void exclusive_scan_i32(const int* in, int* out, int n, int* d_total, void* tmp, size_t tmp_bytes,
-                        cudaStream_t st);
+// out[0..n] = exclusive scan of in[0..n) (arrays 16-byte aligned); `clear` zeroes the input as it is
+// read.  Returns the launches made.
+int exclusive_scan_i32(int* in, int* out, int n, void* tmp, bool clear, cudaStream_t st);
 size_t scan_tmp_bytes(int n);
 
 // neighbours
@@ -176,37 +177,39 @@ struct CellGrid {
   double lo[3], span[3];   // non-periodic axes: frac range mapped onto the grid
   int n_centres;      // atoms [0, n_centres) are centres; the rest (ghosts) only neighbours
 };
-void nb_bin(const double* pos, int n, const CellGrid& g, int* cell_of, int* wrap, int* cell_count,
+// cell_count: zero on entry; cell_rank[i]: atom i's arrival order in its cell
+void nb_bin(const double* pos, int n, const CellGrid& g, int* cell_of, int* wrap, int* cell_count, int* cell_rank,
             cudaStream_t st);
-void nb_place(const int* cell_of, int n, const int* cell_start, int* cell_cursor, int* sorted,
-              cudaStream_t st);
-void nb_sort_cells(const int* cell_start, int n_cells, int* sorted, cudaStream_t st);
-// pos4[s].w carries the model species of atom sorted[s] (its bits)
-// pos4 / pw / wraps: wrapped float32 (with the species bits) and float64 positions and the
-// wrap counts, all in cell order
-void nb_pos4(const double* pos, const int* species, int n, const CellGrid& g, const int* wrap, const int* sorted,
-             float4* pos4, double* pw, int4* wraps, cudaStream_t st);
+// sorted[start[seg_of[i]] + rank[i]] = i for i in [0, n)
+void nb_place(const int* seg_of, const int* rank, int n, const int* start, int* sorted, cudaStream_t st);
+// each cell's atoms in index order, and pos4 / pw / wraps: wrapped float32 (with the model species'
+// bits in w) and float64 positions and the wrap counts, all in cell order
+void nb_sort_cells(const double* pos, const int* species, const CellGrid& g, int n_cells, const int* cell_start,
+                   const int* wrap, int* sorted, float4* pos4, double* pw, int4* wraps, cudaStream_t st);
 // pair_rc2: null, or device [ns * ns] squared cutoffs per ordered species pair
-// (each <= rc2, the search radius; `band` is the prefilter band of rc2)
-void nb_search(bool fill, const double* pos, int n, const CellGrid& g, const int* cell_of,
+// (each <= rc2, the search radius; `band` is the prefilter band of rc2).  The fill passes also count
+// every edge into its neighbour's column (col_count, zero on entry) and keep its arrival order there
+// (col_rank[e]); nb_search returns false when it left that to nb_col_rank.
+bool nb_search(bool fill, const double* pos, int n, const CellGrid& g, const int* cell_of,
                const int4* wraps, const int* cell_start, const int* sorted, const float4* pos4, const double* pw,
                double rc2, float band, const double* pair_rc2, int ns, int* count, const int* row_ptr, int* ej,
-               int* ei, int* eS, double* ed, int* d_err, cudaStream_t st);
+               int* ei, int* eS, double* ed, int* col_count, int* col_rank, int* d_err, cudaStream_t st);
 void nb_bruteforce_batched(bool fill, const double* pos, const int64_t* offs, int nstruct,
                            const double* cells, const int* pbc, const int* nimg, double rc2,
                            const int* species, const double* pair_rc2, int ns,
                            const int* atom_struct, int n, int* count, const int* row_ptr, int* ej,
-                           int* ei, int* eS, double* ed, int* d_err, cudaStream_t st);
+                           int* ei, int* eS, double* ed, int* col_count, int* col_rank, int* d_err,
+                           cudaStream_t st);
 // Verlet-skin reuse: count (fill = false, into count[i]) or write (fill = true, rows at row_ptr[i]) the
 // candidates of a list built at r_c + skin (sk_row / sk_j / sk_S) that pass the exact rule now
 void nb_skin_filter(bool fill, const double* pos, int n, const double* d_cell, const int* sk_row, const int* sk_j,
                     const int* sk_S, double rc2, const double* pair_rc2, const int* species, int ns, int* count,
-                    const int* row_ptr, int* ej, int* ei, int* eS, double* ed, cudaStream_t st);
+                    const int* row_ptr, int* ej, int* ei, int* eS, double* ed, int* col_count, int* col_rank,
+                    cudaStream_t st);
 // max_i |pos_i - ref_i|^2 as the bits of a double in *out (cleared first)
 void nb_max_disp2(const double* pos, const double* ref, int n, unsigned long long* out, cudaStream_t st);
-void nb_columns(const int* ej, int E, int n, int* col_count, cudaStream_t st);
-void nb_fill_columns(const int* ej, int E, const int* col_ptr, int* cursor, int* col_edge,
-                     cudaStream_t st);
+void nb_col_rank(const int* ej, int E, int* col_count, int* col_rank, cudaStream_t st);
+// each column's edges in ascending order
 void nb_sort_columns(const int* col_ptr, int n, int* col_edge, cudaStream_t st);
 void nb_struct_span(const double* pos, const int64_t* offs, const double* inv, int nstruct, double* span,
                     cudaStream_t st);
@@ -244,6 +247,7 @@ void atom_reduce(int n, int n_centres, const int* row_ptr, const int* col_ptr, c
                  const float* g, const double* ed, const int* species, const double* sigma, const double* mu,
                  bool want_forces, double* E_atom, double* F, double* Wat, const int* ei, const int* ej,
                  const Arch& a, cudaStream_t st);
+constexpr int kStructScratch = 12 * 1024;   // doubles of its scratch, zero before the first call
 void struct_reduce(int nstruct, const int64_t* offs, const double* E_atom, const double* Wat, const double* F,
                    bool want_w, double* E_out, double* W_out, int* d_err, double* scratch, int64_t n_atoms,
                    cudaStream_t st);
@@ -293,11 +297,11 @@ struct GenRowIO {
   int ldxs[kGenMaxLayers + 1] = {}, xs_off[kGenMaxLayers + 1] = {};
   const void* sbar[kGenMaxLayers + 1] = {};
   int ldsbar[kGenMaxLayers + 1] = {}, sbar_off[kGenMaxLayers + 1] = {};
-  // L = 1..nl, per atom [na][C][S]: Gamma^L (nu applied), Q^L, Gammabar^L
+  // L = 1..nl, per atom [na][S][C]: Gamma^L (nu applied), Q^L, Gammabar^L
   float* G[kGenMaxLayers + 1] = {};
   float* Q[kGenMaxLayers + 1] = {};
   float* Gb[kGenMaxLayers + 1] = {};
-  float* Qb = nullptr;                            // [na][C][S] scratch
+  float* Qb = nullptr;                            // [na][S][C] scratch
   float* Ybar = nullptr;                          // [Ec][S]
   // layer tensors W^k, k = 1..nl: their values (host memory) at the candidate nonzeros that
   // gen_pack_values lists, layers 1..nl concatenated; the kernels take them as launch parameters

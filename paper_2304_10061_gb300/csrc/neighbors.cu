@@ -26,51 +26,80 @@ __device__ __forceinline__ int floordiv(int a, int b) {
 }
 
 // ---------------------------------------------------------------------------
-// exclusive scan of int32 (out has n+1 entries; out[n] = total)
+// exclusive scan of int32 (out has n+1 entries; out[n] = total).  With `clear`
+// the input is zeroed as it is read (the counters the next build adds to).
 // ---------------------------------------------------------------------------
-constexpr int kScanBlock = 1024;   // elements per block (256 threads x 4)
+constexpr int kScanBlock = 1024;   // elements per block of the large scan (256 threads x 4)
 
-__global__ void scan_block_kernel(const int* __restrict__ in, int* __restrict__ out, int n,
-                                  int* __restrict__ block_sums) {
-  __shared__ int warp_tot[8];
-  const int base = blockIdx.x * kScanBlock;
-  const int t = threadIdx.x;
-  int v[4];
-  int s = 0;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    int idx = base + t * 4 + k;
-    v[k] = (idx < n && in) ? in[idx] : 0;
-    s += v[k];
-  }
-  // warp inclusive scan of per-thread sums
-  int lane = t & 31, w = t >> 5;
-  int x = s;
+__device__ __forceinline__ int warp_inclusive(int x, int lane) {
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    int y = __shfl_up_sync(0xffffffffu, x, o);
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
     if (lane >= o) x += y;
   }
+  return x;
+}
+
+// THREADS x PER elements by one block, thread t the elements [t PER, (t + 1) PER) of its tile
+// (PER a multiple of 4: 16-byte accesses; both arrays start 16-byte aligned at a tile's first element)
+template <int THREADS, int PER>
+__device__ __forceinline__ int block_scan_tile(int* __restrict__ in, int* __restrict__ out, int n, int base,
+                                               bool clear) {
+  constexpr int kWarps = THREADS / 32;
+  __shared__ int warp_tot[kWarps];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int b = base + t * PER;
+  int v[PER];
+#pragma unroll
+  for (int k = 0; k < PER; k += 4) {
+    if (b + k + 3 < n) {
+      const int4 x = *reinterpret_cast<const int4*>(in + b + k);
+      v[k] = x.x; v[k + 1] = x.y; v[k + 2] = x.z; v[k + 3] = x.w;
+      if (clear) *reinterpret_cast<int4*>(in + b + k) = make_int4(0, 0, 0, 0);
+    } else {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        v[k + q] = (b + k + q < n) ? in[b + k + q] : 0;
+        if (clear && b + k + q < n) in[b + k + q] = 0;
+      }
+    }
+  }
+  int s = 0;
+#pragma unroll
+  for (int k = 0; k < PER; ++k) s += v[k];
+  const int x = warp_inclusive(s, lane);
   if (lane == 31) warp_tot[w] = x;
   __syncthreads();
   if (w == 0) {
-    int wt = (lane < 8) ? warp_tot[lane] : 0;
-#pragma unroll
-    for (int o = 1; o < 8; o <<= 1) {
-      int y = __shfl_up_sync(0xffffffffu, wt, o);
-      if (lane >= o) wt += y;
-    }
-    if (lane < 8) warp_tot[lane] = wt;
+    const int wt = warp_inclusive(lane < kWarps ? warp_tot[lane] : 0, lane);
+    if (lane < kWarps) warp_tot[lane] = wt;
   }
   __syncthreads();
   int excl = x - s + (w > 0 ? warp_tot[w - 1] : 0);
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    int idx = base + t * 4 + k;
-    if (idx <= n) out[idx] = excl;
-    excl += v[k];
+  for (int k = 0; k < PER; k += 4) {
+    int4 y;
+    y.x = excl; y.y = y.x + v[k]; y.z = y.y + v[k + 1]; y.w = y.z + v[k + 2];
+    excl = y.w + v[k + 3];
+    if (b + k + 3 <= n) {
+      *reinterpret_cast<int4*>(out + b + k) = y;
+    } else {
+      if (b + k <= n) out[b + k] = y.x;
+      if (b + k + 1 <= n) out[b + k + 1] = y.y;
+      if (b + k + 2 <= n) out[b + k + 2] = y.z;
+    }
   }
-  if (t == 255 && block_sums) block_sums[blockIdx.x] = warp_tot[7];
+  return warp_tot[kWarps - 1];
+}
+
+template <int PER>
+__global__ void __launch_bounds__(1024) scan_one_kernel(int* in, int* out, int n, bool clear) {
+  block_scan_tile<1024, PER>(in, out, n, 0, clear);
+}
+
+__global__ void scan_block_kernel(int* in, int* out, int n, int* __restrict__ block_sums, bool clear) {
+  const int total = block_scan_tile<256, 4>(in, out, n, blockIdx.x * kScanBlock, clear);
+  if (threadIdx.x == 255) block_sums[blockIdx.x] = total;
 }
 
 __global__ void scan_add_kernel(int* __restrict__ out, int n, const int* __restrict__ block_pref) {
@@ -82,37 +111,46 @@ __global__ void scan_add_kernel(int* __restrict__ out, int n, const int* __restr
   }
 }
 
+// ints of a scan's block sums (or prefixes), rounded so that the next array stays 16-byte aligned
+static int scan_pitch(int nb) { return (nb + 1 + 3) / 4 * 4; }
+
 size_t scan_tmp_bytes(int n) {
   size_t total = 0;
   int m = n + 1;
   while (m > 1) {
     int nb = (m + kScanBlock - 1) / kScanBlock;
-    total += (size_t)(nb + 1) * 2 * sizeof(int) + 256;
+    total += (size_t)scan_pitch(nb) * 2 * sizeof(int) + 256;
     m = nb;
   }
   return total + 256;
 }
 
-// Scans in[0..n) into out[0..n] (out[n] = total); in == nullptr means zeros.
-static void scan_rec(const int* in, int* out, int n, char* tmp, cudaStream_t st) {
-  int nb = (n + 1 + kScanBlock - 1) / kScanBlock;
-  if (nb == 1) {
-    scan_block_kernel<<<1, 256, 0, st>>>(in, out, n, nullptr);
+// Scans in[0..n) into out[0..n] (out[n] = total).  Up to 32 x 1024 elements one block does it in
+// one launch (about 3 us against 6 for the three launches of the block-wise scan at 16k elements:
+// the launches are the time at these sizes); above, block sums, their scan, and an add.
+static void scan_rec(int* in, int* out, int n, char* tmp, bool clear, cudaStream_t st) {
+  if (n < 4 * 1024) {
+    scan_one_kernel<4><<<1, 1024, 0, st>>>(in, out, n, clear);
     return;
   }
+  if (n < 32 * 1024) {
+    scan_one_kernel<32><<<1, 1024, 0, st>>>(in, out, n, clear);
+    return;
+  }
+  const int nb = (n + 1 + kScanBlock - 1) / kScanBlock;
   int* sums = reinterpret_cast<int*>(tmp);
-  int* pref = sums + (nb + 1);
-  char* next = reinterpret_cast<char*>(pref + (nb + 1)) + 256;
-  scan_block_kernel<<<nb, 256, 0, st>>>(in, out, n, sums);
-  scan_rec(sums, pref, nb, next, st);
+  int* pref = sums + scan_pitch(nb);
+  char* next = reinterpret_cast<char*>(pref + scan_pitch(nb)) + 256;
+  scan_block_kernel<<<nb, 256, 0, st>>>(in, out, n, sums, clear);
+  scan_rec(sums, pref, nb, next, false, st);
   scan_add_kernel<<<nb, 256, 0, st>>>(out, n, pref);
 }
 
-void exclusive_scan_i32(const int* in, int* out, int n, int* d_total, void* tmp, size_t tmp_bytes,
-                        cudaStream_t st) {
-  (void)tmp_bytes;
-  scan_rec(in, out, n, reinterpret_cast<char*>(tmp), st);
-  if (d_total) cudaMemcpyAsync(d_total, out + n, sizeof(int), cudaMemcpyDeviceToDevice, st);
+int exclusive_scan_i32(int* in, int* out, int n, void* tmp, bool clear, cudaStream_t st) {
+  scan_rec(in, out, n, reinterpret_cast<char*>(tmp), clear, st);
+  int launches = 1;
+  for (int m = n; m >= 32 * 1024; m = (m + 1 + kScanBlock - 1) / kScanBlock) launches += 2;
+  return launches;
 }
 
 // ---------------------------------------------------------------------------
@@ -182,7 +220,7 @@ void nb_minmax_frac(const double* pos, int n, const double* inv, double* d_minma
 }
 
 __global__ void bin_kernel(const double* __restrict__ pos, int n, CellGrid g, int* __restrict__ cell_of,
-                           int* __restrict__ wrap, int* __restrict__ cell_count) {
+                           int* __restrict__ wrap, int* __restrict__ cell_count, int* __restrict__ cell_rank) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   double f[3];
@@ -206,54 +244,107 @@ __global__ void bin_kernel(const double* __restrict__ pos, int n, CellGrid g, in
   }
   int id = (c[0] * g.n[1] + c[1]) * g.n[2] + c[2];
   cell_of[i] = id;
-  atomicAdd(&cell_count[id], 1);
+  cell_rank[i] = atomicAdd(&cell_count[id], 1);
 }
 
-void nb_bin(const double* pos, int n, const CellGrid& g, int* cell_of, int* wrap, int* cell_count,
+void nb_bin(const double* pos, int n, const CellGrid& g, int* cell_of, int* wrap, int* cell_count, int* cell_rank,
             cudaStream_t st) {
   if (n <= 0) return;
-  bin_kernel<<<(n + 255) / 256, 256, 0, st>>>(pos, n, g, cell_of, wrap, cell_count);
+  bin_kernel<<<(n + 255) / 256, 256, 0, st>>>(pos, n, g, cell_of, wrap, cell_count, cell_rank);
 }
 
-__global__ void place_kernel(const int* __restrict__ cell_of, int n, const int* __restrict__ cell_start,
-                             int* __restrict__ cursor, int* __restrict__ sorted) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  int c = cell_of[i];
-  int k = atomicAdd(&cursor[c], 1);
-  sorted[cell_start[c] + k] = i;
+__global__ void place_kernel(const int* __restrict__ seg_of, const int* __restrict__ rank, int n,
+                             const int* __restrict__ start, int* __restrict__ sorted) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) sorted[start[seg_of[i]] + rank[i]] = i;
 }
 
-void nb_place(const int* cell_of, int n, const int* cell_start, int* cell_cursor, int* sorted,
-              cudaStream_t st) {
+void nb_place(const int* seg_of, const int* rank, int n, const int* start, int* sorted, cudaStream_t st) {
   if (n <= 0) return;
-  place_kernel<<<(n + 255) / 256, 256, 0, st>>>(cell_of, n, cell_start, cell_cursor, sorted);
+  place_kernel<<<(n + 255) / 256, 256, 0, st>>>(seg_of, rank, n, start, sorted);
 }
 
-// insertion sort of each segment [start[s], start[s+1]) (segments are short)
-__global__ void sort_segments_kernel(const int* __restrict__ start, int nseg, int* __restrict__ v) {
-  int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= nseg) return;
-  int b = start[s], e = start[s + 1];
-  for (int x = b + 1; x < e; ++x) {
-    int key = v[x];
-    int y = x - 1;
-    while (y >= b && v[y] > key) {
-      v[y + 1] = v[y];
-      --y;
+// Sort each segment [start[s], start[s+1]) of distinct values: G lanes per segment hold up to 4 G
+// values in registers and each value's rank is the number of smaller ones (a broadcast per value),
+// so a segment takes a few dependent loads instead of an insertion sort's chain through memory.
+// Longer segments (never met at liquid densities) are insertion-sorted by one lane.
+// done(place, value) is called for every element of the segment.
+template <int G, int K, typename Done>
+__device__ __forceinline__ void sort_in_registers(int b, int len, int* __restrict__ v, unsigned mask, Done&& done) {
+  const int lane = threadIdx.x & (G - 1);
+  int x[K], r[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    x[k] = (k * G + lane < len) ? v[b + k * G + lane] : 0x7fffffff;
+    r[k] = 0;
+  }
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int m = min(G, len - k * G);
+    for (int q = 0; q < m; ++q) {
+      const int y = __shfl_sync(mask, x[k], q, G);
+#pragma unroll
+      for (int p = 0; p < K; ++p) r[p] += (y < x[p]) ? 1 : 0;
     }
-    v[y + 1] = key;
+  }
+#pragma unroll
+  for (int k = 0; k < K; ++k)
+    if (k * G + lane < len) {
+      v[b + r[k]] = x[k];
+      done(b + r[k], x[k]);
+    }
+}
+
+template <int G, typename Done>
+__device__ __forceinline__ void sort_segment(int b, int len, int* __restrict__ v, Done&& done) {
+  const int lane = threadIdx.x & (G - 1);
+  const unsigned mask = ((1u << G) - 1u) << (threadIdx.x & 31 & ~(G - 1));
+  if (len <= G) {
+    sort_in_registers<G, 1>(b, len, v, mask, done);
+  } else if (len <= 2 * G) {
+    sort_in_registers<G, 2>(b, len, v, mask, done);
+  } else if (len <= 4 * G) {
+    sort_in_registers<G, 4>(b, len, v, mask, done);
+  } else {
+    if (lane == 0)
+      for (int p = b + 1; p < b + len; ++p) {
+        const int key = v[p];
+        int y = p - 1;
+        while (y >= b && v[y] > key) {
+          v[y + 1] = v[y];
+          --y;
+        }
+        v[y + 1] = key;
+      }
+    __syncwarp(mask);
+    for (int p = lane; p < len; p += G) done(b + p, v[b + p]);
   }
 }
 
-void nb_sort_cells(const int* cell_start, int n_cells, int* sorted, cudaStream_t st) {
-  if (n_cells <= 0) return;
-  sort_segments_kernel<<<(n_cells + 255) / 256, 256, 0, st>>>(cell_start, n_cells, sorted);
+// 16 lanes per column (about 25 edges at the density of water and a cutoff of 4 Angstrom)
+__global__ void __launch_bounds__(256) sort_columns_kernel(const int* __restrict__ start, int n, int* __restrict__ v) {
+  const int s = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 4);
+  if (s >= n) return;
+  const int b = start[s];
+  sort_segment<16>(b, start[s + 1] - b, v, [](int, int) {});
+}
+
+// Arrival order of every edge in its column, as a pass of its own: at large sizes the atomics cost
+// the fill pass more than they cost here (1,048,576 atoms: fill 2.51 -> 3.09 ms with them).
+__global__ void __launch_bounds__(256) col_rank_kernel(const int* __restrict__ ej, int E, int* __restrict__ col_count,
+                                                       int* __restrict__ col_rank) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < E) col_rank[e] = atomicAdd(&col_count[ej[e]], 1);
+}
+
+void nb_col_rank(const int* ej, int E, int* col_count, int* col_rank, cudaStream_t st) {
+  if (E <= 0) return;
+  col_rank_kernel<<<(E + 255) / 256, 256, 0, st>>>(ej, E, col_count, col_rank);
 }
 
 void nb_sort_columns(const int* col_ptr, int n, int* col_edge, cudaStream_t st) {
   if (n <= 0) return;
-  sort_segments_kernel<<<(n + 255) / 256, 256, 0, st>>>(col_ptr, n, col_edge);
+  sort_columns_kernel<<<(unsigned)(((int64_t)n * 16 + 255) / 256), 256, 0, st>>>(col_ptr, n, col_edge);
 }
 
 // ---------------------------------------------------------------------------
@@ -288,7 +379,8 @@ __global__ void skin_filter_kernel(const double* __restrict__ pos, int n, const 
                                    const int* __restrict__ sk_S, double rc2, const double* __restrict__ pair_rc2,
                                    const int* __restrict__ species, int ns, int* __restrict__ count,
                                    const int* __restrict__ row_ptr, int* __restrict__ ej, int* __restrict__ ei,
-                                   int* __restrict__ eS, double* __restrict__ ed) {
+                                   int* __restrict__ eS, double* __restrict__ ed, int* __restrict__ col_count,
+                                   int* __restrict__ col_rank) {
   const int lane = threadIdx.x & 31;
   const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (i >= n) return;
@@ -314,6 +406,7 @@ __global__ void skin_filter_kernel(const double* __restrict__ pos, int n, const 
     const unsigned m = __ballot_sync(0xffffffffu, keep);
     if (fill && keep) {
       const int o = out + __popc(m & ((1u << lane) - 1u));
+      col_rank[o] = atomicAdd(&col_count[j], 1);
       ej[o] = j;
       ei[o] = i;
       eS[3 * (size_t)o] = S0; eS[3 * (size_t)o + 1] = S1; eS[3 * (size_t)o + 2] = S2;
@@ -326,15 +419,16 @@ __global__ void skin_filter_kernel(const double* __restrict__ pos, int n, const 
 
 void nb_skin_filter(bool fill, const double* pos, int n, const double* d_cell, const int* sk_row, const int* sk_j,
                     const int* sk_S, double rc2, const double* pair_rc2, const int* species, int ns, int* count,
-                    const int* row_ptr, int* ej, int* ei, int* eS, double* ed, cudaStream_t st) {
+                    const int* row_ptr, int* ej, int* ei, int* eS, double* ed, int* col_count, int* col_rank,
+                    cudaStream_t st) {
   if (n <= 0) return;
   const int threads = 256, blocks = (int)(((int64_t)n * 32 + threads - 1) / threads);
   if (fill)
     skin_filter_kernel<true><<<blocks, threads, 0, st>>>(pos, n, d_cell, sk_row, sk_j, sk_S, rc2, pair_rc2, species,
-                                                         ns, count, row_ptr, ej, ei, eS, ed);
+                                                         ns, count, row_ptr, ej, ei, eS, ed, col_count, col_rank);
   else
     skin_filter_kernel<false><<<blocks, threads, 0, st>>>(pos, n, d_cell, sk_row, sk_j, sk_S, rc2, pair_rc2,
-                                                          species, ns, count, row_ptr, ej, ei, eS, ed);
+                                                          species, ns, count, row_ptr, ej, ei, eS, ed, col_count, col_rank);
 }
 
 // Largest squared displacement of any atom since the reference positions, as
@@ -360,27 +454,41 @@ void nb_max_disp2(const double* pos, const double* ref, int n, unsigned long lon
   max_disp2_kernel<<<(n + 255) / 256, 256, 0, st>>>(pos, ref, n, out);
 }
 
-// Wrapped positions pw = pos - wrap . cell in cell-sorted order (pos4[s] and
-// pw[3 s ..] belong to atom sorted[s]): float32 for the prefilter, float64 for
-// the displacements of accepted edges.
-__global__ void pos4_kernel(const double* __restrict__ pos, const int* __restrict__ species, int n, CellGrid g,
-                            const int* __restrict__ wrap, const int* __restrict__ sorted,
-                            float4* __restrict__ pos4, double* __restrict__ pw, int4* __restrict__ wraps) {
-  int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= n) return;
-  const int j = sorted[s];
-  double p[3];
+// The cell lists in atom order, and with them the wrapped positions pw = pos - wrap . cell in
+// cell-sorted order (pos4[s] and pw[3 s ..] belong to atom sorted[s]): float32 for the prefilter,
+// float64 for the displacements of accepted edges.  Eight lanes per cell (about 6.4 atoms at the
+// density of water).
+__global__ void __launch_bounds__(256) sort_cells_kernel(const double* __restrict__ pos,
+                                                         const int* __restrict__ species, CellGrid g, int n_cells,
+                                                         const int* __restrict__ cell_start,
+                                                         const int* __restrict__ wrap, int* __restrict__ sorted,
+                                                         float4* __restrict__ pos4, double* __restrict__ pw,
+                                                         int4* __restrict__ wraps) {
+  const int c = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3);
+  if (c >= n_cells) return;
+  const int b = cell_start[c];
+  sort_segment<8>(b, cell_start[c + 1] - b, sorted, [&](int s, int j) {
+    double p[3];
+    const int wj[3] = {wrap[3 * (size_t)j], wrap[3 * (size_t)j + 1], wrap[3 * (size_t)j + 2]};
 #pragma unroll
-  for (int x = 0; x < 3; ++x) {
-    p[x] = pos[3 * (size_t)j + x];
+    for (int x = 0; x < 3; ++x) {
+      p[x] = pos[3 * (size_t)j + x];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) p[x] -= (double)wrap[3 * (size_t)j + k] * g.cell[k * 3 + x];
-  }
-  pos4[s] = make_float4((float)p[0], (float)p[1], (float)p[2], __int_as_float(species[j]));
-  pw[3 * (size_t)s] = p[0];
-  pw[3 * (size_t)s + 1] = p[1];
-  pw[3 * (size_t)s + 2] = p[2];
-  wraps[s] = make_int4(wrap[3 * (size_t)j], wrap[3 * (size_t)j + 1], wrap[3 * (size_t)j + 2], 0);
+      for (int k = 0; k < 3; ++k) p[x] -= (double)wj[k] * g.cell[k * 3 + x];
+    }
+    pos4[s] = make_float4((float)p[0], (float)p[1], (float)p[2], __int_as_float(species[j]));
+    pw[3 * (size_t)s] = p[0];
+    pw[3 * (size_t)s + 1] = p[1];
+    pw[3 * (size_t)s + 2] = p[2];
+    wraps[s] = make_int4(wj[0], wj[1], wj[2], 0);
+  });
+}
+
+void nb_sort_cells(const double* pos, const int* species, const CellGrid& g, int n_cells, const int* cell_start,
+                   const int* wrap, int* sorted, float4* pos4, double* pw, int4* wraps, cudaStream_t st) {
+  if (n_cells <= 0) return;
+  sort_cells_kernel<<<(unsigned)(((int64_t)n_cells * 8 + 255) / 256), 256, 0, st>>>(pos, species, g, n_cells, cell_start,
+                                                                                    wrap, sorted, pos4, pw, wraps);
 }
 
 // Neighbour search.  A float32 prefilter on the wrapped positions decides
@@ -392,14 +500,12 @@ __global__ void pos4_kernel(const double* __restrict__ pos, const int* __restric
 // from the exact test inside the band, else (pw_j + q . cell) - pw_i from the
 // float64 wrapped positions (the same vector up to float64 rounding; the
 // edge's image shift is S = q - w_j + w_i).
-// The fill pass writes through shared memory: a lane records each accepted
-// candidate of its row (cell-order index s, image q, whether it took the exact
-// test) in its warp's staging area, then the warp writes the 32 rows one after
-// another with its lanes on consecutive edges of a row, so each store covers
-// consecutive addresses (a row per lane would scatter every store over 32
-// rows).  Edges past kFillStage in a row are written by their lane directly.
 constexpr int kSearchThreads = 128;
-constexpr int kFillStage = 32;
+// Up to this many atoms a warp per centre, above it a thread per centre (both list the same edges in
+// the same order).  Count and fill pass, us, warp / thread: 64 atoms 13 + 13 / 37 + 77; 3,072 atoms
+// 19 + 22 / 81 + 124; 23,552 atoms 49 + 79 / 81 + 143; 65,536 atoms 104 + 196 / 93 + 212; 1,048,576 atoms
+// 1,553 + 3,298 / 804 + 2,517 (the warp form issues more instructions per candidate).
+constexpr int kSearchWarpAtoms = 65536;
 
 // The displacement of pair_test (the same float64 operations in the same order).
 __device__ __forceinline__ void pair_disp(const double* __restrict__ pi, const double* __restrict__ pj,
@@ -413,14 +519,212 @@ __device__ __forceinline__ void pair_disp(const double* __restrict__ pi, const d
   }
 }
 
-// image q (three signed 9-bit fields) and the exact-test flag of a staged edge
+// image q (three signed 10-bit fields) and the exact-test flag of a staged edge
 __device__ __forceinline__ int pack_q(int q0, int q1, int q2, bool exact) {
-  return (q0 & 511) | ((q1 & 511) << 9) | ((q2 & 511) << 18) | (exact ? (1 << 27) : 0);
+  return (q0 & 1023) | ((q1 & 1023) << 10) | ((q2 & 1023) << 20) | (exact ? (1 << 30) : 0);
 }
-__device__ __forceinline__ int unpack_q(int v, int f) { return ((v >> (9 * f)) << 23) >> 23; }
+__device__ __forceinline__ int unpack_q(int v, int f) { return (int)((unsigned)v << (22 - 10 * f)) >> 22; }
+
+// One warp per centre atom (cell order).  Up to 32 cells of the stencil at a
+// time: lane c looks up cell c's range and image offset, a warp scan of the
+// range lengths flattens their atoms into one candidate sequence (stencil
+// order, then cell order), and the lanes test 32 consecutive candidates per
+// round; a ballot places the accepted ones, so rows keep that order.  Accepted
+// candidates are compacted into a 64-entry stage in shared memory and written
+// 32 at a time with lanes on consecutive edges: the float64 displacements (a
+// slow unit on this part) run on full warps and the stores cover consecutive
+// addresses.
+// Bound: latency of the dependent loads (cell ranges, then positions), and at
+// large sizes instruction issue.  Why a warp per atom: a thread per atom walks
+// its ~190 candidates one after another.
+struct SearchCell {
+  float ox, oy, oz;   // image offset of the cell minus the centre's position (float32)
+  int q;              // packed image
+};
 
 template <bool fill>
 __global__ void __launch_bounds__(kSearchThreads) search_kernel(
+    const double* __restrict__ pos, int n, CellGrid g, const int* __restrict__ cell_of,
+    const int4* __restrict__ wraps, const int* __restrict__ cell_start, const int* __restrict__ sorted,
+    const float4* __restrict__ pos4, const double* __restrict__ pw, double rc2, float band,
+    const double* __restrict__ pair_rc2, int ns, int* __restrict__ count, const int* __restrict__ row_ptr,
+    int* __restrict__ ej, int* __restrict__ ei, int* __restrict__ eS, double* __restrict__ ed,
+    int* __restrict__ col_count, int* __restrict__ col_rank, int* __restrict__ d_err) {
+  constexpr int kWarps = kSearchThreads / 32;
+  __shared__ SearchCell s_cell[kWarps][32];
+  __shared__ int s_pref[kWarps][32];    // candidates before the cell
+  __shared__ int s_first[kWarps][32];   // cell_start - candidates before it
+  __shared__ int2 s_stage[kWarps][fill ? 64 : 1];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int t = blockIdx.x * kWarps + w;
+  if (t >= n) return;
+  const int i = sorted[t];
+  if (i >= g.n_centres) {   // ghost atoms (spatial decomposition) are neighbours only, never centres
+    if (!fill && lane == 0) count[i] = 0;
+    return;
+  }
+  const int ci = cell_of[i];
+  const int4 wi = wraps[t];
+  const float4 pi4 = pos4[t];
+  const double pi[3] = {pos[3 * (size_t)i], pos[3 * (size_t)i + 1], pos[3 * (size_t)i + 2]};
+  const int c2 = ci % g.n[2], c1 = (ci / g.n[2]) % g.n[1], c0 = ci / (g.n[2] * g.n[1]);
+  const float rc2f = (float)rc2;
+  const float lo2 = rc2f - band, hi2 = rc2f + band;
+  // per-ordered-pair cutoffs: row of the centre's species (the band of the largest
+  // cutoff bounds the float32 error of every smaller one)
+  const double* prow = pair_rc2 ? pair_rc2 + (size_t)__float_as_int(pi4.w) * ns : nullptr;
+  const int base = fill ? row_ptr[i] : 0;
+  const int cap = fill ? (row_ptr[i + 1] - base) : 0;
+  int k = 0;         // accepted so far
+  int nst = 0;       // staged, not yet written (they are edges [k - nst, k))
+  // the first m (<= 32) staged edges, to base + k0 + lane
+  auto write = [&](int k0, int m) {
+    if (lane < m && k0 + lane < cap) {
+      const int2 en = s_stage[w][lane];
+      const int s = en.x;
+      const int q0 = unpack_q(en.y, 0), q1 = unpack_q(en.y, 1), q2 = unpack_q(en.y, 2);
+      const int j = sorted[s];
+      const int4 wj = wraps[s];
+      const int S0 = g.pbc[0] ? q0 - wj.x + wi.x : 0;
+      const int S1 = g.pbc[1] ? q1 - wj.y + wi.y : 0;
+      const int S2 = g.pbc[2] ? q2 - wj.z + wi.z : 0;
+      double d[3];
+      if ((en.y >> 30) & 1) {
+        pair_disp(pi, pos + 3 * (size_t)j, g.cell, S0, S1, S2, d);
+      } else {
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+          const double qoff = (q0 | q1 | q2) ? ((double)q0 * g.cell[x] + (double)q1 * g.cell[3 + x]) +
+                                                   (double)q2 * g.cell[6 + x]
+                                             : 0.0;
+          d[x] = (pw[3 * (size_t)s + x] + qoff) - pw[3 * (size_t)t + x];
+        }
+      }
+      const size_t o = (size_t)base + k0 + lane;
+      col_rank[o] = atomicAdd(&col_count[j], 1);
+      ej[o] = j;
+      ei[o] = i;
+      eS[3 * o] = S0; eS[3 * o + 1] = S1; eS[3 * o + 2] = S2;
+      ed[3 * o] = d[0]; ed[3 * o + 1] = d[1]; ed[3 * o + 2] = d[2];
+    }
+  };
+  const int n1 = 2 * g.R[1] + 1, n2 = 2 * g.R[2] + 1;
+  const int ncell = (2 * g.R[0] + 1) * n1 * n2;
+  for (int m0 = 0; m0 < ncell; m0 += 32) {
+    const int m = m0 + lane;
+    int b = 0, cnt = 0;
+    SearchCell sc = {0.f, 0.f, 0.f, 0};
+    if (m < ncell) {
+      int cc[3] = {c0 + m / (n1 * n2) - g.R[0], c1 + (m / n2) % n1 - g.R[1], c2 + m % n2 - g.R[2]};
+      int q[3] = {0, 0, 0};
+      bool in = true;
+#pragma unroll
+      for (int x = 0; x < 3; ++x) {
+        if (g.pbc[x]) {
+          q[x] = floordiv(cc[x], g.n[x]);
+          cc[x] -= q[x] * g.n[x];
+        } else if (cc[x] < 0 || cc[x] >= g.n[x]) {
+          in = false;
+        }
+      }
+      if (in) {
+        const int cell = (cc[0] * g.n[1] + cc[1]) * g.n[2] + cc[2];
+        b = cell_start[cell];
+        cnt = cell_start[cell + 1] - b;
+        const float q0 = (float)q[0], q1 = (float)q[1], q2 = (float)q[2];
+        sc.ox = q0 * (float)g.cell[0] + q1 * (float)g.cell[3] + q2 * (float)g.cell[6] - pi4.x;
+        sc.oy = q0 * (float)g.cell[1] + q1 * (float)g.cell[4] + q2 * (float)g.cell[7] - pi4.y;
+        sc.oz = q0 * (float)g.cell[2] + q1 * (float)g.cell[5] + q2 * (float)g.cell[8] - pi4.z;
+        sc.q = pack_q(q[0], q[1], q[2], false);
+      }
+    }
+    int incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    __syncwarp();
+    s_cell[w][lane] = sc;
+    s_pref[w][lane] = incl - cnt;
+    s_first[w][lane] = b - (incl - cnt);
+    __syncwarp();
+    for (int r0 = 0; r0 < total; r0 += 32) {
+      const int r = r0 + lane;
+      bool keep = false;
+      int2 en = make_int2(0, 0);
+      if (r < total) {
+        int o = 0;   // the last cell with s_pref <= r
+#pragma unroll
+        for (int h = 16; h > 0; h >>= 1)
+          if (s_pref[w][o + h] <= r) o += h;
+        const SearchCell ce = s_cell[w][o];
+        const int s = s_first[w][o] + r;
+        const float4 pj = pos4[s];
+        const float dx = pj.x + ce.ox, dy = pj.y + ce.oy, dz = pj.z + ce.oz;
+        const float r2f = dx * dx + dy * dy + dz * dz;
+        double rc2p = rc2;
+        float lo2p = lo2, hi2p = hi2;
+        if (prow) {
+          rc2p = prow[__float_as_int(pj.w)];
+          const float rc2pf = (float)rc2p;
+          lo2p = rc2pf - band;
+          hi2p = fminf(hi2, rc2pf + band);
+        }
+        if (!(r2f > hi2p)) {
+          bool exact = r2f >= lo2p;
+          keep = true;
+          if (s == t || exact) {
+            const int4 wj = wraps[s];
+            const int S0 = g.pbc[0] ? unpack_q(ce.q, 0) - wj.x + wi.x : 0;
+            const int S1 = g.pbc[1] ? unpack_q(ce.q, 1) - wj.y + wi.y : 0;
+            const int S2 = g.pbc[2] ? unpack_q(ce.q, 2) - wj.z + wi.z : 0;
+            if (s == t && S0 == 0 && S1 == 0 && S2 == 0) keep = false;   // (s = t: j = i)
+            double d[3];
+            if (keep && exact) keep = pair_test(pi, pos + 3 * (size_t)sorted[s], g.cell, S0, S1, S2, rc2p, d);
+          }
+          en = make_int2(s, ce.q | (exact ? (1 << 30) : 0));
+        }
+      }
+      const unsigned mask = __ballot_sync(0xffffffffu, keep);
+      const int nk = __popc(mask);
+      if constexpr (fill) {
+        if (keep) s_stage[w][nst + __popc(mask & ((1u << lane) - 1u))] = en;
+        nst += nk;
+        if (nst >= 32) {
+          __syncwarp();
+          write(k + nk - nst, 32);
+          nst -= 32;
+          const int2 rest = s_stage[w][32 + lane];
+          __syncwarp();
+          s_stage[w][lane] = rest;
+          __syncwarp();
+        }
+      }
+      k += nk;
+    }
+  }
+  if constexpr (fill) {
+    __syncwarp();
+    write(k - nst, nst);
+    if (lane == 0 && k != cap) atomicOr(d_err, kErrNeighbor);
+  } else {
+    if (lane == 0) count[i] = k;
+  }
+}
+
+// One thread per centre atom, for systems that fill the GPU with threads: neighbouring lanes share
+// their stencil cells, so a candidate costs a warp a few instructions for 32 centres.  The fill pass
+// writes through shared memory: a lane records each accepted candidate of its row (cell-order index s,
+// image q, whether it took the exact test) in its warp's staging area, then the warp writes the 32 rows
+// one after another with its lanes on consecutive edges of a row, so each store covers consecutive
+// addresses (a row per lane would scatter every store over 32 rows).  Edges past kFillStage in a row
+// are written by their lane directly.
+constexpr int kFillStage = 32;
+
+template <bool fill>
+__global__ void __launch_bounds__(kSearchThreads) search_thread_kernel(
     const double* __restrict__ pos, int n, CellGrid g, const int* __restrict__ cell_of,
     const int4* __restrict__ wraps, const int* __restrict__ cell_start, const int* __restrict__ sorted,
     const float4* __restrict__ pos4, const double* __restrict__ pw, double rc2, float band,
@@ -555,7 +859,7 @@ __global__ void __launch_bounds__(kSearchThreads) search_kernel(
         const int2 en = stage[w0 + r][kk];
         const int s = en.x;
         const int q0 = unpack_q(en.y, 0), q1 = unpack_q(en.y, 1), q2 = unpack_q(en.y, 2);
-        const bool exact = (en.y >> 27) & 1;
+        const bool exact = (en.y >> 30) & 1;
         const int j = sorted[s];
         const int4 wj = wraps[s];
         const int S0 = g.pbc[0] ? q0 - wj.x + wx : 0;
@@ -583,23 +887,23 @@ __global__ void __launch_bounds__(kSearchThreads) search_kernel(
   }
 }
 
-void nb_pos4(const double* pos, const int* species, int n, const CellGrid& g, const int* wrap, const int* sorted,
-             float4* pos4, double* pw, int4* wraps, cudaStream_t st) {
-  if (n <= 0) return;
-  pos4_kernel<<<(n + 255) / 256, 256, 0, st>>>(pos, species, n, g, wrap, sorted, pos4, pw, wraps);
-}
-
-void nb_search(bool fill, const double* pos, int n, const CellGrid& g, const int* cell_of,
+bool nb_search(bool fill, const double* pos, int n, const CellGrid& g, const int* cell_of,
                const int4* wraps, const int* cell_start, const int* sorted, const float4* pos4, const double* pw,
                double rc2, float band, const double* pair_rc2, int ns, int* count, const int* row_ptr, int* ej,
-               int* ei, int* eS, double* ed, int* d_err, cudaStream_t st) {
-  if (n <= 0) return;
-  if (fill)
-    search_kernel<true><<<(n + kSearchThreads - 1) / kSearchThreads, kSearchThreads, 0, st>>>(pos, n, g, cell_of, wraps, cell_start, sorted, pos4, pw, rc2,
-                                                         band, pair_rc2, ns, count, row_ptr, ej, ei, eS, ed, d_err);
-  else
-    search_kernel<false><<<(n + kSearchThreads - 1) / kSearchThreads, kSearchThreads, 0, st>>>(pos, n, g, cell_of, wraps, cell_start, sorted, pos4, pw, rc2,
-                                                          band, pair_rc2, ns, count, row_ptr, ej, ei, eS, ed, d_err);
+               int* ei, int* eS, double* ed, int* col_count, int* col_rank, int* d_err, cudaStream_t st) {
+  if (n <= 0) return true;
+  if (n <= kSearchWarpAtoms) {
+    auto kernel = fill ? search_kernel<true> : search_kernel<false>;
+    kernel<<<(n + kSearchThreads / 32 - 1) / (kSearchThreads / 32), kSearchThreads, 0, st>>>(
+        pos, n, g, cell_of, wraps, cell_start, sorted, pos4, pw, rc2, band, pair_rc2, ns, count, row_ptr, ej, ei, eS, ed,
+        col_count, col_rank, d_err);
+    return true;
+  }
+  auto kernel = fill ? search_thread_kernel<true> : search_thread_kernel<false>;
+  kernel<<<(n + kSearchThreads - 1) / kSearchThreads, kSearchThreads, 0, st>>>(
+      pos, n, g, cell_of, wraps, cell_start, sorted, pos4, pw, rc2, band, pair_rc2, ns, count, row_ptr, ej, ei, eS, ed,
+      d_err);
+  return false;
 }
 
 // ---------------------------------------------------------------------------
@@ -613,7 +917,8 @@ __global__ void brute_batched_kernel(bool fill, const double* __restrict__ pos,
                                      const int* __restrict__ atom_struct, int n,
                                      int* __restrict__ count, const int* __restrict__ row_ptr,
                                      int* __restrict__ ej, int* __restrict__ ei, int* __restrict__ eS,
-                                     double* __restrict__ ed, int* __restrict__ d_err) {
+                                     double* __restrict__ ed, int* __restrict__ col_count,
+                                     int* __restrict__ col_rank, int* __restrict__ d_err) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int b = atom_struct[i];
@@ -638,6 +943,7 @@ __global__ void brute_batched_kernel(bool fill, const double* __restrict__ pos,
           if (!pair_test(pi, pos + 3 * (size_t)j, cell, S0, S1, S2, rc2p, d)) continue;
           if (fill && k < cap) {
             size_t o = (size_t)base + k;
+            col_rank[o] = atomicAdd(&col_count[j], 1);
             ej[o] = j;
             ei[o] = i;
             eS[3 * o] = S0; eS[3 * o + 1] = S1; eS[3 * o + 2] = S2;
@@ -657,12 +963,12 @@ void nb_bruteforce_batched(bool fill, const double* pos, const int64_t* offs, in
                            const double* cells, const int* pbc, const int* nimg, double rc2,
                            const int* species, const double* pair_rc2, int ns,
                            const int* atom_struct, int n, int* count, const int* row_ptr, int* ej,
-                           int* ei, int* eS, double* ed, int* d_err, cudaStream_t st) {
+                           int* ei, int* eS, double* ed, int* col_count, int* col_rank, int* d_err, cudaStream_t st) {
   (void)nstruct;
   if (n <= 0) return;
   brute_batched_kernel<<<(n + 127) / 128, 128, 0, st>>>(fill, pos, offs, cells, pbc, nimg, rc2, species, pair_rc2,
                                                         ns, atom_struct, n, count, row_ptr, ej, ei, eS, ed,
-                                                        d_err);
+                                                        col_count, col_rank, d_err);
 }
 
 // Per structure: spread (max - min) of the fractional coordinates, so the
@@ -697,35 +1003,6 @@ void nb_struct_span(const double* pos, const int64_t* offs, const double* inv, i
                     cudaStream_t st) {
   if (nstruct <= 0) return;
   struct_span_kernel<<<nstruct, 128, 0, st>>>(pos, offs, inv, span);
-}
-
-// ---------------------------------------------------------------------------
-// CSC index: edges grouped by neighbour atom j
-// ---------------------------------------------------------------------------
-__global__ void col_count_kernel(const int* __restrict__ ej, int E, int* __restrict__ col_count) {
-  int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < E) atomicAdd(&col_count[ej[e]], 1);
-}
-
-void nb_columns(const int* ej, int E, int n, int* col_count, cudaStream_t st) {
-  (void)n;
-  if (E <= 0) return;
-  col_count_kernel<<<(E + 255) / 256, 256, 0, st>>>(ej, E, col_count);
-}
-
-__global__ void col_fill_kernel(const int* __restrict__ ej, int E, const int* __restrict__ col_ptr,
-                                int* __restrict__ cursor, int* __restrict__ col_edge) {
-  int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= E) return;
-  int j = ej[e];
-  int k = atomicAdd(&cursor[j], 1);
-  col_edge[col_ptr[j] + k] = e;
-}
-
-void nb_fill_columns(const int* ej, int E, const int* col_ptr, int* cursor, int* col_edge,
-                     cudaStream_t st) {
-  if (E <= 0) return;
-  col_fill_kernel<<<(E + 255) / 256, 256, 0, st>>>(ej, E, col_ptr, cursor, col_edge);
 }
 
 }  // namespace alg
