@@ -24,8 +24,14 @@
 // wbar^L is written then; w^0bar and Ybar, sums over all layers, are formed
 // once, after layer 1.
 //
-// Layout: per atom [atom][channel][S] float32; per edge the activation-type
-// arrays of the MLP side (w, s, sbar, wbar) and float32 Y / Ybar / w^0bar.
+// Layout: per atom [atom][S][channel] float32, so that a warp on 32 consecutive
+// channels reads and writes each component as one 128-byte line (with the
+// channel outside, each of a thread's S accesses touched 32 lines); per edge the
+// activation-type arrays of the MLP side (w, s, sbar, wbar) and float32 Y /
+// Ybar / w^0bar.  With this layout and the asynchronous rings below, all row
+// kernels of the forward pass take 4.37 ms (7.18 with the channel outside and
+// loads through registers) and of the adjoint 10.3 ms (14.8) at 65,536 atoms,
+// three layers, l_max 3, 128 channels in bf16.
 // Row kernels: one warp per centre atom with C / 32 channels per lane (the
 // environment sums, s, Qbar, the upper layers' wbar: a lane's harmonics loads
 // serve all its channels), or, for the per-edge adjoint that combines every
@@ -132,6 +138,66 @@ __device__ __forceinline__ float warp_sum16(float (&v)[16]) {
     }
   }
   return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+// ---------------------------------------------------------------------------
+// Asynchronous copies of an edge's rows into shared memory, so that a warp has
+// several edges' loads in flight without holding them in registers (the row
+// kernels keep 64 to 100 floats of per-channel state, which leaves 8 to 16
+// warps per SM: with one or two edges in flight each they waited on latency).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// `bytes` (even) contiguous bytes at src to dst (16-byte aligned) by the warp; `al` = the low four bits of src and
+// bytes or'ed: 16-byte copies when they are zero, else 4-byte ones, else plain 2-byte copies (latent
+// widths that are odd in bf16)
+__device__ __forceinline__ void warp_copy(unsigned char* dst, const unsigned char* src, int bytes, unsigned al) {
+  const int lane = threadIdx.x & 31;
+  if (al == 0) {
+    for (int k = lane * 16; k < bytes; k += 512) cp_async16(dst + k, src + k);
+  } else if ((al & 3) == 0) {
+    for (int k = lane * 4; k < bytes; k += 128) cp_async4(dst + k, src + k);
+  } else {
+    for (int k = lane * 2; k < bytes; k += 64)
+      *reinterpret_cast<unsigned short*>(dst + k) = *reinterpret_cast<const unsigned short*>(src + k);
+  }
+}
+
+constexpr int kRing = 4;   // edges in flight per warp (stages of its shared-memory ring)
+
+__host__ __device__ constexpr int round16(int x) { return (x + 15) / 16 * 16; }
+
+// A warp's ring over its row's edges.  copy(e, slot) queues edge e's rows into a slot; for each edge
+// in order, use(e, slot) runs once the edge's rows have arrived, with the next kRing - 1 edges queued.
+template <int STAGE, typename Copy, typename Use>
+__device__ __forceinline__ void ring_over(unsigned char* ring, int rb, int re, Copy&& copy, Use&& use) {
+#pragma unroll
+  for (int p = 0; p < kRing - 1; ++p) {
+    if (rb + p < re) copy(rb + p, ring + p * STAGE);
+    cp_async_commit();
+  }
+  int slot = 0;
+  for (int e = rb; e < re; ++e) {
+    cp_async_wait<kRing - 2>();
+    __syncwarp();   // every lane's copies of edge e have landed, and no lane still reads the slot before it
+    const int nslot = (slot + kRing - 1) % kRing;
+    if (e + kRing - 1 < re) copy(e + kRing - 1, ring + nslot * STAGE);
+    cp_async_commit();
+    use(e, ring + slot * STAGE);
+    slot = (slot + 1) % kRing;
+  }
 }
 
 constexpr int kChainThreads = 128;   // (atom, channel) pairs per block of the chain kernels
@@ -324,12 +390,12 @@ __global__ void __launch_bounds__(kChainThreads) gen_chain_fwd_kernel(GenRowIO i
   constexpr int S = (LMAX + 1) * (LMAX + 1);
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= io.na * io.C) return;
-  const size_t o = (size_t)t * S;
+  const size_t o = (size_t)(t / io.C) * S * io.C + t % io.C;
   float G[L][S];
 #pragma unroll
   for (int k = 0; k < L; ++k)
 #pragma unroll
-    for (int b = 0; b < S; ++b) G[k][b] = io.G[k + 1][o + b];
+    for (int b = 0; b < S; ++b) G[k][b] = io.G[k + 1][o + (size_t)b * io.C];
   float x[kGenMaxD], y[kGenMaxD];
   chain_mv<LMAX, NL, L, true>(w.v, G[L - 1], x, y);
   if constexpr (L >= 2) {
@@ -341,7 +407,7 @@ __global__ void __launch_bounds__(kChainThreads) gen_chain_fwd_kernel(GenRowIO i
   const float* q = (L == 2) ? x : y;
   float* out = io.Q[L] + o;
 #pragma unroll
-  for (int a = 0; a < S; ++a) out[a] = q[a];
+  for (int a = 0; a < S; ++a) out[(size_t)a * io.C] = q[a];
 }
 
 // Gb[b] += sum over layer K's candidates of W^K[a][b][c] rb[a] r[c] (r = e_0 when E0) and, unless
@@ -369,18 +435,18 @@ __device__ __forceinline__ void chain_adj(const float* v, const float (&G)[D], c
   }, std::make_integer_sequence<int, P::n>{});
 }
 
-// Back along the chain of Q^L: Gammabar^k += ..., k = 1..L
+// Back along the chain of Q^L: Gammabar^k += ..., k = 1..L (the last layer, which comes first, writes them)
 template <int LMAX, int NL, int L>
 __global__ void __launch_bounds__(kChainThreads) gen_chain_bwd_kernel(GenRowIO io, const __grid_constant__ GenVals<LMAX, NL> w) {
   constexpr int S = (LMAX + 1) * (LMAX + 1);
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= io.na * io.C) return;
-  const size_t o = (size_t)t * S;
+  const size_t o = (size_t)(t / io.C) * S * io.C + t % io.C;
   float G[L][S];
 #pragma unroll
   for (int k = 0; k < L; ++k)
 #pragma unroll
-    for (int b = 0; b < S; ++b) G[k][b] = io.G[k + 1][o + b];
+    for (int b = 0; b < S; ++b) G[k][b] = io.G[k + 1][o + (size_t)b * io.C];
   // r_{L+1} = e_0, r_k = M^k r_{k+1}: r[k - 2] holds r_k for k = 2..L
   float r[L > 1 ? L - 1 : 1][kGenMaxD];
   float dummy[kGenMaxD];
@@ -388,12 +454,15 @@ __global__ void __launch_bounds__(kChainThreads) gen_chain_bwd_kernel(GenRowIO i
   if constexpr (L >= 3) chain_mv<LMAX, NL, L - 1, false>(w.v, G[L - 2], r[L - 2], r[L - 3]);
   float rb[kGenMaxD], nb[kGenMaxD], gb[S];
 #pragma unroll
-  for (int a = 0; a < S; ++a) rb[a] = io.Qb[o + a];
+  for (int a = 0; a < S; ++a) rb[a] = io.Qb[o + (size_t)a * io.C];
   // k = 1 .. L: Gammabar^k, and rbar_{k+1} for k < L
   auto flush = [&](int k) {
     float* g = io.Gb[k] + o;
 #pragma unroll
-    for (int b = 0; b < S; ++b) g[b] += gb[b];
+    for (int b = 0; b < S; ++b) {
+      float* p = g + (size_t)b * io.C;
+      *p = (L == NL) ? gb[b] : *p + gb[b];
+    }
   };
   if constexpr (L == 1) {
     chain_adj<LMAX, NL, 1, true, false>(w.v, G[0], rb, dummy, gb, nb);
@@ -432,15 +501,42 @@ __global__ void __launch_bounds__(kMaxChannels) gen_edge_final_kernel(GenRowIO i
   const int rb = io.row_ptr[io.a0 + ia] - io.e0, re = io.row_ptr[io.a0 + ia + 1] - io.e0;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = (int)(blockDim.x >> 5);
   float q[NL][S], gb[NL][S];
-  const size_t o = ((size_t)ia * io.C + (act ? u : 0)) * S;
+  const size_t o = (size_t)ia * S * io.C + (act ? u : 0);
 #pragma unroll
   for (int L = 0; L < NL; ++L)
 #pragma unroll
     for (int a = 0; a < S; ++a) {
-      q[L][a] = act ? io.Q[L + 1][o + a] : 0.0f;
-      gb[L][a] = act ? io.nu * io.Gb[L + 1][o + a] : 0.0f;
+      q[L][a] = act ? io.Q[L + 1][o + (size_t)a * io.C] : 0.0f;
+      gb[L][a] = act ? io.nu * io.Gb[L + 1][o + (size_t)a * io.C] : 0.0f;
     }
-  const T* w0 = reinterpret_cast<const T*>(io.w[0]);
+  // the warp's ring: per edge its 32 channels of w^0 .. w^NL, of sbar^1 .. sbar^NL, and Y
+  constexpr int kW = 32 * LM * (int)sizeof(T), kSb = 32 * (int)sizeof(T);
+  constexpr int kOffS = (NL + 1) * kW, kOffY = kOffS + NL * kSb, kStage = round16(kOffY + S * 4);
+  __shared__ __align__(16) unsigned char rings[kMaxChannels / 32][kRing * kStage];
+  const int nch = min(32, io.C);   // channels of a warp
+  const unsigned char* wsrc[NL + 1];
+  const unsigned char* ssrc[NL];
+  unsigned sal[NL];
+#pragma unroll
+  for (int L = 0; L <= NL; ++L)
+    wsrc[L] = reinterpret_cast<const unsigned char*>(reinterpret_cast<const T*>(io.w[L]) + io.wcol[L] + wid * 32 * LM);
+#pragma unroll
+  for (int L = 0; L < NL; ++L) {
+    ssrc[L] = reinterpret_cast<const unsigned char*>(reinterpret_cast<const T*>(io.sbar[L + 1]) + io.sbar_off[L + 1] +
+                                                     wid * 32);
+    sal[L] = (unsigned)((reinterpret_cast<uintptr_t>(ssrc[L]) | (io.ldsbar[L + 1] * sizeof(T)) | (nch * sizeof(T))) & 15);
+  }
+  auto copy = [&](int e, unsigned char* st) {
+    // the w rows are 16-byte aligned (pitches of 8 elements, columns at multiples of 8 (l_max + 1))
+#pragma unroll
+    for (int L = 0; L <= NL; ++L)
+      for (int k = lane * 16; k < nch * LM * (int)sizeof(T); k += 512)
+        cp_async16(st + L * kW + k, wsrc[L] + (size_t)e * io.ldw[L] * sizeof(T) + k);
+#pragma unroll
+    for (int L = 0; L < NL; ++L)
+      warp_copy(st + kOffS + L * kSb, ssrc[L] + (size_t)e * io.ldsbar[L + 1] * sizeof(T), nch * (int)sizeof(T), sal[L]);
+    if (lane < S) cp_async4(st + kOffY + lane * 4, io.Y + (size_t)e * S + lane);
+  };
   T* w0b = reinterpret_cast<T*>(io.wbar[0]);
   T* w1b = reinterpret_cast<T*>(io.wbar[1]);
   float gmax = 0.0f;
@@ -453,10 +549,13 @@ __global__ void __launch_bounds__(kMaxChannels) gen_edge_final_kernel(GenRowIO i
       io.Ybar[(size_t)(eb + j) * S + a] = sum;
     }
   };
-  for (int e = rb, buf = 0; e < re; ++e) {
+  int buf = 0;
+  ring_over<kStage>(rings[wid], rb, re, copy, [&](int e, const unsigned char* st) {
     const int j = (e - rb) % kEdgeBatch;
+    const T* ws = reinterpret_cast<const T*>(st);
+    const T* ss = reinterpret_cast<const T*>(st + kOffS);
     float y[S];
-    load_y<S>(io.Y + (size_t)e * S, y);
+    load_y<S>(reinterpret_cast<const float*>(st + kOffY), y);
     float yc[16];
 #pragma unroll
     for (int a = 0; a < 16; ++a) yc[a] = 0.0f;
@@ -466,18 +565,16 @@ __global__ void __launch_bounds__(kMaxChannels) gen_edge_final_kernel(GenRowIO i
       for (int a = 0; a < S; ++a) qs[a] = 0.0f;
 #pragma unroll
       for (int L = 0; L < NL; ++L) {
-        const float sb = gld(reinterpret_cast<const T*>(io.sbar[L + 1]) + (size_t)e * io.ldsbar[L + 1] +
-                             io.sbar_off[L + 1] + u);
+        const float sb = gld(ss + L * 32 + lane);
         float wl[LM];
-        load_lm<T, LM>(reinterpret_cast<const T*>(io.w[L + 1]) + (size_t)e * io.ldw[L + 1] + io.wcol[L + 1] + u * LM,
-                       wl);
+        load_lm<T, LM>(ws + (L + 1) * 32 * LM + lane * LM, wl);
 #pragma unroll
         for (int a = 0; a < S; ++a) {
           qs[a] = fmaf(sb, q[L][a], qs[a]);
           yc[a] = fmaf(wl[l_of(a)], gb[L][a], yc[a]);
         }
       }
-      load_lm<T, LM>(w0 + (size_t)e * io.ldw[0] + io.wcol[0] + u * LM, w0l);
+      load_lm<T, LM>(ws + lane * LM, w0l);
 #pragma unroll
       for (int a = 0; a < S; ++a) {
         const float ya = y[a];
@@ -498,7 +595,7 @@ __global__ void __launch_bounds__(kMaxChannels) gen_edge_final_kernel(GenRowIO i
       flush(e - j, j + 1, buf);
       buf ^= 1;
     }
-  }
+  });
   record_amax(io.amax_wbar, gmax);
 }
 
@@ -532,70 +629,78 @@ __device__ __forceinline__ bool gen_lane(const GenRowIO& io, GenLane& g) {
 template <typename T, int LMAX, int CPL>
 __global__ void __launch_bounds__(32 * kGenWarps) gen_env_w_kernel(GenRowIO io, int L) {
   constexpr int S = (LMAX + 1) * (LMAX + 1), LM = LMAX + 1;
+  constexpr int kW = 32 * CPL * LM * (int)sizeof(T), kStage = round16(kW + S * 4);
+  __shared__ __align__(16) unsigned char rings[kGenWarps][kRing * kStage];
   GenLane g;
-  if (!gen_lane<CPL>(io, g) || !g.act) return;
-  const T* __restrict__ w = reinterpret_cast<const T*>(io.w[L]) + io.wcol[L] + g.lane * LM;
-  const float* __restrict__ Y = io.Y;
-  const int ldw = io.ldw[L];
+  if (!gen_lane<CPL>(io, g)) return;
+  const T* __restrict__ w = reinterpret_cast<const T*>(io.w[L]) + io.wcol[L];
+  const int ldw = io.ldw[L], row_bytes = io.C * LM * (int)sizeof(T);
   float G[CPL][S];
 #pragma unroll
   for (int c = 0; c < CPL; ++c)
 #pragma unroll
     for (int b = 0; b < S; ++b) G[c][b] = 0.0f;
-#pragma unroll 2
-  for (int e = g.rb; e < g.re; ++e) {
+  auto copy = [&](int e, unsigned char* st) {
+    warp_copy(st, reinterpret_cast<const unsigned char*>(w + (size_t)e * ldw), row_bytes, 0);
+    if (g.lane < S) cp_async4(st + kW + g.lane * 4, io.Y + (size_t)e * S + g.lane);
+  };
+  ring_over<kStage>(rings[threadIdx.x >> 5], g.rb, g.re, copy, [&](int, const unsigned char* st) {
+    if (!g.act) return;
     float y[S];
-    load_y<S>(Y + (size_t)e * S, y);
+    load_y<S>(reinterpret_cast<const float*>(st + kW), y);
 #pragma unroll
     for (int c = 0; c < CPL; ++c) {
       float wl[LM];
-      load_lm<T, LM>(w + (size_t)e * ldw + 32 * c * LM, wl);
+      load_lm<T, LM>(reinterpret_cast<const T*>(st) + (g.lane + 32 * c) * LM, wl);
 #pragma unroll
       for (int b = 0; b < S; ++b) G[c][b] = fmaf(wl[l_of(b)], y[b], G[c][b]);
     }
-  }
-  float* out = io.G[L] + ((size_t)g.ia * io.C + g.lane) * S;
+  });
+  if (!g.act) return;
+  float* out = io.G[L] + (size_t)g.ia * S * io.C + g.lane;
 #pragma unroll
   for (int c = 0; c < CPL; ++c)
 #pragma unroll
-    for (int b = 0; b < S; ++b) out[32 * c * S + b] = G[c][b] * io.nu;
+    for (int b = 0; b < S; ++b) out[(size_t)b * io.C + 32 * c] = G[c][b] * io.nu;
 }
 
 // s^L_e[u] = sum_a w^0_{e,u,l(a)} Y_e[a] Q^L[i][u][a], into the s columns of the latent input
 template <typename T, int LMAX, int CPL>
 __global__ void __launch_bounds__(32 * kGenWarps) gen_s_w_kernel(GenRowIO io, int L) {
   constexpr int S = (LMAX + 1) * (LMAX + 1), LM = LMAX + 1;
+  constexpr int kW = 32 * CPL * LM * (int)sizeof(T), kStage = round16(kW + S * 4);
+  __shared__ __align__(16) unsigned char rings[kGenWarps][kRing * kStage];
   GenLane g;
-  if (!gen_lane<CPL>(io, g) || !g.act) return;
-  const T* __restrict__ w0 = reinterpret_cast<const T*>(io.w[0]) + io.wcol[0] + g.lane * LM;
-  const float* __restrict__ Y = io.Y;
+  if (!gen_lane<CPL>(io, g)) return;
+  const T* __restrict__ w0 = reinterpret_cast<const T*>(io.w[0]) + io.wcol[0];
   float q[CPL][S];
-  const float* Q = io.Q[L] + ((size_t)g.ia * io.C + g.lane) * S;
+  const float* Q = io.Q[L] + (size_t)g.ia * S * io.C + (g.act ? g.lane : 0);
 #pragma unroll
   for (int c = 0; c < CPL; ++c)
 #pragma unroll
-    for (int a = 0; a < S; ++a) q[c][a] = Q[32 * c * S + a];
+    for (int a = 0; a < S; ++a) q[c][a] = Q[(size_t)a * io.C + 32 * c];
   T* __restrict__ xs = reinterpret_cast<T*>(io.xs[L]) + io.xs_off[L] + g.lane;
-  const int ldw0 = io.ldw[0], ldxs = io.ldxs[L];
+  const int ldw0 = io.ldw[0], ldxs = io.ldxs[L], row_bytes = io.C * LM * (int)sizeof(T);
   float smax = 0.0f;
-  // the loads of an edge's weights and harmonics are all issued before its stores
-#pragma unroll 2
-  for (int e = g.rb; e < g.re; ++e) {
-    float y[S], wl[CPL][LM];
-    load_y<S>(Y + (size_t)e * S, y);
-#pragma unroll
-    for (int c = 0; c < CPL; ++c) load_lm<T, LM>(w0 + (size_t)e * ldw0 + 32 * c * LM, wl[c]);
-    float sv[CPL];
+  auto copy = [&](int e, unsigned char* st) {
+    warp_copy(st, reinterpret_cast<const unsigned char*>(w0 + (size_t)e * ldw0), row_bytes, 0);
+    if (g.lane < S) cp_async4(st + kW + g.lane * 4, io.Y + (size_t)e * S + g.lane);
+  };
+  ring_over<kStage>(rings[threadIdx.x >> 5], g.rb, g.re, copy, [&](int e, const unsigned char* st) {
+    if (!g.act) return;
+    float y[S];
+    load_y<S>(reinterpret_cast<const float*>(st + kW), y);
 #pragma unroll
     for (int c = 0; c < CPL; ++c) {
-      sv[c] = 0.0f;
+      float wl[LM];
+      load_lm<T, LM>(reinterpret_cast<const T*>(st) + (g.lane + 32 * c) * LM, wl);
+      float sv = 0.0f;
 #pragma unroll
-      for (int a = 0; a < S; ++a) sv[c] = fmaf(wl[c][l_of(a)] * y[a], q[c][a], sv[c]);
-      smax = fmaxf(smax, fabsf(sv[c]));
+      for (int a = 0; a < S; ++a) sv = fmaf(wl[l_of(a)] * y[a], q[c][a], sv);
+      smax = fmaxf(smax, fabsf(sv));
+      gst(xs + (size_t)e * ldxs + 32 * c, sv);
     }
-#pragma unroll
-    for (int c = 0; c < CPL; ++c) gst(xs + (size_t)e * ldxs + 32 * c, sv[c]);
-  }
+  });
   record_amax(io.amax_s, smax);
 }
 
@@ -603,55 +708,69 @@ __global__ void __launch_bounds__(32 * kGenWarps) gen_s_w_kernel(GenRowIO io, in
 template <typename T, int LMAX, int CPL>
 __global__ void __launch_bounds__(32 * kGenWarps) gen_qbar_w_kernel(GenRowIO io, int L) {
   constexpr int S = (LMAX + 1) * (LMAX + 1), LM = LMAX + 1;
+  constexpr int kW = 32 * CPL * LM * (int)sizeof(T), kSb = 32 * CPL * (int)sizeof(T), kStage = round16(kW + kSb + S * 4);
+  __shared__ __align__(16) unsigned char rings[kGenWarps][kRing * kStage];
   GenLane g;
-  if (!gen_lane<CPL>(io, g) || !g.act) return;
-  const T* __restrict__ w0 = reinterpret_cast<const T*>(io.w[0]) + io.wcol[0] + g.lane * LM;
-  const T* __restrict__ sb = reinterpret_cast<const T*>(io.sbar[L]) + io.sbar_off[L] + g.lane;
-  const float* __restrict__ Y = io.Y;
+  if (!gen_lane<CPL>(io, g)) return;
+  const T* __restrict__ w0 = reinterpret_cast<const T*>(io.w[0]) + io.wcol[0];
+  const T* __restrict__ sb = reinterpret_cast<const T*>(io.sbar[L]) + io.sbar_off[L];
+  const int ldw0 = io.ldw[0], ldsb = io.ldsbar[L], row_bytes = io.C * LM * (int)sizeof(T);
+  const unsigned sal =
+      (unsigned)((reinterpret_cast<uintptr_t>(sb) | (ldsb * sizeof(T)) | (io.C * sizeof(T))) & 15);
   float acc[CPL][S];
 #pragma unroll
   for (int c = 0; c < CPL; ++c)
 #pragma unroll
     for (int a = 0; a < S; ++a) acc[c][a] = 0.0f;
-#pragma unroll 2
-  for (int e = g.rb; e < g.re; ++e) {
+  auto copy = [&](int e, unsigned char* st) {
+    warp_copy(st, reinterpret_cast<const unsigned char*>(w0 + (size_t)e * ldw0), row_bytes, 0);
+    warp_copy(st + kW, reinterpret_cast<const unsigned char*>(sb + (size_t)e * ldsb), io.C * (int)sizeof(T), sal);
+    if (g.lane < S) cp_async4(st + kW + kSb + g.lane * 4, io.Y + (size_t)e * S + g.lane);
+  };
+  ring_over<kStage>(rings[threadIdx.x >> 5], g.rb, g.re, copy, [&](int, const unsigned char* st) {
+    if (!g.act) return;
     float y[S];
-    load_y<S>(Y + (size_t)e * S, y);
+    load_y<S>(reinterpret_cast<const float*>(st + kW + kSb), y);
 #pragma unroll
     for (int c = 0; c < CPL; ++c) {
-      const float sv = gld(sb + (size_t)e * io.ldsbar[L] + 32 * c);
+      const float sv = gld(reinterpret_cast<const T*>(st + kW) + g.lane + 32 * c);
       float wl[LM];
-      load_lm<T, LM>(w0 + (size_t)e * io.ldw[0] + 32 * c * LM, wl);
+      load_lm<T, LM>(reinterpret_cast<const T*>(st) + (g.lane + 32 * c) * LM, wl);
 #pragma unroll
       for (int a = 0; a < S; ++a) acc[c][a] = fmaf(wl[l_of(a)] * sv, y[a], acc[c][a]);
     }
-  }
-  float* out = io.Qb + ((size_t)g.ia * io.C + g.lane) * S;
+  });
+  if (!g.act) return;
+  float* out = io.Qb + (size_t)g.ia * S * io.C + g.lane;
 #pragma unroll
   for (int c = 0; c < CPL; ++c)
 #pragma unroll
-    for (int a = 0; a < S; ++a) out[32 * c * S + a] = acc[c][a];
+    for (int a = 0; a < S; ++a) out[(size_t)a * io.C + 32 * c] = acc[c][a];
 }
 
 // wbar^L_{e,u,l} = nu sum_m Gammabar^L[i][u][lm] Y_e[lm], for a layer L >= 2
 template <typename T, int LMAX, int CPL>
 __global__ void __launch_bounds__(32 * kGenWarps) gen_wbar_w_kernel(GenRowIO io, int L) {
   constexpr int S = (LMAX + 1) * (LMAX + 1), LM = LMAX + 1;
+  constexpr int kStage = round16(S * 4);
+  __shared__ __align__(16) unsigned char rings[kGenWarps][kRing * kStage];
   GenLane g;
-  if (!gen_lane<CPL>(io, g) || !g.act) return;
+  if (!gen_lane<CPL>(io, g)) return;
   float gb[CPL][S];
-  const float* G = io.Gb[L] + ((size_t)g.ia * io.C + g.lane) * S;
+  const float* G = io.Gb[L] + (size_t)g.ia * S * io.C + (g.act ? g.lane : 0);
 #pragma unroll
   for (int c = 0; c < CPL; ++c)
 #pragma unroll
-    for (int a = 0; a < S; ++a) gb[c][a] = io.nu * G[32 * c * S + a];
+    for (int a = 0; a < S; ++a) gb[c][a] = io.nu * G[(size_t)a * io.C + 32 * c];
   T* __restrict__ wLb = reinterpret_cast<T*>(io.wbar[L]) + io.wbcol[L] + g.lane * LM;
-  const float* __restrict__ Y = io.Y;
   float gmax = 0.0f;
-#pragma unroll 2
-  for (int e = g.rb; e < g.re; ++e) {
+  auto copy = [&](int e, unsigned char* st) {
+    if (g.lane < S) cp_async4(st + g.lane * 4, io.Y + (size_t)e * S + g.lane);
+  };
+  ring_over<kStage>(rings[threadIdx.x >> 5], g.rb, g.re, copy, [&](int e, const unsigned char* st) {
+    if (!g.act) return;
     float y[S];
-    load_y<S>(Y + (size_t)e * S, y);
+    load_y<S>(reinterpret_cast<const float*>(st), y);
 #pragma unroll
     for (int c = 0; c < CPL; ++c) {
       float o[LM] = {};
@@ -661,7 +780,7 @@ __global__ void __launch_bounds__(32 * kGenWarps) gen_wbar_w_kernel(GenRowIO io,
       for (int l = 0; l < LM; ++l) gmax = fmaxf(gmax, fabsf(o[l]));
       store_lm<T, LM>(wLb + (size_t)e * io.ldwbar[L] + 32 * c * LM, o);
     }
-  }
+  });
   record_amax(io.amax_wbar, gmax);
 }
 
@@ -725,10 +844,6 @@ static void fwd_lmax(const GenRowIO& io, int L, cudaStream_t st) {
 template <typename T, int LMAX>
 static void bwd_lmax(const GenRowIO& io, int L, cudaStream_t st) {
   const int bl = block_of(io.C);
-  if (L == io.nl) {
-    for (int k = 1; k <= io.nl; ++k)
-      cudaMemsetAsync(io.Gb[k], 0, (size_t)io.na * io.C * io.S * sizeof(float), st);
-  }
   GEN_W_LAUNCH(gen_qbar_w_kernel, io, L);
   chain_bwd_nl<LMAX>(io, L, st);
   if (L >= 2) GEN_W_LAUNCH(gen_wbar_w_kernel, io, L);
