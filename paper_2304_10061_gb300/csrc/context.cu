@@ -40,19 +40,39 @@ inline size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 // ------------------------------------------------------------------------
 // small kernels
 // ------------------------------------------------------------------------
-__global__ void map_types_kernel(const int* __restrict__ types, const double* __restrict__ pos, int n,
-                                 const int* __restrict__ map, int nmap, int* __restrict__ species,
-                                 int* __restrict__ err) {
+// The caller's positions and types into the context: positions copied (unless they are there
+// already), types mapped to model species, both checked.
+__global__ void stage_atoms_kernel(const int* __restrict__ types, const double* pos_in, int n,
+                                   const int* __restrict__ map, int nmap, double* pos, int* __restrict__ species,
+                                   int* __restrict__ err) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   int t = types[i];
   bool bad = (t < 0 || t >= nmap);
   int s = bad ? 0 : map[t];
   if (s < 0) bad = true;
-  double x = pos[3 * (size_t)i], y = pos[3 * (size_t)i + 1], z = pos[3 * (size_t)i + 2];
+  const double x = pos_in[3 * (size_t)i], y = pos_in[3 * (size_t)i + 1], z = pos_in[3 * (size_t)i + 2];
   if (!(isfinite(x) && isfinite(y) && isfinite(z))) bad = true;
   if (bad) atomicOr(err, kErrBadInput);
   species[i] = bad ? 0 : s;
+  if (pos != pos_in) {
+    pos[3 * (size_t)i] = x; pos[3 * (size_t)i + 1] = y; pos[3 * (size_t)i + 2] = z;
+  }
+}
+
+// The results into the caller's device arrays (null: not wanted) in one launch.
+__global__ void copy_results_kernel(const double* __restrict__ E, const double* __restrict__ Ea,
+                                    const double* __restrict__ F, const double* __restrict__ W, long long nb, long long n,
+                                    double* __restrict__ oE, double* __restrict__ oEa, double* __restrict__ oF,
+                                    double* __restrict__ oW) {
+  const long long stride = (long long)gridDim.x * blockDim.x, t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  for (long long k = t0; k < nb; k += stride) oE[k] = E[k];
+  if (oEa)
+    for (long long k = t0; k < n; k += stride) oEa[k] = Ea[k];
+  if (oF)
+    for (long long k = t0; k < 3 * n; k += stride) oF[k] = F[k];
+  if (oW)
+    for (long long k = t0; k < 9 * nb; k += stride) oW[k] = W[k];
 }
 
 __global__ void atom_struct_kernel(const int64_t* __restrict__ offs, int nstruct, int* __restrict__ atom_struct) {
@@ -69,6 +89,17 @@ bool is_device_ptr(const void* p) {
     return false;
   }
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+}
+
+// plain device memory of `device` (a kernel of that device may address it directly)
+bool is_own_device_ptr(const void* p, int device) {
+  if (!p) return false;
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == device;
 }
 
 // Per-launch timing of the library's kernels (CUDA events on the launching
@@ -150,7 +181,10 @@ struct allegro_ctx {
   int64_t n_centres = 0;                   // atoms [0, n_centres) are centres (the rest are ghosts)
   int nstruct = 0;
   bool batched = false;
-  std::vector<int> h_row_ptr;              // host copy of row_ptr (for chunking)
+  std::vector<int> h_row_ptr;              // host copy of row_ptr (for chunking), once host_rows fetched it
+  bool rows_on_host = false;
+  int64_t bytes_per_edge = 0;              // chunk workspace per edge (0: not computed yet)
+  int* h_pin = nullptr;                    // pinned words the waits read {error word, edge count} into
 
   // capacities and policy
   int64_t atom_cap = 0, edge_cap = 0;
@@ -777,13 +811,20 @@ allegro_status stage_atoms(allegro_ctx* c, int64_t n, const double* pos, const i
     c->scan_tmp_cap = st * 2;
   }
   if (n > 0) {
-    cudaMemcpyKind kp = is_device_ptr(pos) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    cudaMemcpyKind kt = is_device_ptr(types) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    CUDA_TRY(c, cudaMemcpyAsync(c->d_pos, pos, (size_t)n * 3 * 8, kp, c->stream));
-    CUDA_TRY(c, cudaMemcpyAsync(c->d_types, types, (size_t)n * 4, kt, c->stream));
+    // device inputs are read where they are; others are copied first
+    const double* ps = pos;
+    const int32_t* ts = types;
+    if (!is_own_device_ptr(pos, c->device)) {
+      CUDA_TRY(c, cudaMemcpyAsync(c->d_pos, pos, (size_t)n * 3 * 8, cudaMemcpyDefault, c->stream));
+      ps = c->d_pos;
+    }
+    if (!is_own_device_ptr(types, c->device)) {
+      CUDA_TRY(c, cudaMemcpyAsync(c->d_types, types, (size_t)n * 4, cudaMemcpyDefault, c->stream));
+      ts = c->d_types;
+    }
     CUDA_TRY(c, cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream));
-    map_types_kernel<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(c->d_types, c->d_pos, (int)n, c->d_map,
-                                                                         c->nmap, c->d_species, c->d_err);
+    stage_atoms_kernel<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(ts, ps, (int)n, c->d_map, c->nmap, c->d_pos,
+                                                                           c->d_species, c->d_err);
     CUDA_TRY(c, cudaGetLastError());
   } else {
     CUDA_TRY(c, cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream));
@@ -820,48 +861,79 @@ allegro_status ensure_edges(allegro_ctx* c, int64_t E) {
   return ALLEGRO_OK;
 }
 
-allegro_status read_err(allegro_ctx* c, int* out) {
-  int h = 0;
-  CUDA_TRY(c, cudaMemcpyAsync(&h, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+// Waits for the stream and reads the device's error word and, when asked, the edge count beside it.
+allegro_status read_err(allegro_ctx* c, int* out, int64_t* n_edges = nullptr) {
+  CUDA_TRY(c, cudaMemcpyAsync(c->h_pin, c->d_err, 2 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  *out = h;
+  *out = c->h_pin[0];
+  if (n_edges) *n_edges = c->h_pin[1];
   return ALLEGRO_OK;
+}
+
+// Edges the list's arrays hold now.
+int64_t edge_room(allegro_ctx* c) {
+  const Caps& k = caps_of(c);
+  return std::min({k.ej.v, k.ei.v, k.eS.v / 3, k.ed.v / 3, k.col_edge.v, k.Ee.v, k.g.v / 3, (int64_t)2000000000});
 }
 
 // Each edge's arrival order in its column, from the fill pass to finish_neighbors: held in the
 // edge-energy array, which the next evaluation writes first.
 int* col_rank(allegro_ctx* c) { return reinterpret_cast<int*>(c->d_Ee); }
 
-// CSC index (from the fill pass's column counts and ranks) and host row_ptr copy, shared by all
-// neighbour paths.
-allegro_status finish_neighbors(allegro_ctx* c, int n, int64_t E, bool ranked = true) {
+// The second half of every neighbour path, once the counts are scanned into row_ptr (their total in
+// d_err[1]): fill(edge_cap) queues the fill pass (true: it counted and ranked the columns), then come
+// the CSC index and one wait for the error word and the edge count.  When the arrays of an earlier
+// list are there all of it is queued before the count is known -- the passes leave a list that does
+// not fit unwritten, and they run again once the arrays have grown -- so a list costs one wait
+// instead of two; the first list waits for the count to size the arrays.
+template <typename Fill>
+allegro_status fill_rows(allegro_ctx* c, int n, int64_t* n_edges_out, Fill&& fill) {
   cudaStream_t st = c->stream;
-  {
-    ProfScope ps(c, "nb_csc", 0.0, (double)E * 16 + (double)n * 16, 0);
-    if (!ranked) {
-      nb_col_rank(c->d_ej, (int)E, c->d_col_count, col_rank(c), st);
-      ++c->launches;
-    }
-    c->launches += exclusive_scan_i32(c->d_col_count, c->d_col_ptr, n, c->d_scan_tmp, true, st);
-    if (E > 0) {
-      nb_place(c->d_ej, col_rank(c), (int)E, c->d_col_ptr, c->d_col_edge, st);
+  int64_t E = 0, room = edge_room(c);
+  int err = 0;
+  allegro_status s;
+  for (bool sized = false;;) {
+    if (room > 0) {
+      const bool ranked = fill((int)room);
+      ProfScope ps(c, "nb_csc", 0.0, (double)(sized ? E : c->n_edges) * 16 + (double)n * 16, 0);
+      if (!ranked) {
+        nb_col_rank(c->d_ej, c->d_row_ptr, n, (int)room, c->d_col_count, col_rank(c), st);
+        ++c->launches;
+      }
+      c->launches += exclusive_scan_i32(c->d_col_count, c->d_col_ptr, n, c->d_scan_tmp, true, nullptr, st);
+      nb_place_edges(c->d_ej, col_rank(c), c->d_row_ptr, n, (int)room, c->d_col_ptr, c->d_col_edge, st);
       nb_sort_columns(c->d_col_ptr, n, c->d_col_edge, st);
       c->launches += 2;
     }
+    CUDA_TRY(c, cudaGetLastError());
+    if ((s = read_err(c, &err, &E)) != ALLEGRO_OK) return s;
+    if (E < 0) return fail(c, ALLEGRO_E_CAPACITY, "edge count overflows int32");
+    if ((s = ensure_edges(c, E)) != ALLEGRO_OK) return s;
+    if (room > 0 && E <= room) break;
+    if (sized) return fail(c, ALLEGRO_E_CUDA, "internal: the edge count changed between two passes");
+    sized = true;
+    room = edge_room(c);
   }
-  CUDA_TRY(c, cudaGetLastError());
-  c->h_row_ptr.resize((size_t)n + 1);
-  CUDA_TRY(c, cudaMemcpyAsync(c->h_row_ptr.data(), c->d_row_ptr, (size_t)(n + 1) * 4, cudaMemcpyDeviceToHost, st));
-  int err = 0;
-  allegro_status s = read_err(c, &err);
-  if (s != ALLEGRO_OK) return s;
   if (err & kErrBadInput)
     return fail(c, ALLEGRO_E_INVALID, "a type is outside the species map or a position is not finite");
   if (err & kErrNeighbor) return fail(c, ALLEGRO_E_CUDA, "internal: neighbour fill pass disagreed with its count");
+  c->rows_on_host = false;
   c->n_atoms = n;
   c->n_centres = n;
   c->n_edges = E;
   c->have_nb = true;
+  if (n_edges_out) *n_edges_out = E;
+  return ALLEGRO_OK;
+}
+
+// The host copy of row_ptr (only a list evaluated in several chunks needs it).
+allegro_status host_rows(allegro_ctx* c) {
+  if (c->rows_on_host) return ALLEGRO_OK;
+  const size_t n = (size_t)c->n_atoms;
+  c->h_row_ptr.resize(n + 1);
+  CUDA_TRY(c, cudaMemcpyAsync(c->h_row_ptr.data(), c->d_row_ptr, (n + 1) * 4, cudaMemcpyDeviceToHost, c->stream));
+  CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  c->rows_on_host = true;
   return ALLEGRO_OK;
 }
 
@@ -1523,41 +1595,56 @@ allegro_status run_chunk_gen(allegro_ctx* c, const WS& w, int a0, int a1, int e0
 // Chunks of whole rows (each centre's environment sum complete inside one
 // chunk), at most `budget` edges each (0: the largest the memory allows).
 struct Plan {
-  std::vector<int> bounds;
+  std::vector<int> bounds;   // first row of each chunk, and n
+  std::vector<int> edges;    // first edge of each chunk, and E
   int64_t maxE = 1, maxA = 1;
 };
 
-Plan plan_chunks(allegro_ctx* c, int64_t budget) {
+allegro_status plan_chunks(allegro_ctx* c, int64_t budget, Plan* plan) {
   const int n = (int)c->n_atoms;
+  Plan& p = *plan;
   if (budget <= 0) {
-    size_t fr = 0, tot = 0;
-    cudaMemGetInfo(&fr, &tot);
-    int64_t per = ws_bytes_per_edge(c);
-    int64_t cap_bytes = std::min<int64_t>((int64_t)(fr * 0.5) + (int64_t)c->ws_bytes, 48ll << 30);
-    budget = std::max<int64_t>(cap_bytes / std::max<int64_t>(per, 1), 1 << 16);
-  }
-  Plan p;
-  p.bounds.push_back(0);
-  int a = 0;
-  while (a < n) {
-    int64_t start = c->h_row_ptr[a];
-    // largest b with row_ptr[b] - start <= budget (at least one row)
-    int lo = a + 1, hi = n;
-    while (lo < hi) {
-      int mid = (lo + hi + 1) / 2;
-      if ((int64_t)c->h_row_ptr[mid] - start <= budget) lo = mid;
-      else hi = mid - 1;
+    if (c->bytes_per_edge == 0) c->bytes_per_edge = std::max<int64_t>(ws_bytes_per_edge(c), 1);
+    const int64_t cap = 48ll << 30;
+    // a list that fits the workspace already held is one chunk whatever memory is free (asking the
+    // driver for that costs more than a small list's kernels)
+    budget = std::max<int64_t>(std::min<int64_t>((int64_t)c->ws_bytes, cap) / c->bytes_per_edge, 1 << 16);
+    if (c->n_edges > budget) {
+      size_t fr = 0, tot = 0;
+      cudaMemGetInfo(&fr, &tot);
+      budget = std::max<int64_t>(std::min<int64_t>((int64_t)(fr * 0.5) + (int64_t)c->ws_bytes, cap) / c->bytes_per_edge,
+                                 1 << 16);
     }
-    int b = std::max(lo, a + 1);
-    p.bounds.push_back(b);
-    a = b;
   }
-  if (n == 0) p.bounds.push_back(0);
+  p.bounds.push_back(0);
+  p.edges.push_back(0);
+  if (c->n_edges <= budget) {
+    p.bounds.push_back(n);
+    p.edges.push_back((int)c->n_edges);
+  } else {
+    allegro_status s = host_rows(c);
+    if (s != ALLEGRO_OK) return s;
+    int a = 0;
+    while (a < n) {
+      int64_t start = c->h_row_ptr[a];
+      // largest b with row_ptr[b] - start <= budget (at least one row)
+      int lo = a + 1, hi = n;
+      while (lo < hi) {
+        int mid = (lo + hi + 1) / 2;
+        if ((int64_t)c->h_row_ptr[mid] - start <= budget) lo = mid;
+        else hi = mid - 1;
+      }
+      int b = std::max(lo, a + 1);
+      p.bounds.push_back(b);
+      p.edges.push_back(c->h_row_ptr[b]);
+      a = b;
+    }
+  }
   for (size_t q = 0; q + 1 < p.bounds.size(); ++q) {
-    p.maxE = std::max<int64_t>(p.maxE, (int64_t)c->h_row_ptr[p.bounds[q + 1]] - c->h_row_ptr[p.bounds[q]]);
+    p.maxE = std::max<int64_t>(p.maxE, (int64_t)p.edges[q + 1] - p.edges[q]);
     p.maxA = std::max<int64_t>(p.maxA, p.bounds[q + 1] - p.bounds[q]);
   }
-  return p;
+  return ALLEGRO_OK;
 }
 
 // The device work of one evaluation (no host synchronisation, no allocation:
@@ -1569,7 +1656,7 @@ allegro_status run_plan(allegro_ctx* c, const Plan& p, const WS& w, bool backwar
   allegro_status s;
   for (size_t q = 0; q + 1 < p.bounds.size(); ++q) {
     int a0 = p.bounds[q], a1 = p.bounds[q + 1];
-    int e0 = c->h_row_ptr[a0], e1 = c->h_row_ptr[a1];
+    int e0 = p.edges[q], e1 = p.edges[q + 1];
     if (c->generic)
       s = bf16_storage(c) ? run_chunk_gen<bf16>(c, w, a0, a1, e0, e1, backward)
                                          : run_chunk_gen<float>(c, w, a0, a1, e0, e1, backward);
@@ -1600,14 +1687,15 @@ allegro_status run_plan(allegro_ctx* c, const Plan& p, const WS& w, bool backwar
 // so one-time set-up such as kernel attributes never happens under capture).
 allegro_status evaluate_once(allegro_ctx* c, bool backward) {
   const int64_t budget = c->chunk_edges_user > 0 ? c->chunk_edges_user : c->tune.chunk_edges;
-  Plan p = plan_chunks(c, budget);
-  WS w;
-  allegro_status s = ensure_ws(c, p.maxE, p.maxA, &w);
+  Plan p;
+  allegro_status s = plan_chunks(c, budget, &p);
   if (s != ALLEGRO_OK) return s;
+  WS w;
+  if ((s = ensure_ws(c, p.maxE, p.maxA, &w)) != ALLEGRO_OK) return s;
   if (!c->use_graphs || c->prof.on) return run_plan(c, p, w, backward);
   allegro_ctx::GraphKey key;
   key.bounds = p.bounds;
-  for (int b : p.bounds) key.bounds.push_back(c->h_row_ptr[b]);   // edge offsets of the chunks too
+  key.bounds.insert(key.bounds.end(), p.edges.begin(), p.edges.end());   // edge offsets of the chunks too
   key.bounds.push_back((int)c->n_centres);
   key.ptrs = {c->d_row_ptr, c->d_col_ptr, c->d_col_edge, c->d_ej, c->d_ei, c->d_eS, c->d_ed, c->d_Ee, c->d_g,
               c->d_species, c->d_Eatom, c->d_F, c->d_Wat, c->d_offs, c->d_Eout, c->d_Wout, c->d_err,
@@ -1830,6 +1918,8 @@ allegro_status allegro_create(const void* weights_blob, size_t blob_bytes, const
   if (cudaMalloc(&c->d_err, 16) != cudaSuccess || cudaMalloc(&c->d_total, 16) != cudaSuccess ||
       cudaMalloc(&c->d_minmax, 12 * 8) != cudaSuccess || cudaMalloc(&c->d_red_scratch, kStructScratch * sizeof(double)) != cudaSuccess)
     return bail(fail(c, ALLEGRO_E_OOM, "scratch allocation failed"));
+  if (cudaHostAlloc(reinterpret_cast<void**>(&c->h_pin), 2 * sizeof(int), cudaHostAllocDefault) != cudaSuccess)
+    return bail(fail(c, ALLEGRO_E_OOM, "pinned words"));
   cudaMemset(c->d_err, 0, 16);
   cudaMemset(c->d_red_scratch, 0, kStructScratch * sizeof(double));
   *out = c;
@@ -2034,7 +2124,7 @@ static allegro_status build_single(allegro_ctx* c, int64_t n_atoms, const double
   {
     ProfScope ps(c, "nb_bin_sort", 0.0, (double)n * 80 + (double)ncell * 16, 3);
     nb_bin(c->d_pos, n, g, c->d_cell_of, c->d_wrap, c->d_cell_count, c->d_count, st);
-    c->launches += exclusive_scan_i32(c->d_cell_count, c->d_cell_start, (int)ncell, c->d_scan_tmp, true, st);
+    c->launches += exclusive_scan_i32(c->d_cell_count, c->d_cell_start, (int)ncell, c->d_scan_tmp, true, nullptr, st);
     nb_place(c->d_cell_of, c->d_count, n, c->d_cell_start, c->d_sorted, st);
     nb_sort_cells(c->d_pos, c->d_species, g, (int)ncell, c->d_cell_start, c->d_wrap, c->d_sorted, c->d_pos4, c->d_pw,
                   c->d_wraps, st);
@@ -2063,25 +2153,17 @@ static allegro_status build_single(allegro_ctx* c, int64_t n_atoms, const double
     ProfScope ps(c, "nb_search_count", 0.0, (double)n * 64);
     nb_search(false, c->d_pos, n, g, c->d_cell_of, c->d_wraps, c->d_cell_start, c->d_sorted, c->d_pos4, c->d_pw, rc2,
               band, pair_rc2, c->arch.ns, c->d_count,
-              nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, c->d_err, st);
-    c->launches += exclusive_scan_i32(c->d_count, c->d_row_ptr, n, c->d_scan_tmp, false, st);
+              nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0, c->d_err, st);
+    c->launches += exclusive_scan_i32(c->d_count, c->d_row_ptr, n, c->d_scan_tmp, false, c->d_err + 1, st);
   }
-  int hE = 0;
-  CUDA_TRY(c, cudaMemcpyAsync(&hE, c->d_row_ptr + n, 4, cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(c, cudaStreamSynchronize(st));
-  CUDA_TRY(c, cudaGetLastError());
-  if (hE < 0) return fail(c, ALLEGRO_E_CAPACITY, "edge count overflows int32");
-  if ((s = ensure_edges(c, hE)) != ALLEGRO_OK) return s;
-  bool ranked = true;
-  {
-    ProfScope ps(c, "nb_search_fill", 0.0, (double)hE * 44 + (double)n * 64);
-    ranked = nb_search(true, c->d_pos, n, g, c->d_cell_of, c->d_wraps, c->d_cell_start, c->d_sorted, c->d_pos4, c->d_pw, rc2,
-              band, pair_rc2, c->arch.ns, nullptr,
-              c->d_row_ptr, c->d_ej, c->d_ei, c->d_eS, c->d_ed, c->d_col_count, col_rank(c), c->d_err, st);
-  }
-  if ((s = finish_neighbors(c, n, hE, ranked)) != ALLEGRO_OK) return s;
+  if ((s = fill_rows(c, n, n_edges_out, [&](int edge_cap) {
+         ProfScope ps(c, "nb_search_fill", 0.0, (double)c->n_edges * 44 + (double)n * 64);
+         return nb_search(true, c->d_pos, n, g, c->d_cell_of, c->d_wraps, c->d_cell_start, c->d_sorted, c->d_pos4,
+                          c->d_pw, rc2, band, pair_rc2, c->arch.ns, nullptr, c->d_row_ptr, c->d_ej, c->d_ei, c->d_eS,
+                          c->d_ed, c->d_col_count, col_rank(c), edge_cap, c->d_err, st);
+       })) != ALLEGRO_OK)
+    return s;
   c->n_centres = g.n_centres;
-  if (n_edges_out) *n_edges_out = hE;
   return ALLEGRO_OK;
 }
 
@@ -2162,26 +2244,31 @@ allegro_status allegro_neighbors_batched(allegro_ctx* c, int32_t n_struct, const
       hn[3 * b + k] = hp[3 * b + k] ? (int)ceil(rc / w[k] + hspan[3 * b + k]) : 0;
     }
   }
-  if (cells) CUDA_TRY(c, cudaMemcpyAsync(c->d_cells, hc.data(), hc.size() * 8, cudaMemcpyHostToDevice, st));
-  CUDA_TRY(c, cudaMemcpyAsync(c->d_pbc, hp.data(), hp.size() * 4, cudaMemcpyHostToDevice, st));
-  CUDA_TRY(c, cudaMemcpyAsync(c->d_nimg, hn.data(), hn.size() * 4, cudaMemcpyHostToDevice, st));
+  if (cells) {   // (without cells no axis is periodic and the search reads none of these)
+    CUDA_TRY(c, cudaMemcpyAsync(c->d_cells, hc.data(), hc.size() * 8, cudaMemcpyHostToDevice, st));
+    CUDA_TRY(c, cudaMemcpyAsync(c->d_pbc, hp.data(), hp.size() * 4, cudaMemcpyHostToDevice, st));
+    CUDA_TRY(c, cudaMemcpyAsync(c->d_nimg, hn.data(), hn.size() * 4, cudaMemcpyHostToDevice, st));
+  }
   atom_struct_kernel<<<n_struct, 128, 0, st>>>(c->d_offs, n_struct, c->d_atom_struct);
   const double rc2 = rc * rc;
-  nb_bruteforce_batched(false, c->d_pos, c->d_offs, n_struct, cells ? c->d_cells : nullptr, c->d_pbc, c->d_nimg, rc2,
-                        c->d_species, c->arch.pair_rc2, c->arch.ns, c->d_atom_struct, n, c->d_count, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
-                        c->d_err, st);
-  c->launches += exclusive_scan_i32(c->d_count, c->d_row_ptr, n, c->d_scan_tmp, false, st);
-  int hE = 0;
-  CUDA_TRY(c, cudaMemcpyAsync(&hE, c->d_row_ptr + n, 4, cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(c, cudaStreamSynchronize(st));
-  CUDA_TRY(c, cudaGetLastError());
-  if ((s = ensure_edges(c, hE)) != ALLEGRO_OK) return s;
-  nb_bruteforce_batched(true, c->d_pos, c->d_offs, n_struct, cells ? c->d_cells : nullptr, c->d_pbc, c->d_nimg, rc2,
-                        c->d_species, c->arch.pair_rc2, c->arch.ns, c->d_atom_struct, n, nullptr, c->d_row_ptr, c->d_ej, c->d_ei, c->d_eS, c->d_ed, c->d_col_count, col_rank(c), c->d_err, st);
-  if ((s = finish_neighbors(c, n, hE)) != ALLEGRO_OK) return s;
+  const double* d_cells = cells ? c->d_cells : nullptr;
+  {
+    ProfScope ps(c, "nb_brute_count", 0.0, (double)n * 64);
+    nb_bruteforce_batched(false, c->d_pos, c->d_offs, n_struct, d_cells, c->d_pbc, c->d_nimg, rc2, c->d_species,
+                          c->arch.pair_rc2, c->arch.ns, c->d_atom_struct, n, c->d_count, nullptr, nullptr, nullptr,
+                          nullptr, nullptr, nullptr, nullptr, 0, c->d_err, st);
+    c->launches += exclusive_scan_i32(c->d_count, c->d_row_ptr, n, c->d_scan_tmp, false, c->d_err + 1, st);
+  }
+  if ((s = fill_rows(c, n, n_edges_out, [&](int edge_cap) {
+         ProfScope ps(c, "nb_brute_fill", 0.0, (double)c->n_edges * 44 + (double)n * 64);
+         nb_bruteforce_batched(true, c->d_pos, c->d_offs, n_struct, d_cells, c->d_pbc, c->d_nimg, rc2, c->d_species,
+                               c->arch.pair_rc2, c->arch.ns, c->d_atom_struct, n, nullptr, c->d_row_ptr, c->d_ej,
+                               c->d_ei, c->d_eS, c->d_ed, c->d_col_count, col_rank(c), edge_cap, c->d_err, st);
+         return true;
+       })) != ALLEGRO_OK)
+    return s;
   c->nstruct = n_struct;
   c->batched = true;
-  if (n_edges_out) *n_edges_out = hE;
   return ALLEGRO_OK;
 }
 
@@ -2194,10 +2281,18 @@ allegro_status allegro_energy_forces(allegro_ctx* c, double* E_total, double* E_
   allegro_status s = evaluate(c, backward);
   if (s != ALLEGRO_OK) return s;
   const size_t n = (size_t)c->n_atoms, B = (size_t)c->nstruct;
-  if ((s = copy_out(c, E_total, c->d_Eout, B * 8)) != ALLEGRO_OK) return s;
-  if ((s = copy_out(c, E_atom, c->d_Eatom, n * 8)) != ALLEGRO_OK) return s;
-  if (F && (s = copy_out(c, F, c->d_F, n * 3 * 8)) != ALLEGRO_OK) return s;
-  if (virial && (s = copy_out(c, virial, c->d_Wout, B * 9 * 8)) != ALLEGRO_OK) return s;
+  auto direct = [&](const void* p) { return !p || is_own_device_ptr(p, c->device); };
+  if (direct(E_total) && direct(E_atom) && direct(F) && direct(virial)) {
+    const unsigned blocks = (unsigned)std::min<size_t>((3 * n + 9 * B + 255) / 256, 152 * 8);
+    copy_results_kernel<<<blocks, 256, 0, c->stream>>>(c->d_Eout, c->d_Eatom, c->d_F, c->d_Wout, (long long)B,
+                                                       (long long)n, E_total, E_atom, F, virial);
+    CUDA_TRY(c, cudaGetLastError());
+  } else {
+    if ((s = copy_out(c, E_total, c->d_Eout, B * 8)) != ALLEGRO_OK) return s;
+    if ((s = copy_out(c, E_atom, c->d_Eatom, n * 8)) != ALLEGRO_OK) return s;
+    if (F && (s = copy_out(c, F, c->d_F, n * 3 * 8)) != ALLEGRO_OK) return s;
+    if (virial && (s = copy_out(c, virial, c->d_Wout, B * 9 * 8)) != ALLEGRO_OK) return s;
+  }
   int err = 0;
   if ((s = read_err(c, &err)) != ALLEGRO_OK) return s;
   if (err & kErrTimeout) return fail(c, ALLEGRO_E_TIMEOUT, "a bounded device wait expired; results are invalid");
@@ -2296,21 +2391,16 @@ allegro_status allegro_md_verlet(allegro_ctx* c, int64_t n_atoms, double* pos, d
       ProfScope ps(c, "nb_skin_filter", 0.0, (double)n * 64);
       nb_skin_filter(false, c->d_pos, n, c->d_cell9, c->d_sk_row, c->d_sk_j, c->d_sk_S, c->arch.rc * c->arch.rc,
                      c->arch.pair_rc2, c->d_species, c->arch.ns, c->d_count, nullptr, nullptr, nullptr, nullptr,
-                     nullptr, nullptr, nullptr, st);
-      c->launches += exclusive_scan_i32(c->d_count, c->d_row_ptr, n, c->d_scan_tmp, false, st);
+                     nullptr, nullptr, nullptr, 0, st);
+      c->launches += exclusive_scan_i32(c->d_count, c->d_row_ptr, n, c->d_scan_tmp, false, c->d_err + 1, st);
     }
-    int hE = 0;
-    CUDA_TRY(c, cudaMemcpyAsync(&hE, c->d_row_ptr + n, 4, cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(c, cudaStreamSynchronize(st));
-    if ((r = ensure_edges(c, hE)) != ALLEGRO_OK) return r;
-    {
-      ProfScope ps(c, "nb_skin_filter", 0.0, (double)hE * 44 + (double)n * 64);
+    return fill_rows(c, n, nullptr, [&](int edge_cap) {
+      ProfScope ps(c, "nb_skin_filter", 0.0, (double)c->n_edges * 44 + (double)n * 64);
       nb_skin_filter(true, c->d_pos, n, c->d_cell9, c->d_sk_row, c->d_sk_j, c->d_sk_S, c->arch.rc * c->arch.rc,
                      c->arch.pair_rc2, c->d_species, c->arch.ns, nullptr, c->d_row_ptr, c->d_ej, c->d_ei, c->d_eS,
-                     c->d_ed, c->d_col_count, col_rank(c), st);
-    }
-    CUDA_TRY(c, cudaGetLastError());
-    return finish_neighbors(c, n, hE);
+                     c->d_ed, c->d_col_count, col_rank(c), edge_cap, st);
+      return true;
+    });
   };
   // forces at the initial positions
   if ((s = neighbours(true)) != ALLEGRO_OK) return s;
@@ -2489,6 +2579,7 @@ void allegro_destroy(allegro_ctx* c) {
                   c->d_sk_S, c->d_sk_ref, c->d_cell9, c->d_maxd, c->d_amax, c->d_wraps};
   for (void* p : bufs)
     if (p) cudaFree(p);
+  if (c->h_pin) cudaFreeHost(c->h_pin);
   if (c->own_stream) cudaStreamDestroy(c->own_stream);
   delete c;
 }

@@ -163,8 +163,8 @@ void fp8_quantize(const float* src, int rows, int cols, int lds, uint8_t* dst, i
 
 // scan / utilities
 // out[0..n] = exclusive scan of in[0..n) (arrays 16-byte aligned); `clear` zeroes the input as it is
-// read.  Returns the launches made.
-int exclusive_scan_i32(int* in, int* out, int n, void* tmp, bool clear, cudaStream_t st);
+// read; `total`, if given, also receives out[n].  Returns the launches made.
+int exclusive_scan_i32(int* in, int* out, int n, void* tmp, bool clear, int* total, cudaStream_t st);
 size_t scan_tmp_bytes(int n);
 
 // neighbours
@@ -193,22 +193,28 @@ void nb_sort_cells(const double* pos, const int* species, const CellGrid& g, int
 bool nb_search(bool fill, const double* pos, int n, const CellGrid& g, const int* cell_of,
                const int4* wraps, const int* cell_start, const int* sorted, const float4* pos4, const double* pw,
                double rc2, float band, const double* pair_rc2, int ns, int* count, const int* row_ptr, int* ej,
-               int* ei, int* eS, double* ed, int* col_count, int* col_rank, int* d_err, cudaStream_t st);
+               int* ei, int* eS, double* ed, int* col_count, int* col_rank, int edge_cap, int* d_err,
+               cudaStream_t st);
 void nb_bruteforce_batched(bool fill, const double* pos, const int64_t* offs, int nstruct,
                            const double* cells, const int* pbc, const int* nimg, double rc2,
                            const int* species, const double* pair_rc2, int ns,
                            const int* atom_struct, int n, int* count, const int* row_ptr, int* ej,
-                           int* ei, int* eS, double* ed, int* col_count, int* col_rank, int* d_err,
-                           cudaStream_t st);
+                           int* ei, int* eS, double* ed, int* col_count, int* col_rank, int edge_cap,
+                           int* d_err, cudaStream_t st);
 // Verlet-skin reuse: count (fill = false, into count[i]) or write (fill = true, rows at row_ptr[i]) the
 // candidates of a list built at r_c + skin (sk_row / sk_j / sk_S) that pass the exact rule now
 void nb_skin_filter(bool fill, const double* pos, int n, const double* d_cell, const int* sk_row, const int* sk_j,
                     const int* sk_S, double rc2, const double* pair_rc2, const int* species, int ns, int* count,
                     const int* row_ptr, int* ej, int* ei, int* eS, double* ed, int* col_count, int* col_rank,
-                    cudaStream_t st);
+                    int edge_cap, cudaStream_t st);
 // max_i |pos_i - ref_i|^2 as the bits of a double in *out (cleared first)
 void nb_max_disp2(const double* pos, const double* ref, int n, unsigned long long* out, cudaStream_t st);
-void nb_col_rank(const int* ej, int E, int* col_count, int* col_rank, cudaStream_t st);
+// Passes over a list of row_ptr[n] edges (all of them, and the fill passes, do nothing when that
+// exceeds edge_cap): col_rank[e] = arrival order of e in its column; col_edge[col_ptr[ej[e]] + rank[e]] = e
+void nb_col_rank(const int* ej, const int* row_ptr, int n, int edge_cap, int* col_count, int* col_rank,
+                 cudaStream_t st);
+void nb_place_edges(const int* ej, const int* rank, const int* row_ptr, int n, int edge_cap, const int* col_ptr,
+                    int* col_edge, cudaStream_t st);
 // each column's edges in ascending order
 void nb_sort_columns(const int* col_ptr, int n, int* col_edge, cudaStream_t st);
 void nb_struct_span(const double* pos, const int64_t* offs, const double* inv, int nstruct, double* span,

@@ -15,6 +15,8 @@
 // (edges grouped by neighbour j, ascending edge id) serves the force gather.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "internal.h"
 
 namespace alg {
@@ -93,8 +95,9 @@ __device__ __forceinline__ int block_scan_tile(int* __restrict__ in, int* __rest
 }
 
 template <int PER>
-__global__ void __launch_bounds__(1024) scan_one_kernel(int* in, int* out, int n, bool clear) {
-  block_scan_tile<1024, PER>(in, out, n, 0, clear);
+__global__ void __launch_bounds__(1024) scan_one_kernel(int* in, int* out, int n, bool clear, int* total) {
+  const int t = block_scan_tile<1024, PER>(in, out, n, 0, clear);
+  if (total && threadIdx.x == 0) *total = t;
 }
 
 __global__ void scan_block_kernel(int* in, int* out, int n, int* __restrict__ block_sums, bool clear) {
@@ -102,12 +105,16 @@ __global__ void scan_block_kernel(int* in, int* out, int n, int* __restrict__ bl
   if (threadIdx.x == 255) block_sums[blockIdx.x] = total;
 }
 
-__global__ void scan_add_kernel(int* __restrict__ out, int n, const int* __restrict__ block_pref) {
+__global__ void scan_add_kernel(int* __restrict__ out, int n, const int* __restrict__ block_pref, int* total) {
   const int base = blockIdx.x * kScanBlock;
   const int add = block_pref[blockIdx.x];
   for (int k = threadIdx.x; k < kScanBlock; k += blockDim.x) {
     int idx = base + k;
-    if (idx <= n) out[idx] += add;
+    if (idx <= n) {
+      const int v = out[idx] + add;
+      out[idx] = v;
+      if (total && idx == n) *total = v;
+    }
   }
 }
 
@@ -128,13 +135,13 @@ size_t scan_tmp_bytes(int n) {
 // Scans in[0..n) into out[0..n] (out[n] = total).  Up to 32 x 1024 elements one block does it in
 // one launch (about 3 us against 6 for the three launches of the block-wise scan at 16k elements:
 // the launches are the time at these sizes); above, block sums, their scan, and an add.
-static void scan_rec(int* in, int* out, int n, char* tmp, bool clear, cudaStream_t st) {
+static void scan_rec(int* in, int* out, int n, char* tmp, bool clear, int* total, cudaStream_t st) {
   if (n < 4 * 1024) {
-    scan_one_kernel<4><<<1, 1024, 0, st>>>(in, out, n, clear);
+    scan_one_kernel<4><<<1, 1024, 0, st>>>(in, out, n, clear, total);
     return;
   }
   if (n < 32 * 1024) {
-    scan_one_kernel<32><<<1, 1024, 0, st>>>(in, out, n, clear);
+    scan_one_kernel<32><<<1, 1024, 0, st>>>(in, out, n, clear, total);
     return;
   }
   const int nb = (n + 1 + kScanBlock - 1) / kScanBlock;
@@ -142,12 +149,12 @@ static void scan_rec(int* in, int* out, int n, char* tmp, bool clear, cudaStream
   int* pref = sums + scan_pitch(nb);
   char* next = reinterpret_cast<char*>(pref + scan_pitch(nb)) + 256;
   scan_block_kernel<<<nb, 256, 0, st>>>(in, out, n, sums, clear);
-  scan_rec(sums, pref, nb, next, false, st);
-  scan_add_kernel<<<nb, 256, 0, st>>>(out, n, pref);
+  scan_rec(sums, pref, nb, next, false, nullptr, st);
+  scan_add_kernel<<<nb, 256, 0, st>>>(out, n, pref, total);
 }
 
-int exclusive_scan_i32(int* in, int* out, int n, void* tmp, bool clear, cudaStream_t st) {
-  scan_rec(in, out, n, reinterpret_cast<char*>(tmp), clear, st);
+int exclusive_scan_i32(int* in, int* out, int n, void* tmp, bool clear, int* total, cudaStream_t st) {
+  scan_rec(in, out, n, reinterpret_cast<char*>(tmp), clear, total, st);
   int launches = 1;
   for (int m = n; m >= 32 * 1024; m = (m + 1 + kScanBlock - 1) / kScanBlock) launches += 2;
   return launches;
@@ -264,6 +271,30 @@ void nb_place(const int* seg_of, const int* rank, int n, const int* start, int* 
   place_kernel<<<(n + 255) / 256, 256, 0, st>>>(seg_of, rank, n, start, sorted);
 }
 
+// The fill passes and what follows them are queued before the host knows the edge count: they take
+// the arrays' capacity and read the count (row_ptr[n]); a list that does not fit is left unwritten.
+__device__ __forceinline__ bool list_fits(const int* __restrict__ row_ptr, int n, int edge_cap) {
+  return (unsigned)row_ptr[n] <= (unsigned)edge_cap;
+}
+
+constexpr int kEdgeBlocks = 152 * 16;   // most blocks of the passes over a list of unknown length
+
+__global__ void __launch_bounds__(256) place_edges_kernel(const int* __restrict__ ej, const int* __restrict__ rank,
+                                                          const int* __restrict__ row_ptr, int n, int edge_cap,
+                                                          const int* __restrict__ col_ptr, int* __restrict__ col_edge) {
+  if (!list_fits(row_ptr, n, edge_cap)) return;
+  const int E = row_ptr[n];
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < E; e += gridDim.x * blockDim.x)
+    col_edge[col_ptr[ej[e]] + rank[e]] = e;
+}
+
+void nb_place_edges(const int* ej, const int* rank, const int* row_ptr, int n, int edge_cap, const int* col_ptr,
+                    int* col_edge, cudaStream_t st) {
+  if (edge_cap <= 0) return;
+  const int blocks = std::min((int)(((int64_t)edge_cap + 255) / 256), kEdgeBlocks);
+  place_edges_kernel<<<blocks, 256, 0, st>>>(ej, rank, row_ptr, n, edge_cap, col_ptr, col_edge);
+}
+
 // Sort each segment [start[s], start[s+1]) of distinct values: G lanes per segment hold up to 4 G
 // values in registers and each value's rank is the number of smaller ones (a broadcast per value),
 // so a segment takes a few dependent loads instead of an insertion sort's chain through memory.
@@ -331,15 +362,20 @@ __global__ void __launch_bounds__(256) sort_columns_kernel(const int* __restrict
 
 // Arrival order of every edge in its column, as a pass of its own: at large sizes the atomics cost
 // the fill pass more than they cost here (1,048,576 atoms: fill 2.51 -> 3.09 ms with them).
-__global__ void __launch_bounds__(256) col_rank_kernel(const int* __restrict__ ej, int E, int* __restrict__ col_count,
+__global__ void __launch_bounds__(256) col_rank_kernel(const int* __restrict__ ej, const int* __restrict__ row_ptr,
+                                                       int n, int edge_cap, int* __restrict__ col_count,
                                                        int* __restrict__ col_rank) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < E) col_rank[e] = atomicAdd(&col_count[ej[e]], 1);
+  if (!list_fits(row_ptr, n, edge_cap)) return;
+  const int E = row_ptr[n];
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < E; e += gridDim.x * blockDim.x)
+    col_rank[e] = atomicAdd(&col_count[ej[e]], 1);
 }
 
-void nb_col_rank(const int* ej, int E, int* col_count, int* col_rank, cudaStream_t st) {
-  if (E <= 0) return;
-  col_rank_kernel<<<(E + 255) / 256, 256, 0, st>>>(ej, E, col_count, col_rank);
+void nb_col_rank(const int* ej, const int* row_ptr, int n, int edge_cap, int* col_count, int* col_rank,
+                 cudaStream_t st) {
+  if (edge_cap <= 0) return;
+  const int blocks = std::min((int)(((int64_t)edge_cap + 255) / 256), kEdgeBlocks);
+  col_rank_kernel<<<blocks, 256, 0, st>>>(ej, row_ptr, n, edge_cap, col_count, col_rank);
 }
 
 void nb_sort_columns(const int* col_ptr, int n, int* col_edge, cudaStream_t st) {
@@ -380,7 +416,8 @@ __global__ void skin_filter_kernel(const double* __restrict__ pos, int n, const 
                                    const int* __restrict__ species, int ns, int* __restrict__ count,
                                    const int* __restrict__ row_ptr, int* __restrict__ ej, int* __restrict__ ei,
                                    int* __restrict__ eS, double* __restrict__ ed, int* __restrict__ col_count,
-                                   int* __restrict__ col_rank) {
+                                   int* __restrict__ col_rank, int edge_cap) {
+  if (fill && !list_fits(row_ptr, n, edge_cap)) return;
   const int lane = threadIdx.x & 31;
   const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (i >= n) return;
@@ -420,15 +457,17 @@ __global__ void skin_filter_kernel(const double* __restrict__ pos, int n, const 
 void nb_skin_filter(bool fill, const double* pos, int n, const double* d_cell, const int* sk_row, const int* sk_j,
                     const int* sk_S, double rc2, const double* pair_rc2, const int* species, int ns, int* count,
                     const int* row_ptr, int* ej, int* ei, int* eS, double* ed, int* col_count, int* col_rank,
-                    cudaStream_t st) {
+                    int edge_cap, cudaStream_t st) {
   if (n <= 0) return;
   const int threads = 256, blocks = (int)(((int64_t)n * 32 + threads - 1) / threads);
   if (fill)
     skin_filter_kernel<true><<<blocks, threads, 0, st>>>(pos, n, d_cell, sk_row, sk_j, sk_S, rc2, pair_rc2, species,
-                                                         ns, count, row_ptr, ej, ei, eS, ed, col_count, col_rank);
+                                                         ns, count, row_ptr, ej, ei, eS, ed, col_count, col_rank,
+                                                         edge_cap);
   else
     skin_filter_kernel<false><<<blocks, threads, 0, st>>>(pos, n, d_cell, sk_row, sk_j, sk_S, rc2, pair_rc2,
-                                                          species, ns, count, row_ptr, ej, ei, eS, ed, col_count, col_rank);
+                                                          species, ns, count, row_ptr, ej, ei, eS, ed, col_count, col_rank,
+                                                         edge_cap);
 }
 
 // Largest squared displacement of any atom since the reference positions, as
@@ -549,7 +588,8 @@ __global__ void __launch_bounds__(kSearchThreads) search_kernel(
     const float4* __restrict__ pos4, const double* __restrict__ pw, double rc2, float band,
     const double* __restrict__ pair_rc2, int ns, int* __restrict__ count, const int* __restrict__ row_ptr,
     int* __restrict__ ej, int* __restrict__ ei, int* __restrict__ eS, double* __restrict__ ed,
-    int* __restrict__ col_count, int* __restrict__ col_rank, int* __restrict__ d_err) {
+    int* __restrict__ col_count, int* __restrict__ col_rank, int edge_cap, int* __restrict__ d_err) {
+  if (fill && !list_fits(row_ptr, n, edge_cap)) return;
   constexpr int kWarps = kSearchThreads / 32;
   __shared__ SearchCell s_cell[kWarps][32];
   __shared__ int s_pref[kWarps][32];    // candidates before the cell
@@ -730,7 +770,8 @@ __global__ void __launch_bounds__(kSearchThreads) search_thread_kernel(
     const float4* __restrict__ pos4, const double* __restrict__ pw, double rc2, float band,
     const double* __restrict__ pair_rc2, int ns, int* __restrict__ count, const int* __restrict__ row_ptr,
     int* __restrict__ ej, int* __restrict__ ei, int* __restrict__ eS, double* __restrict__ ed,
-    int* __restrict__ d_err) {
+    int edge_cap, int* __restrict__ d_err) {
+  if (fill && !list_fits(row_ptr, n, edge_cap)) return;
   __shared__ int2 stage[fill ? kSearchThreads : 1][fill ? kFillStage : 1];
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   bool act = t < n;
@@ -890,19 +931,20 @@ __global__ void __launch_bounds__(kSearchThreads) search_thread_kernel(
 bool nb_search(bool fill, const double* pos, int n, const CellGrid& g, const int* cell_of,
                const int4* wraps, const int* cell_start, const int* sorted, const float4* pos4, const double* pw,
                double rc2, float band, const double* pair_rc2, int ns, int* count, const int* row_ptr, int* ej,
-               int* ei, int* eS, double* ed, int* col_count, int* col_rank, int* d_err, cudaStream_t st) {
+               int* ei, int* eS, double* ed, int* col_count, int* col_rank, int edge_cap, int* d_err,
+               cudaStream_t st) {
   if (n <= 0) return true;
   if (n <= kSearchWarpAtoms) {
     auto kernel = fill ? search_kernel<true> : search_kernel<false>;
     kernel<<<(n + kSearchThreads / 32 - 1) / (kSearchThreads / 32), kSearchThreads, 0, st>>>(
         pos, n, g, cell_of, wraps, cell_start, sorted, pos4, pw, rc2, band, pair_rc2, ns, count, row_ptr, ej, ei, eS, ed,
-        col_count, col_rank, d_err);
+        col_count, col_rank, edge_cap, d_err);
     return true;
   }
   auto kernel = fill ? search_thread_kernel<true> : search_thread_kernel<false>;
   kernel<<<(n + kSearchThreads - 1) / kSearchThreads, kSearchThreads, 0, st>>>(
       pos, n, g, cell_of, wraps, cell_start, sorted, pos4, pw, rc2, band, pair_rc2, ns, count, row_ptr, ej, ei, eS, ed,
-      d_err);
+      edge_cap, d_err);
   return false;
 }
 
@@ -918,7 +960,8 @@ __global__ void brute_batched_kernel(bool fill, const double* __restrict__ pos,
                                      int* __restrict__ count, const int* __restrict__ row_ptr,
                                      int* __restrict__ ej, int* __restrict__ ei, int* __restrict__ eS,
                                      double* __restrict__ ed, int* __restrict__ col_count,
-                                     int* __restrict__ col_rank, int* __restrict__ d_err) {
+                                     int* __restrict__ col_rank, int edge_cap, int* __restrict__ d_err) {
+  if (fill && !list_fits(row_ptr, n, edge_cap)) return;
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int b = atom_struct[i];
@@ -959,16 +1002,79 @@ __global__ void brute_batched_kernel(bool fill, const double* __restrict__ pos,
   }
 }
 
+// The same search for structures without cells (molecules): 16 lanes per centre test 16 atoms of its
+// structure at a time and a ballot places the accepted ones in the same order.  Without images a
+// test is 8 float64 operations instead of 26 (the offset is zero), and the rows are written with
+// lanes on consecutive edges.  Bound: float64 issue.
+template <bool fill>
+__global__ void __launch_bounds__(128) brute_nocell_kernel(const double* __restrict__ pos,
+                                                           const int64_t* __restrict__ offs, double rc2,
+                                                           const int* __restrict__ species,
+                                                           const double* __restrict__ pair_rc2, int ns,
+                                                           const int* __restrict__ atom_struct, int n,
+                                                           int* __restrict__ count, const int* __restrict__ row_ptr,
+                                                           int* __restrict__ ej, int* __restrict__ ei,
+                                                           int* __restrict__ eS, double* __restrict__ ed,
+                                                           int* __restrict__ col_count, int* __restrict__ col_rank,
+                                                           int edge_cap, int* __restrict__ d_err) {
+  if (fill && !list_fits(row_ptr, n, edge_cap)) return;
+  const int i = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 4);
+  if (i >= n) return;
+  const int lane = threadIdx.x & 15, half = threadIdx.x & 16;
+  const unsigned mask = 0xffffu << half;
+  const int b = atom_struct[i];
+  const int j0 = (int)offs[b], j1 = (int)offs[b + 1];
+  const double pi[3] = {pos[3 * (size_t)i], pos[3 * (size_t)i + 1], pos[3 * (size_t)i + 2]};
+  const double* prow = pair_rc2 ? pair_rc2 + (size_t)species[i] * ns : nullptr;
+  const int base = fill ? row_ptr[i] : 0;
+  const int cap = fill ? (row_ptr[i + 1] - base) : 0;
+  int k = 0;
+  for (int jb = j0; jb < j1; jb += 16) {
+    const int j = jb + lane;
+    bool keep = false;
+    double d[3] = {0.0, 0.0, 0.0};
+    if (j < j1 && j != i) {
+#pragma unroll
+      for (int x = 0; x < 3; ++x) d[x] = __dsub_rn(pos[3 * (size_t)j + x], pi[x]);
+      const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1])), __dmul_rn(d[2], d[2]));
+      keep = r2 < (prow ? prow[species[j]] : rc2);   // the ordered pair's cutoff
+    }
+    const unsigned m = __ballot_sync(mask, keep) >> half;
+    const int kk = k + __popc(m & ((1u << lane) - 1u));
+    if (fill && keep && kk < cap) {
+      const size_t o = (size_t)base + kk;
+      col_rank[o] = atomicAdd(&col_count[j], 1);
+      ej[o] = j;
+      ei[o] = i;
+      eS[3 * o] = 0; eS[3 * o + 1] = 0; eS[3 * o + 2] = 0;
+      ed[3 * o] = d[0]; ed[3 * o + 1] = d[1]; ed[3 * o + 2] = d[2];
+    }
+    k += __popc(m);
+  }
+  if (lane == 0) {
+    if (!fill) count[i] = k;
+    else if (k != cap) atomicOr(d_err, kErrNeighbor);
+  }
+}
+
 void nb_bruteforce_batched(bool fill, const double* pos, const int64_t* offs, int nstruct,
                            const double* cells, const int* pbc, const int* nimg, double rc2,
                            const int* species, const double* pair_rc2, int ns,
                            const int* atom_struct, int n, int* count, const int* row_ptr, int* ej,
-                           int* ei, int* eS, double* ed, int* col_count, int* col_rank, int* d_err, cudaStream_t st) {
+                           int* ei, int* eS, double* ed, int* col_count, int* col_rank, int edge_cap, int* d_err,
+                           cudaStream_t st) {
   (void)nstruct;
   if (n <= 0) return;
+  if (!cells) {
+    auto kernel = fill ? brute_nocell_kernel<true> : brute_nocell_kernel<false>;
+    kernel<<<(unsigned)(((int64_t)n * 16 + 127) / 128), 128, 0, st>>>(pos, offs, rc2, species, pair_rc2, ns, atom_struct,
+                                                                      n, count, row_ptr, ej, ei, eS, ed, col_count,
+                                                                      col_rank, edge_cap, d_err);
+    return;
+  }
   brute_batched_kernel<<<(n + 127) / 128, 128, 0, st>>>(fill, pos, offs, cells, pbc, nimg, rc2, species, pair_rc2,
                                                         ns, atom_struct, n, count, row_ptr, ej, ei, eS, ed,
-                                                        col_count, col_rank, d_err);
+                                                        col_count, col_rank, edge_cap, d_err);
 }
 
 // Per structure: spread (max - min) of the fractional coordinates, so the
