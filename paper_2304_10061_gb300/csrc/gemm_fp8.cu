@@ -17,12 +17,15 @@
 // rounding (3 mantissa bits) remains.
 //
 // gemm_fp8_kernel<BN>: persistent, one CTA per SM walking 128 x BN tiles.
-//   warp 0      TMA: B k-blocks (BN rows x 128 E4M3 bytes) into the operand
-//               ring, A k-blocks as two 128 x 64 bf16 halves into a staging ring
+//   warp 0      TMA: B k-blocks (BN rows x 128 E4M3 bytes) into the operand ring
+//   warp 14     TMA: A k-blocks as two 128 x 64 bf16 halves into a staging ring (a
+//               producer of its own, so that A, which comes from HBM, runs up to
+//               three k-blocks ahead whatever the two-deep B ring, filled from L2, waits for)
 //   warp 1      TMEM (two BN-column accumulators), tcgen05.mma kind::f8f6f4
 //               (M = 128, N = BN, K = 32 per instruction) from one thread
 //   warps 2-9   epilogue: tcgen05.ld, times sA sB, the float32/bf16 epilogue,
-//               16-byte row stores, the output's amax
+//               32 x 32 boxes through shared memory (pre-activations fetched a
+//               chunk ahead, outputs stored by TMA), the output's amax
 //   warps 10-13 converters: each staging half -> E4M3 (times 1/sA) into the
 //               operand ring's A slot in the 128-byte-swizzled K-major layout
 //               the tensor core reads (16 E4M3 per 16-byte unit, unit u of
@@ -37,6 +40,7 @@
 #include <cstring>
 
 #include "amax.cuh"
+#include "epi_stage.cuh"
 #include "epilogue.cuh"
 #include "internal.h"
 #include "tc_ptx.cuh"
@@ -44,12 +48,14 @@
 namespace alg {
 
 constexpr int kF8BK = 128;                          // E4M3 elements per operand k-block (one 128-byte row)
-constexpr int kF8Stages = 3;                        // operand ring depth (k-blocks)
-constexpr int kF8Stg = 4;                           // bf16 staging ring depth (64-column halves)
+constexpr int kF8Stages = 2;                        // operand ring depth (k-blocks)
+constexpr int kF8Stg = 6;                           // bf16 staging ring depth (64-column halves)
 constexpr int kF8EpiWarps = 8;
+constexpr uint32_t kF8EpiSlot = 4096;               // staging per epilogue warp: two bf16 boxes or one float32 box
 constexpr int kF8ConvWarps = 4;
 constexpr int kF8ConvWarp0 = 2 + kF8EpiWarps;      // first converter warp
-constexpr int kF8Threads = 32 * (kF8ConvWarp0 + kF8ConvWarps);
+constexpr int kF8AWarp = kF8ConvWarp0 + kF8ConvWarps;   // TMA producer of the A staging halves
+constexpr int kF8Threads = 32 * (kF8AWarp + 1);
 constexpr uint32_t kF8ABytes = 128 * kF8BK;         // one E4M3 A k-block
 constexpr uint32_t kF8StgBytes = 128 * 64 * 2;      // one bf16 staging half
 constexpr float kF8Target = 224.0f;                 // largest |A| / sA (half of the E4M3 maximum 448)
@@ -64,7 +70,8 @@ __host__ __device__ constexpr int f8_tmem_cols() {
 }
 template <int BN>
 __host__ __device__ constexpr int f8_smem_bytes() {
-  return kF8Stages * (int)(kF8ABytes + f8_b_bytes<BN>()) + kF8Stg * (int)kF8StgBytes + 1024 + 1024;
+  return kF8Stages * (int)(kF8ABytes + f8_b_bytes<BN>()) + kF8Stg * (int)kF8StgBytes + kF8EpiWarps * (int)kF8EpiSlot + 1024 +
+         1024;
 }
 
 // Instruction descriptor, kind::f8f6f4: D float32 (bits 4-5 = 1), A and B E4M3
@@ -113,7 +120,7 @@ __device__ __forceinline__ float f8_sigmoid(float z) {
 }
 
 // 32 consecutive columns [n, n + 32) of row m (v already times sA sB): the epilogue of
-// the bf16-storage path with plain stores; returns max|output| of an activation output
+// the bf16-storage path with plain stores (rows that TMA cannot move); returns max|output| of an activation output
 // (0 for the float32 output)
 __device__ __forceinline__ float f8_epilogue(const EpiParams& ep, int m, int n, int N, float (&v)[32]) {
   const bool full = (n + 32 <= N) && ep.vec;
@@ -204,6 +211,7 @@ __device__ __forceinline__ void fence_async_smem_f8() {
 
 struct F8Params {
   int M, N, K, K1;              // A columns [0, K1) from tmA, [K1, K) from tmA2
+  int maps;                     // 1: every epilogue array can be moved by TMA
   float sB;                     // the weights' scale
   const unsigned* amax_a;       // amax slots of A and A2 (float bits)
   const unsigned* amax_a2;
@@ -214,7 +222,8 @@ struct F8Params {
 template <int BN>
 __global__ void __launch_bounds__(kF8Threads, 1)
     gemm_fp8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA2,
-                    const __grid_constant__ CUtensorMap tmB, EpiParams ep, F8Params fp) {
+                    const __grid_constant__ CUtensorMap tmB, const __grid_constant__ EpiMaps em, EpiParams ep,
+                    F8Params fp) {
   constexpr uint32_t B_BYTES = f8_b_bytes<BN>();
   constexpr uint32_t COLS = f8_tmem_cols<BN>();
   extern __shared__ uint8_t smem_raw[];
@@ -222,14 +231,16 @@ __global__ void __launch_bounds__(kF8Threads, 1)
   uint8_t* sA = smem;                                  // [kF8Stages] E4M3 A k-blocks
   uint8_t* sB = sA + kF8Stages * kF8ABytes;            // [kF8Stages] E4M3 B k-blocks
   uint8_t* sS = sB + kF8Stages * B_BYTES;              // [kF8Stg] bf16 staging halves
-  uint64_t* full = reinterpret_cast<uint64_t*>(sS + kF8Stg * kF8StgBytes);   // B landed
+  uint8_t* sE = sS + kF8Stg * kF8StgBytes;             // epilogue staging
+  uint64_t* full = reinterpret_cast<uint64_t*>(sE + kF8EpiWarps * kF8EpiSlot);   // B landed
   uint64_t* afull = full + kF8Stages;                  // A converted (one arrival per converter warp)
   uint64_t* empty = afull + kF8Stages;                 // the MMAs of the stage are complete
   uint64_t* sfull = empty + kF8Stages;                 // staging half landed
   uint64_t* sempty = sfull + kF8Stg;                   // staging half read (one arrival per converter warp)
   uint64_t* tfull = sempty + kF8Stg;                   // [2] accumulator ready
   uint64_t* tempty = tfull + 2;                        // [2] accumulator drained (one arrival per epilogue warp)
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(tempty + 2);
+  uint64_t* inbar = tempty + 2;                        // [kF8EpiWarps] input box filled
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(inbar + kF8EpiWarps);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -256,6 +267,7 @@ __global__ void __launch_bounds__(kF8Threads, 1)
       mbar_init(&tfull[b], 1);
       mbar_init(&tempty[b], kF8EpiWarps);
     }
+    for (int w = 0; w < kF8EpiWarps; ++w) mbar_init(&inbar[w], 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -274,7 +286,7 @@ __global__ void __launch_bounds__(kF8Threads, 1)
       uint32_t g = 0;   // global k-block counter
       bool ok = true;
       for (int t = blockIdx.x; t < ntiles && ok && !*abort_flag; t += gridDim.x) {
-        const int m0 = tm0(t), n0 = tn0(t);
+        const int n0 = tn0(t);
         for (int kb = 0; kb < nk; ++kb, ++g) {
           const uint32_t s = g % kF8Stages, r = g / kF8Stages;
           if (g >= (uint32_t)kF8Stages && !mbar_wait(&empty[s], (r - 1) & 1)) {
@@ -283,19 +295,30 @@ __global__ void __launch_bounds__(kF8Threads, 1)
           }
           mbar_expect_tx(&full[s], B_BYTES);
           tma_load_2d(sB + s * B_BYTES, &tmB, &full[s], kb * kF8BK, n0);
-          for (int h = 0; h < 2 && ok; ++h) {
-            const uint32_t g2 = 2 * g + h, s2 = g2 % kF8Stg, r2 = g2 / kF8Stg;
-            if (g2 >= (uint32_t)kF8Stg && !mbar_wait(&sempty[s2], (r2 - 1) & 1)) {
-              ok = false;
-              break;
-            }
-            mbar_expect_tx(&sfull[s2], kF8StgBytes);
-            // first column of this half: A1 below K1, A2 up to K, past K (read as zero) from A1's map
-            const int kc = kb * kF8BK + 64 * h;
-            if (kc < fp.K1 || kc >= K) tma_load_2d(sS + s2 * kF8StgBytes, &tmA, &sfull[s2], kc, m0);
-            else tma_load_2d(sS + s2 * kF8StgBytes, &tmA2, &sfull[s2], kc - fp.K1, m0);
+        }
+      }
+      if (!ok) {
+        atomicOr(fp.err, kErrTimeout);
+        *abort_flag = 1;
+      }
+    }
+  } else if (warp == kF8AWarp) {
+    if (lane == 0) {
+      uint32_t g2 = 0;   // global half counter
+      bool ok = true;
+      for (int t = blockIdx.x; t < ntiles && ok && !*abort_flag; t += gridDim.x) {
+        const int m0 = tm0(t);
+        for (int hb = 0; hb < 2 * nk; ++hb, ++g2) {
+          const uint32_t s2 = g2 % kF8Stg, r2 = g2 / kF8Stg;
+          if (g2 >= (uint32_t)kF8Stg && !mbar_wait(&sempty[s2], (r2 - 1) & 1)) {
+            ok = false;
+            break;
           }
-          if (!ok) break;
+          mbar_expect_tx(&sfull[s2], kF8StgBytes);
+          // first column of this half: A1 below K1, A2 up to K, past K (read as zero) from A1's map
+          const int kc = 64 * hb;
+          if (kc < fp.K1 || kc >= K) tma_load_2d(sS + s2 * kF8StgBytes, &tmA, &sfull[s2], kc, m0);
+          else tma_load_2d(sS + s2 * kF8StgBytes, &tmA2, &sfull[s2], kc - fp.K1, m0);
         }
       }
       if (!ok) {
@@ -341,7 +364,21 @@ __global__ void __launch_bounds__(kF8Threads, 1)
   } else if (warp < kF8ConvWarp0) {
     // epilogue: 2 warps per TMEM lane quarter, alternating 32-column chunks
     const int q = warp & 3;
-    const int h = (warp - 2) >> 2;
+    const int ew = warp - 2;
+    const int h = ew >> 2;
+    // staging: the output box (2 KB bf16, 4 KB float32), then the pre-activation box, stored or fetched
+    uint8_t* box0 = sE + ew * kF8EpiSlot;
+    uint8_t* box1 = box0 + 2048;
+    const bool store_pre = fp.maps && ep.epi == EPI_FWD_SILU && ep.pre;
+    const bool input = fp.maps && ep.epi == EPI_BWD_SILU;
+    uint32_t in_par = 0;
+    auto nch_of = [&](int tt) { return (min(BN, N - tn0(tt)) + 31) / 32; };
+    auto fetch = [&](int tt, int cc) {   // pre-activation box of chunk cc of tile tt
+      if (!input || lane != 0) return;
+      mbar_expect_tx(&inbar[ew], 2048);
+      tma_load_2d(box1, &em.pre, &inbar[ew], tn0(tt) + 32 * cc, tm0(tt) + q * 32);
+    };
+    if (h < nch_of(blockIdx.x)) fetch(blockIdx.x, h);
     float scA, invA;
     f8_scale(f8_amax_bits(fp.amax_a, fp.amax_a2), scA, invA);
     const float sab = scA * fp.sB;
@@ -359,18 +396,68 @@ __global__ void __launch_bounds__(kF8Threads, 1)
       const int m0 = tm0(t), n0 = tn0(t);
       const int m = m0 + q * 32 + lane;
       const uint32_t base = tmem + (uint32_t)(b * COLS) + ((uint32_t)(q * 32) << 16);
-      const int nch = (min(BN, N - n0) + 31) / 32;
+      const int nch = nch_of(t);
+      const float rs = (ep.rowscale && m < M) ? ep.rowscale[m] : 1.0f;
       for (int c = h; c < nch; c += 2) {
         float v[32];
+        uint32_t zw[16];
+        if (input) {
+          if (!mbar_wait(&inbar[ew], in_par)) {
+            if (lane == 0) atomicOr(fp.err, kErrTimeout);
+            *abort_flag = 1;
+          }
+          in_par ^= 1u;
+          ld_bf16_row_raw(box1, lane, zw);
+          // the box's generic reads are ordered before the next TMA write into it
+          fence_async_smem();
+          __syncwarp();
+          if (c + 2 < nch) fetch(t, c + 2);
+          else if (t + (int)gridDim.x < ntiles && h < nch_of(t + gridDim.x)) fetch(t + gridDim.x, h);
+        }
         tc_ld32(base + (uint32_t)(32 * c), v);
 #pragma unroll
         for (int j = 0; j < 32; ++j) v[j] *= sab;
-        if (m < M) amx = fmaxf(amx, f8_epilogue(ep, m, n0 + 32 * c, N, v));
+        if (!fp.maps) {
+          if (m < M) amx = fmaxf(amx, f8_epilogue(ep, m, n0 + 32 * c, N, v));
+          continue;
+        }
+        // the boxes are free once the store that used them has read them
+        if (lane == 0) bulk_wait_read0();
+        __syncwarp();
+        if (ep.epi == EPI_F32) {
+          st_f32_row(box0, lane, v);
+        } else {
+          if (ep.epi == EPI_FWD_SILU) {
+            if (store_pre) st_bf16_row(box1, lane, v);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] = v[j] * f8_sigmoid(v[j]) * rs;
+          } else if (ep.epi == EPI_BWD_SILU) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+              const float z = bf16_word_elem(zw, j);
+              const float sg = f8_sigmoid(z);
+              v[j] = v[j] * sg * (1.0f + z * (1.0f - sg));
+            }
+          }
+          // (rows past M and columns past N are zero here: their operands are read as zero)
+#pragma unroll
+          for (int j = 0; j < 32; ++j) amx = fmaxf(amx, fabsf(v[j]));
+          st_bf16_row(box0, lane, v);
+        }
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+          tma_store_2d(&em.out, box0, n0 + 32 * c, m0 + q * 32);
+          if (store_pre) tma_store_2d(&em.pre, box1, n0 + 32 * c, m0 + q * 32);
+          bulk_commit();
+        }
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&tempty[b]);
     }
+    if (lane == 0) bulk_wait_all();
+    __syncwarp();
     record_amax(fp.amax_out, amx);
   } else {
     // converters: staging halves (bf16, 128-byte swizzle: 8-element unit u of row r at
@@ -479,9 +566,18 @@ static bool launch_fp8(const GemmArgs& g, const uint8_t* B8, int ldb8, float sB,
   fp.amax_a = g.amax_a; fp.amax_a2 = g.A2 ? g.amax_a2 : nullptr;
   fp.amax_out = g.amax_out;
   fp.err = d_err;
+  const EpiParams ep = make_epi(g);
+  EpiMaps em;
+  memset(&em, 0, sizeof em);
+  fp.maps = ep.vec && !g.add;
+  if (fp.maps && (!tc_box_map(&em.out, g.out, g.N, g.M, g.ldo, g.epi == EPI_F32 ? 4 : 2) ||
+                  (g.pre && !tc_box_map(&em.pre, g.pre, g.N, g.M, g.ldp, 2)))) {
+    if (why) *why = "cuTensorMapEncodeTiled failed (FP8 GEMM epilogue)";
+    return false;
+  }
   const int tiles = ((g.M + 127) / 128) * ((g.N + BN - 1) / BN);
   const int grid = tiles < nsm[dev] ? tiles : nsm[dev];
-  gemm_fp8_kernel<BN><<<grid, kF8Threads, smem, st>>>(ta, ta2, tb, make_epi(g), fp);
+  gemm_fp8_kernel<BN><<<grid, kF8Threads, smem, st>>>(ta, ta2, tb, em, ep, fp);
   return true;
 }
 

@@ -28,6 +28,7 @@
 #include <cstdint>
 #include <cstring>
 
+#include "epi_stage.cuh"
 #include "epilogue.cuh"
 #include "internal.h"
 #include "tc_ptx.cuh"
@@ -82,6 +83,18 @@ bool tc_tensor_map_2d(CUtensorMap* tm, CUtensorMapDataType dtype, int esize, con
   return r == CUDA_SUCCESS;
 }
 
+
+bool tc_box_map(CUtensorMap* tm, const void* base, int cols, int rows, int ld, int esize) {
+  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+  cuuint64_t strides[1] = {(cuuint64_t)ld * esize};
+  cuuint32_t box[2] = {32, 32};
+  cuuint32_t estr[2] = {1, 1};
+  CUresult r = g_encode(tm, esize == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
+                        const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                        esize == 2 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                        CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS;
+}
 
 // Instruction descriptor, kind::f16: D f32, A bf16, B bf16, both K-major, M = 128, N = BN.
 template <int BN>
@@ -144,73 +157,6 @@ static size_t tc_smem_bytes(const TcLayout& L) {
   return (size_t)L.stages * tc_stage_bytes<BN>() + (size_t)4 * EPQ * L.epi_slot + 1024 + kTcMisc;
 }
 
-// --- epilogue staging: 32 x 32 boxes moved by TMA --------------------------
-// bf16 box rows are 64 bytes (64-byte swizzle), float32 box rows 128 bytes
-// (128-byte swizzle); the 16-byte unit u of row r sits at unit u ^ f(r) so the
-// row-per-lane accesses spread over all banks.
-__device__ __forceinline__ uint32_t sw64(int r, int u) { return r * 64 + ((u ^ ((r >> 1) & 3)) << 4); }
-__device__ __forceinline__ uint32_t sw128(int r, int u) { return r * 128 + ((u ^ (r & 7)) << 4); }
-
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap* tm, const void* src, int c0, int c1) {
-  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(
-                   reinterpret_cast<uint64_t>(tm)),
-               "r"(smem_u32(src)), "r"(c0), "r"(c1)
-               : "memory");
-}
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_read1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_read0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-__device__ __forceinline__ void st_bf16_row(uint8_t* box, int r, const float (&v)[32]) {
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    uint4 x = make_uint4(pack_bf16x2(v[8 * u + 0], v[8 * u + 1]), pack_bf16x2(v[8 * u + 2], v[8 * u + 3]),
-                         pack_bf16x2(v[8 * u + 4], v[8 * u + 5]), pack_bf16x2(v[8 * u + 6], v[8 * u + 7]));
-    *reinterpret_cast<uint4*>(box + sw64(r, u)) = x;
-  }
-}
-__device__ __forceinline__ void ld_bf16_row(const uint8_t* box, int r, float (&v)[32]) {
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    uint4 x = *reinterpret_cast<const uint4*>(box + sw64(r, u));
-    uint32_t w[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      float2 f = __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&w[t]));
-      v[8 * u + 2 * t] = f.x;
-      v[8 * u + 2 * t + 1] = f.y;
-    }
-  }
-}
-__device__ __forceinline__ void st_f32_row(uint8_t* box, int r, const float (&v)[32]) {
-#pragma unroll
-  for (int u = 0; u < 8; ++u)
-    *reinterpret_cast<float4*>(box + sw128(r, u)) = make_float4(v[4 * u], v[4 * u + 1], v[4 * u + 2], v[4 * u + 3]);
-}
-__device__ __forceinline__ void ld_f32_row(const uint8_t* box, int r, float (&v)[32]) {
-#pragma unroll
-  for (int u = 0; u < 8; ++u) {
-    float4 x = *reinterpret_cast<const float4*>(box + sw128(r, u));
-    v[4 * u] = x.x; v[4 * u + 1] = x.y; v[4 * u + 2] = x.z; v[4 * u + 3] = x.w;
-  }
-}
-
-// 16 columns (half hh of a 32-column box row) into the swizzled staging boxes.
-__device__ __forceinline__ void st_bf16_half(uint8_t* box, int r, int hh, const float (&v)[16]) {
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    uint4 x = make_uint4(pack_bf16x2(v[8 * u + 0], v[8 * u + 1]), pack_bf16x2(v[8 * u + 2], v[8 * u + 3]),
-                         pack_bf16x2(v[8 * u + 4], v[8 * u + 5]), pack_bf16x2(v[8 * u + 6], v[8 * u + 7]));
-    *reinterpret_cast<uint4*>(box + sw64(r, 2 * hh + u)) = x;
-  }
-}
-__device__ __forceinline__ void st_f32_half(uint8_t* box, int r, int hh, const float (&v)[16]) {
-#pragma unroll
-  for (int u = 0; u < 4; ++u)
-    *reinterpret_cast<float4*>(box + sw128(r, 4 * hh + u)) = make_float4(v[4 * u], v[4 * u + 1], v[4 * u + 2], v[4 * u + 3]);
-}
 __device__ __forceinline__ void load_bf16x16(const bf16* p, float (&v)[16]) {
   const uint4* q = reinterpret_cast<const uint4*>(p);
 #pragma unroll
@@ -257,23 +203,6 @@ __device__ __forceinline__ float2 bf16_word_pair(uint32_t x) {
   return make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u));
 }
 
-struct EpiMaps {
-  CUtensorMap out, pre, add;
-};
-
-// Raw bf16 words of one 32-column row of a swizzled bf16 32x32 box (16 words).
-__device__ __forceinline__ void ld_bf16_row_raw(const uint8_t* box, int r, uint32_t (&w)[16]) {
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const uint4 x = *reinterpret_cast<const uint4*>(box + sw64(r, u));
-    w[4 * u] = x.x; w[4 * u + 1] = x.y; w[4 * u + 2] = x.z; w[4 * u + 3] = x.w;
-  }
-}
-// element j (0..31) of such a row
-__device__ __forceinline__ float bf16_word_elem(const uint32_t (&w)[16], int j) {
-  const uint32_t x = w[j >> 1];
-  return __uint_as_float((j & 1) ? (x & 0xffff0000u) : (x << 16));
-}
 
 // Persistent kernel: CTA b handles tiles b, b + gridDim.x, ...  Two TMEM
 // accumulator buffers: the MMA warp fills buffer (t & 1) while the epilogue
@@ -1126,20 +1055,6 @@ static bool smem_opt_in(K kernel, int bytes, bool (&done)[kMaxDevices], int dev,
   return true;
 }
 
-// 2-D tensor map over a row-major [rows][ld] array of `esize`-byte elements,
-// box 32 x 32, swizzle matched to the row width of the box.
-static bool make_box_map(CUtensorMap* tm, const void* base, int cols, int rows, int ld, int esize) {
-  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)ld * esize};
-  cuuint32_t box[2] = {32, 32};
-  cuuint32_t estr[2] = {1, 1};
-  CUresult r = g_encode(tm, esize == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
-                        const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        esize == 2 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
-                        CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS;
-}
-
 template <int BN, int EPQ>
 static bool launch_bn(const GemmArgs& g, const bf16* B, int ldb, cudaStream_t st, int* d_err, std::string* why) {
   static bool attr_set[kMaxDevices] = {};
@@ -1158,9 +1073,9 @@ static bool launch_bn(const GemmArgs& g, const bf16* B, int ldb, cudaStream_t st
   EpiMaps em;
   memset(&em, 0, sizeof em);
   const bool f32out = (g.epi == EPI_F32);
-  bool ok = make_box_map(&em.out, g.out, g.N, g.M, g.ldo, f32out ? 4 : 2);
-  if (ok && g.pre) ok = make_box_map(&em.pre, g.pre, g.N, g.M, g.ldp, 2);
-  if (ok && g.add) ok = make_box_map(&em.add, g.add, g.N, g.M, g.ld_add, 2);
+  bool ok = tc_box_map(&em.out, g.out, g.N, g.M, g.ldo, f32out ? 4 : 2);
+  if (ok && g.pre) ok = tc_box_map(&em.pre, g.pre, g.N, g.M, g.ldp, 2);
+  if (ok && g.add) ok = tc_box_map(&em.add, g.add, g.N, g.M, g.ld_add, 2);
   if (!ok) {
     if (why) *why = "cuTensorMapEncodeTiled failed for an epilogue operand";
     return false;
@@ -1236,11 +1151,11 @@ static bool launch_chain_pipe(const GemmArgs& g1, const GemmArgs& g2, const bf16
                       (uint64_t)(g1.A2 ? g1.lda2 : g1.lda) * 2, kTcBK, kTcBM) &&
             make_tmap(&cm.b1, B1, (uint64_t)g1.K, (uint64_t)g1.N, (uint64_t)ldb1 * 2, kTcBK, kCfJobN) &&
             make_tmap(&cm.b2, B2, (uint64_t)g2.K, (uint64_t)g2.N, (uint64_t)ldb2 * 2, kTcBK, N2);
-  if (ok && g1.pre) ok = make_box_map(&cm.pre1, g1.pre, g1.N, g1.M, g1.ldp, 2);
-  if (ok && g1.epi == EPI_BWD_SILU) ok = make_box_map(&cm.out1, g1.out, g1.N, g1.M, g1.ldo, 2);
+  if (ok && g1.pre) ok = tc_box_map(&cm.pre1, g1.pre, g1.N, g1.M, g1.ldp, 2);
+  if (ok && g1.epi == EPI_BWD_SILU) ok = tc_box_map(&cm.out1, g1.out, g1.N, g1.M, g1.ldo, 2);
   if (ok && g2.pre && (g2.epi == EPI_FWD_SILU || g2.epi == EPI_BWD_SILU))
-    ok = make_box_map(&cm.pre2, g2.pre, g2.N, g2.M, g2.ldp, 2);
-  if (ok) ok = make_box_map(&cm.out2, g2.out, g2.N, g2.M, g2.ldo, 2);
+    ok = tc_box_map(&cm.pre2, g2.pre, g2.N, g2.M, g2.ldp, 2);
+  if (ok) ok = tc_box_map(&cm.out2, g2.out, g2.N, g2.M, g2.ldo, 2);
   if (!ok) {
     if (why) *why = "cuTensorMapEncodeTiled failed (chain)";
     return false;
@@ -1306,7 +1221,11 @@ bool gemm_chain_bf16(const GemmArgs& g1, const GemmArgs& g2, cudaStream_t st, in
 // shared-memory ring, warp 1 owns two BN-column TMEM accumulators and issues
 // tcgen05.mma.kind::tf32 (K = 8 per instruction) from one thread, 8 epilogue
 // warps (2 per TMEM lane quarter, alternating 32-column chunks) read the
-// accumulator with tcgen05.ld and write their rows with 16-byte stores.
+// accumulator with tcgen05.ld, fetch their inputs (pre-activation or addend) by
+// TMA a chunk ahead and write 32 x 32 boxes through shared memory with TMA
+// stores.  The epilogue's memory accesses bound this kernel: with a row per lane
+// in global memory a 128 x 256 SiLU tile took 16,000 LSU cycles against 600 per
+// 32-column k-block of MMAs.
 // ---------------------------------------------------------------------------
 constexpr int kT32BK = 32;                     // float32 elements per 128-byte operand row
 constexpr int kT32Threads = 64 + 8 * 32;
@@ -1331,17 +1250,17 @@ template <int BN>
 __host__ __device__ constexpr int t32_stage_bytes() {
   return 128 * kT32BK * 4 + BN * kT32BK * 4;
 }
+constexpr int kT32EpiWarps = 8;
+constexpr int kT32Box = 32 * 32 * 4;           // one float32 staging box
+// operand stages beside `epi_slot` bytes of staging per epilogue warp
 template <int BN>
-__host__ __device__ constexpr int t32_stages() {
-  return (kTcSmemMax - 1024 - 1024) / t32_stage_bytes<BN>() > 6 ? 6
-                                                               : (kTcSmemMax - 1024 - 1024) / t32_stage_bytes<BN>();
-}
-template <int BN>
-__host__ __device__ constexpr int t32_smem_bytes() {
-  return t32_stages<BN>() * t32_stage_bytes<BN>() + 1024 + 1024;
+static int t32_stages(int epi_slot) {
+  const int st = (kTcSmemMax - 1024 - 1024 - kT32EpiWarps * epi_slot) / t32_stage_bytes<BN>();
+  return st > 6 ? 6 : st;
 }
 
-// 32 consecutive float32 columns of one row: epilogue of the float32 path
+// 32 consecutive float32 columns of one row: epilogue of the float32 path (rows that TMA cannot
+// move: a start or pitch that is not a multiple of 16 bytes)
 __device__ __forceinline__ void t32_epilogue(const EpiParams& ep, int m, int n, int N, float (&v)[32]) {
   const bool full = (n + 32 <= N) && ep.vec;
   if (ep.epi == EPI_FWD_SILU) {
@@ -1408,9 +1327,9 @@ __device__ __forceinline__ void t32_epilogue(const EpiParams& ep, int m, int n, 
 
 template <int BN>
 __global__ void __launch_bounds__(kT32Threads, 1)
-    gemm_tf32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, EpiParams ep,
-                     int M, int N, int K, int* __restrict__ err) {
-  constexpr int STAGES = t32_stages<BN>();
+    gemm_tf32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                     const __grid_constant__ EpiMaps em, EpiParams ep, int STAGES, int epi_slot, int M, int N, int K,
+                     int* __restrict__ err) {
   constexpr uint32_t A_BYTES = 128 * kT32BK * 4;
   constexpr uint32_t B_BYTES = BN * kT32BK * 4;
   constexpr uint32_t COLS = tc_tmem_cols<BN>();
@@ -1418,11 +1337,13 @@ __global__ void __launch_bounds__(kT32Threads, 1)
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = smem;
   uint8_t* sB = smem + STAGES * A_BYTES;
-  uint64_t* full = reinterpret_cast<uint64_t*>(sB + STAGES * B_BYTES);
+  uint8_t* sE = sB + STAGES * B_BYTES;                       // epilogue staging (1024-aligned)
+  uint64_t* full = reinterpret_cast<uint64_t*>(sE + kT32EpiWarps * epi_slot);
   uint64_t* empty = full + STAGES;
   uint64_t* tfull = empty + STAGES;   // [2]
   uint64_t* tempty = tfull + 2;       // [2]
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(tempty + 2);
+  uint64_t* inbar = tempty + 2;       // [kT32EpiWarps]: input box filled
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(inbar + kT32EpiWarps);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1439,8 +1360,9 @@ __global__ void __launch_bounds__(kT32Threads, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&tfull[b], 1);
-      mbar_init(&tempty[b], 8);
+      mbar_init(&tempty[b], kT32EpiWarps);
     }
+    for (int w = 0; w < kT32EpiWarps; ++w) mbar_init(&inbar[w], 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -1509,7 +1431,22 @@ __global__ void __launch_bounds__(kT32Threads, 1)
     __syncwarp();
   } else {
     const int q = warp & 3;        // TMEM lane quarter this warp may access
-    const int h = (warp - 2) >> 2; // 0 or 1: alternating 32-column chunks
+    const int ew = warp - 2;
+    const int h = ew >> 2;         // 0 or 1: alternating 32-column chunks
+    // staging: the output box, then the pre-activation box (stored) or the input box (fetched)
+    uint8_t* box0 = sE + ew * epi_slot;
+    uint8_t* box1 = box0 + kT32Box;
+    const bool maps = epi_slot != 0;   // else every access by the lanes themselves
+    const bool store_pre = maps && ep.epi == EPI_FWD_SILU && ep.pre;
+    const bool input = maps && (ep.epi == EPI_BWD_SILU || (ep.epi == EPI_F32 && ep.add));
+    uint32_t in_par = 0;
+    auto nch_of = [&](int tt) { return (min(BN, N - tn0(tt)) + 31) / 32; };
+    auto fetch = [&](int tt, int cc) {   // input box of chunk cc of tile tt
+      if (!input || lane != 0) return;
+      mbar_expect_tx(&inbar[ew], kT32Box);
+      tma_load_2d(box1, ep.epi == EPI_BWD_SILU ? &em.pre : &em.add, &inbar[ew], tn0(tt) + 32 * cc, tm0(tt) + q * 32);
+    };
+    if (h < nch_of(blockIdx.x)) fetch(blockIdx.x, h);
     int lt = 0;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++lt) {
       const int b = lt & 1, use = lt >> 1;
@@ -1523,16 +1460,62 @@ __global__ void __launch_bounds__(kT32Threads, 1)
       const int m0 = tm0(t), n0 = tn0(t);
       const int m = m0 + q * 32 + lane;
       const uint32_t base = tmem + (uint32_t)(b * COLS) + ((uint32_t)(q * 32) << 16);
-      const int nch = (min(BN, N - n0) + 31) / 32;
+      const int nch = nch_of(t);
+      const float rs = (ep.rowscale && m < M) ? ep.rowscale[m] : 1.0f;
       for (int c = h; c < nch; c += 2) {
-        float v[32];
+        float v[32], z[32];
+        if (input) {
+          if (!mbar_wait(&inbar[ew], in_par)) {
+            if (lane == 0) atomicOr(err, kErrTimeout);
+            *abort_flag = 1;
+          }
+          in_par ^= 1u;
+          ld_f32_row(box1, lane, z);
+          // the box's generic reads are ordered before the next TMA write into it
+          fence_async_smem();
+          __syncwarp();
+          if (c + 2 < nch) fetch(t, c + 2);
+          else if (t + (int)gridDim.x < ntiles && h < nch_of(t + gridDim.x)) fetch(t + gridDim.x, h);
+        }
         tc_ld32(base + (uint32_t)(32 * c), v);
-        if (m < M) t32_epilogue(ep, m, n0 + 32 * c, N, v);
+        if (!maps) {
+          if (m < M) t32_epilogue(ep, m, n0 + 32 * c, N, v);
+          continue;
+        }
+        // the boxes are free once the store that used them has read them
+        if (lane == 0) bulk_wait_read0();
+        __syncwarp();
+        if (ep.epi == EPI_FWD_SILU) {
+          if (store_pre) st_f32_row(box1, lane, v);
+#pragma unroll
+          for (int j = 0; j < 32; ++j) v[j] = v[j] * epi_sigmoid(v[j]) * rs;
+        } else if (ep.epi == EPI_F32) {
+          if (input) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] += z[j];
+          }
+        } else if (ep.epi == EPI_BWD_SILU) {
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            const float sg = epi_sigmoid(z[j]);
+            v[j] = v[j] * sg * (1.0f + z[j] * (1.0f - sg));
+          }
+        }
+        st_f32_row(box0, lane, v);
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+          tma_store_2d(&em.out, box0, n0 + 32 * c, m0 + q * 32);
+          if (store_pre) tma_store_2d(&em.pre, box1, n0 + 32 * c, m0 + q * 32);
+          bulk_commit();
+        }
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&tempty[b]);
     }
+    if (lane == 0) bulk_wait_all();
+    __syncwarp();
   }
   tc_fence_before();
   __syncthreads();
@@ -1559,9 +1542,7 @@ template <int BN>
 static bool launch_tf32(const GemmArgs& g, const float* B, int ldb, cudaStream_t st, int* d_err, std::string* why) {
   static bool attr_set[kMaxDevices] = {};
   const int dev = current_device();
-  constexpr int smem = t32_smem_bytes<BN>();
-  static_assert(smem <= kTcSmemMax, "tf32 GEMM shared memory");
-  if (!smem_opt_in(gemm_tf32_kernel<BN>, smem, attr_set, dev, why)) return false;
+  if (!smem_opt_in(gemm_tf32_kernel<BN>, kTcSmemMax, attr_set, dev, why)) return false;
   CUtensorMap ta, tb;
   if (!make_tmap_f32(&ta, g.A, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.lda * 4, kT32BK, 128) ||
       !make_tmap_f32(&tb, B, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)ldb * 4, kT32BK, BN)) {
@@ -1571,7 +1552,24 @@ static bool launch_tf32(const GemmArgs& g, const float* B, int ldb, cudaStream_t
   const int tiles = ((g.M + 127) / 128) * ((g.N + BN - 1) / BN);
   const int nsm = num_sms(dev);
   const int grid = tiles < nsm ? tiles : nsm;
-  gemm_tf32_kernel<BN><<<grid, kT32Threads, smem, st>>>(ta, tb, make_epi(g), g.M, g.N, g.K, d_err);
+  // staging when TMA can move every epilogue array: one box for the output, one for what is stored or
+  // fetched beside it
+  const EpiParams ep = make_epi(g);
+  EpiMaps em;
+  memset(&em, 0, sizeof em);
+  int epi_slot = 0;
+  if (ep.vec) {
+    const bool pre = g.pre && g.epi != EPI_F32 && g.epi != EPI_LINEAR, add = g.add && g.epi == EPI_F32;
+    epi_slot = (pre || add) ? 2 * kT32Box : kT32Box;
+    if (!tc_box_map(&em.out, g.out, g.N, g.M, g.ldo, 4) || (pre && !tc_box_map(&em.pre, g.pre, g.N, g.M, g.ldp, 4)) ||
+        (add && !tc_box_map(&em.add, g.add, g.N, g.M, g.ld_add, 4))) {
+      if (why) *why = "cuTensorMapEncodeTiled failed (tf32 epilogue)";
+      return false;
+    }
+  }
+  const int stages = t32_stages<BN>(epi_slot);
+  const int smem = stages * t32_stage_bytes<BN>() + kT32EpiWarps * epi_slot + 1024 + 1024;
+  gemm_tf32_kernel<BN><<<grid, kT32Threads, smem, st>>>(ta, tb, em, ep, stages, epi_slot, g.M, g.N, g.K, d_err);
   return true;
 }
 

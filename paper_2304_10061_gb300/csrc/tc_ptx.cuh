@@ -19,6 +19,10 @@ namespace alg {
 bool tc_tensor_map_2d(CUtensorMap* tm, CUtensorMapDataType dtype, int esize, const void* base, uint64_t inner,
                       uint64_t outer, uint64_t row_bytes, uint32_t box_inner, uint32_t box_outer);
 
+// 2-D tensor map over a row-major [rows][ld] array of `esize`-byte elements, box 32 x 32, swizzle
+// matched to the row width of the box (64 bytes for 2-byte, 128 for 4-byte elements).
+bool tc_box_map(CUtensorMap* tm, const void* base, int cols, int rows, int ld, int esize);
+
 // ---------------------------------------------------------------------------
 // PTX wrappers
 // ---------------------------------------------------------------------------
