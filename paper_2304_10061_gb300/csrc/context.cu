@@ -863,6 +863,7 @@ allegro_status ensure_edges(allegro_ctx* c, int64_t E) {
 
 // Waits for the stream and reads the device's error word and, when asked, the edge count beside it.
 allegro_status read_err(allegro_ctx* c, int* out, int64_t* n_edges = nullptr) {
+  if (!c->h_pin) CUDA_TRY(c, cudaHostAlloc(reinterpret_cast<void**>(&c->h_pin), 2 * sizeof(int), cudaHostAllocDefault));
   CUDA_TRY(c, cudaMemcpyAsync(c->h_pin, c->d_err, 2 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   *out = c->h_pin[0];
@@ -1918,8 +1919,6 @@ allegro_status allegro_create(const void* weights_blob, size_t blob_bytes, const
   if (cudaMalloc(&c->d_err, 16) != cudaSuccess || cudaMalloc(&c->d_total, 16) != cudaSuccess ||
       cudaMalloc(&c->d_minmax, 12 * 8) != cudaSuccess || cudaMalloc(&c->d_red_scratch, kStructScratch * sizeof(double)) != cudaSuccess)
     return bail(fail(c, ALLEGRO_E_OOM, "scratch allocation failed"));
-  if (cudaHostAlloc(reinterpret_cast<void**>(&c->h_pin), 2 * sizeof(int), cudaHostAllocDefault) != cudaSuccess)
-    return bail(fail(c, ALLEGRO_E_OOM, "pinned words"));
   cudaMemset(c->d_err, 0, 16);
   cudaMemset(c->d_red_scratch, 0, kStructScratch * sizeof(double));
   *out = c;

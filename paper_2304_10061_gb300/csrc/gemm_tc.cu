@@ -25,6 +25,7 @@
 #include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <cstring>
 
@@ -96,10 +97,10 @@ bool tc_box_map(CUtensorMap* tm, const void* base, int cols, int rows, int ld, i
   return r == CUDA_SUCCESS;
 }
 
-// Instruction descriptor, kind::f16: D f32, A bf16, B bf16, both K-major, M = 128, N = BN.
-template <int BN>
+// Instruction descriptor, kind::f16: D f32, A bf16, B bf16, both K-major, M = MM, N = BN.
+template <int BN, int MM = 128>
 __device__ __forceinline__ constexpr uint32_t idesc_bf16() {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(MM >> 4) << 24);
 }
 
 constexpr int kTcBM = 128, kTcBK = 64;
@@ -129,9 +130,10 @@ struct TcLayout {
   int epi_slot;    // n_out * out_box + in_slot
 };
 
-template <int BN>
+// (a CTA of a pair holds half the rows of B)
+template <int BN, bool PAIR = false>
 __host__ __device__ constexpr int tc_stage_bytes() {
-  return kTcBM * kTcBK * 2 + BN * kTcBK * 2;
+  return kTcBM * kTcBK * 2 + BN * kTcBK * 2 / (PAIR ? 2 : 1);
 }
 
 template <int BN>
@@ -139,7 +141,7 @@ __host__ __device__ constexpr int tc_tmem_cols() {   // one accumulator buffer
   return BN <= 32 ? 32 : (BN <= 64 ? 64 : (BN <= 128 ? 128 : 256));
 }
 
-template <int BN, int EPQ>
+template <int BN, int EPQ, bool PAIR>
 static TcLayout tc_layout(int epi, bool pre) {
   TcLayout L;
   const bool wide_out = (epi == EPI_F32) || (epi == EPI_FWD_SILU && pre);
@@ -148,13 +150,13 @@ static TcLayout tc_layout(int epi, bool pre) {
   L.in_slot = (epi == EPI_BWD_SILU) ? 2048 : (epi == EPI_HEAD ? 4096 : 0);
   L.epi_slot = L.n_out * L.out_box + L.in_slot;
   const int epi_smem = 4 * EPQ * L.epi_slot;
-  const int st = (kTcSmemMax - 1024 - kTcMisc - epi_smem) / tc_stage_bytes<BN>();
+  const int st = (kTcSmemMax - 1024 - kTcMisc - epi_smem) / tc_stage_bytes<BN, PAIR>();
   L.stages = st > kTcMaxStages ? kTcMaxStages : st;
   return L;
 }
-template <int BN, int EPQ>
+template <int BN, int EPQ, bool PAIR>
 static size_t tc_smem_bytes(const TcLayout& L) {
-  return (size_t)L.stages * tc_stage_bytes<BN>() + (size_t)4 * EPQ * L.epi_slot + 1024 + kTcMisc;
+  return (size_t)L.stages * tc_stage_bytes<BN, PAIR>() + (size_t)4 * EPQ * L.epi_slot + 1024 + kTcMisc;
 }
 
 __device__ __forceinline__ void load_bf16x16(const bf16* p, float (&v)[16]) {
@@ -216,7 +218,17 @@ __device__ __forceinline__ float2 bf16_word_pair(uint32_t x) {
 // quarter's partial row sums in a fixed warp order.
 // With 18 warps (EPQ = 4) five share one SM sub-partition's 16K registers: at
 // most 96 per thread.
-template <int BN, int EPQ>
+//
+// PAIR: the two CTAs of a cluster share one 256 x BN tile (tcgen05.mma
+// cta_group::2, M = 256): each loads its own 128 rows of A and half the rows of
+// B, the CTA of rank 0 issues the MMAs once both have landed (all loads complete
+// on its barriers; its commits arrive on both CTAs' barriers), and each drains
+// its own 128 rows of the accumulator.  A CTA of its own reads 128 A rows and
+// BN B rows per tile, 768 bytes of shared memory (and as much from L2) per k
+// column for 2 x 128 x 256 FLOP: at these widths the operand traffic, not the
+// tensor pipe, sets the rate (1.14 PFLOP/s on 1024-wide layers); the pair halves
+// the B part of it.
+template <int BN, int EPQ, bool PAIR>
 __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA2,
                    const __grid_constant__ CUtensorMap tmB, const __grid_constant__ EpiMaps em, EpiParams ep,
@@ -226,7 +238,7 @@ __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
   const int kEpiSlot = lay.epi_slot;
   const int kNOut = lay.n_out;
   constexpr uint32_t A_BYTES = kTcBM * kTcBK * 2;
-  constexpr uint32_t B_BYTES = BN * kTcBK * 2;
+  constexpr uint32_t B_BYTES = BN * kTcBK * 2 / (PAIR ? 2 : 1);
   constexpr uint32_t COLS = tc_tmem_cols<BN>();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -244,13 +256,17 @@ __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
   float* rowpart = reinterpret_cast<float*>(tslot + 4);   // [4 quarters][2 buffers][EPQ - 1][32] partial row sums
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = PAIR ? cluster_ctarank() : 0;
+  // tiles of this CTA (or pair): t0, t0 + tstep, ...
+  const int t0 = PAIR ? (int)blockIdx.x >> 1 : (int)blockIdx.x, tstep = PAIR ? (int)gridDim.x >> 1 : (int)gridDim.x;
+  constexpr int TM = PAIR ? 2 * kTcBM : kTcBM;
   const int nk = (K + kTcBK - 1) / kTcBK;
-  const int tiles_m = (M + kTcBM - 1) / kTcBM, tiles_n = (N + BN - 1) / BN;
+  const int tiles_m = (M + TM - 1) / TM, tiles_n = (N + BN - 1) / BN;
   const int ntiles = tiles_m * tiles_n;
   // tile t -> (row block t / tiles_n, column block t % tiles_n): the column
   // blocks of one row block run on neighbouring CTAs at the same time, so the
   // A rows they share come from L2 after the first read
-  auto tm0 = [&](int tt) { return (tt / tiles_n) * kTcBM; };
+  auto tm0 = [&](int tt) { return (tt / tiles_n) * TM + (int)rank * kTcBM; };
   auto tn0 = [&](int tt) { return (tt % tiles_n) * BN; };
 
   if (threadIdx.x == 0) {
@@ -260,7 +276,7 @@ __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&tfull[b], 1);
-      mbar_init(&tempty[b], kEpiWarps);
+      mbar_init(&tempty[b], kEpiWarps * (PAIR ? 2 : 1));
     }
     for (int q = 0; q < 8; ++q) mbar_init(&rsbar[q], EPQ - 1);
     for (int q = 0; q < kEpiWarps; ++q) mbar_init(&inbar[q], 1);
@@ -269,18 +285,24 @@ __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   if (warp == 1) {
-    tc_alloc(tslot, 2 * COLS);
-    tc_relinquish();
+    if constexpr (PAIR) {
+      tc_alloc_pair(tslot, 2 * COLS);
+      tc_relinquish_pair();
+    } else {
+      tc_alloc(tslot, 2 * COLS);
+      tc_relinquish();
+    }
   }
   tc_fence_before();
   __syncthreads();
+  if constexpr (PAIR) cluster_sync();   // both CTAs' barriers exist before either is signalled
   tc_fence_after();
   const uint32_t tmem = *tslot;
 
   if (warp == 0) {
     if (lane == 0) {
       uint32_t g = 0;   // global k-block counter (ring position)
-      for (int t = blockIdx.x; t < ntiles && !*abort_flag; t += gridDim.x) {
+      for (int t = t0; t < ntiles && !*abort_flag; t += tstep) {
         const int m0 = tm0(t), n0 = tn0(t);
         for (int kb = 0; kb < nk; ++kb, ++g) {
           const uint32_t s = g % STAGES, r = g / STAGES;
@@ -289,19 +311,28 @@ __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
             *abort_flag = 1;
             break;
           }
-          mbar_expect_tx(&full[s], A_BYTES + B_BYTES);
-          if (kb * kTcBK < K1) tma_load_2d(sA + s * A_BYTES, &tmA, &full[s], kb * kTcBK, m0);
-          else tma_load_2d(sA + s * A_BYTES, &tmA2, &full[s], kb * kTcBK - K1, m0);   // columns of A2
-          tma_load_2d(sB + s * B_BYTES, &tmB, &full[s], kb * kTcBK, n0);
+          const bool first = kb * kTcBK < K1;   // else columns of A2
+          const int kc = first ? kb * kTcBK : kb * kTcBK - K1;
+          if constexpr (PAIR) {
+            // both CTAs' loads complete on the barrier of rank 0, which expects them all
+            const uint32_t bar = mapa_u32(&full[s], 0);
+            if (rank == 0) mbar_expect_tx(&full[s], 2 * (A_BYTES + B_BYTES));
+            tma_load_2d_pair(sA + s * A_BYTES, first ? &tmA : &tmA2, bar, kc, m0);
+            tma_load_2d_pair(sB + s * B_BYTES, &tmB, bar, kb * kTcBK, n0 + (int)rank * (BN / 2));
+          } else {
+            mbar_expect_tx(&full[s], A_BYTES + B_BYTES);
+            tma_load_2d(sA + s * A_BYTES, first ? &tmA : &tmA2, &full[s], kc, m0);
+            tma_load_2d(sB + s * B_BYTES, &tmB, &full[s], kb * kTcBK, n0);
+          }
         }
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = idesc_bf16<BN>();
+    if (lane == 0 && rank == 0) {
+      constexpr uint32_t idesc = idesc_bf16<BN, TM>();
       uint32_t g = 0;
       int lt = 0;
-      for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++lt) {
+      for (int t = t0; t < ntiles; t += tstep, ++lt) {
         const int b = lt & 1, use = lt >> 1;
         bool ok = !*abort_flag && mbar_wait(&tempty[b], (use & 1) ^ 1);
         if (ok) {
@@ -316,17 +347,21 @@ __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
             tc_fence_after();
             const uint32_t a_addr = smem_u32(sA + s * A_BYTES), b_addr = smem_u32(sB + s * B_BYTES);
 #pragma unroll
-            for (int k = 0; k < kTcBK / 16; ++k)
-              tc_mma(dt, sdesc_sw128(a_addr + k * 32), sdesc_sw128(b_addr + k * 32), idesc,
-                     (kb > 0 || k > 0) ? 1u : 0u);
-            tc_commit(&empty[s]);
+            for (int k = 0; k < kTcBK / 16; ++k) {
+              const uint64_t da = sdesc_sw128(a_addr + k * 32), db = sdesc_sw128(b_addr + k * 32);
+              if constexpr (PAIR) tc_mma_pair(dt, da, db, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+              else tc_mma(dt, da, db, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+            }
+            if constexpr (PAIR) tc_commit_pair(&empty[s]);
+            else tc_commit(&empty[s]);
           }
         }
         if (!ok) {
           atomicOr(err, kErrTimeout);
           *abort_flag = 1;
         }
-        tc_commit(&tfull[b]);
+        if constexpr (PAIR) tc_commit_pair(&tfull[b]);
+        else tc_commit(&tfull[b]);
         if (!ok) break;
       }
     }
@@ -355,10 +390,16 @@ __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
       }
     };
     auto nch_of = [&](int tt) { return (min(BN, N - tn0(tt)) + 31) / 32; };
+    // this warp has drained accumulator bb (the MMA thread is in the CTA of rank 0)
+    auto release = [&](int bb) {
+      if (lane != 0) return;
+      if constexpr (PAIR) mbar_arrive_cluster(mapa_u32(&tempty[bb], 0));
+      else mbar_arrive(&tempty[bb]);
+    };
     int lt = 0;
     int oc = 0;                        // output chunks issued (buffer = oc % kNOut)
-    if (h < nch_of(blockIdx.x)) fetch(blockIdx.x, h);
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++lt) {
+    if (t0 < ntiles && h < nch_of(t0)) fetch(t0, h);
+    for (int t = t0; t < ntiles; t += tstep, ++lt) {
       const int b = lt & 1, use = lt >> 1;
       const bool ok = mbar_wait(&tfull[b], use & 1);
       if (!ok) {
@@ -394,7 +435,7 @@ __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
           __syncwarp();
           // prefetch this warp's next chunk (possibly in its next tile)
           if (c + EPQ < nch) fetch(t, c + EPQ);
-          else if (t + (int)gridDim.x < ntiles && h < nch_of(t + gridDim.x)) fetch(t + gridDim.x, h);
+          else if (t + tstep < ntiles && h < nch_of(t + tstep)) fetch(t + tstep, h);
         }
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
@@ -472,7 +513,7 @@ __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
       tc_fence_before();
       __syncwarp();
       if (!rowsums) {
-        if (lane == 0) mbar_arrive(&tempty[b]);
+        release(b);
       } else {
         // combine the quarter's partial row sums in a fixed order (h = 0, 1, 2, 3).
         // Warp h = 0 releases the TMEM buffer only after reading the partials,
@@ -485,8 +526,8 @@ __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
           __syncwarp();
           if (lane == 0) {
             mbar_arrive(&rsbar[q * 2 + b]);
-            mbar_arrive(&tempty[b]);
           }
+          release(b);
         } else {
           if (!mbar_wait(&rsbar[q * 2 + b], use & 1)) {
             if (lane == 0) atomicOr(err, kErrTimeout);
@@ -505,7 +546,7 @@ __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
             }
           }
           __syncwarp();
-          if (lane == 0) mbar_arrive(&tempty[b]);
+          release(b);
         }
       }
     }
@@ -514,9 +555,12 @@ __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
   }
   tc_fence_before();
   __syncthreads();
+  // neither CTA leaves while the other may still signal its barriers or read its operands
+  if constexpr (PAIR) cluster_sync();
   if (warp == 1) {
     tc_fence_after();
-    tc_dealloc(tmem, 2 * COLS);
+    if constexpr (PAIR) tc_dealloc_pair(tmem, 2 * COLS);
+    else tc_dealloc(tmem, 2 * COLS);
   }
 }
 
@@ -1055,18 +1099,18 @@ static bool smem_opt_in(K kernel, int bytes, bool (&done)[kMaxDevices], int dev,
   return true;
 }
 
-template <int BN, int EPQ>
+template <int BN, int EPQ, bool PAIR = false>
 static bool launch_bn(const GemmArgs& g, const bf16* B, int ldb, cudaStream_t st, int* d_err, std::string* why) {
   static bool attr_set[kMaxDevices] = {};
   const int dev = current_device();
-  if (!smem_opt_in(gemm_tc_kernel<BN, EPQ>, kTcSmemMax, attr_set, dev, why)) return false;
+  if (!smem_opt_in(gemm_tc_kernel<BN, EPQ, PAIR>, kTcSmemMax, attr_set, dev, why)) return false;
   const int nsm = num_sms(dev);
   CUtensorMap ta, ta2, tb;
   const int K1 = g.A2 ? g.K1 : g.K;
   if (!make_tmap(&ta, g.A, (uint64_t)K1, (uint64_t)g.M, (uint64_t)g.lda * 2, kTcBK, kTcBM) ||
       !make_tmap(&ta2, g.A2 ? g.A2 : g.A, (uint64_t)(g.A2 ? g.K - K1 : K1), (uint64_t)g.M,
                  (uint64_t)(g.A2 ? g.lda2 : g.lda) * 2, kTcBK, kTcBM) ||
-      !make_tmap(&tb, B, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)ldb * 2, kTcBK, BN)) {
+      !make_tmap(&tb, B, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)ldb * 2, kTcBK, PAIR ? BN / 2 : BN)) {
     if (why) *why = "cuTensorMapEncodeTiled failed (alignment or extent)";
     return false;
   }
@@ -1080,16 +1124,37 @@ static bool launch_bn(const GemmArgs& g, const bf16* B, int ldb, cudaStream_t st
     if (why) *why = "cuTensorMapEncodeTiled failed for an epilogue operand";
     return false;
   }
-  const TcLayout lay = tc_layout<BN, EPQ>(g.epi, g.pre != nullptr);
+  const TcLayout lay = tc_layout<BN, EPQ, PAIR>(g.epi, g.pre != nullptr);
   if (lay.stages < 2) {
     if (why) *why = "tcgen05 GEMM: shared memory too small for two operand stages";
     return false;
   }
-  const size_t smem = tc_smem_bytes<BN, EPQ>(lay);
-  const int tiles = ((g.M + kTcBM - 1) / kTcBM) * ((g.N + BN - 1) / BN);
-  const int grid = tiles < nsm ? tiles : nsm;
-  gemm_tc_kernel<BN, EPQ><<<grid, tc_threads<EPQ>(), smem, st>>>(ta, ta2, tb, em, make_epi(g), lay, g.M, g.N, g.K,
-                                                                  K1, d_err);
+  const size_t smem = tc_smem_bytes<BN, EPQ, PAIR>(lay);
+  if constexpr (PAIR) {
+    const int tiles = ((g.M + 2 * kTcBM - 1) / (2 * kTcBM)) * ((g.N + BN - 1) / BN);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * std::min(tiles, nsm / 2));
+    cfg.blockDim = dim3(tc_threads<EPQ>());
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 2;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_tc_kernel<BN, EPQ, true>, ta, ta2, tb, em, make_epi(g), lay, g.M,
+                                             g.N, g.K, K1, d_err);
+    if (e != cudaSuccess) {
+      if (why) *why = std::string("cudaLaunchKernelEx: ") + cudaGetErrorString(e);
+      return false;
+    }
+  } else {
+    const int tiles = ((g.M + kTcBM - 1) / kTcBM) * ((g.N + BN - 1) / BN);
+    const int grid = tiles < nsm ? tiles : nsm;
+    gemm_tc_kernel<BN, EPQ, false><<<grid, tc_threads<EPQ>(), smem, st>>>(ta, ta2, tb, em, make_epi(g), lay, g.M, g.N,
+                                                                          g.K, K1, d_err);
+  }
   return true;
 }
 
@@ -1129,6 +1194,13 @@ bool gemm_tc_bf16(const GemmArgs& g, cudaStream_t st, int* d_err, std::string* w
     case 192: return launch_bn<192, 2>(g, B, ldb, st, d_err, why);
     case 224: return launch_bn<224, 2>(g, B, ldb, st, d_err, why);
     default:
+      // CTA pairs for long sums, once there is a tile for every pair of SMs.  ms alone / paired at
+      // 1.64 million rows: K = 1536, N = 512 2.16 / 1.89, K = 1024, N = 512 1.55 / 1.39; K = 640 1.07 /
+      // 1.07, K = 512 0.95 / 1.03 (HBM-bound, and the two epilogues wait for each other); 184,600 rows,
+      // K = N = 1024 0.342 / 0.307
+      if (g.K >= 768 && g.N > 256 && (int64_t)((g.M + 255) / 256) * tiles >= num_sms(current_device()) / 2)
+        return wide ? launch_bn<256, 4, true>(g, B, ldb, st, d_err, why)
+                    : launch_bn<256, 2, true>(g, B, ldb, st, d_err, why);
       return wide ? launch_bn<256, 4>(g, B, ldb, st, d_err, why) : launch_bn<256, 2>(g, B, ldb, st, d_err, why);
   }
 }
