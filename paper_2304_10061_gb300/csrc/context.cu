@@ -1938,11 +1938,12 @@ allegro_status allegro_set_pair_cutoffs(allegro_ctx* c, const double* pair_rc, i
   if (!pair_rc) {
     c->arch.pair_basis = nullptr;
     c->arch.pair_rc2 = nullptr;
+    c->arch.pair_rc2f = nullptr;
     return ALLEGRO_OK;
   }
   const int ns = c->arch.ns;
   if (n_species != ns) return fail(c, ALLEGRO_E_INVALID, "n_species %d differs from the model's %d", n_species, ns);
-  std::vector<float> basis(2 * (size_t)ns * ns);
+  std::vector<float> basis(3 * (size_t)ns * ns);   // {1/rc, sqrt(2/rc)} per pair, then rc^2 per pair
   std::vector<double> rc2((size_t)ns * ns);
   for (int q = 0; q < ns * ns; ++q) {
     const double rc = pair_rc[q];
@@ -1952,9 +1953,10 @@ allegro_status allegro_set_pair_cutoffs(allegro_ctx* c, const double* pair_rc, i
     basis[2 * q] = (float)(1.0 / rc);
     basis[2 * q + 1] = (float)std::sqrt(2.0 / rc);
     rc2[q] = rc * rc;
+    basis[2 * (size_t)ns * ns + q] = (float)rc2[q];
   }
   if (!c->d_pair_basis) {
-    CUDA_TRY(c, cudaMalloc(&c->d_pair_basis, 2 * sizeof(float) * kMaxSpecies * kMaxSpecies));
+    CUDA_TRY(c, cudaMalloc(&c->d_pair_basis, 3 * sizeof(float) * kMaxSpecies * kMaxSpecies));
     CUDA_TRY(c, cudaMalloc(&c->d_pair_rc2, sizeof(double) * kMaxSpecies * kMaxSpecies));
   }
   CUDA_TRY(c, cudaMemcpyAsync(c->d_pair_basis, basis.data(), basis.size() * sizeof(float), cudaMemcpyHostToDevice,
@@ -1964,6 +1966,7 @@ allegro_status allegro_set_pair_cutoffs(allegro_ctx* c, const double* pair_rc, i
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   c->arch.pair_basis = c->d_pair_basis;
   c->arch.pair_rc2 = c->d_pair_rc2;
+  c->arch.pair_rc2f = c->d_pair_basis + 2 * (size_t)ns * ns;
   return ALLEGRO_OK;
 }
 
@@ -2148,17 +2151,19 @@ static allegro_status build_single(allegro_ctx* c, int64_t n_atoms, const double
     if (!(band > 0) || !std::isfinite(band) || band > 0.25 * rc * rc) band = 1e30f;   // prefilter off
   }
   const double rc2 = rc * rc;
+  for (int q = 0; q < 9; ++q) g.cellf[q] = (float)g.cell[q];
+  g.rc2f = (float)rc2;
   {
     ProfScope ps(c, "nb_search_count", 0.0, (double)n * 64);
     nb_search(false, c->d_pos, n, g, c->d_cell_of, c->d_wraps, c->d_cell_start, c->d_sorted, c->d_pos4, c->d_pw, rc2,
-              band, pair_rc2, c->arch.ns, c->d_count,
+              band, pair_rc2, c->arch.pair_rc2f, c->arch.ns, c->d_count,
               nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0, c->d_err, st);
     c->launches += exclusive_scan_i32(c->d_count, c->d_row_ptr, n, c->d_scan_tmp, false, c->d_err + 1, st);
   }
   if ((s = fill_rows(c, n, n_edges_out, [&](int edge_cap) {
          ProfScope ps(c, "nb_search_fill", 0.0, (double)c->n_edges * 44 + (double)n * 64);
          return nb_search(true, c->d_pos, n, g, c->d_cell_of, c->d_wraps, c->d_cell_start, c->d_sorted, c->d_pos4,
-                          c->d_pw, rc2, band, pair_rc2, c->arch.ns, nullptr, c->d_row_ptr, c->d_ej, c->d_ei, c->d_eS,
+                          c->d_pw, rc2, band, pair_rc2, c->arch.pair_rc2f, c->arch.ns, nullptr, c->d_row_ptr, c->d_ej, c->d_ei, c->d_eS,
                           c->d_ed, c->d_col_count, col_rank(c), edge_cap, c->d_err, st);
        })) != ALLEGRO_OK)
     return s;

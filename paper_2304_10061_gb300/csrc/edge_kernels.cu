@@ -123,20 +123,22 @@ template <> __device__ __forceinline__ float path_sigmoid<bf16>(float z) {
   return fmaf(0.5f, t, 0.5f);
 }
 
-// Edge geometry, basis and the first two-body layer, one block of kGeomBlock
-// edges.  The layer's input row [onehot(Z_i) | onehot(Z_j) | B(r)] is never
-// formed: z_k = W0[k][Z_i] + W0[k][ns + Z_j] + sum_n W0[k][2 ns + n] B_n(r),
-// with W0 read as its transpose W0t[input][output] from shared memory, 32
-// output columns at a time.  Outputs: Y, u, sigma_{Z_i}, the pre-activation
-// z and the activation silu(z) (times u when the layer is the MLP's last), all
-// staged in shared memory and written back as contiguous runs (per-thread
-// records would scatter over partial sectors).
+// Edge geometry, basis and the first two-body layer.  The layer's input row
+// [onehot(Z_i) | onehot(Z_j) | B(r)] is never formed: z_k = W0[k][Z_i] +
+// W0[k][ns + Z_j] + sum_n W0[k][2 ns + n] B_n(r), with W0 read as its transpose
+// W0t[input][output].  Outputs: Y, u, sigma_{Z_i}, the pre-activation z and the
+// activation silu(z) (times u when the layer is the MLP's last).
+// Persistent blocks over tiles of kGeomBlock edges, two phases per tile: a thread
+// per edge for the geometry and the basis (B_n, species and scale to shared
+// memory, Y through shared memory to contiguous runs), then 16 lanes per edge for
+// the layer, four columns per lane with their Bessel weights in registers, so that
+// a row of z or silu(z) is written as one contiguous run.
+// Bound: HBM (24 + 8 + 8 + 4 S + 4 N0 bytes per edge in bf16) beside shared-memory
+// wavefronts: a thread per edge for the layer too reads ten 16-byte weights of
+// shared memory per four outputs (640 wavefronts per 32 edges at N0 = 64, which
+// set its time), this form five per 64 outputs of one edge (about 320).
 constexpr int kGeomBlock = 128;
-constexpr int kGeomCols = 32;                   // output columns per pass
-constexpr int kGeomWPad = kGeomCols + 4;        // padded shared row of W0t (float4-aligned, bank-spread)
-
-template <typename T>
-__host__ __device__ constexpr int geom_stage_ld() { return kGeomCols + 16 / (int)sizeof(T); }   // padded row, 16-byte multiple
+constexpr int kGeomFwdBlocksPerSM = 6;
 
 // four consecutive activation-type values from floats (8- or 16-byte aligned)
 __device__ __forceinline__ void st4_act(float* p, const float (&v)[4]) {
@@ -147,52 +149,35 @@ __device__ __forceinline__ void st4_act(bf16* p, const float (&v)[4]) {
   *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<uint32_t*>(&a), *reinterpret_cast<uint32_t*>(&b));
 }
 
-template <typename T>
-__device__ __forceinline__ void copy_rows_out(const T* src, int lds, T* dst, int ldd, int c0, int nrows, int nc) {
-  // rows of nc elements from shared (row pitch lds) to global (row pitch ldd, column offset c0)
-  const bool vec = ((nc * (int)sizeof(T)) % 16 == 0) && ((c0 * (int)sizeof(T)) % 16 == 0) &&
-                   ((ldd * (int)sizeof(T)) % 16 == 0);
-  if (vec) {
-    const int per = nc * (int)sizeof(T) / 16;
-    for (int q = threadIdx.x; q < nrows * per; q += blockDim.x) {
-      const int rr = q / per, cc = q - rr * per;
-      reinterpret_cast<uint4*>(dst + (size_t)rr * ldd + c0)[cc] = reinterpret_cast<const uint4*>(src + rr * lds)[cc];
-    }
-  } else {
-    for (int q = threadIdx.x; q < nrows * nc; q += blockDim.x) {
-      const int rr = q / nc, cc = q - rr * nc;
-      dst[(size_t)rr * ldd + c0 + cc] = src[rr * lds + cc];
-    }
-  }
-}
-
-// AMAX: record max|activation| for the FP8 per-tensor scale (the other paths skip the work)
-template <typename T, bool AMAX>
+// NB: Bessel functions the kernel holds weights for (8 or kMaxBessel); AMAX: record max|activation|
+// for the FP8 per-tensor scale (the other paths skip the work)
+template <typename T, int NB, bool AMAX>
 __global__ void __launch_bounds__(kGeomBlock)
     geom_fwd_kernel(int Ec, int e0, const double* __restrict__ ed, const int* __restrict__ ei,
                     const int* __restrict__ ej, const int* __restrict__ species, BasisConst bc,
                     float* __restrict__ Yout, float* __restrict__ uout, const double* __restrict__ sigma,
                     float* __restrict__ sig, const float* __restrict__ W0t, int ldW, int N0, T* __restrict__ Zout,
-                    int ldZ, T* __restrict__ Hout, int ldH, int scale_u, unsigned* __restrict__ amax) {
-  constexpr int LDS = geom_stage_ld<T>();
-  extern __shared__ __align__(16) uint8_t geom_sm[];
-  const int K0 = 2 * bc.ns + bc.nb;
-  const int WP = kGeomWPad;   // shared row pitch of W0t (floats)
-  float* sY = reinterpret_cast<float*>(geom_sm);                                  // [kGeomBlock][kMaxS]
-  float* sW = sY + kGeomBlock * kMaxS;                                            // [K0][WP]
-  T* sZ = reinterpret_cast<T*>(sW + K0 * WP);                                     // [kGeomBlock][LDS]
-  T* sH = sZ + kGeomBlock * LDS;                                                  // [kGeomBlock][LDS]
+                    int ldZ, T* __restrict__ Hout, int ldH, int scale_u, int vec, unsigned* __restrict__ amax) {
+  __shared__ float sY[kGeomBlock * kMaxS];
+  __shared__ float4 sB[kGeomBlock][NB / 4];
+  __shared__ int4 sI[kGeomBlock];   // species of i and j, scale of the activation (float bits)
   const int tl = threadIdx.x;
+  const int hl = tl & 15, hw = tl >> 4;   // lane in its half-warp, half-warp
   const int ntiles = (Ec + kGeomBlock - 1) / kGeomBlock;
   float hmax = 0.0f;   // max |activation| written (FP8 per-tensor scale)
+  float4 w[NB];        // Bessel weights of this lane's four columns
+  auto load_w = [&](int c) {
+#pragma unroll
+    for (int n = 0; n < NB; ++n)
+      w[n] = (n < bc.nb && c < N0) ? __ldg(reinterpret_cast<const float4*>(W0t + (size_t)(2 * bc.ns + n) * ldW + c))
+                                   : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  };
+  load_w(4 * hl);
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int eb = tile * kGeomBlock;
     const int nloc = min(kGeomBlock, Ec - eb);
     const int e = eb + tl;
-    float B[kMaxBessel];
-    float u = 0.0f;
-    int zi = 0, zj = 0;
-    __syncthreads();   // the previous tile's Y staging has been copied out
+    __syncthreads();   // the previous tile's shared arrays have been read
     if (tl < nloc) {
       const size_t eg = (size_t)e0 + e;
       const double dx = ed[3 * eg], dy = ed[3 * eg + 1], dz = ed[3 * eg + 2];
@@ -207,76 +192,85 @@ __global__ void __launch_bounds__(kGeomBlock)
 #pragma unroll
       for (int a = 0; a < kMaxS; ++a)
         if (a < bc.S) sY[tl * bc.S + a] = Y[a];
-      zi = species[ei[eg]];
-      zj = species[ej[eg]];
+      const int zi = species[ei[eg]], zj = species[ej[eg]];
       const float2 pb = pair_basis(bc, zi, zj);   // the pair's 1/rc and sqrt(2/rc)
       const float xr = r * pb.x;
+      float u = 0.0f;
       if (xr < 1.0f) {
         const float xp = ipow(xr, bc.p);
         u = 1.0f - xp * (bc.c0 - xr * (bc.c1 - bc.c2 * xr));
       }
       uout[e] = u;
       if (sig) sig[e] = (float)sigma[zi];
+      sI[tl] = make_int4(zi, zj, __float_as_int(scale_u ? u : 1.0f), 0);
       // sin(n pi x) for n = 1..nb by the angle-addition recurrence from one
       // sincospi: (s, c)_{n+1} = (s_n c_1 + c_n s_1, c_n c_1 - s_n s_1)
       float s1, c1;
       sincospif(xr, &s1, &c1);
-      float sn = s1, cn = c1;
+      float sn = s1, cn = c1, B[NB];
 #pragma unroll
-      for (int n = 0; n < kMaxBessel; ++n) {
+      for (int n = 0; n < NB; ++n) {
         B[n] = (n < bc.nb) ? pb.y * sn * ir32 : 0.0f;
         const float s2 = fmaf(sn, c1, cn * s1);
         cn = fmaf(cn, c1, -(sn * s1));
         sn = s2;
       }
-    }
-    const float rsc = scale_u ? u : 1.0f;
-    for (int c0 = 0; c0 < N0; c0 += kGeomCols) {
-      const int nc = min(kGeomCols, N0 - c0);
-      __syncthreads();   // the previous pass's staging has been copied out
-      for (int q = tl; q < K0 * kGeomCols; q += kGeomBlock) {
-        const int rr = q / kGeomCols, cc = q - rr * kGeomCols;
-        sW[rr * kGeomWPad + cc] = (cc < nc) ? W0t[(size_t)rr * ldW + c0 + cc] : 0.0f;
-      }
-      __syncthreads();
-      if (tl < nloc) {
-        const float* wi = sW + zi * WP;
-        const float* wj = sW + (bc.ns + zj) * WP;
-        const float* wb = sW + 2 * bc.ns * WP;
-#pragma unroll 2
-        for (int c4 = 0; c4 < kGeomCols; c4 += 4) {
-          const float4 a = *reinterpret_cast<const float4*>(wi + c4);
-          const float4 b = *reinterpret_cast<const float4*>(wj + c4);
-          // column pairs in packed fp32 (FFMA2 / FMUL2: each half the ordinary
-          // IEEE fp32 fma / multiply, so the results equal the scalar ones)
-          float2 z01 = make_float2(a.x + b.x, a.y + b.y), z23 = make_float2(a.z + b.z, a.w + b.w);
 #pragma unroll
-          for (int n = 0; n < kMaxBessel; ++n) {
+      for (int n = 0; n < NB / 4; ++n) sB[tl][n] = make_float4(B[4 * n], B[4 * n + 1], B[4 * n + 2], B[4 * n + 3]);
+    }
+    __syncthreads();
+    for (int c0 = 0; c0 < N0; c0 += 64) {
+      const int c = c0 + 4 * hl;
+      if (N0 > 64) load_w(c);
+      if (c >= N0) continue;
+#pragma unroll 2
+      for (int q = hw; q < nloc; q += kGeomBlock / 16) {
+        const int4 in = sI[q];
+        const float4 a = __ldg(reinterpret_cast<const float4*>(W0t + (size_t)in.x * ldW + c));
+        const float4 b = __ldg(reinterpret_cast<const float4*>(W0t + (size_t)(bc.ns + in.y) * ldW + c));
+        // column pairs in packed fp32 (FFMA2 / FMUL2: each half the ordinary
+        // IEEE fp32 fma / multiply, so the results equal the scalar ones)
+        float2 z01 = make_float2(a.x + b.x, a.y + b.y), z23 = make_float2(a.z + b.z, a.w + b.w);
+#pragma unroll
+        for (int n4 = 0; n4 < NB / 4; ++n4) {
+          const float4 b4 = sB[q][n4];
+          const float bn[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int n = 4 * n4 + k;
             if (n < bc.nb) {
-              const float4 w = *reinterpret_cast<const float4*>(wb + n * WP + c4);
-              const float2 bn = make_float2(B[n], B[n]);
-              z01 = __ffma2_rn(bn, make_float2(w.x, w.y), z01);
-              z23 = __ffma2_rn(bn, make_float2(w.z, w.w), z23);
+              const float2 bb = make_float2(bn[k], bn[k]);
+              z01 = __ffma2_rn(bb, make_float2(w[n].x, w[n].y), z01);
+              z23 = __ffma2_rn(bb, make_float2(w[n].z, w[n].w), z23);
             }
           }
-          const float2 rs2 = make_float2(rsc, rsc);
-          const float2 g01 = make_float2(path_sigmoid<T>(z01.x), path_sigmoid<T>(z01.y));
-          const float2 g23 = make_float2(path_sigmoid<T>(z23.x), path_sigmoid<T>(z23.y));
-          const float2 h01 = __fmul2_rn(__fmul2_rn(z01, g01), rs2);
-          const float2 h23 = __fmul2_rn(__fmul2_rn(z23, g23), rs2);
-          const float acc[4] = {z01.x, z01.y, z23.x, z23.y};
-          const float hv[4] = {h01.x, h01.y, h23.x, h23.y};
-          if constexpr (AMAX) {
+        }
+        const float rsc = __int_as_float(in.z);
+        const float2 rs2 = make_float2(rsc, rsc);
+        const float2 g01 = make_float2(path_sigmoid<T>(z01.x), path_sigmoid<T>(z01.y));
+        const float2 g23 = make_float2(path_sigmoid<T>(z23.x), path_sigmoid<T>(z23.y));
+        const float2 h01 = __fmul2_rn(__fmul2_rn(z01, g01), rs2);
+        const float2 h23 = __fmul2_rn(__fmul2_rn(z23, g23), rs2);
+        const float acc[4] = {z01.x, z01.y, z23.x, z23.y};
+        const float hv[4] = {h01.x, h01.y, h23.x, h23.y};
+        if constexpr (AMAX) {   // (columns past N0 read zero weights)
 #pragma unroll
-            for (int k = 0; k < 4; ++k) hmax = fmaxf(hmax, fabsf(hv[k]));
-          }
-          st4_act(sZ + tl * LDS + c4, acc);
-          st4_act(sH + tl * LDS + c4, hv);
+          for (int k = 0; k < 4; ++k) hmax = fmaxf(hmax, fabsf(hv[k]));
+        }
+        T* zo = Zout + (size_t)(eb + q) * ldZ + c;
+        T* ho = Hout + (size_t)(eb + q) * ldH + c;
+        if (vec) {
+          st4_act(zo, acc);
+          st4_act(ho, hv);
+        } else {
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (c + k < N0) {
+              zo[k] = to_act<T>(acc[k]);
+              ho[k] = to_act<T>(hv[k]);
+            }
         }
       }
-      __syncthreads();
-      copy_rows_out<T>(sZ, LDS, Zout + (size_t)eb * ldZ, ldZ, c0, nloc, nc);
-      copy_rows_out<T>(sH, LDS, Hout + (size_t)eb * ldH, ldH, c0, nloc, nc);
     }
     // Y: nloc * S floats starting at float eb * S (4-byte aligned only): scalar, coalesced
     float* dst = Yout + (size_t)eb * bc.S;
@@ -290,20 +284,26 @@ void edge_geom_fwd(int Ec, int e0, const double* ed, const int* ei, const int* e
                    const Arch& a, float* Y, float* u, const double* sigma, float* sig, const float* W0t, int ldW,
                    T* Z0, int ldZ, T* H0, int ldH, bool scale_u, cudaStream_t st, unsigned* amax) {
   if (Ec <= 0) return;
-  const int N0 = a.tb[0], K0 = a.K0in();
-  const size_t stage = (size_t)kGeomBlock * kMaxS * 4 + 2 * (size_t)kGeomBlock * geom_stage_ld<T>() * sizeof(T);
+  const int N0 = a.tb[0];
+  int dev = 0, nsm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const int tiles = (Ec + kGeomBlock - 1) / kGeomBlock;
-  // one tile per block, 32 weight columns staged per pass (measured faster than persistent
-  // blocks holding all of W0t)
-  const size_t smem = stage + (size_t)K0 * kGeomWPad * 4;
+  const int grid = std::min(tiles, std::max(nsm, 1) * kGeomFwdBlocksPerSM);
+  // whole groups of four columns at 16-byte (8-byte in bf16) boundaries
+  auto al = [](const void* p) { return reinterpret_cast<uintptr_t>(p) % (4 * sizeof(T)) == 0; };
+  const int vec = N0 % 4 == 0 && ldZ % 4 == 0 && ldH % 4 == 0 && al(Z0) && al(H0);
   auto launch = [&](auto kern) {
-    if (smem > 48 * 1024)   // many species: opt in to more than the default dynamic shared memory
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    kern<<<tiles, kGeomBlock, smem, st>>>(Ec, e0, ed, ei, ej, species, make_basis(a), Y, u, sigma, sig, W0t, ldW, N0,
-                                          Z0, ldZ, H0, ldH, scale_u ? 1 : 0, amax);
+    kern<<<grid, kGeomBlock, 0, st>>>(Ec, e0, ed, ei, ej, species, make_basis(a), Y, u, sigma, sig, W0t, ldW, N0, Z0,
+                                      ldZ, H0, ldH, scale_u ? 1 : 0, vec, amax);
   };
-  if (amax) launch(geom_fwd_kernel<T, true>);
-  else launch(geom_fwd_kernel<T, false>);
+  if (a.nb <= 8) {
+    if (amax) launch(geom_fwd_kernel<T, 8, true>);
+    else launch(geom_fwd_kernel<T, 8, false>);
+  } else {
+    if (amax) launch(geom_fwd_kernel<T, kMaxBessel, true>);
+    else launch(geom_fwd_kernel<T, kMaxBessel, false>);
+  }
 }
 template void edge_geom_fwd<float>(int, int, const double*, const int*, const int*, const int*, const Arch&,
                                    float*, float*, const double*, float*, const float*, int, float*, int, float*,

@@ -38,9 +38,10 @@ struct Arch {
   // per-ordered-species-pair cutoffs (Sec. "Species-dependent cutoffs"), set by
   // allegro_set_pair_cutoffs: device [ns * ns][2] = {1/rc, sqrt(2/rc)} of pair
   // (Z_i, Z_j) for the basis and envelope, and device [ns * ns] rc^2 for the
-  // neighbour test; null: the model cutoff rc for every pair
+  // neighbour test (and its float32 rounding for the prefilter); null: the model cutoff rc for every pair
   const float* pair_basis = nullptr;
   const double* pair_rc2 = nullptr;
+  const float* pair_rc2f = nullptr;
   // ZBL repulsion (Sec. "Training details"), set by allegro_set_zbl: device
   // [ns * ns][2] = {k_e Z_a Z_b / 2, 1 / a_s} per ordered species pair; null: no ZBL term
   const float* zbl = nullptr;
@@ -176,6 +177,11 @@ struct CellGrid {
   int R[3];           // stencil radius per axis
   double lo[3], span[3];   // non-periodic axes: frac range mapped onto the grid
   int n_centres;      // atoms [0, n_centres) are centres; the rest (ghosts) only neighbours
+  // float32 values of `cell` and of the squared search radius, rounded on the host: the conversions
+  // are float64 instructions, the slow unit of this part (ten of them per warp took half of the
+  // warp-per-atom count pass)
+  float cellf[9];
+  float rc2f;
 };
 // cell_count: zero on entry; cell_rank[i]: atom i's arrival order in its cell
 void nb_bin(const double* pos, int n, const CellGrid& g, int* cell_of, int* wrap, int* cell_count, int* cell_rank,
@@ -186,13 +192,13 @@ void nb_place(const int* seg_of, const int* rank, int n, const int* start, int* 
 // bits in w) and float64 positions and the wrap counts, all in cell order
 void nb_sort_cells(const double* pos, const int* species, const CellGrid& g, int n_cells, const int* cell_start,
                    const int* wrap, int* sorted, float4* pos4, double* pw, int4* wraps, cudaStream_t st);
-// pair_rc2: null, or device [ns * ns] squared cutoffs per ordered species pair
-// (each <= rc2, the search radius; `band` is the prefilter band of rc2).  The fill passes also count
+// pair_rc2 (and pair_rc2f, its float32 rounding): null, or device [ns * ns] squared cutoffs per
+// ordered species pair (each <= rc2, the search radius; `band` is the prefilter band of rc2).  The fill passes also count
 // every edge into its neighbour's column (col_count, zero on entry) and keep its arrival order there
 // (col_rank[e]); nb_search returns false when it left that to nb_col_rank.
 bool nb_search(bool fill, const double* pos, int n, const CellGrid& g, const int* cell_of,
                const int4* wraps, const int* cell_start, const int* sorted, const float4* pos4, const double* pw,
-               double rc2, float band, const double* pair_rc2, int ns, int* count, const int* row_ptr, int* ej,
+               double rc2, float band, const double* pair_rc2, const float* pair_rc2f, int ns, int* count, const int* row_ptr, int* ej,
                int* ei, int* eS, double* ed, int* col_count, int* col_rank, int edge_cap, int* d_err,
                cudaStream_t st);
 void nb_bruteforce_batched(bool fill, const double* pos, const int64_t* offs, int nstruct,

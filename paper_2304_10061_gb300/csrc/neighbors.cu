@@ -386,16 +386,28 @@ void nb_sort_columns(const int* col_ptr, int n, int* col_edge, cudaStream_t st) 
 // ---------------------------------------------------------------------------
 // exact pair test (float64, explicitly rounded, no contraction)
 // ---------------------------------------------------------------------------
+// (of the home image the offset is zero and adding it leaves pos_j as it is: float64 is the slow unit
+// here, so a warp without images skips the 15 operations that form it)
+__device__ __forceinline__ void pair_disp(const double* __restrict__ pi, const double* __restrict__ pj,
+                                          const double* cell, int S0, int S1, int S2, double d[3]) {
+  double p[3] = {pj[0], pj[1], pj[2]};
+  if (S0 | S1 | S2) {
+    const double s0 = (double)S0, s1 = (double)S1, s2 = (double)S2;
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+      const double off = __dadd_rn(__dadd_rn(__dmul_rn(s0, cell[0 * 3 + x]), __dmul_rn(s1, cell[1 * 3 + x])),
+                                   __dmul_rn(s2, cell[2 * 3 + x]));
+      p[x] = __dadd_rn(p[x], off);
+    }
+  }
+#pragma unroll
+  for (int x = 0; x < 3; ++x) d[x] = __dsub_rn(p[x], pi[x]);
+}
+
 __device__ __forceinline__ bool pair_test(const double* __restrict__ pi, const double* __restrict__ pj,
                                           const double* cell, int S0, int S1, int S2, double rc2,
                                           double d[3]) {
-  double s0 = (double)S0, s1 = (double)S1, s2 = (double)S2;
-#pragma unroll
-  for (int x = 0; x < 3; ++x) {
-    double off = __dadd_rn(__dadd_rn(__dmul_rn(s0, cell[0 * 3 + x]), __dmul_rn(s1, cell[1 * 3 + x])),
-                           __dmul_rn(s2, cell[2 * 3 + x]));
-    d[x] = __dsub_rn(__dadd_rn(pj[x], off), pi[x]);
-  }
+  pair_disp(pi, pj, cell, S0, S1, S2, d);
   double r2 = __dadd_rn(__dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1])), __dmul_rn(d[2], d[2]));
   return r2 < rc2;
 }
@@ -546,18 +558,6 @@ constexpr int kSearchThreads = 128;
 // 1,553 + 3,298 / 804 + 2,517 (the warp form issues more instructions per candidate).
 constexpr int kSearchWarpAtoms = 65536;
 
-// The displacement of pair_test (the same float64 operations in the same order).
-__device__ __forceinline__ void pair_disp(const double* __restrict__ pi, const double* __restrict__ pj,
-                                          const double* cell, int S0, int S1, int S2, double d[3]) {
-  double s0 = (double)S0, s1 = (double)S1, s2 = (double)S2;
-#pragma unroll
-  for (int x = 0; x < 3; ++x) {
-    double off = __dadd_rn(__dadd_rn(__dmul_rn(s0, cell[0 * 3 + x]), __dmul_rn(s1, cell[1 * 3 + x])),
-                           __dmul_rn(s2, cell[2 * 3 + x]));
-    d[x] = __dsub_rn(__dadd_rn(pj[x], off), pi[x]);
-  }
-}
-
 // image q (three signed 10-bit fields) and the exact-test flag of a staged edge
 __device__ __forceinline__ int pack_q(int q0, int q1, int q2, bool exact) {
   return (q0 & 1023) | ((q1 & 1023) << 10) | ((q2 & 1023) << 20) | (exact ? (1 << 30) : 0);
@@ -586,8 +586,8 @@ __global__ void __launch_bounds__(kSearchThreads) search_kernel(
     const double* __restrict__ pos, int n, CellGrid g, const int* __restrict__ cell_of,
     const int4* __restrict__ wraps, const int* __restrict__ cell_start, const int* __restrict__ sorted,
     const float4* __restrict__ pos4, const double* __restrict__ pw, double rc2, float band,
-    const double* __restrict__ pair_rc2, int ns, int* __restrict__ count, const int* __restrict__ row_ptr,
-    int* __restrict__ ej, int* __restrict__ ei, int* __restrict__ eS, double* __restrict__ ed,
+    const double* __restrict__ pair_rc2, const float* __restrict__ pair_rc2f, int ns, int* __restrict__ count,
+    const int* __restrict__ row_ptr, int* __restrict__ ej, int* __restrict__ ei, int* __restrict__ eS, double* __restrict__ ed,
     int* __restrict__ col_count, int* __restrict__ col_rank, int edge_cap, int* __restrict__ d_err) {
   if (fill && !list_fits(row_ptr, n, edge_cap)) return;
   constexpr int kWarps = kSearchThreads / 32;
@@ -608,11 +608,11 @@ __global__ void __launch_bounds__(kSearchThreads) search_kernel(
   const float4 pi4 = pos4[t];
   const double pi[3] = {pos[3 * (size_t)i], pos[3 * (size_t)i + 1], pos[3 * (size_t)i + 2]};
   const int c2 = ci % g.n[2], c1 = (ci / g.n[2]) % g.n[1], c0 = ci / (g.n[2] * g.n[1]);
-  const float rc2f = (float)rc2;
-  const float lo2 = rc2f - band, hi2 = rc2f + band;
+  const float lo2 = g.rc2f - band, hi2 = g.rc2f + band;
   // per-ordered-pair cutoffs: row of the centre's species (the band of the largest
   // cutoff bounds the float32 error of every smaller one)
   const double* prow = pair_rc2 ? pair_rc2 + (size_t)__float_as_int(pi4.w) * ns : nullptr;
+  const float* prowf = pair_rc2f + (size_t)(pair_rc2 ? __float_as_int(pi4.w) : 0) * ns;
   const int base = fill ? row_ptr[i] : 0;
   const int cap = fill ? (row_ptr[i + 1] - base) : 0;
   int k = 0;         // accepted so far
@@ -634,10 +634,10 @@ __global__ void __launch_bounds__(kSearchThreads) search_kernel(
       } else {
 #pragma unroll
         for (int x = 0; x < 3; ++x) {
-          const double qoff = (q0 | q1 | q2) ? ((double)q0 * g.cell[x] + (double)q1 * g.cell[3 + x]) +
-                                                   (double)q2 * g.cell[6 + x]
-                                             : 0.0;
-          d[x] = (pw[3 * (size_t)s + x] + qoff) - pw[3 * (size_t)t + x];
+          double pj = pw[3 * (size_t)s + x];
+          if (q0 | q1 | q2)
+            pj += ((double)q0 * g.cell[x] + (double)q1 * g.cell[3 + x]) + (double)q2 * g.cell[6 + x];
+          d[x] = pj - pw[3 * (size_t)t + x];
         }
       }
       const size_t o = (size_t)base + k0 + lane;
@@ -672,9 +672,9 @@ __global__ void __launch_bounds__(kSearchThreads) search_kernel(
         b = cell_start[cell];
         cnt = cell_start[cell + 1] - b;
         const float q0 = (float)q[0], q1 = (float)q[1], q2 = (float)q[2];
-        sc.ox = q0 * (float)g.cell[0] + q1 * (float)g.cell[3] + q2 * (float)g.cell[6] - pi4.x;
-        sc.oy = q0 * (float)g.cell[1] + q1 * (float)g.cell[4] + q2 * (float)g.cell[7] - pi4.y;
-        sc.oz = q0 * (float)g.cell[2] + q1 * (float)g.cell[5] + q2 * (float)g.cell[8] - pi4.z;
+        sc.ox = q0 * g.cellf[0] + q1 * g.cellf[3] + q2 * g.cellf[6] - pi4.x;
+        sc.oy = q0 * g.cellf[1] + q1 * g.cellf[4] + q2 * g.cellf[7] - pi4.y;
+        sc.oz = q0 * g.cellf[2] + q1 * g.cellf[5] + q2 * g.cellf[8] - pi4.z;
         sc.q = pack_q(q[0], q[1], q[2], false);
       }
     }
@@ -704,11 +704,9 @@ __global__ void __launch_bounds__(kSearchThreads) search_kernel(
         const float4 pj = pos4[s];
         const float dx = pj.x + ce.ox, dy = pj.y + ce.oy, dz = pj.z + ce.oz;
         const float r2f = dx * dx + dy * dy + dz * dz;
-        double rc2p = rc2;
         float lo2p = lo2, hi2p = hi2;
         if (prow) {
-          rc2p = prow[__float_as_int(pj.w)];
-          const float rc2pf = (float)rc2p;
+          const float rc2pf = prowf[__float_as_int(pj.w)];
           lo2p = rc2pf - band;
           hi2p = fminf(hi2, rc2pf + band);
         }
@@ -722,7 +720,9 @@ __global__ void __launch_bounds__(kSearchThreads) search_kernel(
             const int S2 = g.pbc[2] ? unpack_q(ce.q, 2) - wj.z + wi.z : 0;
             if (s == t && S0 == 0 && S1 == 0 && S2 == 0) keep = false;   // (s = t: j = i)
             double d[3];
-            if (keep && exact) keep = pair_test(pi, pos + 3 * (size_t)sorted[s], g.cell, S0, S1, S2, rc2p, d);
+            if (keep && exact)
+              keep = pair_test(pi, pos + 3 * (size_t)sorted[s], g.cell, S0, S1, S2,
+                               prow ? prow[__float_as_int(pj.w)] : rc2, d);
           }
           en = make_int2(s, ce.q | (exact ? (1 << 30) : 0));
         }
@@ -768,8 +768,8 @@ __global__ void __launch_bounds__(kSearchThreads) search_thread_kernel(
     const double* __restrict__ pos, int n, CellGrid g, const int* __restrict__ cell_of,
     const int4* __restrict__ wraps, const int* __restrict__ cell_start, const int* __restrict__ sorted,
     const float4* __restrict__ pos4, const double* __restrict__ pw, double rc2, float band,
-    const double* __restrict__ pair_rc2, int ns, int* __restrict__ count, const int* __restrict__ row_ptr,
-    int* __restrict__ ej, int* __restrict__ ei, int* __restrict__ eS, double* __restrict__ ed,
+    const double* __restrict__ pair_rc2, const float* __restrict__ pair_rc2f, int ns, int* __restrict__ count,
+    const int* __restrict__ row_ptr, int* __restrict__ ej, int* __restrict__ ei, int* __restrict__ eS, double* __restrict__ ed,
     int edge_cap, int* __restrict__ d_err) {
   if (fill && !list_fits(row_ptr, n, edge_cap)) return;
   __shared__ int2 stage[fill ? kSearchThreads : 1][fill ? kFillStage : 1];
@@ -799,14 +799,12 @@ __global__ void __launch_bounds__(kSearchThreads) search_thread_kernel(
       pwi[x] = pw[3 * (size_t)t + x];
     }
     const float4 pi4 = pos4[t];
-    const float rc2f = (float)rc2;
-    const float lo2 = rc2f - band, hi2 = rc2f + band;
+    const float lo2 = g.rc2f - band, hi2 = g.rc2f + band;
     // per-ordered-pair cutoffs: row of the centre's species (the band of the largest
     // cutoff bounds the float32 error of every smaller one)
     const double* prow = pair_rc2 ? pair_rc2 + (size_t)__float_as_int(pi4.w) * ns : nullptr;
-    float cf[9];
-#pragma unroll
-    for (int q = 0; q < 9; ++q) cf[q] = (float)g.cell[q];
+    const float* prowf = pair_rc2f + (size_t)(pair_rc2 ? __float_as_int(pi4.w) : 0) * ns;
+    const float* cf = g.cellf;
     base = fill ? row_ptr[i] : 0;
     cap = fill ? (row_ptr[i + 1] - base) : 0;
     for (int d0 = -g.R[0]; d0 <= g.R[0]; ++d0) {
@@ -832,11 +830,9 @@ __global__ void __launch_bounds__(kSearchThreads) search_thread_kernel(
             const float dx = pj.x + ox, dy = pj.y + oy, dz = pj.z + oz;
             const float r2f = dx * dx + dy * dy + dz * dz;
             if (r2f > hi2) continue;
-            double rc2p = rc2;
             float lo2p = lo2;
             if (prow) {
-              rc2p = prow[__float_as_int(pj.w)];
-              const float rc2pf = (float)rc2p;
+              const float rc2pf = prowf[__float_as_int(pj.w)];
               if (r2f > rc2pf + band) continue;
               lo2p = rc2pf - band;
             }
@@ -847,7 +843,9 @@ __global__ void __launch_bounds__(kSearchThreads) search_thread_kernel(
             if (s == t && S0 == 0 && S1 == 0 && S2 == 0) continue;   // (s = t: j = i)
             const bool exact = r2f >= lo2p;
             double d[3];
-            if (exact && !pair_test(pi, pos + 3 * (size_t)sorted[s], g.cell, S0, S1, S2, rc2p, d)) continue;
+            if (exact && !pair_test(pi, pos + 3 * (size_t)sorted[s], g.cell, S0, S1, S2,
+                                    prow ? prow[__float_as_int(pj.w)] : rc2, d))
+              continue;
             if constexpr (fill) {
               if (k < kFillStage) {
                 stage[threadIdx.x][k] = make_int2(s, pack_q(q0, q1, q2, exact));
@@ -930,20 +928,20 @@ __global__ void __launch_bounds__(kSearchThreads) search_thread_kernel(
 
 bool nb_search(bool fill, const double* pos, int n, const CellGrid& g, const int* cell_of,
                const int4* wraps, const int* cell_start, const int* sorted, const float4* pos4, const double* pw,
-               double rc2, float band, const double* pair_rc2, int ns, int* count, const int* row_ptr, int* ej,
-               int* ei, int* eS, double* ed, int* col_count, int* col_rank, int edge_cap, int* d_err,
+               double rc2, float band, const double* pair_rc2, const float* pair_rc2f, int ns, int* count, const int* row_ptr,
+               int* ej,               int* ei, int* eS, double* ed, int* col_count, int* col_rank, int edge_cap, int* d_err,
                cudaStream_t st) {
   if (n <= 0) return true;
   if (n <= kSearchWarpAtoms) {
     auto kernel = fill ? search_kernel<true> : search_kernel<false>;
     kernel<<<(n + kSearchThreads / 32 - 1) / (kSearchThreads / 32), kSearchThreads, 0, st>>>(
-        pos, n, g, cell_of, wraps, cell_start, sorted, pos4, pw, rc2, band, pair_rc2, ns, count, row_ptr, ej, ei, eS, ed,
+        pos, n, g, cell_of, wraps, cell_start, sorted, pos4, pw, rc2, band, pair_rc2, pair_rc2f, ns, count, row_ptr, ej, ei, eS, ed,
         col_count, col_rank, edge_cap, d_err);
     return true;
   }
   auto kernel = fill ? search_thread_kernel<true> : search_thread_kernel<false>;
   kernel<<<(n + kSearchThreads - 1) / kSearchThreads, kSearchThreads, 0, st>>>(
-      pos, n, g, cell_of, wraps, cell_start, sorted, pos4, pw, rc2, band, pair_rc2, ns, count, row_ptr, ej, ei, eS, ed,
+      pos, n, g, cell_of, wraps, cell_start, sorted, pos4, pw, rc2, band, pair_rc2, pair_rc2f, ns, count, row_ptr, ej, ei, eS, ed,
       edge_cap, d_err);
   return false;
 }
