@@ -447,6 +447,15 @@ __global__ void __launch_bounds__(kChainThreads) gen_chain_bwd_kernel(GenRowIO i
   for (int k = 0; k < L; ++k)
 #pragma unroll
     for (int b = 0; b < S; ++b) G[k][b] = io.G[k + 1][o + (size_t)b * io.C];
+  // what the layers above left in Gammabar, loaded with the operands (left to the additions at the
+  // end, these loads' latency was 80 % of the two-layer chain's time)
+  float old[L < NL ? L : 1][S];
+  if constexpr (L < NL) {
+#pragma unroll
+    for (int k = 0; k < L; ++k)
+#pragma unroll
+      for (int b = 0; b < S; ++b) old[k][b] = io.Gb[k + 1][o + (size_t)b * io.C];
+  }
   // r_{L+1} = e_0, r_k = M^k r_{k+1}: r[k - 2] holds r_k for k = 2..L
   float r[L > 1 ? L - 1 : 1][kGenMaxD];
   float dummy[kGenMaxD];
@@ -459,10 +468,7 @@ __global__ void __launch_bounds__(kChainThreads) gen_chain_bwd_kernel(GenRowIO i
   auto flush = [&](int k) {
     float* g = io.Gb[k] + o;
 #pragma unroll
-    for (int b = 0; b < S; ++b) {
-      float* p = g + (size_t)b * io.C;
-      *p = (L == NL) ? gb[b] : *p + gb[b];
-    }
+    for (int b = 0; b < S; ++b) g[(size_t)b * io.C] = (L == NL) ? gb[b] : old[L < NL ? k - 1 : 0][b] + gb[b];
   };
   if constexpr (L == 1) {
     chain_adj<LMAX, NL, 1, true, false>(w.v, G[0], rb, dummy, gb, nb);
@@ -487,9 +493,12 @@ __global__ void __launch_bounds__(kChainThreads) gen_chain_bwd_kernel(GenRowIO i
 //   wbar^1_{e,u,l} = nu sum_{a in l} Gammabar^1[a] Y_e[a]
 //   Ybar_e[a]      = sum_u (w^0_{e,u,l(a)} qs[a] + nu sum_L w^L_{e,u,l(a)} Gammabar^L[a])
 // The channel sums of Ybar: warp halving sums, then the warps' partials in a fixed order.
-template <typename T, int LMAX, int NL>
+// AMAX: record max|wbar| (FP8 precision).
+// Bound: instruction issue (the 16-component halving sums and the unpacking of the bf16 operands
+// beside the multiply-adds, which run on component pairs in packed fp32).
+template <typename T, int LMAX, int NL, bool AMAX>
 __global__ void __launch_bounds__(kMaxChannels) gen_edge_final_kernel(GenRowIO io) {
-  constexpr int S = (LMAX + 1) * (LMAX + 1), LM = LMAX + 1;
+  constexpr int S = (LMAX + 1) * (LMAX + 1), LM = LMAX + 1, S2 = (S + 1) / 2;
   static_assert(S <= 16, "halving sums of 16 components");
   // per-warp channel partials of Ybar for batches of kEdgeBatch edges, double-buffered:
   // one barrier per batch
@@ -500,41 +509,73 @@ __global__ void __launch_bounds__(kMaxChannels) gen_edge_final_kernel(GenRowIO i
   const bool act = u < io.C;
   const int rb = io.row_ptr[io.a0 + ia] - io.e0, re = io.row_ptr[io.a0 + ia + 1] - io.e0;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = (int)(blockDim.x >> 5);
-  float q[NL][S], gb[NL][S];
+  float2 q[NL][S2], gb[NL][S2];   // component pairs (2 i, 2 i + 1); an odd S is padded with zeros
   const size_t o = (size_t)ia * S * io.C + (act ? u : 0);
 #pragma unroll
   for (int L = 0; L < NL; ++L)
 #pragma unroll
-    for (int a = 0; a < S; ++a) {
-      q[L][a] = act ? io.Q[L + 1][o + (size_t)a * io.C] : 0.0f;
-      gb[L][a] = act ? io.nu * io.Gb[L + 1][o + (size_t)a * io.C] : 0.0f;
+    for (int i = 0; i < S2; ++i) {
+      auto at = [&](const float* p, int a) { return (act && a < S) ? p[o + (size_t)a * io.C] : 0.0f; };
+      q[L][i] = make_float2(at(io.Q[L + 1], 2 * i), at(io.Q[L + 1], 2 * i + 1));
+      gb[L][i] = make_float2(io.nu * at(io.Gb[L + 1], 2 * i), io.nu * at(io.Gb[L + 1], 2 * i + 1));
     }
   // the warp's ring: per edge its 32 channels of w^0 .. w^NL, of sbar^1 .. sbar^NL, and Y
   constexpr int kW = 32 * LM * (int)sizeof(T), kSb = 32 * (int)sizeof(T);
   constexpr int kOffS = (NL + 1) * kW, kOffY = kOffS + NL * kSb, kStage = round16(kOffY + S * 4);
   __shared__ __align__(16) unsigned char rings[kMaxChannels / 32][kRing * kStage];
   const int nch = min(32, io.C);   // channels of a warp
-  const unsigned char* wsrc[NL + 1];
-  const unsigned char* ssrc[NL];
-  unsigned sal[NL];
+  auto wsrc = [&](int L) {
+    return reinterpret_cast<const unsigned char*>(reinterpret_cast<const T*>(io.w[L]) + io.wcol[L] + wid * 32 * LM);
+  };
+  auto ssrc = [&](int L) {
+    return reinterpret_cast<const unsigned char*>(reinterpret_cast<const T*>(io.sbar[L + 1]) + io.sbar_off[L + 1] +
+                                                  wid * 32);
+  };
+  auto sal = [&](int L) {
+    return (unsigned)((reinterpret_cast<uintptr_t>(ssrc(L)) | (io.ldsbar[L + 1] * sizeof(T)) | (nch * sizeof(T))) & 15);
+  };
+  // With whole warps of channels and aligned sbar rows a lane's share of an edge is the same
+  // 16-byte pieces every time: kNW of w, and one of sbar or Y.  Their addresses are kept and moved
+  // on by a row per edge.
+  constexpr int kCW = kW / 16, kNW = ((NL + 1) * kCW + 31) / 32, kCS = kSb / 16, kCY = S % 4 == 0 ? S / 4 : 0;
+  static_assert(NL * kCS + kCY <= 32, "one piece of sbar or Y per lane");
+  bool fast = io.C >= 32;
 #pragma unroll
-  for (int L = 0; L <= NL; ++L)
-    wsrc[L] = reinterpret_cast<const unsigned char*>(reinterpret_cast<const T*>(io.w[L]) + io.wcol[L] + wid * 32 * LM);
+  for (int L = 0; L < NL; ++L) fast = fast && sal(L) == 0;
+  const unsigned char* wp[kNW];
+  int wpitch[kNW];
 #pragma unroll
-  for (int L = 0; L < NL; ++L) {
-    ssrc[L] = reinterpret_cast<const unsigned char*>(reinterpret_cast<const T*>(io.sbar[L + 1]) + io.sbar_off[L + 1] +
-                                                     wid * 32);
-    sal[L] = (unsigned)((reinterpret_cast<uintptr_t>(ssrc[L]) | (io.ldsbar[L + 1] * sizeof(T)) | (nch * sizeof(T))) & 15);
+  for (int k = 0; k < kNW; ++k) {
+    const int id = lane + 32 * k, L = min(id / kCW, NL);
+    wpitch[k] = io.ldw[L] * (int)sizeof(T);
+    wp[k] = wsrc(L) + (size_t)rb * wpitch[k] + id % kCW * 16;
   }
+  const bool isS = lane < NL * kCS, isY = kCY > 0 && !isS && lane < NL * kCS + kCY;
+  const int sl = min(lane / kCS, NL - 1);
+  int xpitch = isS ? io.ldsbar[sl + 1] * (int)sizeof(T) : S * 4;
+  const unsigned char* xp = isS ? ssrc(sl) + lane % kCS * 16
+                                : reinterpret_cast<const unsigned char*>(io.Y) + (isY ? (lane - NL * kCS) * 16 : 0);
+  xp += (size_t)rb * xpitch;
   auto copy = [&](int e, unsigned char* st) {
+    if (fast) {
+#pragma unroll
+      for (int k = 0; k < kNW; ++k) {
+        if ((NL + 1) * kCW % 32 == 0 || lane + 32 * k < (NL + 1) * kCW) cp_async16(st + (lane + 32 * k) * 16, wp[k]);
+        wp[k] += wpitch[k];
+      }
+      if (isS || isY) cp_async16(st + kOffS + lane * 16, xp);
+      xp += xpitch;
+      if (kCY == 0 && lane < S) cp_async4(st + kOffY + lane * 4, io.Y + (size_t)e * S + lane);
+      return;
+    }
     // the w rows are 16-byte aligned (pitches of 8 elements, columns at multiples of 8 (l_max + 1))
 #pragma unroll
     for (int L = 0; L <= NL; ++L)
       for (int k = lane * 16; k < nch * LM * (int)sizeof(T); k += 512)
-        cp_async16(st + L * kW + k, wsrc[L] + (size_t)e * io.ldw[L] * sizeof(T) + k);
+        cp_async16(st + L * kW + k, wsrc(L) + (size_t)e * io.ldw[L] * sizeof(T) + k);
 #pragma unroll
     for (int L = 0; L < NL; ++L)
-      warp_copy(st + kOffS + L * kSb, ssrc[L] + (size_t)e * io.ldsbar[L + 1] * sizeof(T), nch * (int)sizeof(T), sal[L]);
+      warp_copy(st + kOffS + L * kSb, ssrc(L) + (size_t)e * io.ldsbar[L + 1] * sizeof(T), nch * (int)sizeof(T), sal(L));
     if (lane < S) cp_async4(st + kOffY + lane * 4, io.Y + (size_t)e * S + lane);
   };
   T* w0b = reinterpret_cast<T*>(io.wbar[0]);
@@ -560,32 +601,44 @@ __global__ void __launch_bounds__(kMaxChannels) gen_edge_final_kernel(GenRowIO i
 #pragma unroll
     for (int a = 0; a < 16; ++a) yc[a] = 0.0f;
     if (act) {
-      float qs[S], w0l[LM], g0[LM] = {}, g1[LM] = {};
+      float2 qs[S2], yp[S2];
+      float w0l[LM], g0[LM] = {}, g1[LM] = {};
 #pragma unroll
-      for (int a = 0; a < S; ++a) qs[a] = 0.0f;
+      for (int i = 0; i < S2; ++i) qs[i] = yp[i] = make_float2(0.0f, 0.0f);
+      // the weights of a component pair
+      auto wpair = [](const float (&x)[LM], int i) {
+        return make_float2(x[l_of(2 * i)], x[2 * i + 1 < S ? l_of(2 * i + 1) : 0]);
+      };
 #pragma unroll
       for (int L = 0; L < NL; ++L) {
         const float sb = gld(ss + L * 32 + lane);
         float wl[LM];
         load_lm<T, LM>(ws + (L + 1) * 32 * LM + lane * LM, wl);
 #pragma unroll
-        for (int a = 0; a < S; ++a) {
-          qs[a] = fmaf(sb, q[L][a], qs[a]);
-          yc[a] = fmaf(wl[l_of(a)], gb[L][a], yc[a]);
+        for (int i = 0; i < S2; ++i) {
+          qs[i] = __ffma2_rn(make_float2(sb, sb), q[L][i], qs[i]);
+          yp[i] = __ffma2_rn(wpair(wl, i), gb[L][i], yp[i]);
         }
       }
       load_lm<T, LM>(ws + lane * LM, w0l);
 #pragma unroll
+      for (int i = 0; i < S2; ++i) {
+        yp[i] = __ffma2_rn(wpair(w0l, i), qs[i], yp[i]);
+        yc[2 * i] = yp[i].x;
+        if (2 * i + 1 < S) yc[2 * i + 1] = yp[i].y;
+      }
+#pragma unroll
       for (int a = 0; a < S; ++a) {
         const float ya = y[a];
-        g0[l_of(a)] = fmaf(ya, qs[a], g0[l_of(a)]);
-        g1[l_of(a)] = fmaf(ya, gb[0][a], g1[l_of(a)]);
-        yc[a] = fmaf(w0l[l_of(a)], qs[a], yc[a]);
+        g0[l_of(a)] = fmaf(ya, (a & 1) ? qs[a / 2].y : qs[a / 2].x, g0[l_of(a)]);
+        g1[l_of(a)] = fmaf(ya, (a & 1) ? gb[0][a / 2].y : gb[0][a / 2].x, g1[l_of(a)]);
       }
       store_lm<T, LM>(w0b + (size_t)e * io.ldwbar[0] + io.wbcol[0] + u * LM, g0);
       store_lm<T, LM>(w1b + (size_t)e * io.ldwbar[1] + io.wbcol[1] + u * LM, g1);
+      if constexpr (AMAX) {
 #pragma unroll
-      for (int l = 0; l < LM; ++l) gmax = fmaxf(gmax, fmaxf(fabsf(g0[l]), fabsf(g1[l])));
+        for (int l = 0; l < LM; ++l) gmax = fmaxf(gmax, fmaxf(fabsf(g0[l]), fabsf(g1[l])));
+      }
     }
     const float t = warp_sum16(yc);   // component lane / 2
     if ((lane & 1) == 0) red[buf][j][wid][lane >> 1] = t;
@@ -596,7 +649,7 @@ __global__ void __launch_bounds__(kMaxChannels) gen_edge_final_kernel(GenRowIO i
       buf ^= 1;
     }
   });
-  record_amax(io.amax_wbar, gmax);
+  if constexpr (AMAX) record_amax(io.amax_wbar, gmax);
 }
 
 // ---------------------------------------------------------------------------
@@ -846,10 +899,17 @@ static void bwd_lmax(const GenRowIO& io, int L, cudaStream_t st) {
   const int bl = block_of(io.C);
   GEN_W_LAUNCH(gen_qbar_w_kernel, io, L);
   chain_bwd_nl<LMAX>(io, L, st);
-  if (L >= 2) GEN_W_LAUNCH(gen_wbar_w_kernel, io, L);
-  else if (io.nl == 1) gen_edge_final_kernel<T, LMAX, 1><<<io.na, bl, 0, st>>>(io);
-  else if (io.nl == 2) gen_edge_final_kernel<T, LMAX, 2><<<io.na, bl, 0, st>>>(io);
-  else gen_edge_final_kernel<T, LMAX, 3><<<io.na, bl, 0, st>>>(io);
+  if (L >= 2) {
+    GEN_W_LAUNCH(gen_wbar_w_kernel, io, L);
+    return;
+  }
+  auto final = [&](auto plain, auto recorded) {
+    if (io.amax_wbar) recorded<<<io.na, bl, 0, st>>>(io);
+    else plain<<<io.na, bl, 0, st>>>(io);
+  };
+  if (io.nl == 1) final(gen_edge_final_kernel<T, LMAX, 1, false>, gen_edge_final_kernel<T, LMAX, 1, true>);
+  else if (io.nl == 2) final(gen_edge_final_kernel<T, LMAX, 2, false>, gen_edge_final_kernel<T, LMAX, 2, true>);
+  else final(gen_edge_final_kernel<T, LMAX, 3, false>, gen_edge_final_kernel<T, LMAX, 3, true>);
 }
 
 template <typename T>
