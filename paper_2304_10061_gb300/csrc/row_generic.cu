@@ -59,6 +59,7 @@
 
 #include "amax.cuh"
 #include "internal.h"
+#include "row_ring.cuh"
 
 namespace alg {
 
@@ -140,65 +141,7 @@ __device__ __forceinline__ float warp_sum16(float (&v)[16]) {
   return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
-// ---------------------------------------------------------------------------
-// Asynchronous copies of an edge's rows into shared memory, so that a warp has
-// several edges' loads in flight without holding them in registers (the row
-// kernels keep 64 to 100 floats of per-channel state, which leaves 8 to 16
-// warps per SM: with one or two edges in flight each they waited on latency).
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
-// `bytes` (even) contiguous bytes at src to dst (16-byte aligned) by the warp; `al` = the low four bits of src and
-// bytes or'ed: 16-byte copies when they are zero, else 4-byte ones, else plain 2-byte copies (latent
-// widths that are odd in bf16)
-__device__ __forceinline__ void warp_copy(unsigned char* dst, const unsigned char* src, int bytes, unsigned al) {
-  const int lane = threadIdx.x & 31;
-  if (al == 0) {
-    for (int k = lane * 16; k < bytes; k += 512) cp_async16(dst + k, src + k);
-  } else if ((al & 3) == 0) {
-    for (int k = lane * 4; k < bytes; k += 128) cp_async4(dst + k, src + k);
-  } else {
-    for (int k = lane * 2; k < bytes; k += 64)
-      *reinterpret_cast<unsigned short*>(dst + k) = *reinterpret_cast<const unsigned short*>(src + k);
-  }
-}
-
 constexpr int kRing = 4;   // edges in flight per warp (stages of its shared-memory ring)
-
-__host__ __device__ constexpr int round16(int x) { return (x + 15) / 16 * 16; }
-
-// A warp's ring over its row's edges.  copy(e, slot) queues edge e's rows into a slot; for each edge
-// in order, use(e, slot) runs once the edge's rows have arrived, with the next kRing - 1 edges queued.
-template <int STAGE, typename Copy, typename Use>
-__device__ __forceinline__ void ring_over(unsigned char* ring, int rb, int re, Copy&& copy, Use&& use) {
-#pragma unroll
-  for (int p = 0; p < kRing - 1; ++p) {
-    if (rb + p < re) copy(rb + p, ring + p * STAGE);
-    cp_async_commit();
-  }
-  int slot = 0;
-  for (int e = rb; e < re; ++e) {
-    cp_async_wait<kRing - 2>();
-    __syncwarp();   // every lane's copies of edge e have landed, and no lane still reads the slot before it
-    const int nslot = (slot + kRing - 1) % kRing;
-    if (e + kRing - 1 < re) copy(e + kRing - 1, ring + nslot * STAGE);
-    cp_async_commit();
-    use(e, ring + slot * STAGE);
-    slot = (slot + 1) % kRing;
-  }
-}
 
 constexpr int kChainThreads = 128;   // (atom, channel) pairs per block of the chain kernels
 
@@ -591,7 +534,7 @@ __global__ void __launch_bounds__(kMaxChannels) gen_edge_final_kernel(GenRowIO i
     }
   };
   int buf = 0;
-  ring_over<kStage>(rings[wid], rb, re, copy, [&](int e, const unsigned char* st) {
+  ring_over<kRing, kStage>(rings[wid], rb, re, copy, [&](int e, const unsigned char* st) {
     const int j = (e - rb) % kEdgeBatch;
     const T* ws = reinterpret_cast<const T*>(st);
     const T* ss = reinterpret_cast<const T*>(st + kOffS);
@@ -697,7 +640,7 @@ __global__ void __launch_bounds__(32 * kGenWarps) gen_env_w_kernel(GenRowIO io, 
     warp_copy(st, reinterpret_cast<const unsigned char*>(w + (size_t)e * ldw), row_bytes, 0);
     if (g.lane < S) cp_async4(st + kW + g.lane * 4, io.Y + (size_t)e * S + g.lane);
   };
-  ring_over<kStage>(rings[threadIdx.x >> 5], g.rb, g.re, copy, [&](int, const unsigned char* st) {
+  ring_over<kRing, kStage>(rings[threadIdx.x >> 5], g.rb, g.re, copy, [&](int, const unsigned char* st) {
     if (!g.act) return;
     float y[S];
     load_y<S>(reinterpret_cast<const float*>(st + kW), y);
@@ -739,7 +682,7 @@ __global__ void __launch_bounds__(32 * kGenWarps) gen_s_w_kernel(GenRowIO io, in
     warp_copy(st, reinterpret_cast<const unsigned char*>(w0 + (size_t)e * ldw0), row_bytes, 0);
     if (g.lane < S) cp_async4(st + kW + g.lane * 4, io.Y + (size_t)e * S + g.lane);
   };
-  ring_over<kStage>(rings[threadIdx.x >> 5], g.rb, g.re, copy, [&](int e, const unsigned char* st) {
+  ring_over<kRing, kStage>(rings[threadIdx.x >> 5], g.rb, g.re, copy, [&](int e, const unsigned char* st) {
     if (!g.act) return;
     float y[S];
     load_y<S>(reinterpret_cast<const float*>(st + kW), y);
@@ -780,7 +723,7 @@ __global__ void __launch_bounds__(32 * kGenWarps) gen_qbar_w_kernel(GenRowIO io,
     warp_copy(st + kW, reinterpret_cast<const unsigned char*>(sb + (size_t)e * ldsb), io.C * (int)sizeof(T), sal);
     if (g.lane < S) cp_async4(st + kW + kSb + g.lane * 4, io.Y + (size_t)e * S + g.lane);
   };
-  ring_over<kStage>(rings[threadIdx.x >> 5], g.rb, g.re, copy, [&](int, const unsigned char* st) {
+  ring_over<kRing, kStage>(rings[threadIdx.x >> 5], g.rb, g.re, copy, [&](int, const unsigned char* st) {
     if (!g.act) return;
     float y[S];
     load_y<S>(reinterpret_cast<const float*>(st + kW + kSb), y);
@@ -820,7 +763,7 @@ __global__ void __launch_bounds__(32 * kGenWarps) gen_wbar_w_kernel(GenRowIO io,
   auto copy = [&](int e, unsigned char* st) {
     if (g.lane < S) cp_async4(st + g.lane * 4, io.Y + (size_t)e * S + g.lane);
   };
-  ring_over<kStage>(rings[threadIdx.x >> 5], g.rb, g.re, copy, [&](int e, const unsigned char* st) {
+  ring_over<kRing, kStage>(rings[threadIdx.x >> 5], g.rb, g.re, copy, [&](int e, const unsigned char* st) {
     if (!g.act) return;
     float y[S];
     load_y<S>(reinterpret_cast<const float*>(st), y);

@@ -28,6 +28,7 @@
 #include <cuda_bf16.h>
 
 #include "internal.h"
+#include "row_ring.cuh"
 
 namespace alg {
 
@@ -330,7 +331,6 @@ __device__ __forceinline__ void edge_batches(int cnt, Load&& load, Comp&& comp) 
 }
 
 constexpr int kBatchLight = 8;   // edges per batch in passes with one weight array
-constexpr int kBatchHeavy = 4;   // first pass of the layer-1 adjoint (weights + two sbar, most live state)
 constexpr int kBatchLast = 6;  // both passes of the last-layer adjoint (measured: 6 beats 8 and 12 there)
 
 // Gamma-type environment sum over the row: G[j][b] = sum_e w[e][j][l(b)] Y[e][b]
@@ -709,56 +709,119 @@ __global__ void __launch_bounds__(32 * kRowWarps) row_bwd_last_kernel(RowIO io, 
 // The second pass reads the row's w^0 and sbar again (from L2: the row was
 // just read) so that each pass keeps only half the per-channel state.
 // ---------------------------------------------------------------------------
+// An edge's rows (w^0 or [w^0 | w^1], sbar^1, sbar^2, Y) come through a per-warp ring of cp.async
+// copies, several edges ahead; the second pass's first edges are queued before the per-atom part.
+// Bound: instruction issue (about 350 warp instructions per edge).  With batches of loads through
+// registers the passes waited between batches (issue 47 % of cycles); ms, batches / ring: 1,048,576
+// atoms 14.06 / 12.57 (bf16), 2,048 molecules 0.718 / 0.665, 3,072 atoms 0.112 / 0.091 (float32).
 template <typename T, int LMAX, int CPL>
-// (at most 128 registers: four blocks per SM; measured faster than the unbounded 157)
-__global__ void __launch_bounds__(32 * kRowWarps, 4) row_bwd_mid_kernel(RowIO io, TPConst tp) {
+// (at most 128 registers, four blocks per SM, where two channels per lane fit them)
+__global__ void __launch_bounds__(32 * kRowWarps, CPL > 2 ? 2 : 4) row_bwd_mid_kernel(RowIO io, TPConst tp) {
   constexpr int S = (LMAX + 1) * (LMAX + 1);
   constexpr int LM = LMAX + 1;
-  __shared__ __align__(16) float ysm[kRowWarps * kYSeg * YStage<S>::P];
+  using WS = WSpan<T, CPL, LM>;
+  using SW = SbarW<T, CPL>;
+  // stage: w rows, sbar^1, sbar^2, Y (a 16-byte record)
+  constexpr int kW = 64 * CPL * LM * (int)sizeof(T), kSb = 32 * CPL * (int)sizeof(T), kY = ((S + 3) & ~3) * 4;
+  constexpr int kOff1 = kW, kOff2 = kW + kSb, kOffY = kW + 2 * kSb, kStage = kOffY + kY;
+  constexpr int D = kStage <= 1536 ? 6 : (kStage <= 3072 ? 4 : 2);   // edges in flight
+  __shared__ __align__(16) unsigned char rings[kRowWarps][D * kStage];
+  static_assert(kRowWarps * D * kStage <= 48 * 1024, "static shared memory");
   RowCtx r;
   if (!row_ctx<CPL>(io, r)) return;
-  const YStage<S> ys{ysm + (threadIdx.x >> 5) * kYSeg * YStage<S>::P};
+  unsigned char* ring = rings[threadIdx.x >> 5];
   const int nw = io.C * LM;
   const T* W01 = reinterpret_cast<const T*>(io.W01);
   T* wb = reinterpret_cast<T*>(io.wbar01);
-  using WS = WSpan<T, CPL, LM>;
+  // the lane's 16-byte pieces of an edge's w and sbar rows, `nwb` bytes of w (addresses kept and moved
+  // on by a row per edge); sbar rows off 16-byte boundaries are copied in smaller pieces
+  constexpr int NP = (kW + 2 * kSb + 511) / 512;
+  const unsigned char* s1p = reinterpret_cast<const unsigned char*>(io.sbar1);
+  const unsigned char* s2p = reinterpret_cast<const unsigned char*>(io.sbar2);
+  const int pw = io.ld01 * (int)sizeof(T), p1 = io.ld_sbar1 * (int)sizeof(T), p2 = io.ld_sbar2 * (int)sizeof(T);
+  const int nsb = io.C * (int)sizeof(T);
+  const unsigned al1 = (unsigned)((reinterpret_cast<uintptr_t>(s1p) | p1) & 15),
+                 al2 = (unsigned)((reinterpret_cast<uintptr_t>(s2p) | p2) & 15);
+  const unsigned char* src[NP];
+  int pitch[NP], dst[NP];
+  auto pieces = [&](int nwb) {
+    const int n0 = nwb / 16, n1 = al1 ? 0 : nsb / 16, n2 = al2 ? 0 : nsb / 16;
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+      int id = r.lane + 32 * k;
+      dst[k] = -1;
+      src[k] = nullptr;
+      pitch[k] = 0;
+      if (id < n0) {
+        src[k] = reinterpret_cast<const unsigned char*>(W01) + id * 16;
+        pitch[k] = pw;
+        dst[k] = id * 16;
+      } else if ((id -= n0) < n1) {
+        src[k] = s1p + id * 16;
+        pitch[k] = p1;
+        dst[k] = kOff1 + id * 16;
+      } else if ((id -= n1) < n2) {
+        src[k] = s2p + id * 16;
+        pitch[k] = p2;
+        dst[k] = kOff2 + id * 16;
+      }
+      src[k] += (size_t)r.rb * pitch[k];
+    }
+  };
+  auto copy = [&](int e, unsigned char* st) {
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+      if (dst[k] >= 0) cp_async16(st + dst[k], src[k]);
+      src[k] += pitch[k];
+    }
+    if (al1) warp_copy(st + kOff1, s1p + (size_t)e * p1, nsb, al1);
+    if (al2) warp_copy(st + kOff2, s2p + (size_t)e * p2, nsb, al2);
+    if (r.lane < S) cp_async4(st + kOffY + r.lane * 4, io.Y + (size_t)e * S + r.lane);
+  };
+  // the lane's words of a staged row
+  auto words = [&](const unsigned char* p, auto& w) {
+    constexpr int NBY = (int)sizeof(w);
+    if (r.act) ld_words<NBY>(p + r.lane * NBY, w);
+    else {
+#pragma unroll
+      for (int q = 0; q < NBY / 4; ++q) w[q] = 0u;
+    }
+  };
+  auto get_y = [&](const unsigned char* st, float (&y)[S]) {
+    YStage<S> ys{reinterpret_cast<float*>(const_cast<unsigned char*>(st + kOffY))};
+    ys.get(0, y);
+  };
   float2 Q1p[CPL / 2][S], Q2p[CPL / 2][S];
 #pragma unroll
   for (int p = 0; p < CPL / 2; ++p)
 #pragma unroll
     for (int b = 0; b < S; ++b) { Q1p[p][b] = bc(0.0f); Q2p[p][b] = bc(0.0f); }
-  int staged = -1;
-  for (int sb = r.rb; sb < r.re; sb += kYSeg) {
-    const int cnt = min(kYSeg, r.re - sb);
-    ys.load(io.Y, sb, cnt, r.lane);
-    staged = sb;
-    uint32_t raw[kBatchLight][WS::NW];
-    uint32_t s1r[kBatchLight][SbarW<T, CPL>::NW], s2r[kBatchLight][SbarW<T, CPL>::NW];
-    edge_batches<kBatchLight>(
-        cnt,
-        [&](int u, int k) {
-          ld_w_raw<T, CPL, LM>(W01, io.ld01, 0, sb + k, r, raw[u]);
-          ld_sbar<T, CPL>(io.sbar1, io.ld_sbar1, sb + k, r, s1r[u]);
-          ld_sbar<T, CPL>(io.sbar2, io.ld_sbar2, sb + k, r, s2r[u]);
-        },
-        [&](int u, int k) {
-          float y[S], w0[WS::N];
-          ys.get(k, y);
-          unpack_span<T, WS::N>(raw[u], w0);
+  pieces(nw * (int)sizeof(T));
+  ring_over<D, kStage>(ring, r.rb, r.re, copy, [&](int, const unsigned char* st) {
+    uint32_t raw[WS::NW], s1r[SW::NW], s2r[SW::NW];
+    words(st, raw);
+    words(st + kOff1, s1r);
+    words(st + kOff2, s2r);
+    float y[S], w0[WS::N];
+    get_y(st, y);
+    unpack_span<T, WS::N>(raw, w0);
 #pragma unroll
-          for (int p = 0; p < CPL / 2; ++p) {
-            const float2 s1 = sbar_pair<T, CPL>(s1r[u], p);
-            const float2 s2 = sbar_pair<T, CPL>(s2r[u], p);
+    for (int p = 0; p < CPL / 2; ++p) {
+      const float2 s1 = sbar_pair<T, CPL>(s1r, p);
+      const float2 s2 = sbar_pair<T, CPL>(s2r, p);
 #pragma unroll
-            for (int b = 0; b < S; ++b) {
-              const int l = lof<LMAX>(b);
-              const float2 v0 = mul2(pk(w0[2 * p * LM + l], w0[(2 * p + 1) * LM + l]), bc(y[b]));
-              Q1p[p][b] = fma2(s1, v0, Q1p[p][b]);
-              Q2p[p][b] = fma2(s2, v0, Q2p[p][b]);
-            }
-          }
-        });
-  }
+      for (int b = 0; b < S; ++b) {
+        const int l = lof<LMAX>(b);
+        const float2 v0 = mul2(pk(w0[2 * p * LM + l], w0[(2 * p + 1) * LM + l]), bc(y[b]));
+        Q1p[p][b] = fma2(s1, v0, Q1p[p][b]);
+        Q2p[p][b] = fma2(s2, v0, Q2p[p][b]);
+      }
+    }
+  });
+  // the second pass reads w^0 and sbar again (from L2) and w^1, which follows w^0 in its rows
+  __syncwarp();
+  pieces(2 * nw * (int)sizeof(T));
+  ring_begin<D, kStage>(ring, r.rb, r.re, copy);
   float Q1[CPL][S], Q2[CPL][S];
 #pragma unroll
   for (int p = 0; p < CPL / 2; ++p)
@@ -814,60 +877,48 @@ __global__ void __launch_bounds__(32 * kRowWarps, 4) row_bwd_mid_kernel(RowIO io
       T2p[p][b] = pk(T2[2 * p][b], T2[2 * p + 1][b]);
       G1bp[p][b] = pk(G1b[2 * p][b], G1b[2 * p + 1][b]);
     }
-  const int nseg = (r.re - r.rb + kYSeg - 1) / kYSeg;
-  for (int q = nseg - 1; q >= 0; --q) {
-    const int sb = r.rb + q * kYSeg, cnt = min(kYSeg, r.re - sb);
-    if (sb != staged) ys.load(io.Y, sb, cnt, r.lane);
-    staged = sb;
-    uint32_t raw0[kBatchHeavy][WS::NW], raw1[kBatchHeavy][WS::NW];
-    uint32_t s1r[kBatchHeavy][SbarW<T, CPL>::NW], s2r[kBatchHeavy][SbarW<T, CPL>::NW];
-    edge_batches<kBatchHeavy>(
-        cnt,
-        [&](int u, int k) {
-          ld_w_raw<T, CPL, LM>(W01, io.ld01, 0, sb + k, r, raw0[u]);
-          ld_w_raw<T, CPL, LM>(W01, io.ld01, nw, sb + k, r, raw1[u]);
-          ld_sbar<T, CPL>(io.sbar1, io.ld_sbar1, sb + k, r, s1r[u]);
-          ld_sbar<T, CPL>(io.sbar2, io.ld_sbar2, sb + k, r, s2r[u]);
-        },
-        [&](int u, int k) {
-          const int e = sb + k;
-          float y[S], w0[WS::N], w1[WS::N], g0[WS::N], g1[WS::N], yc[S];
-          float2 yc2[S];
-          ys.get(k, y);
-          unpack_span<T, WS::N>(raw0[u], w0);
-          unpack_span<T, WS::N>(raw1[u], w1);
+  ring_loop<D, kStage>(ring, r.rb, r.re, copy, [&](int e, const unsigned char* st) {
+    uint32_t raw0[WS::NW], raw1[WS::NW], s1r[SW::NW], s2r[SW::NW];
+    words(st, raw0);
+    words(st + nw * (int)sizeof(T), raw1);
+    words(st + kOff1, s1r);
+    words(st + kOff2, s2r);
+    float y[S], w0[WS::N], w1[WS::N], g0[WS::N], g1[WS::N], yc[S];
+    float2 yc2[S];
+    get_y(st, y);
+    unpack_span<T, WS::N>(raw0, w0);
+    unpack_span<T, WS::N>(raw1, w1);
 #pragma unroll
-          for (int b = 0; b < S; ++b) yc2[b] = bc(0.0f);
+    for (int b = 0; b < S; ++b) yc2[b] = bc(0.0f);
 #pragma unroll
-          for (int p = 0; p < CPL / 2; ++p) {
-            const float2 s1 = sbar_pair<T, CPL>(s1r[u], p);
-            const float2 s2 = sbar_pair<T, CPL>(s2r[u], p);
-            float2 a0[LM], a1[LM];
+    for (int p = 0; p < CPL / 2; ++p) {
+      const float2 s1 = sbar_pair<T, CPL>(s1r, p);
+      const float2 s2 = sbar_pair<T, CPL>(s2r, p);
+      float2 a0[LM], a1[LM];
 #pragma unroll
-            for (int l = 0; l < LM; ++l) { a0[l] = bc(0.0f); a1[l] = bc(0.0f); }
+      for (int l = 0; l < LM; ++l) { a0[l] = bc(0.0f); a1[l] = bc(0.0f); }
 #pragma unroll
-            for (int b = 0; b < S; ++b) {
-              const int l = lof<LMAX>(b);
-              const float2 yy = bc(y[b]);
-              const float2 v0b = fma2(s2, T2p[p][b], mul2(s1, T1p[p][b]));
-              a0[l] = fma2(v0b, yy, a0[l]);
-              a1[l] = fma2(G1bp[p][b], yy, a1[l]);
-              yc2[b] = fma2(pk(w0[2 * p * LM + l], w0[(2 * p + 1) * LM + l]), v0b, yc2[b]);
-              yc2[b] = fma2(pk(w1[2 * p * LM + l], w1[(2 * p + 1) * LM + l]), G1bp[p][b], yc2[b]);
-            }
+      for (int b = 0; b < S; ++b) {
+        const int l = lof<LMAX>(b);
+        const float2 yy = bc(y[b]);
+        const float2 v0b = fma2(s2, T2p[p][b], mul2(s1, T1p[p][b]));
+        a0[l] = fma2(v0b, yy, a0[l]);
+        a1[l] = fma2(G1bp[p][b], yy, a1[l]);
+        yc2[b] = fma2(pk(w0[2 * p * LM + l], w0[(2 * p + 1) * LM + l]), v0b, yc2[b]);
+        yc2[b] = fma2(pk(w1[2 * p * LM + l], w1[(2 * p + 1) * LM + l]), G1bp[p][b], yc2[b]);
+      }
 #pragma unroll
-            for (int l = 0; l < LM; ++l) {
-              g0[2 * p * LM + l] = a0[l].x; g0[(2 * p + 1) * LM + l] = a0[l].y;
-              g1[2 * p * LM + l] = a1[l].x; g1[(2 * p + 1) * LM + l] = a1[l].y;
-            }
-          }
+      for (int l = 0; l < LM; ++l) {
+        g0[2 * p * LM + l] = a0[l].x; g0[(2 * p + 1) * LM + l] = a0[l].y;
+        g1[2 * p * LM + l] = a1[l].x; g1[(2 * p + 1) * LM + l] = a1[l].y;
+      }
+    }
 #pragma unroll
-          for (int b = 0; b < S; ++b) yc[b] = yc2[b].x + yc2[b].y;
-          st_w<T, CPL, LM>(wb, io.ld_wbar01, 0, e, r, g0);
-          st_w<T, CPL, LM>(wb, io.ld_wbar01, nw, e, r, g1);
-          warp_channel_sum<S>(yc, r.lane, io.Ybar[1] + (size_t)e * S);
-        });
-  }
+    for (int b = 0; b < S; ++b) yc[b] = yc2[b].x + yc2[b].y;
+    st_w<T, CPL, LM>(wb, io.ld_wbar01, 0, e, r, g0);
+    st_w<T, CPL, LM>(wb, io.ld_wbar01, nw, e, r, g1);
+    warp_channel_sum<S>(yc, r.lane, io.Ybar[1] + (size_t)e * S);
+  });
 }
 
 // ---------------------------------------------------------------------------
