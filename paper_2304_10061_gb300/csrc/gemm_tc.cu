@@ -115,11 +115,15 @@ template <int EPQ> __host__ __device__ constexpr int tc_threads() { return 64 + 
 // mbarriers, flags and partial row sums.  The epilogue part depends on the
 // mode (TcLayout, chosen on the host): a bf16 32x32 output box is 2 KB, a
 // float32 box or an activation + pre-activation pair 4 KB; two output buffers
-// (double-buffered TMA stores) with two warps per quarter, one with four; an
+// (double-buffered TMA stores) with two warps per quarter, one with four and in
+// CTA pairs (whose rate hangs on the ring's depth: latent layers of K = N = 1024
+// 0.324 / 0.315 / 0.312 ms with 4 / 5 / 6 stages, float32 outputs at K = 1408
+// 0.404 / 0.376 / 0.367); an
 // input slot of 2 KB per bf16 input (pre-activation, addend).  The ring takes
 // the rest, up to kTcMaxStages k-blocks.
 constexpr int kTcSmemMax = 232448;           // dynamic shared memory per block (227 KB)
 constexpr int kTcMisc = 4096;                // mbarriers, TMEM slot, flags, partial row sums
+constexpr int kTcMiscPair = 1024;            // the same for CTA pairs (no row sums)
 constexpr int kTcMaxStages = 8;
 
 struct TcLayout {
@@ -146,17 +150,17 @@ static TcLayout tc_layout(int epi, bool pre) {
   TcLayout L;
   const bool wide_out = (epi == EPI_F32) || (epi == EPI_FWD_SILU && pre);
   L.out_box = wide_out ? 4096 : 2048;
-  L.n_out = (EPQ == 2) ? 2 : 1;
+  L.n_out = (EPQ == 2 && !PAIR) ? 2 : 1;
   L.in_slot = (epi == EPI_BWD_SILU) ? 2048 : (epi == EPI_HEAD ? 4096 : 0);
   L.epi_slot = L.n_out * L.out_box + L.in_slot;
   const int epi_smem = 4 * EPQ * L.epi_slot;
-  const int st = (kTcSmemMax - 1024 - kTcMisc - epi_smem) / tc_stage_bytes<BN, PAIR>();
+  const int st = (kTcSmemMax - 1024 - (PAIR ? kTcMiscPair : kTcMisc) - epi_smem) / tc_stage_bytes<BN, PAIR>();
   L.stages = st > kTcMaxStages ? kTcMaxStages : st;
   return L;
 }
 template <int BN, int EPQ, bool PAIR>
 static size_t tc_smem_bytes(const TcLayout& L) {
-  return (size_t)L.stages * tc_stage_bytes<BN, PAIR>() + (size_t)4 * EPQ * L.epi_slot + 1024 + kTcMisc;
+  return (size_t)L.stages * tc_stage_bytes<BN, PAIR>() + (size_t)4 * EPQ * L.epi_slot + 1024 + (PAIR ? kTcMiscPair : kTcMisc);
 }
 
 __device__ __forceinline__ void load_bf16x16(const bf16* p, float (&v)[16]) {
@@ -445,18 +449,25 @@ __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
           float o2[16];
           if (ep.epi == EPI_FWD_SILU) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              o2[j] = v[j];
-              v[j] = v[j] * fast_sigmoid(v[j]) * rs;
+            for (int j = 0; j < 16; ++j) o2[j] = v[j];
+            // column pairs in packed fp32 (the scalar operations, two per instruction)
+#pragma unroll
+            for (int j = 0; j < 16; j += 2) {
+              const float2 z = make_float2(v[j], v[j + 1]);
+              const float2 x = f2_mul(f2_mul(z, fast_sigmoid2(z)), f2_bc(rs));
+              v[j] = x.x;
+              v[j + 1] = x.y;
             }
           } else if (ep.epi == EPI_F32 || ep.epi == EPI_LINEAR) {
             // the accumulator as it is (float32 or activation type)
           } else if (ep.epi == EPI_BWD_SILU) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const float z = bf16_word_elem(zw, 16 * hh + j);
-              const float sgm = fast_sigmoid(z);
-              v[j] = v[j] * sgm * (1.0f + z * (1.0f - sgm));
+            for (int j = 0; j < 16; j += 2) {
+              const float2 z = bf16_word_pair(zw[8 * hh + j / 2]);
+              const float2 sg2 = fast_sigmoid2(z);
+              const float2 x = f2_mul(f2_mul(make_float2(v[j], v[j + 1]), sg2), dsilu_factor2(z, sg2));
+              v[j] = x.x;
+              v[j + 1] = x.y;
             }
           } else if (ep.epi == EPI_HEAD) {
 #pragma unroll
@@ -1197,10 +1208,10 @@ bool gemm_tc_bf16(const GemmArgs& g, cudaStream_t st, int* d_err, std::string* w
       // CTA pairs for long sums, once there is a tile for every pair of SMs.  ms alone / paired at
       // 1.64 million rows: K = 1536, N = 512 2.16 / 1.89, K = 1024, N = 512 1.55 / 1.39; K = 640 1.07 /
       // 1.07, K = 512 0.95 / 1.03 (HBM-bound, and the two epilogues wait for each other); 184,600 rows,
-      // K = N = 1024 0.342 / 0.307
+      // K = N = 1024 0.342 / 0.293.  Two epilogue warps per quarter in every mode: four leave the ring
+      // four stages (SiLU 0.340, its adjoint 0.321 against 0.306)
       if (g.K >= 768 && g.N > 256 && (int64_t)((g.M + 255) / 256) * tiles >= num_sms(current_device()) / 2)
-        return wide ? launch_bn<256, 4, true>(g, B, ldb, st, d_err, why)
-                    : launch_bn<256, 2, true>(g, B, ldb, st, d_err, why);
+        return launch_bn<256, 2, true>(g, B, ldb, st, d_err, why);
       return wide ? launch_bn<256, 4>(g, B, ldb, st, d_err, why) : launch_bn<256, 2>(g, B, ldb, st, d_err, why);
   }
 }
