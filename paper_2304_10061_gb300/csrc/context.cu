@@ -29,6 +29,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "launch.cuh"
 
 using namespace alg;
 
@@ -45,6 +46,7 @@ inline size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 __global__ void stage_atoms_kernel(const int* __restrict__ types, const double* pos_in, int n,
                                    const int* __restrict__ map, int nmap, double* pos, int* __restrict__ species,
                                    int* __restrict__ err) {
+  pdl_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   int t = types[i];
@@ -65,6 +67,7 @@ __global__ void copy_results_kernel(const double* __restrict__ E, const double* 
                                     const double* __restrict__ F, const double* __restrict__ W, long long nb, long long n,
                                     double* __restrict__ oE, double* __restrict__ oEa, double* __restrict__ oF,
                                     double* __restrict__ oW) {
+  pdl_wait();
   const long long stride = (long long)gridDim.x * blockDim.x, t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   for (long long k = t0; k < nb; k += stride) oE[k] = E[k];
   if (oEa)
@@ -76,6 +79,7 @@ __global__ void copy_results_kernel(const double* __restrict__ E, const double* 
 }
 
 __global__ void atom_struct_kernel(const int64_t* __restrict__ offs, int nstruct, int* __restrict__ atom_struct) {
+  pdl_wait();
   int b = blockIdx.x;
   if (b >= nstruct) return;
   for (long long i = offs[b] + threadIdx.x; i < offs[b + 1]; i += blockDim.x) atom_struct[i] = b;
@@ -823,7 +827,7 @@ allegro_status stage_atoms(allegro_ctx* c, int64_t n, const double* pos, const i
       ts = c->d_types;
     }
     CUDA_TRY(c, cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream));
-    stage_atoms_kernel<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(ts, ps, (int)n, c->d_map, c->nmap, c->d_pos,
+    launch(stage_atoms_kernel, (unsigned)((n + 255) / 256), 256, 0, c->stream, ts, ps, (int)n, c->d_map, c->nmap, c->d_pos,
                                                                            c->d_species, c->d_err);
     CUDA_TRY(c, cudaGetLastError());
   } else {
@@ -2253,7 +2257,7 @@ allegro_status allegro_neighbors_batched(allegro_ctx* c, int32_t n_struct, const
     CUDA_TRY(c, cudaMemcpyAsync(c->d_pbc, hp.data(), hp.size() * 4, cudaMemcpyHostToDevice, st));
     CUDA_TRY(c, cudaMemcpyAsync(c->d_nimg, hn.data(), hn.size() * 4, cudaMemcpyHostToDevice, st));
   }
-  atom_struct_kernel<<<n_struct, 128, 0, st>>>(c->d_offs, n_struct, c->d_atom_struct);
+  launch(atom_struct_kernel, n_struct, 128, 0, st, c->d_offs, n_struct, c->d_atom_struct);
   const double rc2 = rc * rc;
   const double* d_cells = cells ? c->d_cells : nullptr;
   {
@@ -2288,7 +2292,7 @@ allegro_status allegro_energy_forces(allegro_ctx* c, double* E_total, double* E_
   auto direct = [&](const void* p) { return !p || is_own_device_ptr(p, c->device); };
   if (direct(E_total) && direct(E_atom) && direct(F) && direct(virial)) {
     const unsigned blocks = (unsigned)std::min<size_t>((3 * n + 9 * B + 255) / 256, 152 * 8);
-    copy_results_kernel<<<blocks, 256, 0, c->stream>>>(c->d_Eout, c->d_Eatom, c->d_F, c->d_Wout, (long long)B,
+    launch(copy_results_kernel, blocks, 256, 0, c->stream, c->d_Eout, c->d_Eatom, c->d_F, c->d_Wout, (long long)B,
                                                        (long long)n, E_total, E_atom, F, virial);
     CUDA_TRY(c, cudaGetLastError());
   } else {

@@ -22,6 +22,7 @@
 
 #include "amax.cuh"
 #include "internal.h"
+#include "launch.cuh"
 
 namespace alg {
 
@@ -158,6 +159,7 @@ __global__ void __launch_bounds__(kGeomBlock)
                     float* __restrict__ Yout, float* __restrict__ uout, const double* __restrict__ sigma,
                     float* __restrict__ sig, const float* __restrict__ W0t, int ldW, int N0, T* __restrict__ Zout,
                     int ldZ, T* __restrict__ Hout, int ldH, int scale_u, int vec, unsigned* __restrict__ amax) {
+  pdl_wait();
   __shared__ float sY[kGeomBlock * kMaxS];
   __shared__ float4 sB[kGeomBlock][NB / 4];
   __shared__ int4 sI[kGeomBlock];   // species of i and j, scale of the activation (float bits)
@@ -293,16 +295,16 @@ void edge_geom_fwd(int Ec, int e0, const double* ed, const int* ei, const int* e
   // whole groups of four columns at 16-byte (8-byte in bf16) boundaries
   auto al = [](const void* p) { return reinterpret_cast<uintptr_t>(p) % (4 * sizeof(T)) == 0; };
   const int vec = N0 % 4 == 0 && ldZ % 4 == 0 && ldH % 4 == 0 && al(Z0) && al(H0);
-  auto launch = [&](auto kern) {
-    kern<<<grid, kGeomBlock, 0, st>>>(Ec, e0, ed, ei, ej, species, make_basis(a), Y, u, sigma, sig, W0t, ldW, N0, Z0,
+  auto go = [&](auto kern) {
+    launch(kern, grid, kGeomBlock, 0, st, Ec, e0, ed, ei, ej, species, make_basis(a), Y, u, sigma, sig, W0t, ldW, N0, Z0,
                                       ldZ, H0, ldH, scale_u ? 1 : 0, vec, amax);
   };
   if (a.nb <= 8) {
-    if (amax) launch(geom_fwd_kernel<T, 8, true>);
-    else launch(geom_fwd_kernel<T, 8, false>);
+    if (amax) go(geom_fwd_kernel<T, 8, true>);
+    else go(geom_fwd_kernel<T, 8, false>);
   } else {
-    if (amax) launch(geom_fwd_kernel<T, kMaxBessel, true>);
-    else launch(geom_fwd_kernel<T, kMaxBessel, false>);
+    if (amax) go(geom_fwd_kernel<T, kMaxBessel, true>);
+    else go(geom_fwd_kernel<T, kMaxBessel, false>);
   }
 }
 template void edge_geom_fwd<float>(int, int, const double*, const int*, const int*, const int*, const Arch&,
@@ -324,6 +326,7 @@ __global__ void __launch_bounds__(kGeomBlock, kGeomBwdBlocksPerSM)
                     const T* __restrict__ zbar0,
                     int ldz, const float* __restrict__ W0t, int ldW, int N0, const float* __restrict__ ubar,
                     YbarParts yb, float* __restrict__ g) {
+  pdl_wait();
   extern __shared__ __align__(16) float wb_sm[];   // [nb][N0]: Bessel rows of W0t
   for (int q = threadIdx.x; q < bc.nb * N0; q += blockDim.x) {
     const int n = q / N0, k = q - n * N0;
@@ -433,8 +436,7 @@ void edge_geom_bwd(int Ec, int e0, const double* ed, const int* ei, const int* e
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const int tiles = (Ec + kGeomBlock - 1) / kGeomBlock;
   const int grid = std::min(tiles, std::max(nsm, 1) * kGeomBwdBlocksPerSM);
-  geom_bwd_kernel<T><<<grid, kGeomBlock, smem, st>>>(
-      Ec, e0, ed, ei, ej, species, make_basis(a), zbar0, ldz, W0t, ldW, a.tb[0], ubar, yb, g);
+  launch(geom_bwd_kernel<T>, grid, kGeomBlock, smem, st, Ec, e0, ed, ei, ej, species, make_basis(a), zbar0, ldz, W0t, ldW, a.tb[0], ubar, yb, g);
 }
 template void edge_geom_bwd<float>(int, int, const double*, const int*, const int*, const int*, const Arch&,
                                    const float*, int, const float*, int, const float*, const YbarParts&, float*,
@@ -478,6 +480,7 @@ __global__ void head_bwd_kernel(int Ec, int K, const float* __restrict__ xbar, i
                                 const float* __restrict__ u, float* __restrict__ ubar, bool ubar_init,
                                 T* __restrict__ zbar, int ld_z, unsigned* __restrict__ amax,
                                 const T* __restrict__ addx, int ld_addx, int vec) {
+  pdl_wait();
   int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   int lane = threadIdx.x & 31;
   if (warp >= Ec) return;
@@ -535,8 +538,7 @@ void mlp_head_bwd(int Ec, int K, const float* xbar, int ld_x, const float* vcons
   constexpr int b4 = 4 * (int)sizeof(T);   // bytes of four activation-type values
   const int vec = al(xbar, 16) && al(vconst, 16) && al(pre, b4) && al(zbar, b4) && al(addx, b4) &&
                   (ld_x % 4 == 0) && (ld_pre % 4 == 0) && (ld_z % 4 == 0) && (!addx || ld_addx % 4 == 0);
-  head_bwd_kernel<T><<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(
-      Ec, K, xbar, ld_x, vconst, ei, species, sigma, e0, pre, ld_pre, u, ubar, ubar_init, zbar, ld_z, amax, addx,
+  launch(head_bwd_kernel<T>, (unsigned)((threads + 255) / 256), 256, 0, st, Ec, K, xbar, ld_x, vconst, ei, species, sigma, e0, pre, ld_pre, u, ubar, ubar_init, zbar, ld_z, amax, addx,
       ld_addx, vec);
 }
 template void mlp_head_bwd<float>(int, int, const float*, int, const float*, const int*, const int*,
@@ -550,6 +552,7 @@ template void mlp_head_bwd<bf16>(int, int, const float*, int, const float*, cons
 template <typename T>
 __global__ void edge_energy_kernel(int Ec, int K, const T* __restrict__ x, int ldx, const float* __restrict__ v,
                                    float* __restrict__ Ee) {
+  pdl_wait();
   int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   int lane = threadIdx.x & 31;
   if (warp >= Ec) return;
@@ -563,7 +566,7 @@ template <typename T>
 void edge_energy(int Ec, int K, const T* x, int ldx, const float* v, float* Ee, cudaStream_t st) {
   if (Ec <= 0) return;
   long long threads = (long long)Ec * 32;
-  edge_energy_kernel<T><<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(Ec, K, x, ldx, v, Ee);
+  launch(edge_energy_kernel<T>, (unsigned)((threads + 255) / 256), 256, 0, st, Ec, K, x, ldx, v, Ee);
 }
 template void edge_energy<float>(int, int, const float*, int, const float*, float*, cudaStream_t);
 template void edge_energy<bf16>(int, int, const bf16*, int, const float*, float*, cudaStream_t);
@@ -614,6 +617,7 @@ __global__ void atom_reduce_kernel(int n, int n_centres, const int* __restrict__
                                    const double* __restrict__ mu, bool want_forces, double* __restrict__ E_atom,
                                    double* __restrict__ F, double* __restrict__ Wat, const int* __restrict__ ei,
                                    const int* __restrict__ ej, const float2* __restrict__ zbl, BasisConst bc) {
+  pdl_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int b = row_ptr[i], e1 = row_ptr[i + 1];
@@ -678,6 +682,7 @@ __global__ void __launch_bounds__(16 * kReduceAtoms) atom_reduce_group_kernel(
     const double* __restrict__ mu, bool want_forces, double* __restrict__ E_atom, double* __restrict__ F,
     double* __restrict__ Wat, const int* __restrict__ ei, const int* __restrict__ ej, const float2* __restrict__ zbl,
     BasisConst bc) {
+  pdl_wait();
   // per edge: -d (3), 1, g (3), E, E_ZBL
   __shared__ double sh[kReduceAtoms][16][9];
   const int q = threadIdx.x & 15, w = threadIdx.x >> 4;
@@ -759,11 +764,10 @@ void atom_reduce(int n, int n_centres, const int* row_ptr, const int* col_ptr, c
   if (n <= 0) return;
   const float2* zbl = reinterpret_cast<const float2*>(a.zbl);
   if (n <= (zbl ? kReduceGroupAtomsZbl : (want_forces ? kReduceGroupAtoms : kReduceGroupAtomsEnergy)))
-    atom_reduce_group_kernel<<<(n + kReduceAtoms - 1) / kReduceAtoms, 16 * kReduceAtoms, 0, st>>>(
-        n, n_centres, row_ptr, col_ptr, col_edge, Ee, g, ed, species, sigma, mu, want_forces, E_atom, F, Wat, ei, ej,
+    launch(atom_reduce_group_kernel, (n + kReduceAtoms - 1) / kReduceAtoms, 16 * kReduceAtoms, 0, st, n, n_centres, row_ptr, col_ptr, col_edge, Ee, g, ed, species, sigma, mu, want_forces, E_atom, F, Wat, ei, ej,
         zbl, make_basis(a));
   else
-    atom_reduce_kernel<<<(n + 127) / 128, 128, 0, st>>>(n, n_centres, row_ptr, col_ptr, col_edge, Ee, g, ed, species,
+    launch(atom_reduce_kernel, (n + 127) / 128, 128, 0, st, n, n_centres, row_ptr, col_ptr, col_edge, Ee, g, ed, species,
                                                         sigma, mu, want_forces, E_atom, F, Wat, ei, ej, zbl,
                                                         make_basis(a));
 }
@@ -789,6 +793,7 @@ __global__ void __launch_bounds__(kStructThreads) struct_reduce_kernel(
     const int64_t* __restrict__ offs, const double* __restrict__ E_atom, const double* __restrict__ Wat,
     const double* __restrict__ F, bool want_w, int parts, double* __restrict__ part, unsigned* __restrict__ ticket,
     double* __restrict__ E_out, double* __restrict__ W_out, int* __restrict__ d_err) {
+  pdl_wait();
   const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
   long long a0, a1;
   if (parts > 1) {
@@ -842,8 +847,7 @@ void struct_reduce(int nstruct, const int64_t* offs, const double* E_atom, const
   if (nstruct <= 0) return;
   static_assert(kStructScratch > 10 * kStructParts, "partials and the ticket");
   const int parts = nstruct == 1 ? (int)std::min<int64_t>(kStructParts, (n_atoms + kStructAtoms - 1) / kStructAtoms) : 1;
-  struct_reduce_kernel<<<parts > 1 ? parts : nstruct, kStructThreads, 0, st>>>(
-      offs, E_atom, Wat, F, want_w, std::max(parts, 1), scratch, reinterpret_cast<unsigned*>(scratch + 10 * kStructParts),
+  launch(struct_reduce_kernel, parts > 1 ? parts : nstruct, kStructThreads, 0, st, offs, E_atom, Wat, F, want_w, std::max(parts, 1), scratch, reinterpret_cast<unsigned*>(scratch + 10 * kStructParts),
       E_out, W_out, d_err);
 }
 
@@ -860,6 +864,7 @@ constexpr double kACC = 9.648533212e-3;
 
 __global__ void inv_mass_kernel(int n, const int* __restrict__ types, const double* __restrict__ masses, int nm,
                                 double* __restrict__ inv_m, int* __restrict__ err) {
+  pdl_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int t = types[i];
@@ -872,6 +877,7 @@ __global__ void inv_mass_kernel(int n, const int* __restrict__ types, const doub
 __global__ void kick_drift_kernel(int n, double* __restrict__ pos, double* __restrict__ vel,
                                   const double* __restrict__ F, const double* __restrict__ inv_m, double dt,
                                   bool drift) {
+  pdl_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double h = 0.5 * dt * kACC * inv_m[i];
@@ -886,6 +892,7 @@ __global__ void kick_drift_kernel(int n, double* __restrict__ pos, double* __res
 // Kinetic energy 0.5 sum m v^2 / kACC in float64, two fixed-order levels.
 __global__ void kinetic_partial_kernel(int n, const double* __restrict__ vel, const double* __restrict__ inv_m,
                                        double* __restrict__ part) {
+  pdl_wait();
   __shared__ double sh[256];
   double acc = 0.0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -902,6 +909,7 @@ __global__ void kinetic_partial_kernel(int n, const double* __restrict__ vel, co
 }
 
 __global__ void kinetic_final_kernel(const double* __restrict__ part, int nparts, double* __restrict__ out) {
+  pdl_wait();
   __shared__ double sh[256];
   double acc = 0.0;
   for (int p = threadIdx.x; p < nparts; p += blockDim.x) acc += part[p];
@@ -915,18 +923,18 @@ __global__ void kinetic_final_kernel(const double* __restrict__ part, int nparts
 }
 
 void md_inv_mass(int n, const int* types, const double* masses, int nm, double* inv_m, int* err, cudaStream_t st) {
-  if (n > 0) inv_mass_kernel<<<(n + 255) / 256, 256, 0, st>>>(n, types, masses, nm, inv_m, err);
+  if (n > 0) launch(inv_mass_kernel, (n + 255) / 256, 256, 0, st, n, types, masses, nm, inv_m, err);
 }
 
 void md_kick(int n, double* pos, double* vel, const double* F, const double* inv_m, double dt, bool drift,
              cudaStream_t st) {
-  if (n > 0) kick_drift_kernel<<<(n + 255) / 256, 256, 0, st>>>(n, pos, vel, F, inv_m, dt, drift);
+  if (n > 0) launch(kick_drift_kernel, (n + 255) / 256, 256, 0, st, n, pos, vel, F, inv_m, dt, drift);
 }
 
 void md_kinetic(int n, const double* vel, const double* inv_m, double* part, double* out, cudaStream_t st) {
   const int parts = 256;
-  kinetic_partial_kernel<<<parts, 256, 0, st>>>(n, vel, inv_m, part);
-  kinetic_final_kernel<<<1, 256, 0, st>>>(part, parts, out);
+  launch(kinetic_partial_kernel, parts, 256, 0, st, n, vel, inv_m, part);
+  launch(kinetic_final_kernel, 1, 256, 0, st, part, parts, out);
 }
 
 }  // namespace alg

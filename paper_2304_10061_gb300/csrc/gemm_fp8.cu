@@ -43,6 +43,7 @@
 #include "epi_stage.cuh"
 #include "epilogue.cuh"
 #include "internal.h"
+#include "launch.cuh"
 #include "tc_ptx.cuh"
 
 namespace alg {
@@ -272,6 +273,7 @@ __global__ void __launch_bounds__(kF8Threads, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  pdl_wait();   // before TMEM is allocated: the kernel before holds its own until it ends
   if (warp == 1) {
     tc_alloc(tslot, 2 * COLS);
     tc_relinquish();
@@ -577,7 +579,7 @@ static bool launch_fp8(const GemmArgs& g, const uint8_t* B8, int ldb8, float sB,
   }
   const int tiles = ((g.M + 127) / 128) * ((g.N + BN - 1) / BN);
   const int grid = tiles < nsm[dev] ? tiles : nsm[dev];
-  gemm_fp8_kernel<BN><<<grid, kF8Threads, smem, st>>>(ta, ta2, tb, em, ep, fp);
+  launch(gemm_fp8_kernel<BN>, grid, kF8Threads, smem, st, ta, ta2, tb, em, ep, fp);
   return true;
 }
 

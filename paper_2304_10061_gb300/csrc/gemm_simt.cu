@@ -25,6 +25,7 @@
 
 #include "epilogue.cuh"
 #include "internal.h"
+#include "launch.cuh"
 
 namespace alg {
 
@@ -75,6 +76,7 @@ template <int BM, int SB_K>
 __global__ void __launch_bounds__(BM) gemm_simt_kernel(
     const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb, int M, int N, int K, EpiParams ep,
     int vecA, int vecB) {
+  pdl_wait();
   constexpr int BN = 64, TM = 8, TN = 8, kThreads = BM;   // BM BN / (TM TN)
   constexpr int kRows = kThreads / (SB_K / 4);    // rows of a slice loaded per pass (four k per thread)
   constexpr int ALOADS = BM / kRows, BLOADS = BN / kRows;
@@ -174,7 +176,7 @@ template <int BM, int SB_K>
 static void launch_simt(const GemmArgs& g, const float* A, const float* B, int ldb, const EpiParams& ep, int vecA,
                         int vecB, cudaStream_t st) {
   const unsigned tiles = (unsigned)((g.M + BM - 1) / BM) * (unsigned)((g.N + 63) / 64);
-  gemm_simt_kernel<BM, SB_K><<<tiles, BM, 0, st>>>(A, g.lda, B, ldb, g.M, g.N, g.K, ep, vecA, vecB);
+  launch(gemm_simt_kernel<BM, SB_K>, tiles, BM, 0, st, A, g.lda, B, ldb, g.M, g.N, g.K, ep, vecA, vecB);
 }
 
 void gemm_simt_f32(const GemmArgs& g, cudaStream_t st) {

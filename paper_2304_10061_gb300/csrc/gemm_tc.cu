@@ -32,6 +32,7 @@
 #include "epi_stage.cuh"
 #include "epilogue.cuh"
 #include "internal.h"
+#include "launch.cuh"
 #include "tc_ptx.cuh"
 
 namespace alg {
@@ -288,6 +289,7 @@ __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  pdl_wait();   // before TMEM is allocated: the kernel before holds its own until it ends
   if (warp == 1) {
     if constexpr (PAIR) {
       tc_alloc_pair(tslot, 2 * COLS);
@@ -692,6 +694,7 @@ __global__ void __launch_bounds__(kCfThreads, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  pdl_wait();   // before TMEM is allocated: the kernel before holds its own until it ends
   if (warp == 1) {
     tc_alloc(tslot, 512);
     tc_relinquish();
@@ -1143,27 +1146,17 @@ static bool launch_bn(const GemmArgs& g, const bf16* B, int ldb, cudaStream_t st
   const size_t smem = tc_smem_bytes<BN, EPQ, PAIR>(lay);
   if constexpr (PAIR) {
     const int tiles = ((g.M + 2 * kTcBM - 1) / (2 * kTcBM)) * ((g.N + BN - 1) / BN);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * std::min(tiles, nsm / 2));
-    cfg.blockDim = dim3(tc_threads<EPQ>());
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at = {};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = 2;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_tc_kernel<BN, EPQ, true>, ta, ta2, tb, em, make_epi(g), lay, g.M,
-                                             g.N, g.K, K1, d_err);
+    const cudaError_t e = launch_cluster(2, gemm_tc_kernel<BN, EPQ, true>, 2 * std::min(tiles, nsm / 2),
+                                         tc_threads<EPQ>(), smem, st, ta, ta2, tb, em, make_epi(g), lay, g.M, g.N, g.K,
+                                         K1, d_err);
     if (e != cudaSuccess) {
-      if (why) *why = std::string("cudaLaunchKernelEx: ") + cudaGetErrorString(e);
+      if (why) *why = std::string("launch: ") + cudaGetErrorString(e);
       return false;
     }
   } else {
     const int tiles = ((g.M + kTcBM - 1) / kTcBM) * ((g.N + BN - 1) / BN);
     const int grid = tiles < nsm ? tiles : nsm;
-    gemm_tc_kernel<BN, EPQ, false><<<grid, tc_threads<EPQ>(), smem, st>>>(ta, ta2, tb, em, make_epi(g), lay, g.M, g.N,
+    launch(gemm_tc_kernel<BN, EPQ, false>, grid, tc_threads<EPQ>(), smem, st, ta, ta2, tb, em, make_epi(g), lay, g.M, g.N,
                                                                           g.K, K1, d_err);
   }
   return true;
@@ -1245,7 +1238,7 @@ static bool launch_chain_pipe(const GemmArgs& g1, const GemmArgs& g2, const bf16
   }
   const int tiles = (g1.M + kTcBM - 1) / kTcBM;
   const int grid = tiles < nsm ? tiles : nsm;
-  gemm_chain_pipe_kernel<N1, N2, E1, E2><<<grid, kCfThreads, smem, st>>>(cm, make_epi(g1), make_epi(g2), g1.M,
+  launch(gemm_chain_pipe_kernel<N1, N2, E1, E2>, grid, kCfThreads, smem, st, cm, make_epi(g1), make_epi(g2), g1.M,
                                                                           g1.K, K1a, d_err);
   return true;
 }
@@ -1450,6 +1443,7 @@ __global__ void __launch_bounds__(kT32Threads, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  pdl_wait();   // before TMEM is allocated: the kernel before holds its own until it ends
   if (warp == 1) {
     tc_alloc(tslot, 2 * COLS);
     tc_relinquish();
@@ -1652,7 +1646,7 @@ static bool launch_tf32(const GemmArgs& g, const float* B, int ldb, cudaStream_t
   }
   const int stages = t32_stages<BN>(epi_slot);
   const int smem = stages * t32_stage_bytes<BN>() + kT32EpiWarps * epi_slot + 1024 + 1024;
-  gemm_tf32_kernel<BN><<<grid, kT32Threads, smem, st>>>(ta, tb, em, ep, stages, epi_slot, g.M, g.N, g.K, d_err);
+  launch(gemm_tf32_kernel<BN>, grid, kT32Threads, smem, st, ta, tb, em, ep, stages, epi_slot, g.M, g.N, g.K, d_err);
   return true;
 }
 

@@ -18,6 +18,7 @@
 #include <algorithm>
 
 #include "internal.h"
+#include "launch.cuh"
 
 namespace alg {
 
@@ -96,16 +97,19 @@ __device__ __forceinline__ int block_scan_tile(int* __restrict__ in, int* __rest
 
 template <int PER>
 __global__ void __launch_bounds__(1024) scan_one_kernel(int* in, int* out, int n, bool clear, int* total) {
+  pdl_wait();
   const int t = block_scan_tile<1024, PER>(in, out, n, 0, clear);
   if (total && threadIdx.x == 0) *total = t;
 }
 
 __global__ void scan_block_kernel(int* in, int* out, int n, int* __restrict__ block_sums, bool clear) {
+  pdl_wait();
   const int total = block_scan_tile<256, 4>(in, out, n, blockIdx.x * kScanBlock, clear);
   if (threadIdx.x == 255) block_sums[blockIdx.x] = total;
 }
 
 __global__ void scan_add_kernel(int* __restrict__ out, int n, const int* __restrict__ block_pref, int* total) {
+  pdl_wait();
   const int base = blockIdx.x * kScanBlock;
   const int add = block_pref[blockIdx.x];
   for (int k = threadIdx.x; k < kScanBlock; k += blockDim.x) {
@@ -137,20 +141,20 @@ size_t scan_tmp_bytes(int n) {
 // the launches are the time at these sizes); above, block sums, their scan, and an add.
 static void scan_rec(int* in, int* out, int n, char* tmp, bool clear, int* total, cudaStream_t st) {
   if (n < 4 * 1024) {
-    scan_one_kernel<4><<<1, 1024, 0, st>>>(in, out, n, clear, total);
+    launch(scan_one_kernel<4>, 1, 1024, 0, st, in, out, n, clear, total);
     return;
   }
   if (n < 32 * 1024) {
-    scan_one_kernel<32><<<1, 1024, 0, st>>>(in, out, n, clear, total);
+    launch(scan_one_kernel<32>, 1, 1024, 0, st, in, out, n, clear, total);
     return;
   }
   const int nb = (n + 1 + kScanBlock - 1) / kScanBlock;
   int* sums = reinterpret_cast<int*>(tmp);
   int* pref = sums + scan_pitch(nb);
   char* next = reinterpret_cast<char*>(pref + scan_pitch(nb)) + 256;
-  scan_block_kernel<<<nb, 256, 0, st>>>(in, out, n, sums, clear);
+  launch(scan_block_kernel, nb, 256, 0, st, in, out, n, sums, clear);
   scan_rec(sums, pref, nb, next, false, nullptr, st);
-  scan_add_kernel<<<nb, 256, 0, st>>>(out, n, pref, total);
+  launch(scan_add_kernel, nb, 256, 0, st, out, n, pref, total);
 }
 
 int exclusive_scan_i32(int* in, int* out, int n, void* tmp, bool clear, int* total, cudaStream_t st) {
@@ -176,6 +180,7 @@ __device__ __forceinline__ unsigned long long dkey(double x) {
 
 __global__ void minmax_frac_kernel(const double* __restrict__ pos, int n, CellGrid g,
                                    unsigned long long* __restrict__ mm) {
+  pdl_wait();
   double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     double f[3];
@@ -200,12 +205,14 @@ __global__ void minmax_frac_kernel(const double* __restrict__ pos, int n, CellGr
 }
 
 __global__ void minmax_init_kernel(unsigned long long* mm) {
+  pdl_wait();
   int k = threadIdx.x;
   if (k < 3) mm[k] = ~0ull;
   else if (k < 6) mm[k] = 0ull;
 }
 
 __global__ void minmax_decode_kernel(const unsigned long long* mm, double* out) {
+  pdl_wait();
   int k = threadIdx.x;
   if (k < 6) {
     unsigned long long b = mm[k];
@@ -218,16 +225,17 @@ void nb_minmax_frac(const double* pos, int n, const double* inv, double* d_minma
   CellGrid g{};
   for (int k = 0; k < 9; ++k) g.inv[k] = inv[k];
   unsigned long long* mm = reinterpret_cast<unsigned long long*>(d_minmax + 6);
-  minmax_init_kernel<<<1, 32, 0, st>>>(mm);
+  launch(minmax_init_kernel, 1, 32, 0, st, mm);
   int blocks = (n + 255) / 256;
   if (blocks > 1184) blocks = 1184;
   if (blocks < 1) blocks = 1;
-  minmax_frac_kernel<<<blocks, 256, 0, st>>>(pos, n, g, mm);
-  minmax_decode_kernel<<<1, 32, 0, st>>>(mm, d_minmax);
+  launch(minmax_frac_kernel, blocks, 256, 0, st, pos, n, g, mm);
+  launch(minmax_decode_kernel, 1, 32, 0, st, mm, d_minmax);
 }
 
 __global__ void bin_kernel(const double* __restrict__ pos, int n, CellGrid g, int* __restrict__ cell_of,
                            int* __restrict__ wrap, int* __restrict__ cell_count, int* __restrict__ cell_rank) {
+  pdl_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   double f[3];
@@ -257,18 +265,19 @@ __global__ void bin_kernel(const double* __restrict__ pos, int n, CellGrid g, in
 void nb_bin(const double* pos, int n, const CellGrid& g, int* cell_of, int* wrap, int* cell_count, int* cell_rank,
             cudaStream_t st) {
   if (n <= 0) return;
-  bin_kernel<<<(n + 255) / 256, 256, 0, st>>>(pos, n, g, cell_of, wrap, cell_count, cell_rank);
+  launch(bin_kernel, (n + 255) / 256, 256, 0, st, pos, n, g, cell_of, wrap, cell_count, cell_rank);
 }
 
 __global__ void place_kernel(const int* __restrict__ seg_of, const int* __restrict__ rank, int n,
                              const int* __restrict__ start, int* __restrict__ sorted) {
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) sorted[start[seg_of[i]] + rank[i]] = i;
 }
 
 void nb_place(const int* seg_of, const int* rank, int n, const int* start, int* sorted, cudaStream_t st) {
   if (n <= 0) return;
-  place_kernel<<<(n + 255) / 256, 256, 0, st>>>(seg_of, rank, n, start, sorted);
+  launch(place_kernel, (n + 255) / 256, 256, 0, st, seg_of, rank, n, start, sorted);
 }
 
 // The fill passes and what follows them are queued before the host knows the edge count: they take
@@ -282,6 +291,7 @@ constexpr int kEdgeBlocks = 152 * 16;   // most blocks of the passes over a list
 __global__ void __launch_bounds__(256) place_edges_kernel(const int* __restrict__ ej, const int* __restrict__ rank,
                                                           const int* __restrict__ row_ptr, int n, int edge_cap,
                                                           const int* __restrict__ col_ptr, int* __restrict__ col_edge) {
+  pdl_wait();
   if (!list_fits(row_ptr, n, edge_cap)) return;
   const int E = row_ptr[n];
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < E; e += gridDim.x * blockDim.x)
@@ -292,7 +302,7 @@ void nb_place_edges(const int* ej, const int* rank, const int* row_ptr, int n, i
                     int* col_edge, cudaStream_t st) {
   if (edge_cap <= 0) return;
   const int blocks = std::min((int)(((int64_t)edge_cap + 255) / 256), kEdgeBlocks);
-  place_edges_kernel<<<blocks, 256, 0, st>>>(ej, rank, row_ptr, n, edge_cap, col_ptr, col_edge);
+  launch(place_edges_kernel, blocks, 256, 0, st, ej, rank, row_ptr, n, edge_cap, col_ptr, col_edge);
 }
 
 // Sort each segment [start[s], start[s+1]) of distinct values: G lanes per segment hold up to 4 G
@@ -354,6 +364,7 @@ __device__ __forceinline__ void sort_segment(int b, int len, int* __restrict__ v
 
 // 16 lanes per column (about 25 edges at the density of water and a cutoff of 4 Angstrom)
 __global__ void __launch_bounds__(256) sort_columns_kernel(const int* __restrict__ start, int n, int* __restrict__ v) {
+  pdl_wait();
   const int s = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 4);
   if (s >= n) return;
   const int b = start[s];
@@ -365,6 +376,7 @@ __global__ void __launch_bounds__(256) sort_columns_kernel(const int* __restrict
 __global__ void __launch_bounds__(256) col_rank_kernel(const int* __restrict__ ej, const int* __restrict__ row_ptr,
                                                        int n, int edge_cap, int* __restrict__ col_count,
                                                        int* __restrict__ col_rank) {
+  pdl_wait();
   if (!list_fits(row_ptr, n, edge_cap)) return;
   const int E = row_ptr[n];
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < E; e += gridDim.x * blockDim.x)
@@ -375,12 +387,12 @@ void nb_col_rank(const int* ej, const int* row_ptr, int n, int edge_cap, int* co
                  cudaStream_t st) {
   if (edge_cap <= 0) return;
   const int blocks = std::min((int)(((int64_t)edge_cap + 255) / 256), kEdgeBlocks);
-  col_rank_kernel<<<blocks, 256, 0, st>>>(ej, row_ptr, n, edge_cap, col_count, col_rank);
+  launch(col_rank_kernel, blocks, 256, 0, st, ej, row_ptr, n, edge_cap, col_count, col_rank);
 }
 
 void nb_sort_columns(const int* col_ptr, int n, int* col_edge, cudaStream_t st) {
   if (n <= 0) return;
-  sort_columns_kernel<<<(unsigned)(((int64_t)n * 16 + 255) / 256), 256, 0, st>>>(col_ptr, n, col_edge);
+  launch(sort_columns_kernel, (unsigned)(((int64_t)n * 16 + 255) / 256), 256, 0, st, col_ptr, n, col_edge);
 }
 
 // ---------------------------------------------------------------------------
@@ -429,6 +441,7 @@ __global__ void skin_filter_kernel(const double* __restrict__ pos, int n, const 
                                    const int* __restrict__ row_ptr, int* __restrict__ ej, int* __restrict__ ei,
                                    int* __restrict__ eS, double* __restrict__ ed, int* __restrict__ col_count,
                                    int* __restrict__ col_rank, int edge_cap) {
+  pdl_wait();
   if (fill && !list_fits(row_ptr, n, edge_cap)) return;
   const int lane = threadIdx.x & 31;
   const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -473,11 +486,11 @@ void nb_skin_filter(bool fill, const double* pos, int n, const double* d_cell, c
   if (n <= 0) return;
   const int threads = 256, blocks = (int)(((int64_t)n * 32 + threads - 1) / threads);
   if (fill)
-    skin_filter_kernel<true><<<blocks, threads, 0, st>>>(pos, n, d_cell, sk_row, sk_j, sk_S, rc2, pair_rc2, species,
+    launch(skin_filter_kernel<true>, blocks, threads, 0, st, pos, n, d_cell, sk_row, sk_j, sk_S, rc2, pair_rc2, species,
                                                          ns, count, row_ptr, ej, ei, eS, ed, col_count, col_rank,
                                                          edge_cap);
   else
-    skin_filter_kernel<false><<<blocks, threads, 0, st>>>(pos, n, d_cell, sk_row, sk_j, sk_S, rc2, pair_rc2,
+    launch(skin_filter_kernel<false>, blocks, threads, 0, st, pos, n, d_cell, sk_row, sk_j, sk_S, rc2, pair_rc2,
                                                           species, ns, count, row_ptr, ej, ei, eS, ed, col_count, col_rank,
                                                          edge_cap);
 }
@@ -486,6 +499,7 @@ void nb_skin_filter(bool fill, const double* pos, int n, const double* d_cell, c
 // the bits of a non-negative double (their order is the values' order).
 __global__ void max_disp2_kernel(const double* __restrict__ pos, const double* __restrict__ ref, int n,
                                  unsigned long long* __restrict__ out) {
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   double v = 0.0;
   if (i < n) {
@@ -502,7 +516,7 @@ __global__ void max_disp2_kernel(const double* __restrict__ pos, const double* _
 void nb_max_disp2(const double* pos, const double* ref, int n, unsigned long long* out, cudaStream_t st) {
   cudaMemsetAsync(out, 0, sizeof(unsigned long long), st);
   if (n <= 0) return;
-  max_disp2_kernel<<<(n + 255) / 256, 256, 0, st>>>(pos, ref, n, out);
+  launch(max_disp2_kernel, (n + 255) / 256, 256, 0, st, pos, ref, n, out);
 }
 
 // The cell lists in atom order, and with them the wrapped positions pw = pos - wrap . cell in
@@ -515,6 +529,7 @@ __global__ void __launch_bounds__(256) sort_cells_kernel(const double* __restric
                                                          const int* __restrict__ wrap, int* __restrict__ sorted,
                                                          float4* __restrict__ pos4, double* __restrict__ pw,
                                                          int4* __restrict__ wraps) {
+  pdl_wait();
   const int c = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3);
   if (c >= n_cells) return;
   const int b = cell_start[c];
@@ -538,7 +553,7 @@ __global__ void __launch_bounds__(256) sort_cells_kernel(const double* __restric
 void nb_sort_cells(const double* pos, const int* species, const CellGrid& g, int n_cells, const int* cell_start,
                    const int* wrap, int* sorted, float4* pos4, double* pw, int4* wraps, cudaStream_t st) {
   if (n_cells <= 0) return;
-  sort_cells_kernel<<<(unsigned)(((int64_t)n_cells * 8 + 255) / 256), 256, 0, st>>>(pos, species, g, n_cells, cell_start,
+  launch(sort_cells_kernel, (unsigned)(((int64_t)n_cells * 8 + 255) / 256), 256, 0, st, pos, species, g, n_cells, cell_start,
                                                                                     wrap, sorted, pos4, pw, wraps);
 }
 
@@ -589,6 +604,7 @@ __global__ void __launch_bounds__(kSearchThreads) search_kernel(
     const double* __restrict__ pair_rc2, const float* __restrict__ pair_rc2f, int ns, int* __restrict__ count,
     const int* __restrict__ row_ptr, int* __restrict__ ej, int* __restrict__ ei, int* __restrict__ eS, double* __restrict__ ed,
     int* __restrict__ col_count, int* __restrict__ col_rank, int edge_cap, int* __restrict__ d_err) {
+  pdl_wait();
   if (fill && !list_fits(row_ptr, n, edge_cap)) return;
   constexpr int kWarps = kSearchThreads / 32;
   __shared__ SearchCell s_cell[kWarps][32];
@@ -771,6 +787,7 @@ __global__ void __launch_bounds__(kSearchThreads) search_thread_kernel(
     const double* __restrict__ pair_rc2, const float* __restrict__ pair_rc2f, int ns, int* __restrict__ count,
     const int* __restrict__ row_ptr, int* __restrict__ ej, int* __restrict__ ei, int* __restrict__ eS, double* __restrict__ ed,
     int edge_cap, int* __restrict__ d_err) {
+  pdl_wait();
   if (fill && !list_fits(row_ptr, n, edge_cap)) return;
   __shared__ int2 stage[fill ? kSearchThreads : 1][fill ? kFillStage : 1];
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -934,14 +951,12 @@ bool nb_search(bool fill, const double* pos, int n, const CellGrid& g, const int
   if (n <= 0) return true;
   if (n <= kSearchWarpAtoms) {
     auto kernel = fill ? search_kernel<true> : search_kernel<false>;
-    kernel<<<(n + kSearchThreads / 32 - 1) / (kSearchThreads / 32), kSearchThreads, 0, st>>>(
-        pos, n, g, cell_of, wraps, cell_start, sorted, pos4, pw, rc2, band, pair_rc2, pair_rc2f, ns, count, row_ptr, ej, ei, eS, ed,
+    launch(kernel, (n + kSearchThreads / 32 - 1) / (kSearchThreads / 32), kSearchThreads, 0, st, pos, n, g, cell_of, wraps, cell_start, sorted, pos4, pw, rc2, band, pair_rc2, pair_rc2f, ns, count, row_ptr, ej, ei, eS, ed,
         col_count, col_rank, edge_cap, d_err);
     return true;
   }
   auto kernel = fill ? search_thread_kernel<true> : search_thread_kernel<false>;
-  kernel<<<(n + kSearchThreads - 1) / kSearchThreads, kSearchThreads, 0, st>>>(
-      pos, n, g, cell_of, wraps, cell_start, sorted, pos4, pw, rc2, band, pair_rc2, pair_rc2f, ns, count, row_ptr, ej, ei, eS, ed,
+  launch(kernel, (n + kSearchThreads - 1) / kSearchThreads, kSearchThreads, 0, st, pos, n, g, cell_of, wraps, cell_start, sorted, pos4, pw, rc2, band, pair_rc2, pair_rc2f, ns, count, row_ptr, ej, ei, eS, ed,
       edge_cap, d_err);
   return false;
 }
@@ -959,6 +974,7 @@ __global__ void brute_batched_kernel(bool fill, const double* __restrict__ pos,
                                      int* __restrict__ ej, int* __restrict__ ei, int* __restrict__ eS,
                                      double* __restrict__ ed, int* __restrict__ col_count,
                                      int* __restrict__ col_rank, int edge_cap, int* __restrict__ d_err) {
+  pdl_wait();
   if (fill && !list_fits(row_ptr, n, edge_cap)) return;
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -1015,6 +1031,7 @@ __global__ void __launch_bounds__(128) brute_nocell_kernel(const double* __restr
                                                            int* __restrict__ eS, double* __restrict__ ed,
                                                            int* __restrict__ col_count, int* __restrict__ col_rank,
                                                            int edge_cap, int* __restrict__ d_err) {
+  pdl_wait();
   if (fill && !list_fits(row_ptr, n, edge_cap)) return;
   const int i = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 4);
   if (i >= n) return;
@@ -1065,12 +1082,12 @@ void nb_bruteforce_batched(bool fill, const double* pos, const int64_t* offs, in
   if (n <= 0) return;
   if (!cells) {
     auto kernel = fill ? brute_nocell_kernel<true> : brute_nocell_kernel<false>;
-    kernel<<<(unsigned)(((int64_t)n * 16 + 127) / 128), 128, 0, st>>>(pos, offs, rc2, species, pair_rc2, ns, atom_struct,
+    launch(kernel, (unsigned)(((int64_t)n * 16 + 127) / 128), 128, 0, st, pos, offs, rc2, species, pair_rc2, ns, atom_struct,
                                                                       n, count, row_ptr, ej, ei, eS, ed, col_count,
                                                                       col_rank, edge_cap, d_err);
     return;
   }
-  brute_batched_kernel<<<(n + 127) / 128, 128, 0, st>>>(fill, pos, offs, cells, pbc, nimg, rc2, species, pair_rc2,
+  launch(brute_batched_kernel, (n + 127) / 128, 128, 0, st, fill, pos, offs, cells, pbc, nimg, rc2, species, pair_rc2,
                                                         ns, atom_struct, n, count, row_ptr, ej, ei, eS, ed,
                                                         col_count, col_rank, edge_cap, d_err);
 }
@@ -1079,6 +1096,7 @@ void nb_bruteforce_batched(bool fill, const double* pos, const int64_t* offs, in
 // image range covers positions that are not wrapped into the cell.
 __global__ void struct_span_kernel(const double* __restrict__ pos, const int64_t* __restrict__ offs,
                                    const double* __restrict__ inv, double* __restrict__ span) {
+  pdl_wait();
   const int b = blockIdx.x;
   __shared__ double lo[3][128], hi[3][128];
   double l[3] = {1e300, 1e300, 1e300}, h[3] = {-1e300, -1e300, -1e300};
@@ -1106,7 +1124,7 @@ __global__ void struct_span_kernel(const double* __restrict__ pos, const int64_t
 void nb_struct_span(const double* pos, const int64_t* offs, const double* inv, int nstruct, double* span,
                     cudaStream_t st) {
   if (nstruct <= 0) return;
-  struct_span_kernel<<<nstruct, 128, 0, st>>>(pos, offs, inv, span);
+  launch(struct_span_kernel, nstruct, 128, 0, st, pos, offs, inv, span);
 }
 
 }  // namespace alg

@@ -59,6 +59,7 @@
 
 #include "amax.cuh"
 #include "internal.h"
+#include "launch.cuh"
 #include "row_ring.cuh"
 
 namespace alg {
@@ -330,6 +331,7 @@ __device__ __forceinline__ void chain_mv(const float* v, const float (&G)[D], co
 // Q^L[i][u][:] = M^1 ... M^L e_0
 template <int LMAX, int NL, int L>
 __global__ void __launch_bounds__(kChainThreads) gen_chain_fwd_kernel(GenRowIO io, const __grid_constant__ GenVals<LMAX, NL> w) {
+  pdl_wait();
   constexpr int S = (LMAX + 1) * (LMAX + 1);
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= io.na * io.C) return;
@@ -381,6 +383,7 @@ __device__ __forceinline__ void chain_adj(const float* v, const float (&G)[D], c
 // Back along the chain of Q^L: Gammabar^k += ..., k = 1..L (the last layer, which comes first, writes them)
 template <int LMAX, int NL, int L>
 __global__ void __launch_bounds__(kChainThreads) gen_chain_bwd_kernel(GenRowIO io, const __grid_constant__ GenVals<LMAX, NL> w) {
+  pdl_wait();
   constexpr int S = (LMAX + 1) * (LMAX + 1);
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= io.na * io.C) return;
@@ -441,6 +444,7 @@ __global__ void __launch_bounds__(kChainThreads) gen_chain_bwd_kernel(GenRowIO i
 // beside the multiply-adds, which run on component pairs in packed fp32).
 template <typename T, int LMAX, int NL, bool AMAX>
 __global__ void __launch_bounds__(kMaxChannels) gen_edge_final_kernel(GenRowIO io) {
+  pdl_wait();
   constexpr int S = (LMAX + 1) * (LMAX + 1), LM = LMAX + 1, S2 = (S + 1) / 2;
   static_assert(S <= 16, "halving sums of 16 components");
   // per-warp channel partials of Ybar for batches of kEdgeBatch edges, double-buffered:
@@ -624,6 +628,7 @@ __device__ __forceinline__ bool gen_lane(const GenRowIO& io, GenLane& g) {
 // Gamma^L[i][u][b] = nu sum_{e in row i} w^L[e][u][l(b)] Y[e][b]
 template <typename T, int LMAX, int CPL>
 __global__ void __launch_bounds__(32 * kGenWarps) gen_env_w_kernel(GenRowIO io, int L) {
+  pdl_wait();
   constexpr int S = (LMAX + 1) * (LMAX + 1), LM = LMAX + 1;
   constexpr int kW = 32 * CPL * LM * (int)sizeof(T), kStage = round16(kW + S * 4);
   __shared__ __align__(16) unsigned char rings[kGenWarps][kRing * kStage];
@@ -663,6 +668,7 @@ __global__ void __launch_bounds__(32 * kGenWarps) gen_env_w_kernel(GenRowIO io, 
 // s^L_e[u] = sum_a w^0_{e,u,l(a)} Y_e[a] Q^L[i][u][a], into the s columns of the latent input
 template <typename T, int LMAX, int CPL>
 __global__ void __launch_bounds__(32 * kGenWarps) gen_s_w_kernel(GenRowIO io, int L) {
+  pdl_wait();
   constexpr int S = (LMAX + 1) * (LMAX + 1), LM = LMAX + 1;
   constexpr int kW = 32 * CPL * LM * (int)sizeof(T), kStage = round16(kW + S * 4);
   __shared__ __align__(16) unsigned char rings[kGenWarps][kRing * kStage];
@@ -703,6 +709,7 @@ __global__ void __launch_bounds__(32 * kGenWarps) gen_s_w_kernel(GenRowIO io, in
 // Qbar^L[i][u][a] = sum_e sbar^L_e[u] w^0_{e,u,l(a)} Y_e[a]
 template <typename T, int LMAX, int CPL>
 __global__ void __launch_bounds__(32 * kGenWarps) gen_qbar_w_kernel(GenRowIO io, int L) {
+  pdl_wait();
   constexpr int S = (LMAX + 1) * (LMAX + 1), LM = LMAX + 1;
   constexpr int kW = 32 * CPL * LM * (int)sizeof(T), kSb = 32 * CPL * (int)sizeof(T), kStage = round16(kW + kSb + S * 4);
   __shared__ __align__(16) unsigned char rings[kGenWarps][kRing * kStage];
@@ -747,6 +754,7 @@ __global__ void __launch_bounds__(32 * kGenWarps) gen_qbar_w_kernel(GenRowIO io,
 // wbar^L_{e,u,l} = nu sum_m Gammabar^L[i][u][lm] Y_e[lm], for a layer L >= 2
 template <typename T, int LMAX, int CPL>
 __global__ void __launch_bounds__(32 * kGenWarps) gen_wbar_w_kernel(GenRowIO io, int L) {
+  pdl_wait();
   constexpr int S = (LMAX + 1) * (LMAX + 1), LM = LMAX + 1;
   constexpr int kStage = round16(S * 4);
   __shared__ __align__(16) unsigned char rings[kGenWarps][kRing * kStage];
@@ -786,9 +794,9 @@ static int block_of(int C) { return (C + 31) / 32 * 32; }
 #define GEN_W_LAUNCH(KERNEL, ...)                                                     \
   do {                                                                                \
     const dim3 grid_((io.na + kGenWarps - 1) / kGenWarps), block_(32 * kGenWarps);    \
-    if (io.C >= 128) KERNEL<T, LMAX, 4><<<grid_, block_, 0, st>>>(__VA_ARGS__);       \
-    else if (io.C >= 64) KERNEL<T, LMAX, 2><<<grid_, block_, 0, st>>>(__VA_ARGS__);   \
-    else KERNEL<T, LMAX, 1><<<grid_, block_, 0, st>>>(__VA_ARGS__);                   \
+    if (io.C >= 128) launch(KERNEL<T, LMAX, 4>, grid_, block_, 0, st, __VA_ARGS__);       \
+    else if (io.C >= 64) launch(KERNEL<T, LMAX, 2>, grid_, block_, 0, st, __VA_ARGS__);   \
+    else launch(KERNEL<T, LMAX, 1>, grid_, block_, 0, st, __VA_ARGS__);                   \
   } while (0)
 
 template <int LMAX, int NL>
@@ -802,18 +810,18 @@ template <int LMAX, int NL>
 static void chain_fwd(const GenRowIO& io, int L, cudaStream_t st) {
   const GenVals<LMAX, NL> w = vals_of<LMAX, NL>(io);
   const int g = (io.na * io.C + kChainThreads - 1) / kChainThreads;
-  if (L == 1) gen_chain_fwd_kernel<LMAX, NL, 1><<<g, kChainThreads, 0, st>>>(io, w);
-  if constexpr (NL >= 2) if (L == 2) gen_chain_fwd_kernel<LMAX, NL, 2><<<g, kChainThreads, 0, st>>>(io, w);
-  if constexpr (NL >= 3) if (L == 3) gen_chain_fwd_kernel<LMAX, NL, 3><<<g, kChainThreads, 0, st>>>(io, w);
+  if (L == 1) launch(gen_chain_fwd_kernel<LMAX, NL, 1>, g, kChainThreads, 0, st, io, w);
+  if constexpr (NL >= 2) if (L == 2) launch(gen_chain_fwd_kernel<LMAX, NL, 2>, g, kChainThreads, 0, st, io, w);
+  if constexpr (NL >= 3) if (L == 3) launch(gen_chain_fwd_kernel<LMAX, NL, 3>, g, kChainThreads, 0, st, io, w);
 }
 
 template <int LMAX, int NL>
 static void chain_bwd(const GenRowIO& io, int L, cudaStream_t st) {
   const GenVals<LMAX, NL> w = vals_of<LMAX, NL>(io);
   const int g = (io.na * io.C + kChainThreads - 1) / kChainThreads;
-  if (L == 1) gen_chain_bwd_kernel<LMAX, NL, 1><<<g, kChainThreads, 0, st>>>(io, w);
-  if constexpr (NL >= 2) if (L == 2) gen_chain_bwd_kernel<LMAX, NL, 2><<<g, kChainThreads, 0, st>>>(io, w);
-  if constexpr (NL >= 3) if (L == 3) gen_chain_bwd_kernel<LMAX, NL, 3><<<g, kChainThreads, 0, st>>>(io, w);
+  if (L == 1) launch(gen_chain_bwd_kernel<LMAX, NL, 1>, g, kChainThreads, 0, st, io, w);
+  if constexpr (NL >= 2) if (L == 2) launch(gen_chain_bwd_kernel<LMAX, NL, 2>, g, kChainThreads, 0, st, io, w);
+  if constexpr (NL >= 3) if (L == 3) launch(gen_chain_bwd_kernel<LMAX, NL, 3>, g, kChainThreads, 0, st, io, w);
 }
 
 // the (l_max, layers) models of the generic path
@@ -847,8 +855,8 @@ static void bwd_lmax(const GenRowIO& io, int L, cudaStream_t st) {
     return;
   }
   auto final = [&](auto plain, auto recorded) {
-    if (io.amax_wbar) recorded<<<io.na, bl, 0, st>>>(io);
-    else plain<<<io.na, bl, 0, st>>>(io);
+    if (io.amax_wbar) launch(recorded, io.na, bl, 0, st, io);
+    else launch(plain, io.na, bl, 0, st, io);
   };
   if (io.nl == 1) final(gen_edge_final_kernel<T, LMAX, 1, false>, gen_edge_final_kernel<T, LMAX, 1, true>);
   else if (io.nl == 2) final(gen_edge_final_kernel<T, LMAX, 2, false>, gen_edge_final_kernel<T, LMAX, 2, true>);

@@ -28,6 +28,7 @@
 #include <cuda_bf16.h>
 
 #include "internal.h"
+#include "launch.cuh"
 #include "row_ring.cuh"
 
 namespace alg {
@@ -422,6 +423,7 @@ __device__ __forceinline__ void scalar_out(const RowIO& io, const RowCtx& r, con
 // ---------------------------------------------------------------------------
 template <typename T, int LMAX, int CPL>
 __global__ void __launch_bounds__(32 * kRowWarps) row_fwd_mid_kernel(RowIO io, TPConst tp) {
+  pdl_wait();
   constexpr int S = (LMAX + 1) * (LMAX + 1);
   __shared__ __align__(16) float ysm[kRowWarps * kYSeg * YStage<S>::P];
   RowCtx r;
@@ -488,6 +490,7 @@ __device__ __forceinline__ void make_T2(const TPConst& tp, const float (&G1)[S],
 // ---------------------------------------------------------------------------
 template <typename T, int LMAX, int NL, int CPL>
 __global__ void __launch_bounds__(32 * kRowWarps) row_fwd_last_kernel(RowIO io, TPConst tp) {
+  pdl_wait();
   constexpr int S = (LMAX + 1) * (LMAX + 1);
   __shared__ __align__(16) float ysm[kRowWarps * kYSeg * YStage<S>::P];
   RowCtx r;
@@ -530,6 +533,7 @@ __global__ void __launch_bounds__(32 * kRowWarps) row_fwd_last_kernel(RowIO io, 
 // ---------------------------------------------------------------------------
 template <typename T, int LMAX, int NL, int CPL>
 __global__ void __launch_bounds__(32 * kRowWarps) row_bwd_last_kernel(RowIO io, TPConst tp) {
+  pdl_wait();
   constexpr int S = (LMAX + 1) * (LMAX + 1);
   constexpr int LM = LMAX + 1;
   __shared__ __align__(16) float ysm[kRowWarps * kYSeg * YStage<S>::P];
@@ -717,6 +721,7 @@ __global__ void __launch_bounds__(32 * kRowWarps) row_bwd_last_kernel(RowIO io, 
 template <typename T, int LMAX, int CPL>
 // (at most 128 registers, four blocks per SM, where two channels per lane fit them)
 __global__ void __launch_bounds__(32 * kRowWarps, CPL > 2 ? 2 : 4) row_bwd_mid_kernel(RowIO io, TPConst tp) {
+  pdl_wait();
   constexpr int S = (LMAX + 1) * (LMAX + 1);
   constexpr int LM = LMAX + 1;
   using WS = WSpan<T, CPL, LM>;
@@ -927,14 +932,14 @@ template <typename T, int CPL>
 void row_fwd_cpl(int layer, int nl, int lmax, const RowIO& io, const TPConst& tp, cudaStream_t st) {
   dim3 grid((io.na + kRowWarps - 1) / kRowWarps), block(32 * kRowWarps);
   if (layer < nl) {
-    if (lmax == 1) row_fwd_mid_kernel<T, 1, CPL><<<grid, block, 0, st>>>(io, tp);
-    else row_fwd_mid_kernel<T, 2, CPL><<<grid, block, 0, st>>>(io, tp);
+    if (lmax == 1) launch(row_fwd_mid_kernel<T, 1, CPL>, grid, block, 0, st, io, tp);
+    else launch(row_fwd_mid_kernel<T, 2, CPL>, grid, block, 0, st, io, tp);
   } else if (nl == 1) {
-    if (lmax == 1) row_fwd_last_kernel<T, 1, 1, CPL><<<grid, block, 0, st>>>(io, tp);
-    else row_fwd_last_kernel<T, 2, 1, CPL><<<grid, block, 0, st>>>(io, tp);
+    if (lmax == 1) launch(row_fwd_last_kernel<T, 1, 1, CPL>, grid, block, 0, st, io, tp);
+    else launch(row_fwd_last_kernel<T, 2, 1, CPL>, grid, block, 0, st, io, tp);
   } else {
-    if (lmax == 1) row_fwd_last_kernel<T, 1, 2, CPL><<<grid, block, 0, st>>>(io, tp);
-    else row_fwd_last_kernel<T, 2, 2, CPL><<<grid, block, 0, st>>>(io, tp);
+    if (lmax == 1) launch(row_fwd_last_kernel<T, 1, 2, CPL>, grid, block, 0, st, io, tp);
+    else launch(row_fwd_last_kernel<T, 2, 2, CPL>, grid, block, 0, st, io, tp);
   }
 }
 
@@ -942,14 +947,14 @@ template <typename T, int CPL>
 void row_bwd_cpl(int layer, int nl, int lmax, const RowIO& io, const TPConst& tp, cudaStream_t st) {
   dim3 grid((io.na + kRowWarps - 1) / kRowWarps), block(32 * kRowWarps);
   if (layer < nl) {
-    if (lmax == 1) row_bwd_mid_kernel<T, 1, CPL><<<grid, block, 0, st>>>(io, tp);
-    else row_bwd_mid_kernel<T, 2, CPL><<<grid, block, 0, st>>>(io, tp);
+    if (lmax == 1) launch(row_bwd_mid_kernel<T, 1, CPL>, grid, block, 0, st, io, tp);
+    else launch(row_bwd_mid_kernel<T, 2, CPL>, grid, block, 0, st, io, tp);
   } else if (nl == 1) {
-    if (lmax == 1) row_bwd_last_kernel<T, 1, 1, CPL><<<grid, block, 0, st>>>(io, tp);
-    else row_bwd_last_kernel<T, 2, 1, CPL><<<grid, block, 0, st>>>(io, tp);
+    if (lmax == 1) launch(row_bwd_last_kernel<T, 1, 1, CPL>, grid, block, 0, st, io, tp);
+    else launch(row_bwd_last_kernel<T, 2, 1, CPL>, grid, block, 0, st, io, tp);
   } else {
-    if (lmax == 1) row_bwd_last_kernel<T, 1, 2, CPL><<<grid, block, 0, st>>>(io, tp);
-    else row_bwd_last_kernel<T, 2, 2, CPL><<<grid, block, 0, st>>>(io, tp);
+    if (lmax == 1) launch(row_bwd_last_kernel<T, 1, 2, CPL>, grid, block, 0, st, io, tp);
+    else launch(row_bwd_last_kernel<T, 2, 2, CPL>, grid, block, 0, st, io, tp);
   }
 }
 }  // namespace
