@@ -998,7 +998,7 @@ const char* gemm_label(allegro_ctx* c, const Lin* W, bool trans, int epi) {
   for (size_t L = 0; L < c->lat.size(); ++L)
     for (size_t k = 0; k < c->lat[L].size(); ++k)
       if (W == &c->lat[L][k]) n = "latent." + std::to_string(L + 1) + "." + std::to_string(k);
-  const char* en[] = {"silu", "f32", "dsilu", "head", "last", "linear"};
+  const char* en[] = {"silu", "f32", "dsilu", "head", "last", "linear", "head"};
   n = std::string(c->prec == ALLEGRO_PREC_BF16 ? "gemm_tc/"
                   : (c->prec == ALLEGRO_PREC_TF32 ? "gemm_tf32/"
                                                   : (c->prec == ALLEGRO_PREC_FP8 ? "gemm_fp8/" : "gemm_simt/"))) +
@@ -1220,8 +1220,7 @@ allegro_status run_chunk(allegro_ctx* c, const WS& w, int a0, int a1, int e0, in
   // layer's pre-activation (into H[0]); it runs paired with the first transposed GEMM.
   auto back_mlp = [&](const std::vector<Lin>& layers, const std::vector<void*>& Z, const std::vector<int>& ldZ,
                       int nlay, void* dst, int ld_dst, int Kin, int epi_dst, int col0, const void** zin,
-                      const GemmArgs* head) -> allegro_status {
-    int cur = 0;
+                      const GemmArgs* head, int cur = 0) -> allegro_status {
     int k = nlay - 1;
     if (head && nlay < 2) {
       allegro_status r = run1(*head);
@@ -1270,6 +1269,18 @@ allegro_status run_chunk(allegro_ctx* c, const WS& w, int a0, int a1, int e0, in
   auto kcat = [&](int L) { return bf16 && c->headB[L - 1] != nullptr; };
   if (bf16 && !fused && (!kcat(1) || (nl == 2 && !kcat(2))))
     return fail(c, ALLEGRO_E_INVALID, "BF16 path with MLPs wider than 256 needs 64-aligned env-weight widths");
+  // Adjoint heads of wide MLPs in the epilogue of the GEMM that forms xbar, where its path has one
+  // (the float32 xbar never reaches HBM); zbar goes to the H buffer that GEMM does not read
+  const bool wide_t = !fused && gemm_head_wide(c->prec, Ec, a.lat.back());
+  const bool wide_0 = !fused && gemm_head_wide(c->prec, Ec, a.tb.back());
+  auto to_wide = [&](GemmArgs& g, const void* pre, int ldp) {
+    const int h = g.A2 == w.H[0] ? 1 : 0;
+    g.epi = EPI_HEAD_WIDE;
+    g.out = w.H[h]; g.ldo = w.ld_H;
+    g.pre = const_cast<void*>(pre); g.ldp = ldp;
+    g.rowscale = w.u; g.ubar = w.ubar;
+    return h;
+  };
   // D (the latent inputs' adjoint) is stored in the activation type: EPI_LINEAR
   const void* zlat[2] = {nullptr, nullptr};
   if ((s = back_mlp(c->lat[nl - 1], w.Zlat[nl - 1], w.ld_Zlat, nlat, w.D[nl - 1], w.ld_D[nl - 1],
@@ -1291,11 +1302,13 @@ allegro_status run_chunk(allegro_ctx* c, const WS& w, int a0, int a1, int e0, in
     // xbar^1 = wbar^2 . env2 + D[1][:, :K1], then the adjoint head of x^1 = u silu(z)
     GemmArgs head1;
     const GemmArgs* head1p = nullptr;
+    int h1 = 0;   // H buffer that holds zbar of the latent MLP's last layer
     if (kcat(2) && !fused) {
       // wide MLPs: xbar^1 in float32 from the K-concatenated GEMM, the head below
       head1 = mk(w.wbar2, w.ld_wbar2, c->headK[1], c->env2, true, EPI_F32, w.xbar, w.ld_xbar, a.lat.back());
       head1.A2 = zlat[1]; head1.lda2 = w.ld_H; head1.K1 = c->headK1[1];
       head1.Bover = c->headB[1]; head1.ldb_over = c->headLd[1];
+      if (wide_t) h1 = to_wide(head1, w.Zlat[0][nlat - 1], w.ld_Zlat[nlat - 1]);
       if ((s = run1(head1)) != ALLEGRO_OK) return s;
     } else if (kcat(2)) {
       head1 = mk(w.wbar2, w.ld_wbar2, c->headK[1], c->env2, true, EPI_HEAD, w.H[0], w.ld_H, a.lat.back(),
@@ -1307,18 +1320,20 @@ allegro_status run_chunk(allegro_ctx* c, const WS& w, int a0, int a1, int e0, in
       if ((s = G(w.wbar2, w.ld_wbar2, nw, c->env2, true, EPI_HEAD, w.H[0], w.ld_H, a.lat.back(),
                  w.Zlat[0][nlat - 1], w.ld_Zlat[nlat - 1], w.u, w.D[1], w.ld_D[1], w.ubar)) != ALLEGRO_OK)
         return s;
-    } else if ((s = G(w.wbar2, w.ld_wbar2, nw, c->env2, true, EPI_F32, w.xbar, w.ld_xbar, a.lat.back(), nullptr,
-                      0, nullptr, w.D[1], w.ld_D[1])) != ALLEGRO_OK) {
-      return s;
+    } else {
+      head1 = mk(w.wbar2, w.ld_wbar2, nw, c->env2, true, EPI_F32, w.xbar, w.ld_xbar, a.lat.back(), nullptr, 0, nullptr,
+                 w.D[1], w.ld_D[1]);
+      if (wide_t) h1 = to_wide(head1, w.Zlat[0][nlat - 1], w.ld_Zlat[nlat - 1]);
+      if ((s = run1(head1)) != ALLEGRO_OK) return s;
     }
-    if (!fused) {
+    if (!fused && !wide_t) {
       ProfScope ps(c, "head_bwd", 0.0, (double)Ec * (a.lat.back() * (4 + 2 * act) + 12));
       mlp_head_bwd<T>(Ec, a.lat.back(), w.xbar, w.ld_xbar, nullptr, c->d_ei, c->d_species, c->d_sigma, e0,
                       (const T*)w.Zlat[0][nlat - 1], w.ld_Zlat[nlat - 1], w.u, w.ubar, false, (T*)w.H[0], w.ld_H,
                       st);
     }
     if ((s = back_mlp(c->lat[0], w.Zlat[0], w.ld_Zlat, nlat, w.D[0], w.ld_D[0], a.Klat(0) + a.C, EPI_LINEAR,
-                      kcat(1) ? a.Klat(0) : 0, &zlat[0], head1p)) != ALLEGRO_OK)
+                      kcat(1) ? a.Klat(0) : 0, &zlat[0], head1p, h1)) != ALLEGRO_OK)
       return s;
     io.sbar1 = (const T*)w.D[0] + a.Klat(0); io.ld_sbar1 = w.ld_D[0];
     auto ps = row_scope("row_bwd_mid", 2.0 * nw * act + 2.0 * C * act + S * 4 + 2.0 * nw * act + S * 4,
@@ -1328,11 +1343,13 @@ allegro_status run_chunk(allegro_ctx* c, const WS& w, int a0, int a1, int e0, in
   // xbar^0 = [wbar^0 | wbar^1] . [W_emb ; W_env1] + D[0][:, :K0], then the head of x^0 = u silu(z)
   GemmArgs head0;
   bool head0_pending = false;
+  int cur0 = 0;   // H buffer that holds zbar of the two-body MLP's last layer
   if (kcat(1) && !fused) {
     // wide MLPs: xbar^0 in float32 from the K-concatenated GEMM, the head below
     head0 = mk(w.wbar01, w.ld_wbar01, c->headK[0], c->w01, true, EPI_F32, w.xbar, w.ld_xbar, a.tb.back());
     head0.A2 = zlat[0]; head0.lda2 = w.ld_H; head0.K1 = c->headK1[0];
     head0.Bover = c->headB[0]; head0.ldb_over = c->headLd[0];
+    if (wide_0) cur0 = to_wide(head0, w.Ztb[ntb - 1], w.ld_Ztb[ntb - 1]);
     if ((s = run1(head0)) != ALLEGRO_OK) return s;
   } else if (kcat(1)) {
     head0 = mk(w.wbar01, w.ld_wbar01, c->headK[0], c->w01, true, EPI_HEAD, w.H[0], w.ld_H, a.tb.back(),
@@ -1345,17 +1362,18 @@ allegro_status run_chunk(allegro_ctx* c, const WS& w, int a0, int a1, int e0, in
     if ((s = G(w.wbar01, w.ld_wbar01, 2 * nw, c->w01, true, EPI_HEAD, w.H[0], w.ld_H, a.tb.back(),
                w.Ztb[ntb - 1], w.ld_Ztb[ntb - 1], w.u, w.D[0], w.ld_D[0], w.ubar)) != ALLEGRO_OK)
       return s;
-  } else if ((s = G(w.wbar01, w.ld_wbar01, 2 * nw, c->w01, true, EPI_F32, w.xbar, w.ld_xbar, a.tb.back(), nullptr,
-                    0, nullptr, w.D[0], w.ld_D[0])) != ALLEGRO_OK) {
-    return s;
+  } else {
+    head0 = mk(w.wbar01, w.ld_wbar01, 2 * nw, c->w01, true, EPI_F32, w.xbar, w.ld_xbar, a.tb.back(), nullptr, 0, nullptr,
+               w.D[0], w.ld_D[0]);
+    if (wide_0) cur0 = to_wide(head0, w.Ztb[ntb - 1], w.ld_Ztb[ntb - 1]);
+    if ((s = run1(head0)) != ALLEGRO_OK) return s;
   }
-  if (!fused) {
+  if (!fused && !wide_0) {
     ProfScope ps(c, "head_bwd", 0.0, (double)Ec * (a.tb.back() * (4 + 2 * act) + 12));
     mlp_head_bwd<T>(Ec, a.tb.back(), w.xbar, w.ld_xbar, nullptr, c->d_ei, c->d_species, c->d_sigma, e0,
                     (const T*)w.Ztb[ntb - 1], w.ld_Ztb[ntb - 1], w.u, w.ubar, false, (T*)w.H[0], w.ld_H, st);
   }
   // two-body MLP adjoint down to zbar0; the first layer's transposed product is folded into geom_bwd
-  int cur0 = 0;
   for (int k = ntb - 1; k >= 1; --k) {
     const Lin& W = c->tb[k];
     GemmArgs g = mk(w.H[cur0], w.ld_H, W.N, W, true, EPI_BWD_SILU, w.H[cur0 ^ 1], w.ld_H, W.K, w.Ztb[k - 1],
@@ -1429,7 +1447,7 @@ allegro_status run_chunk_gen(allegro_ctx* c, const WS& w, int a0, int a1, int e0
     if (fp8) {
       g.amax_a = slot_of(g.A);
       g.amax_a2 = slot_of(g.A2);
-      if (g.epi == EPI_FWD_SILU || g.epi == EPI_BWD_SILU) {
+      if (g.epi == EPI_FWD_SILU || g.epi == EPI_BWD_SILU || g.epi == EPI_HEAD_WIDE) {
         g.amax_out = fresh(g.out);
         if (!g.amax_out) return fail(c, ALLEGRO_E_INVALID, "FP8: more than %d activation arrays in a chunk", kAmaxSlots);
       }
@@ -1456,8 +1474,7 @@ allegro_status run_chunk_gen(allegro_ctx* c, const WS& w, int a0, int a1, int e0
   };
   // adjoint of an MLP from zbar of its last layer (in H[0]) to its input's adjoint, columns [col0, Kin)
   auto back_mlp = [&](const std::vector<Lin>& layers, const std::vector<void*>& Z, const std::vector<int>& ldZ,
-                      void* dst, int ld_dst, int Kin, int col0, const void** zin) -> allegro_status {
-    int cur = 0;
+                      void* dst, int ld_dst, int Kin, int col0, const void** zin, int cur) -> allegro_status {
     for (int k = (int)layers.size() - 1; k >= 0; --k) {
       const Lin& W = layers[k];
       allegro_status r;
@@ -1541,11 +1558,12 @@ allegro_status run_chunk_gen(allegro_ctx* c, const WS& w, int a0, int a1, int e0
                     (const T*)w.Zlat[nl - 1][nlat - 1], w.ld_Zlat[nlat - 1], w.u, w.ubar, true, (T*)w.H[0], w.ld_H,
                     st, fresh(w.H[0]));
   }
+  int hz = 0;   // H buffer that holds zbar of the MLP to go back through next
   for (int L = nl; L >= 1; --L) {
     const bool kc = bf16 && c->headB[L - 1] != nullptr && (!fp8 || c->headB8[L - 1] != nullptr);
     const void* zlat = nullptr;
     if ((s = back_mlp(c->lat[L - 1], w.Zlat[L - 1], w.ld_Zlat, w.D[L - 1], w.ld_D[L - 1], a.Klat(L - 1) + a.C,
-                      kc ? a.Klat(L - 1) : 0, &zlat)) != ALLEGRO_OK)
+                      kc ? a.Klat(L - 1) : 0, &zlat, hz)) != ALLEGRO_OK)
       return s;
     {
       ProfScope ps(c, "row_gen_bwd", 0.0, (double)Ec * (4.0 * nw * act + 2 * S * 4 + a.C * act) + (double)Ac * a.C * S * 16.0, 3);
@@ -1570,15 +1588,26 @@ allegro_status run_chunk_gen(allegro_ctx* c, const WS& w, int a0, int a1, int e0
       hd = mk(wbL[L], (L == 1) ? w.ld_wbar01 : w.ld_wbar2, K1, *env[L], true, EPI_F32, w.xbar, w.ld_xbar,
               a.Klat(L - 1), nullptr, 0, nullptr, w.D[L - 1], w.ld_D[L - 1]);
     }
-    if ((s = run1(hd)) != ALLEGRO_OK) return s;
     const void* pre = (L == 1) ? w.Ztb[ntb - 1] : w.Zlat[L - 2][nlat - 1];
     const int ldp = (L == 1) ? w.ld_Ztb[ntb - 1] : w.ld_Zlat[nlat - 1];
+    hz = 0;
+    if ((kc || !bf16) && gemm_head_wide(c->prec, Ec, a.Klat(L - 1))) {
+      // the head in the GEMM's epilogue; zbar goes to the H buffer the GEMM does not read
+      hz = hd.A2 == w.H[0] ? 1 : 0;
+      hd.epi = EPI_HEAD_WIDE;
+      hd.out = w.H[hz]; hd.ldo = w.ld_H;
+      hd.pre = const_cast<void*>(pre); hd.ldp = ldp;
+      hd.rowscale = w.u; hd.ubar = w.ubar;
+      if ((s = run1(hd)) != ALLEGRO_OK) return s;
+      continue;
+    }
+    if ((s = run1(hd)) != ALLEGRO_OK) return s;
     ProfScope ps(c, "head_bwd", 0.0, (double)Ec * (a.Klat(L - 1) * (4 + 2 * act) + 12));
     mlp_head_bwd<T>(Ec, a.Klat(L - 1), w.xbar, w.ld_xbar, nullptr, c->d_ei, c->d_species, c->d_sigma, e0,
                     (const T*)pre, ldp, w.u, w.ubar, false, (T*)w.H[0], w.ld_H, st, fresh(w.H[0]),
                     (bf16 && !kc) ? (const T*)w.D[L - 1] : nullptr, w.ld_D[L - 1]);
   }
-  int cur0 = 0;
+  int cur0 = hz;
   for (int k = ntb - 1; k >= 1; --k) {
     const Lin& W = c->tb[k];
     if ((s = run1(mk(w.H[cur0], w.ld_H, W.N, W, true, EPI_BWD_SILU, w.H[cur0 ^ 1], w.ld_H, W.K, w.Ztb[k - 1],

@@ -241,7 +241,8 @@ __global__ void __launch_bounds__(kF8Threads, 1)
   uint64_t* tfull = sempty + kF8Stg;                   // [2] accumulator ready
   uint64_t* tempty = tfull + 2;                        // [2] accumulator drained (one arrival per epilogue warp)
   uint64_t* inbar = tempty + 2;                        // [kF8EpiWarps] input box filled
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(inbar + kF8EpiWarps);
+  uint64_t* hbar = inbar + kF8EpiWarps;                // [4 quarters][2] EPI_HEAD_WIDE partial sums ready / used
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(hbar + 8);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -253,6 +254,11 @@ __global__ void __launch_bounds__(kF8Threads, 1)
   // block run on neighbouring CTAs, so their A rows come from L2 after the first read
   auto tm0 = [&](int tt) { return (tt / tiles_n) * 128; };
   auto tn0 = [&](int tt) { return (tt % tiles_n) * BN; };
+  // EPI_HEAD_WIDE: a CTA takes whole row blocks, their column tiles one after another
+  constexpr bool kWide = BN == 256;
+  const bool wide = kWide && ep.epi == EPI_HEAD_WIDE;
+  const int tstep = gridDim.x, tfirst = wide ? (int)blockIdx.x * tiles_n : (int)blockIdx.x;
+  auto next = [&](int tt) { return !wide ? tt + tstep : ((tt + 1) % tiles_n ? tt + 1 : tt + 1 + (tstep - 1) * tiles_n); };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kF8Stages; ++s) {
@@ -269,6 +275,7 @@ __global__ void __launch_bounds__(kF8Threads, 1)
       mbar_init(&tempty[b], kF8EpiWarps);
     }
     for (int w = 0; w < kF8EpiWarps; ++w) mbar_init(&inbar[w], 1);
+    for (int w = 0; w < 8; ++w) mbar_init(&hbar[w], 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -287,7 +294,7 @@ __global__ void __launch_bounds__(kF8Threads, 1)
     if (lane == 0) {
       uint32_t g = 0;   // global k-block counter
       bool ok = true;
-      for (int t = blockIdx.x; t < ntiles && ok && !*abort_flag; t += gridDim.x) {
+      for (int t = tfirst; t < ntiles && ok && !*abort_flag; t = next(t)) {
         const int n0 = tn0(t);
         for (int kb = 0; kb < nk; ++kb, ++g) {
           const uint32_t s = g % kF8Stages, r = g / kF8Stages;
@@ -308,7 +315,7 @@ __global__ void __launch_bounds__(kF8Threads, 1)
     if (lane == 0) {
       uint32_t g2 = 0;   // global half counter
       bool ok = true;
-      for (int t = blockIdx.x; t < ntiles && ok && !*abort_flag; t += gridDim.x) {
+      for (int t = tfirst; t < ntiles && ok && !*abort_flag; t = next(t)) {
         const int m0 = tm0(t);
         for (int hb = 0; hb < 2 * nk; ++hb, ++g2) {
           const uint32_t s2 = g2 % kF8Stg, r2 = g2 / kF8Stg;
@@ -333,7 +340,7 @@ __global__ void __launch_bounds__(kF8Threads, 1)
       constexpr uint32_t idesc = idesc_e4m3<BN>();
       uint32_t g = 0;
       int lt = 0;
-      for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++lt) {
+      for (int t = tfirst; t < ntiles; t = next(t), ++lt) {
         const int b = lt & 1, use = lt >> 1;
         bool ok = !*abort_flag && mbar_wait(&tempty[b], (use & 1) ^ 1);
         if (ok) {
@@ -372,7 +379,9 @@ __global__ void __launch_bounds__(kF8Threads, 1)
     uint8_t* box0 = sE + ew * kF8EpiSlot;
     uint8_t* box1 = box0 + 2048;
     const bool store_pre = fp.maps && ep.epi == EPI_FWD_SILU && ep.pre;
-    const bool input = fp.maps && ep.epi == EPI_BWD_SILU;
+    const bool input = fp.maps && (ep.epi == EPI_BWD_SILU || wide);
+    HeadSums hs;   // EPI_HEAD_WIDE: this row's partial sums, row blocks finished
+    int nrow = 0;
     uint32_t in_par = 0;
     auto nch_of = [&](int tt) { return (min(BN, N - tn0(tt)) + 31) / 32; };
     auto fetch = [&](int tt, int cc) {   // pre-activation box of chunk cc of tile tt
@@ -380,13 +389,13 @@ __global__ void __launch_bounds__(kF8Threads, 1)
       mbar_expect_tx(&inbar[ew], 2048);
       tma_load_2d(box1, &em.pre, &inbar[ew], tn0(tt) + 32 * cc, tm0(tt) + q * 32);
     };
-    if (h < nch_of(blockIdx.x)) fetch(blockIdx.x, h);
+    if (tfirst < ntiles && h < nch_of(tfirst)) fetch(tfirst, h);
     float scA, invA;
     f8_scale(f8_amax_bits(fp.amax_a, fp.amax_a2), scA, invA);
     const float sab = scA * fp.sB;
     float amx = 0.0f;
     int lt = 0;
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++lt) {
+    for (int t = tfirst; t < ntiles; t = next(t), ++lt) {
       const int b = lt & 1, use = lt >> 1;
       if (!mbar_wait(&tfull[b], use & 1)) {
         if (lane == 0) atomicOr(fp.err, kErrTimeout);
@@ -400,6 +409,62 @@ __global__ void __launch_bounds__(kF8Threads, 1)
       const uint32_t base = tmem + (uint32_t)(b * COLS) + ((uint32_t)(q * 32) << 16);
       const int nch = nch_of(t);
       const float rs = (ep.rowscale && m < M) ? ep.rowscale[m] : 1.0f;
+      if constexpr (kWide) {
+        if (wide) {
+          if (n0 == 0) {
+            hs.clear();
+            if (!head_start(h, &hbar[q * 2 + 1], nrow)) {
+              if (lane == 0) atomicOr(fp.err, kErrTimeout);
+              *abort_flag = 1;
+            }
+          }
+          auto chunk = [&](int c, float (&d)[8]) {
+            float v[32];
+            uint32_t zw[16];
+            if (!mbar_wait(&inbar[ew], in_par)) {
+              if (lane == 0) atomicOr(fp.err, kErrTimeout);
+              *abort_flag = 1;
+            }
+            in_par ^= 1u;
+            ld_bf16_row_raw(box1, lane, zw);
+            fence_async_smem();
+            __syncwarp();
+            if (c + 2 < nch) fetch(t, c + 2);
+            else if (next(t) < ntiles && h < nch_of(next(t))) fetch(next(t), h);
+            tc_ld32(base + (uint32_t)(32 * c), v);
+            if (lane == 0) bulk_wait_read0();
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+              v[j] = head_elem(v[j] * sab, bf16_word_elem(zw, j), rs, d[j / 4]);
+              amx = fmaxf(amx, fabsf(v[j]));
+            }
+            st_bf16_row(box0, lane, v);
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+              tma_store_2d(&em.out, box0, n0 + 32 * c, m0 + q * 32);
+              bulk_commit();
+            }
+          };
+          for (int c = h; c < nch; c += 4) {
+            chunk(c, hs.d0);
+            if (c + 2 < nch) chunk(c + 2, hs.d1);
+          }
+          if (n0 + BN >= N) {
+            uint8_t* xbox = h ? box0 : box0 + 4 * kF8EpiSlot;
+            if (!head_finish(h, lane, hs, xbox, &hbar[q * 2], &hbar[q * 2 + 1], nrow, m < M ? ep.ubar + m : nullptr)) {
+              if (lane == 0) atomicOr(fp.err, kErrTimeout);
+              *abort_flag = 1;
+            }
+            ++nrow;
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&tempty[b]);
+          continue;
+        }
+      }
       for (int c = h; c < nch; c += 2) {
         float v[32];
         uint32_t zw[16];
@@ -414,7 +479,7 @@ __global__ void __launch_bounds__(kF8Threads, 1)
           fence_async_smem();
           __syncwarp();
           if (c + 2 < nch) fetch(t, c + 2);
-          else if (t + (int)gridDim.x < ntiles && h < nch_of(t + gridDim.x)) fetch(t + gridDim.x, h);
+          else if (next(t) < ntiles && h < nch_of(next(t))) fetch(next(t), h);
         }
         tc_ld32(base + (uint32_t)(32 * c), v);
 #pragma unroll
@@ -469,7 +534,7 @@ __global__ void __launch_bounds__(kF8Threads, 1)
     f8_scale(f8_amax_bits(fp.amax_a, fp.amax_a2), scA, invA);
     uint32_t g = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+    for (int t = tfirst; t < ntiles && ok; t = next(t)) {
       for (int kb = 0; kb < nk; ++kb, ++g) {
         const uint32_t s = g % kF8Stages, r = g / kF8Stages;
         if (*abort_flag || (g >= (uint32_t)kF8Stages && !mbar_wait(&empty[s], (r - 1) & 1))) {
@@ -586,7 +651,9 @@ static bool launch_fp8(const GemmArgs& g, const uint8_t* B8, int ldb8, float sB,
 bool gemm_tc_fp8(const GemmArgs& g, cudaStream_t st, int* d_err, std::string* why) {
   if (g.M <= 0 || g.N <= 0) return true;
   if (!gemm_tc_init(why)) return false;
-  if (!(g.epi == EPI_FWD_SILU || g.epi == EPI_F32 || g.epi == EPI_BWD_SILU || g.epi == EPI_LINEAR)) {
+  const bool wide_ok = g.epi == EPI_HEAD_WIDE && gemm_head_fits(ALLEGRO_PREC_FP8, g.N) && g.pre && g.ubar &&
+                       g.rowscale && !g.add && make_epi(g).vec;
+  if (!(g.epi == EPI_FWD_SILU || g.epi == EPI_F32 || g.epi == EPI_BWD_SILU || g.epi == EPI_LINEAR || wide_ok)) {
     if (why) *why = "FP8 GEMM: unsupported epilogue";
     return false;
   }

@@ -152,7 +152,7 @@ static TcLayout tc_layout(int epi, bool pre) {
   const bool wide_out = (epi == EPI_F32) || (epi == EPI_FWD_SILU && pre);
   L.out_box = wide_out ? 4096 : 2048;
   L.n_out = (EPQ == 2 && !PAIR) ? 2 : 1;
-  L.in_slot = (epi == EPI_BWD_SILU) ? 2048 : (epi == EPI_HEAD ? 4096 : 0);
+  L.in_slot = (epi == EPI_BWD_SILU || epi == EPI_HEAD_WIDE) ? 2048 : (epi == EPI_HEAD ? 4096 : 0);
   L.epi_slot = L.n_out * L.out_box + L.in_slot;
   const int epi_smem = 4 * EPQ * L.epi_slot;
   const int st = (kTcSmemMax - 1024 - (PAIR ? kTcMiscPair : kTcMisc) - epi_smem) / tc_stage_bytes<BN, PAIR>();
@@ -273,6 +273,11 @@ __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
   // A rows they share come from L2 after the first read
   auto tm0 = [&](int tt) { return (tt / tiles_n) * TM + (int)rank * kTcBM; };
   auto tn0 = [&](int tt) { return (tt % tiles_n) * BN; };
+  // EPI_HEAD_WIDE: a CTA (pair) takes whole row blocks, their column tiles one after another
+  constexpr bool kWide = BN == 256 && EPQ == 2;
+  const bool wide = kWide && ep.epi == EPI_HEAD_WIDE;
+  const int tfirst = wide ? t0 * tiles_n : t0;
+  auto next = [&](int tt) { return !wide ? tt + tstep : ((tt + 1) % tiles_n ? tt + 1 : tt + 1 + (tstep - 1) * tiles_n); };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -308,7 +313,7 @@ __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
   if (warp == 0) {
     if (lane == 0) {
       uint32_t g = 0;   // global k-block counter (ring position)
-      for (int t = t0; t < ntiles && !*abort_flag; t += tstep) {
+      for (int t = tfirst; t < ntiles && !*abort_flag; t = next(t)) {
         const int m0 = tm0(t), n0 = tn0(t);
         for (int kb = 0; kb < nk; ++kb, ++g) {
           const uint32_t s = g % STAGES, r = g / STAGES;
@@ -338,7 +343,7 @@ __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
       constexpr uint32_t idesc = idesc_bf16<BN, TM>();
       uint32_t g = 0;
       int lt = 0;
-      for (int t = t0; t < ntiles; t += tstep, ++lt) {
+      for (int t = tfirst; t < ntiles; t = next(t), ++lt) {
         const int b = lt & 1, use = lt >> 1;
         bool ok = !*abort_flag && mbar_wait(&tempty[b], (use & 1) ^ 1);
         if (ok) {
@@ -378,7 +383,7 @@ __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
     const int h = ew >> 2;             // 0..EPQ-1 within the quarter
     uint8_t* my_out = sE + ew * kEpiSlot;
     uint8_t* my_in = my_out + kNOut * lay.out_box;
-    const bool need_pre = (ep.epi == EPI_BWD_SILU || ep.epi == EPI_HEAD);
+    const bool need_pre = (ep.epi == EPI_BWD_SILU || ep.epi == EPI_HEAD || wide);
     const bool need_add = (ep.add != nullptr) && (ep.epi == EPI_HEAD);
     const uint32_t in_bytes = (need_pre ? 2048u : 0u) + (need_add ? 2048u : 0u);
     const bool out_f32 = (ep.epi == EPI_F32);
@@ -404,8 +409,10 @@ __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
     };
     int lt = 0;
     int oc = 0;                        // output chunks issued (buffer = oc % kNOut)
-    if (t0 < ntiles && h < nch_of(t0)) fetch(t0, h);
-    for (int t = t0; t < ntiles; t += tstep, ++lt) {
+    HeadSums hs;                       // EPI_HEAD_WIDE: this row's partial sums, row blocks finished
+    int nrow = 0;
+    if (tfirst < ntiles && h < nch_of(tfirst)) fetch(tfirst, h);
+    for (int t = tfirst; t < ntiles; t = next(t), ++lt) {
       const int b = lt & 1, use = lt >> 1;
       const bool ok = mbar_wait(&tfull[b], use & 1);
       if (!ok) {
@@ -424,6 +431,70 @@ __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
       float acc1 = 0.0f;
       const uint32_t base = tmem + (uint32_t)(b * COLS) + ((uint32_t)(q * 32) << 16);
       const int nch = nch_of(t);
+      if constexpr (kWide) {
+        if (wide) {
+          if (n0 == 0) {
+            hs.clear();
+            if (!head_start(h, &rsbar[q * 2 + 1], nrow)) {
+              if (lane == 0) atomicOr(err, kErrTimeout);
+              *abort_flag = 1;
+            }
+          }
+          auto chunk = [&](int c, float (&d)[8]) {
+            uint8_t* ob = my_out + (oc % kNOut) * lay.out_box;
+            uint32_t zw[16];
+            if (!mbar_wait(&inbar[ew], in_par)) {
+              if (lane == 0) atomicOr(err, kErrTimeout);
+              *abort_flag = 1;
+            }
+            in_par ^= 1u;
+            ld_bf16_row_raw(my_in, lane, zw);
+            fence_async_smem();
+            __syncwarp();
+            if (c + 2 < nch) fetch(t, c + 2);
+            else if (next(t) < ntiles && h < nch_of(next(t))) fetch(next(t), h);
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh) {
+              float v[16];
+              tc_ld16(base + (uint32_t)(32 * c + 16 * hh), v);
+#pragma unroll
+              for (int j = 0; j < 16; ++j)
+                v[j] = head_elem(v[j], bf16_word_elem(zw, 16 * hh + j), rs, d[(16 * hh + j) / 4]);
+              if (hh == 0) {
+                if (lane == 0) {
+                  if (kNOut == 1) bulk_wait_read0();
+                  else bulk_wait_read1();
+                }
+                __syncwarp();
+              }
+              st_bf16_half(ob, lane, hh, v);
+            }
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+              tma_store_2d(&em.out, ob, n0 + 32 * c, mrow);
+              bulk_commit();
+            }
+            ++oc;
+          };
+          for (int c = h; c < nch; c += 4) {
+            chunk(c, hs.d0);
+            if (c + 2 < nch) chunk(c + 2, hs.d1);
+          }
+          if (n0 + BN >= N) {
+            uint8_t* xbox = h ? my_out : my_out + 4 * kEpiSlot;
+            if (!head_finish(h, lane, hs, xbox, &rsbar[q * 2], &rsbar[q * 2 + 1], nrow, live ? ep.ubar + m : nullptr)) {
+              if (lane == 0) atomicOr(err, kErrTimeout);
+              *abort_flag = 1;
+            }
+            ++nrow;
+          }
+          tc_fence_before();
+          __syncwarp();
+          release(b);
+          continue;
+        }
+      }
       for (int c = h; c < nch; c += EPQ) {
         uint8_t* ob = my_out + (oc % kNOut) * lay.out_box;
         // inputs of this chunk, kept as packed bf16 words
@@ -441,7 +512,7 @@ __global__ void __launch_bounds__(tc_threads<EPQ>(), 1)
           __syncwarp();
           // prefetch this warp's next chunk (possibly in its next tile)
           if (c + EPQ < nch) fetch(t, c + EPQ);
-          else if (t + tstep < ntiles && h < nch_of(t + tstep)) fetch(t + tstep, h);
+          else if (next(t) < ntiles && h < nch_of(next(t))) fetch(next(t), h);
         }
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
@@ -1162,6 +1233,29 @@ static bool launch_bn(const GemmArgs& g, const bf16* B, int ldb, cudaStream_t st
   return true;
 }
 
+bool gemm_head_fits(int prec, int N) {
+  // whole tiles (the bf16 path takes rows of one tile by EPI_HEAD)
+  if (prec == ALLEGRO_PREC_BF16) return N % 256 == 0 && N > 256;
+  if (prec == ALLEGRO_PREC_FP8) return N % 256 == 0;
+  return prec == ALLEGRO_PREC_TF32 && N % 128 == 0;
+}
+
+// A CTA that sums over a row runs the row block's column tiles one after another, which costs the
+// waves that the last row blocks leave SMs idle in; the separate form costs a launch and the float32
+// xbar written and read (8 B per element, from L2 while it fits).  Waves (row blocks whole / tiles
+// dealt out) and us per step, separate / fused: 1024 columns bf16, 45 row blocks 4 / 2 waves 653 / 685;
+// 82 4 / 3 797 / 808; 132 4 / 4 942 / 921; 353 12 / 10 1,864 / 1,838; 703 20 / 19 3,181 / 3,072.  512
+// columns: 175 4 / 3 1,000 / 1,010 (fp8 1,083 / 1,108); 290 4 / 4 1,293 / 1,239; 784 12 / 11 2,758 / 2,654
+// (fp8 2,947 / 2,859).  TF32: 256 columns, 137 2 / 2 527 / 537; 333 6 / 5 811 / 814; 486 8 / 7 1,043 / 1,031;
+// 962 14 / 13 1,694 / 1,640; 1024 columns, 225 16 / 12 2,283 / 2,287; 703 40 / 37 6,229 / 6,128.
+bool gemm_head_wide(int prec, int64_t M, int N) {
+  if (!gemm_head_fits(prec, N)) return false;
+  const bool tf32 = prec == ALLEGRO_PREC_TF32;
+  const int64_t nsm = num_sms(current_device()), rb = (M + 127) / 128, tn = N / (tf32 ? 128 : 256);
+  const int64_t whole = (rb + nsm - 1) / nsm * tn, dealt = (rb * tn + nsm - 1) / nsm;
+  return tf32 ? rb >= nsm && 7 * whole <= 8 * dealt : 4 * whole <= 5 * dealt;
+}
+
 bool gemm_tc_bf16(const GemmArgs& g, cudaStream_t st, int* d_err, std::string* why) {
   if (g.M <= 0 || g.N <= 0) return true;
   if (!gemm_tc_init(why)) return false;
@@ -1179,6 +1273,10 @@ bool gemm_tc_bf16(const GemmArgs& g, cudaStream_t st, int* d_err, std::string* w
     return false;
   }
   const int tiles = (g.N + 255) / 256;
+  if (g.epi == EPI_HEAD_WIDE && !(gemm_head_fits(ALLEGRO_PREC_BF16, g.N) && g.pre && g.ubar && g.rowscale)) {
+    if (why) *why = "wide head epilogues need whole 256-column tiles";
+    return false;
+  }
   if ((g.epi == EPI_HEAD || g.epi == EPI_LAST) && tiles != 1) {
     if (why) *why = "fused head epilogues need N <= 256";
     return false;
@@ -1419,7 +1517,8 @@ __global__ void __launch_bounds__(kT32Threads, 1)
   uint64_t* tfull = empty + STAGES;   // [2]
   uint64_t* tempty = tfull + 2;       // [2]
   uint64_t* inbar = tempty + 2;       // [kT32EpiWarps]: input box filled
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(inbar + kT32EpiWarps);
+  uint64_t* hbar = inbar + kT32EpiWarps;   // [4 quarters][2]: EPI_HEAD_WIDE partial sums ready / used
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(hbar + 8);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1428,6 +1527,11 @@ __global__ void __launch_bounds__(kT32Threads, 1)
   const int ntiles = tiles_m * tiles_n;
   auto tm0 = [&](int tt) { return (tt / tiles_n) * 128; };
   auto tn0 = [&](int tt) { return (tt % tiles_n) * BN; };
+  // EPI_HEAD_WIDE: a CTA takes whole row blocks, their column tiles one after another
+  constexpr bool kWide = BN == 128;
+  const bool wide = kWide && ep.epi == EPI_HEAD_WIDE;
+  const int tstep = gridDim.x, tfirst = wide ? (int)blockIdx.x * tiles_n : (int)blockIdx.x;
+  auto next = [&](int tt) { return !wide ? tt + tstep : ((tt + 1) % tiles_n ? tt + 1 : tt + 1 + (tstep - 1) * tiles_n); };
 
   if (threadIdx.x == 0) {
     for (int q = 0; q < STAGES; ++q) {
@@ -1439,6 +1543,7 @@ __global__ void __launch_bounds__(kT32Threads, 1)
       mbar_init(&tempty[b], kT32EpiWarps);
     }
     for (int w = 0; w < kT32EpiWarps; ++w) mbar_init(&inbar[w], 1);
+    for (int w = 0; w < 8; ++w) mbar_init(&hbar[w], 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -1456,7 +1561,7 @@ __global__ void __launch_bounds__(kT32Threads, 1)
   if (warp == 0) {
     if (lane == 0) {
       uint32_t g = 0;
-      for (int t = blockIdx.x; t < ntiles && !*abort_flag; t += gridDim.x) {
+      for (int t = tfirst; t < ntiles && !*abort_flag; t = next(t)) {
         const int m0 = tm0(t), n0 = tn0(t);
         for (int kb = 0; kb < nk; ++kb, ++g) {
           const uint32_t q = g % STAGES, r = g / STAGES;
@@ -1476,7 +1581,7 @@ __global__ void __launch_bounds__(kT32Threads, 1)
       constexpr uint32_t idesc = idesc_tf32<BN>();
       uint32_t g = 0;
       int lt = 0;
-      for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++lt) {
+      for (int t = tfirst; t < ntiles; t = next(t), ++lt) {
         const int b = lt & 1, use = lt >> 1;
         bool ok = !*abort_flag && mbar_wait(&tempty[b], (use & 1) ^ 1);
         if (ok) {
@@ -1510,22 +1615,29 @@ __global__ void __launch_bounds__(kT32Threads, 1)
     const int q = warp & 3;        // TMEM lane quarter this warp may access
     const int ew = warp - 2;
     const int h = ew >> 2;         // 0 or 1: alternating 32-column chunks
-    // staging: the output box, then the pre-activation box (stored) or the input box (fetched)
+    // staging: the output box, then the pre-activation box (stored) or the input box (fetched), and
+    // for the head a third box for its addend
     uint8_t* box0 = sE + ew * epi_slot;
     uint8_t* box1 = box0 + kT32Box;
+    uint8_t* box2 = box1 + kT32Box;
+    const bool head_add = wide && ep.add;
+    HeadSums hs;   // EPI_HEAD_WIDE: this row's partial sums, row blocks finished
+    int nrow = 0;
     const bool maps = epi_slot != 0;   // else every access by the lanes themselves
     const bool store_pre = maps && ep.epi == EPI_FWD_SILU && ep.pre;
-    const bool input = maps && (ep.epi == EPI_BWD_SILU || (ep.epi == EPI_F32 && ep.add));
+    const bool input = maps && (ep.epi == EPI_BWD_SILU || wide || (ep.epi == EPI_F32 && ep.add));
     uint32_t in_par = 0;
     auto nch_of = [&](int tt) { return (min(BN, N - tn0(tt)) + 31) / 32; };
     auto fetch = [&](int tt, int cc) {   // input box of chunk cc of tile tt
       if (!input || lane != 0) return;
-      mbar_expect_tx(&inbar[ew], kT32Box);
-      tma_load_2d(box1, ep.epi == EPI_BWD_SILU ? &em.pre : &em.add, &inbar[ew], tn0(tt) + 32 * cc, tm0(tt) + q * 32);
+      const int nb = tn0(tt) + 32 * cc, mb = tm0(tt) + q * 32;
+      mbar_expect_tx(&inbar[ew], head_add ? 2 * kT32Box : kT32Box);
+      tma_load_2d(box1, ep.epi == EPI_F32 ? &em.add : &em.pre, &inbar[ew], nb, mb);
+      if (head_add) tma_load_2d(box2, &em.add, &inbar[ew], nb, mb);
     };
-    if (h < nch_of(blockIdx.x)) fetch(blockIdx.x, h);
+    if (tfirst < ntiles && h < nch_of(tfirst)) fetch(tfirst, h);
     int lt = 0;
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++lt) {
+    for (int t = tfirst; t < ntiles; t = next(t), ++lt) {
       const int b = lt & 1, use = lt >> 1;
       if (!mbar_wait(&tfull[b], use & 1)) {
         if (lane == 0) atomicOr(err, kErrTimeout);
@@ -1539,6 +1651,63 @@ __global__ void __launch_bounds__(kT32Threads, 1)
       const uint32_t base = tmem + (uint32_t)(b * COLS) + ((uint32_t)(q * 32) << 16);
       const int nch = nch_of(t);
       const float rs = (ep.rowscale && m < M) ? ep.rowscale[m] : 1.0f;
+      if constexpr (kWide) {
+        if (wide) {
+          if (n0 == 0) {
+            hs.clear();
+            if (!head_start(h, &hbar[q * 2 + 1], nrow)) {
+              if (lane == 0) atomicOr(err, kErrTimeout);
+              *abort_flag = 1;
+            }
+          }
+          auto chunk = [&](int c, float (&d)[8]) {
+            float v[32], z[32];
+            if (!mbar_wait(&inbar[ew], in_par)) {
+              if (lane == 0) atomicOr(err, kErrTimeout);
+              *abort_flag = 1;
+            }
+            in_par ^= 1u;
+            tc_ld32(base + (uint32_t)(32 * c), v);
+            if (head_add) {
+              ld_f32_row(box2, lane, z);
+#pragma unroll
+              for (int j = 0; j < 32; ++j) v[j] += z[j];
+            }
+            ld_f32_row(box1, lane, z);
+            fence_async_smem();
+            __syncwarp();
+            if (c + 2 < nch) fetch(t, c + 2);
+            else if (next(t) < ntiles && h < nch_of(next(t))) fetch(next(t), h);
+            if (lane == 0) bulk_wait_read0();
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] = head_elem(v[j], z[j], rs, d[j / 4]);
+            st_f32_row(box0, lane, v);
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+              tma_store_2d(&em.out, box0, n0 + 32 * c, m0 + q * 32);
+              bulk_commit();
+            }
+          };
+          for (int c = h; c < nch; c += 4) {
+            chunk(c, hs.d0);
+            if (c + 2 < nch) chunk(c + 2, hs.d1);
+          }
+          if (n0 + BN >= N) {
+            uint8_t* xbox = h ? box0 : box0 + 4 * epi_slot;
+            if (!head_finish(h, lane, hs, xbox, &hbar[q * 2], &hbar[q * 2 + 1], nrow, m < M ? ep.ubar + m : nullptr)) {
+              if (lane == 0) atomicOr(err, kErrTimeout);
+              *abort_flag = 1;
+            }
+            ++nrow;
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&tempty[b]);
+          continue;
+        }
+      }
       for (int c = h; c < nch; c += 2) {
         float v[32], z[32];
         if (input) {
@@ -1552,7 +1721,7 @@ __global__ void __launch_bounds__(kT32Threads, 1)
           fence_async_smem();
           __syncwarp();
           if (c + 2 < nch) fetch(t, c + 2);
-          else if (t + (int)gridDim.x < ntiles && h < nch_of(t + gridDim.x)) fetch(t + gridDim.x, h);
+          else if (next(t) < ntiles && h < nch_of(next(t))) fetch(next(t), h);
         }
         tc_ld32(base + (uint32_t)(32 * c), v);
         if (!maps) {
@@ -1636,8 +1805,9 @@ static bool launch_tf32(const GemmArgs& g, const float* B, int ldb, cudaStream_t
   memset(&em, 0, sizeof em);
   int epi_slot = 0;
   if (ep.vec) {
-    const bool pre = g.pre && g.epi != EPI_F32 && g.epi != EPI_LINEAR, add = g.add && g.epi == EPI_F32;
-    epi_slot = (pre || add) ? 2 * kT32Box : kT32Box;
+    const bool wide = g.epi == EPI_HEAD_WIDE;
+    const bool pre = g.pre && g.epi != EPI_F32 && g.epi != EPI_LINEAR, add = g.add && (g.epi == EPI_F32 || wide);
+    epi_slot = (1 + (pre ? 1 : 0) + (add ? 1 : 0)) * kT32Box;
     if (!tc_box_map(&em.out, g.out, g.N, g.M, g.ldo, 4) || (pre && !tc_box_map(&em.pre, g.pre, g.N, g.M, g.ldp, 4)) ||
         (add && !tc_box_map(&em.add, g.add, g.N, g.M, g.ld_add, 4))) {
       if (why) *why = "cuTensorMapEncodeTiled failed (tf32 epilogue)";
@@ -1654,8 +1824,13 @@ bool gemm_tc_tf32(const GemmArgs& g, cudaStream_t st, int* d_err, std::string* w
   if (g.M <= 0 || g.N <= 0) return true;
   if (!gemm_tc_init(why)) return false;
   if (g.A2 || g.Bover || g.b_row0 || !(g.epi == EPI_FWD_SILU || g.epi == EPI_F32 || g.epi == EPI_BWD_SILU ||
-                                       g.epi == EPI_LINEAR)) {
+                                       g.epi == EPI_LINEAR || g.epi == EPI_HEAD_WIDE)) {
     if (why) *why = "tf32 GEMM: unsupported operand form or epilogue";
+    return false;
+  }
+  if (g.epi == EPI_HEAD_WIDE &&
+      !(gemm_head_fits(ALLEGRO_PREC_TF32, g.N) && g.pre && g.ubar && g.rowscale && make_epi(g).vec)) {
+    if (why) *why = "wide head epilogues need whole 128-column tiles and 16-byte rows";
     return false;
   }
   const float* B = g.trans ? g.W->f32T : g.W->f32;
@@ -1668,6 +1843,7 @@ bool gemm_tc_tf32(const GemmArgs& g, cudaStream_t st, int* d_err, std::string* w
   const int tiles = (g.N + 255) / 256;
   int bn = (g.N + tiles - 1) / tiles;
   bn = (bn + 31) / 32 * 32;
+  if (g.epi == EPI_HEAD_WIDE) bn = 128;   // (three boxes per epilogue warp: four stages beside 128 columns)
   switch (bn) {
     case 32: return launch_tf32<32>(g, B, ldb, st, d_err, why);
     case 64: return launch_tf32<64>(g, B, ldb, st, d_err, why);

@@ -116,6 +116,9 @@ enum Epi : int {
   // out = sigma_m v u silu'(z)  (the gradient w.r.t. z, input of the adjoint GEMMs).
   EPI_LAST = 4,
   EPI_LINEAR = 5,     // out = acc in the activation type (bf16 on the BF16 path)
+  // EPI_HEAD for rows of several column tiles (tcgen05 paths), the operations and the order of the row
+  // sum those of head_bwd_kernel: xbar = acc (+ add); out = xbar u silu'(z); ubar[m] += sum_n xbar_n silu(z_n)
+  EPI_HEAD_WIDE = 6,
 };
 
 struct GemmArgs {
@@ -158,6 +161,9 @@ bool gemm_chain_bf16(const GemmArgs& g1, const GemmArgs& g2, cudaStream_t st, in
 // E4M3 operands with per-tensor scales read by tcgen05 kind::f8f6f4 (bf16 activations converted on
 // chip), float32 accumulation, bf16 / float32 epilogues (FWD_SILU, F32, BWD_SILU, LINEAR)
 bool gemm_tc_fp8(const GemmArgs& g, cudaStream_t st, int* d_err, std::string* why);
+// whether `prec`'s tcgen05 path has EPI_HEAD_WIDE for N columns, and whether it is the faster form for M rows
+bool gemm_head_fits(int prec, int N);
+bool gemm_head_wide(int prec, int64_t M, int N);
 // dst[r][k] = e4m3(src[r][k] * inv_scale) for k < cols, 0 for cols <= k < ldd (rows x ldd bytes)
 void fp8_quantize(const float* src, int rows, int cols, int lds, uint8_t* dst, int ldd, float inv_scale,
                   cudaStream_t st);
