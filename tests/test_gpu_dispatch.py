@@ -13,6 +13,7 @@ import pytest
 from gpu_util import BF16_F_RMS, FP32_E, FP32_F, FP32_W, assert_same_edges, errors, lib_model
 from oracle.allegro import AllegroOracle
 from oracle.neighbors import neighbor_list
+from paper_2304_10061_gb300 import AllegroError
 from synth import ARCHS, Arch, lattice_box, make_weights, weights_to_blob
 
 pytestmark = pytest.mark.gpu
@@ -114,11 +115,12 @@ def test_atom_sums(model, n, zbl):
 
 
 # widths: no multiple of four, eight or thirty-two; several column tiles, whole and ragged; the generic
-# row path.  900 atoms: enough tiles for CTA pairs, a ragged last row block; chunks of 2500 edges: too few
+# row path.  1500 atoms: enough tiles for CTA pairs, and row blocks in whole waves for the head epilogues of
+# wide rows, the last block ragged; chunks of 2500 edges: too few for either
 WIDTHS = {
     "odd": Arch(n_species=2, lmax=1, n_layers=2, channels=16, two_body=(18, 37), latent=(45, 33), edge=(7,)),
     "ragged_tiles": Arch(n_species=2, lmax=1, n_layers=2, channels=64, two_body=(60, 520), latent=(392, 328), edge=(12,)),
-    "whole_tiles": Arch(n_species=2, lmax=1, n_layers=2, channels=64, two_body=(96, 512), latent=(512, 768), edge=()),
+    "whole_tiles": Arch(n_species=2, lmax=1, n_layers=2, channels=64, two_body=(96, 512), latent=(768, 768), edge=()),
     "generic_whole_tiles": Arch(n_species=2, lmax=2, n_layers=3, channels=64, two_body=(64, 512), latent=(512,), edge=(16,)),
     "generic_128": Arch(n_species=2, lmax=2, n_layers=3, channels=32, two_body=(40, 128), latent=(128,), edge=()),
     "basis_12": Arch(n_species=2, lmax=2, n_layers=1, channels=8, two_body=(19, 32), latent=(32,), edge=(), n_bessel=12),
@@ -131,7 +133,7 @@ def _reference(name):
     if name not in _REF:
         arch = WIDTHS[name]
         w = make_weights(arch, 21)
-        s = lattice_box(900 if "tiles" in name else 330, ((900 if "tiles" in name else 330) / 0.1) ** (1 / 3), seed=17)
+        s = _box(1500 if "tiles" in name else 330, seed=17)
         s.species = s.species % 2
         i, j, S = neighbor_list(s.pos, s.cell, s.pbc, arch.r_c)
         _REF[name] = (arch, w, s, AllegroOracle(arch, w).energy_forces(s.pos, s.species, s.cell, i, j, S))
@@ -142,6 +144,14 @@ def _reference(name):
 @pytest.mark.parametrize("name", list(WIDTHS))
 def test_mlp_widths(name, prec):
     arch, w, s, (E0, Ea0, F0, W0) = _reference(name)
+    if (name, prec) == ("odd", "bf16"):
+        # [x | s] with s at an odd column: no TMA box starts there, the call is refused
+        m = lib_model(weights_to_blob(arch, w), precision=prec)
+        m.neighbors(s.pos, s.species, s.cell)
+        with pytest.raises(AllegroError):
+            m.energy_forces()
+        m.close()
+        return
     runs = []
     for chunk in (0, 2500):
         m = lib_model(weights_to_blob(arch, w), precision=prec)
