@@ -568,9 +568,9 @@ void nb_sort_cells(const double* pos, const int* species, const CellGrid& g, int
 // edge's image shift is S = q - w_j + w_i).
 constexpr int kSearchThreads = 128;
 // Up to this many atoms a warp per centre, above it a thread per centre (both list the same edges in
-// the same order).  Count and fill pass, us, warp / thread: 64 atoms 13 + 13 / 37 + 77; 3,072 atoms
-// 19 + 22 / 81 + 124; 23,552 atoms 49 + 79 / 81 + 143; 65,536 atoms 104 + 196 / 93 + 212; 1,048,576 atoms
-// 1,553 + 3,298 / 804 + 2,517 (the warp form issues more instructions per candidate).
+// the same order).  Count and fill pass, us, warp / thread: 64 atoms 11 + 12 / 37 + 77; 3,072 atoms
+// 17 + 18 / 81 + 124; 23,552 atoms 44 + 53 / 81 + 143; 65,536 atoms 89 + 124 / 93 + 212; 1,048,576 atoms
+// 1,553 + 3,298 / 518 + 2,426 (the warp form issues more instructions per candidate).
 constexpr int kSearchWarpAtoms = 65536;
 
 // image q (three signed 10-bit fields) and the exact-test flag of a staged edge

@@ -31,7 +31,7 @@
 // Ybar / w^0bar.  With this layout and the asynchronous rings below, all row
 // kernels of the forward pass take 4.37 ms (7.18 with the channel outside and
 // loads through registers) and of the adjoint 10.3 ms (14.8) at 65,536 atoms,
-// three layers, l_max 3, 128 channels in bf16.
+// three layers, l_max 3, 128 channels in bf16 (with what the kernels' own comments name, less now).
 // Row kernels: one warp per centre atom with C / 32 channels per lane (the
 // environment sums, s, Qbar, the upper layers' wbar: a lane's harmonics loads
 // serve all its channels), or, for the per-edge adjoint that combines every
@@ -625,36 +625,93 @@ __device__ __forceinline__ bool gen_lane(const GenRowIO& io, GenLane& g) {
   return true;
 }
 
+// An edge's row of w (C LM values, in 16-byte pieces: the rows' pitches and first columns are multiples of
+// 8 elements) and its harmonics, each written twice so that a 16-byte read gives two (y, y) operands of the
+// packed multiply-adds.  The lane's piece addresses are kept and moved on by a row per edge; copies are
+// queued for consecutive edges from rb.
+template <typename T, int CPL, int LM, int S>
+struct GenRow {
+  static constexpr int kW = 32 * CPL * LM * (int)sizeof(T);   // bytes of w
+  static constexpr int kY = (S + 1) / 2 * 16;                 // bytes of the doubled harmonics
+  static constexpr int kN = (kW + 511) / 512;
+  const unsigned char* wp;
+  const float* yp;
+  int pitch, pieces, lane;
+  __device__ __forceinline__ GenRow(const T* w, int ld, int row_bytes, const float* Y, int rb, int ln) {
+    lane = ln;
+    pitch = ld * (int)sizeof(T);
+    pieces = row_bytes / 16;
+    wp = reinterpret_cast<const unsigned char*>(w) + (size_t)rb * pitch + lane * 16;
+    yp = Y + (size_t)rb * S + lane / 2;
+  }
+  __device__ __forceinline__ void copy_w(unsigned char* st) {
+#pragma unroll
+    for (int k = 0; k < kN; ++k)
+      if (lane + 32 * k < pieces) cp_async16(st + (lane + 32 * k) * 16, wp + 512 * k);
+    wp += pitch;
+  }
+  __device__ __forceinline__ void copy_y(unsigned char* st) {
+    if (lane < 2 * S) cp_async4(st + lane * 4, yp);
+    yp += S;
+  }
+};
+// the doubled harmonics of a stage
+template <int S>
+__device__ __forceinline__ void load_yy(const unsigned char* st, float2 (&y)[(S + 1) / 2 * 2]) {
+#pragma unroll
+  for (int k = 0; k < (S + 1) / 2; ++k) {
+    const float4 v = *reinterpret_cast<const float4*>(st + 16 * k);
+    y[2 * k] = make_float2(v.x, v.y);
+    y[2 * k + 1] = make_float2(v.z, v.w);
+  }
+}
+// the LM weights of the channel pair (lane + 64 p, lane + 64 p + 32); a lane's only channel pairs with zeros
+template <typename T, int CPL, int LM>
+__device__ __forceinline__ void load_pair(const unsigned char* st, int lane, int p, float2 (&w)[LM]) {
+  const T* ws = reinterpret_cast<const T*>(st);
+  float a[LM], b[LM] = {};
+  load_lm<T, LM>(ws + (lane + 64 * p) * LM, a);
+  if constexpr (CPL > 1) load_lm<T, LM>(ws + (lane + 64 * p + 32) * LM, b);
+#pragma unroll
+  for (int l = 0; l < LM; ++l) w[l] = make_float2(a[l], b[l]);
+}
+
+// The per-edge loops run on channel pairs in packed fp32 (two IEEE operations per instruction).
+// Bound: HBM (84 to 90 % of the copy rate for the sums, s and Qbar; wbar 75 %).  12,000 atoms, 3 layers,
+// l_max 3, 128 channels in bf16, us, scalar arithmetic with addresses formed per edge / now: Gamma 77 / 69,
+// s 106 / 84, Qbar 88 / 80, wbar 70 / 70 (instructions per edge 203 / 150, 281 / 172, 234 / 175, 151 / 111);
+// 65,536 atoms 34.10 / 33.56 ms per step.
+
 // Gamma^L[i][u][b] = nu sum_{e in row i} w^L[e][u][l(b)] Y[e][b]
 template <typename T, int LMAX, int CPL>
 __global__ void __launch_bounds__(32 * kGenWarps) gen_env_w_kernel(GenRowIO io, int L) {
   pdl_wait();
-  constexpr int S = (LMAX + 1) * (LMAX + 1), LM = LMAX + 1;
-  constexpr int kW = 32 * CPL * LM * (int)sizeof(T), kStage = round16(kW + S * 4);
+  constexpr int S = (LMAX + 1) * (LMAX + 1), LM = LMAX + 1, NP = (CPL + 1) / 2;
+  using Row = GenRow<T, CPL, LM, S>;
+  constexpr int kStage = Row::kW + Row::kY;
   __shared__ __align__(16) unsigned char rings[kGenWarps][kRing * kStage];
   GenLane g;
   if (!gen_lane<CPL>(io, g)) return;
-  const T* __restrict__ w = reinterpret_cast<const T*>(io.w[L]) + io.wcol[L];
-  const int ldw = io.ldw[L], row_bytes = io.C * LM * (int)sizeof(T);
-  float G[CPL][S];
+  Row row(reinterpret_cast<const T*>(io.w[L]) + io.wcol[L], io.ldw[L], io.C * LM * (int)sizeof(T), io.Y, g.rb, g.lane);
+  float2 G[NP][S];
 #pragma unroll
-  for (int c = 0; c < CPL; ++c)
+  for (int p = 0; p < NP; ++p)
 #pragma unroll
-    for (int b = 0; b < S; ++b) G[c][b] = 0.0f;
-  auto copy = [&](int e, unsigned char* st) {
-    warp_copy(st, reinterpret_cast<const unsigned char*>(w + (size_t)e * ldw), row_bytes, 0);
-    if (g.lane < S) cp_async4(st + kW + g.lane * 4, io.Y + (size_t)e * S + g.lane);
+    for (int b = 0; b < S; ++b) G[p][b] = make_float2(0.0f, 0.0f);
+  auto copy = [&](int, unsigned char* st) {
+    row.copy_w(st);
+    row.copy_y(st + Row::kW);
   };
   ring_over<kRing, kStage>(rings[threadIdx.x >> 5], g.rb, g.re, copy, [&](int, const unsigned char* st) {
     if (!g.act) return;
-    float y[S];
-    load_y<S>(reinterpret_cast<const float*>(st + kW), y);
+    float2 y[(S + 1) / 2 * 2];
+    load_yy<S>(st + Row::kW, y);
 #pragma unroll
-    for (int c = 0; c < CPL; ++c) {
-      float wl[LM];
-      load_lm<T, LM>(reinterpret_cast<const T*>(st) + (g.lane + 32 * c) * LM, wl);
+    for (int p = 0; p < NP; ++p) {
+      float2 w[LM];
+      load_pair<T, CPL, LM>(st, g.lane, p, w);
 #pragma unroll
-      for (int b = 0; b < S; ++b) G[c][b] = fmaf(wl[l_of(b)], y[b], G[c][b]);
+      for (int b = 0; b < S; ++b) G[p][b] = __ffma2_rn(w[l_of(b)], y[b], G[p][b]);
     }
   });
   if (!g.act) return;
@@ -662,46 +719,50 @@ __global__ void __launch_bounds__(32 * kGenWarps) gen_env_w_kernel(GenRowIO io, 
 #pragma unroll
   for (int c = 0; c < CPL; ++c)
 #pragma unroll
-    for (int b = 0; b < S; ++b) out[(size_t)b * io.C + 32 * c] = G[c][b] * io.nu;
+    for (int b = 0; b < S; ++b) out[(size_t)b * io.C + 32 * c] = ((c & 1) ? G[c / 2][b].y : G[c / 2][b].x) * io.nu;
 }
 
 // s^L_e[u] = sum_a w^0_{e,u,l(a)} Y_e[a] Q^L[i][u][a], into the s columns of the latent input
 template <typename T, int LMAX, int CPL>
 __global__ void __launch_bounds__(32 * kGenWarps) gen_s_w_kernel(GenRowIO io, int L) {
   pdl_wait();
-  constexpr int S = (LMAX + 1) * (LMAX + 1), LM = LMAX + 1;
-  constexpr int kW = 32 * CPL * LM * (int)sizeof(T), kStage = round16(kW + S * 4);
+  constexpr int S = (LMAX + 1) * (LMAX + 1), LM = LMAX + 1, NP = (CPL + 1) / 2;
+  using Row = GenRow<T, CPL, LM, S>;
+  constexpr int kStage = Row::kW + Row::kY;
   __shared__ __align__(16) unsigned char rings[kGenWarps][kRing * kStage];
   GenLane g;
   if (!gen_lane<CPL>(io, g)) return;
-  const T* __restrict__ w0 = reinterpret_cast<const T*>(io.w[0]) + io.wcol[0];
-  float q[CPL][S];
+  Row row(reinterpret_cast<const T*>(io.w[0]) + io.wcol[0], io.ldw[0], io.C * LM * (int)sizeof(T), io.Y, g.rb, g.lane);
+  float2 q[NP][S];
   const float* Q = io.Q[L] + (size_t)g.ia * S * io.C + (g.act ? g.lane : 0);
 #pragma unroll
-  for (int c = 0; c < CPL; ++c)
+  for (int p = 0; p < NP; ++p)
 #pragma unroll
-    for (int a = 0; a < S; ++a) q[c][a] = Q[(size_t)a * io.C + 32 * c];
-  T* __restrict__ xs = reinterpret_cast<T*>(io.xs[L]) + io.xs_off[L] + g.lane;
-  const int ldw0 = io.ldw[0], ldxs = io.ldxs[L], row_bytes = io.C * LM * (int)sizeof(T);
+    for (int a = 0; a < S; ++a)
+      q[p][a] = make_float2(Q[(size_t)a * io.C + 64 * p], CPL > 1 ? Q[(size_t)a * io.C + 64 * p + 32] : 0.0f);
+  T* __restrict__ xs = reinterpret_cast<T*>(io.xs[L]) + io.xs_off[L] + g.lane + (size_t)g.rb * io.ldxs[L];
+  const int ldxs = io.ldxs[L];
+  const bool amax = io.amax_s != nullptr;
   float smax = 0.0f;
-  auto copy = [&](int e, unsigned char* st) {
-    warp_copy(st, reinterpret_cast<const unsigned char*>(w0 + (size_t)e * ldw0), row_bytes, 0);
-    if (g.lane < S) cp_async4(st + kW + g.lane * 4, io.Y + (size_t)e * S + g.lane);
+  auto copy = [&](int, unsigned char* st) {
+    row.copy_w(st);
+    row.copy_y(st + Row::kW);
   };
-  ring_over<kRing, kStage>(rings[threadIdx.x >> 5], g.rb, g.re, copy, [&](int e, const unsigned char* st) {
+  ring_over<kRing, kStage>(rings[threadIdx.x >> 5], g.rb, g.re, copy, [&](int, const unsigned char* st) {
     if (!g.act) return;
-    float y[S];
-    load_y<S>(reinterpret_cast<const float*>(st + kW), y);
+    float2 y[(S + 1) / 2 * 2];
+    load_yy<S>(st + Row::kW, y);
 #pragma unroll
-    for (int c = 0; c < CPL; ++c) {
-      float wl[LM];
-      load_lm<T, LM>(reinterpret_cast<const T*>(st) + (g.lane + 32 * c) * LM, wl);
-      float sv = 0.0f;
+    for (int p = 0; p < NP; ++p) {
+      float2 w[LM], sv = make_float2(0.0f, 0.0f);
+      load_pair<T, CPL, LM>(st, g.lane, p, w);
 #pragma unroll
-      for (int a = 0; a < S; ++a) sv = fmaf(wl[l_of(a)] * y[a], q[c][a], sv);
-      smax = fmaxf(smax, fabsf(sv));
-      gst(xs + (size_t)e * ldxs + 32 * c, sv);
+      for (int a = 0; a < S; ++a) sv = __ffma2_rn(__fmul2_rn(w[l_of(a)], y[a]), q[p][a], sv);
+      if (amax) smax = fmaxf(smax, fmaxf(fabsf(sv.x), fabsf(sv.y)));
+      gst(xs + 64 * p, sv.x);
+      if constexpr (CPL > 1) gst(xs + 64 * p + 32, sv.y);
     }
+    xs += ldxs;
   });
   record_amax(io.amax_s, smax);
 }
@@ -710,37 +771,46 @@ __global__ void __launch_bounds__(32 * kGenWarps) gen_s_w_kernel(GenRowIO io, in
 template <typename T, int LMAX, int CPL>
 __global__ void __launch_bounds__(32 * kGenWarps) gen_qbar_w_kernel(GenRowIO io, int L) {
   pdl_wait();
-  constexpr int S = (LMAX + 1) * (LMAX + 1), LM = LMAX + 1;
-  constexpr int kW = 32 * CPL * LM * (int)sizeof(T), kSb = 32 * CPL * (int)sizeof(T), kStage = round16(kW + kSb + S * 4);
+  constexpr int S = (LMAX + 1) * (LMAX + 1), LM = LMAX + 1, NP = (CPL + 1) / 2;
+  using Row = GenRow<T, CPL, LM, S>;
+  constexpr int kSb = 32 * CPL * (int)sizeof(T), kOffY = Row::kW + kSb, kStage = kOffY + Row::kY;
   __shared__ __align__(16) unsigned char rings[kGenWarps][kRing * kStage];
   GenLane g;
   if (!gen_lane<CPL>(io, g)) return;
-  const T* __restrict__ w0 = reinterpret_cast<const T*>(io.w[0]) + io.wcol[0];
-  const T* __restrict__ sb = reinterpret_cast<const T*>(io.sbar[L]) + io.sbar_off[L];
-  const int ldw0 = io.ldw[0], ldsb = io.ldsbar[L], row_bytes = io.C * LM * (int)sizeof(T);
-  const unsigned sal =
-      (unsigned)((reinterpret_cast<uintptr_t>(sb) | (ldsb * sizeof(T)) | (io.C * sizeof(T))) & 15);
-  float acc[CPL][S];
+  Row row(reinterpret_cast<const T*>(io.w[0]) + io.wcol[0], io.ldw[0], io.C * LM * (int)sizeof(T), io.Y, g.rb, g.lane);
+  const int nsb = io.C * (int)sizeof(T), psb = io.ldsbar[L] * (int)sizeof(T);
+  const unsigned char* sp =
+      reinterpret_cast<const unsigned char*>(reinterpret_cast<const T*>(io.sbar[L]) + io.sbar_off[L]) + (size_t)g.rb * psb;
+  const unsigned sal = (unsigned)((reinterpret_cast<uintptr_t>(sp) | psb | nsb) & 15);
+  float2 acc[NP][S];
 #pragma unroll
-  for (int c = 0; c < CPL; ++c)
+  for (int p = 0; p < NP; ++p)
 #pragma unroll
-    for (int a = 0; a < S; ++a) acc[c][a] = 0.0f;
-  auto copy = [&](int e, unsigned char* st) {
-    warp_copy(st, reinterpret_cast<const unsigned char*>(w0 + (size_t)e * ldw0), row_bytes, 0);
-    warp_copy(st + kW, reinterpret_cast<const unsigned char*>(sb + (size_t)e * ldsb), io.C * (int)sizeof(T), sal);
-    if (g.lane < S) cp_async4(st + kW + kSb + g.lane * 4, io.Y + (size_t)e * S + g.lane);
+    for (int a = 0; a < S; ++a) acc[p][a] = make_float2(0.0f, 0.0f);
+  auto copy = [&](int, unsigned char* st) {
+    row.copy_w(st);
+    if (sal == 0) {   // (at most 512 bytes: one piece per lane)
+      if (g.lane * 16 < nsb) cp_async16(st + Row::kW + g.lane * 16, sp + g.lane * 16);
+    } else {
+      warp_copy(st + Row::kW, sp, nsb, sal);
+    }
+    sp += psb;
+    row.copy_y(st + kOffY);
   };
   ring_over<kRing, kStage>(rings[threadIdx.x >> 5], g.rb, g.re, copy, [&](int, const unsigned char* st) {
     if (!g.act) return;
-    float y[S];
-    load_y<S>(reinterpret_cast<const float*>(st + kW + kSb), y);
+    float2 y[(S + 1) / 2 * 2];
+    load_yy<S>(st + kOffY, y);
+    const T* ss = reinterpret_cast<const T*>(st + Row::kW) + g.lane;
 #pragma unroll
-    for (int c = 0; c < CPL; ++c) {
-      const float sv = gld(reinterpret_cast<const T*>(st + kW) + g.lane + 32 * c);
-      float wl[LM];
-      load_lm<T, LM>(reinterpret_cast<const T*>(st) + (g.lane + 32 * c) * LM, wl);
+    for (int p = 0; p < NP; ++p) {
+      const float2 sv = make_float2(gld(ss + 64 * p), CPL > 1 ? gld(ss + 64 * p + (CPL > 1 ? 32 : 0)) : 0.0f);
+      float2 w[LM];
+      load_pair<T, CPL, LM>(st, g.lane, p, w);
 #pragma unroll
-      for (int a = 0; a < S; ++a) acc[c][a] = fmaf(wl[l_of(a)] * sv, y[a], acc[c][a]);
+      for (int l = 0; l < LM; ++l) w[l] = __fmul2_rn(w[l], sv);
+#pragma unroll
+      for (int a = 0; a < S; ++a) acc[p][a] = __ffma2_rn(w[l_of(a)], y[a], acc[p][a]);
     }
   });
   if (!g.act) return;
@@ -748,42 +818,58 @@ __global__ void __launch_bounds__(32 * kGenWarps) gen_qbar_w_kernel(GenRowIO io,
 #pragma unroll
   for (int c = 0; c < CPL; ++c)
 #pragma unroll
-    for (int a = 0; a < S; ++a) out[(size_t)a * io.C + 32 * c] = acc[c][a];
+    for (int a = 0; a < S; ++a) out[(size_t)a * io.C + 32 * c] = (c & 1) ? acc[c / 2][a].y : acc[c / 2][a].x;
 }
 
 // wbar^L_{e,u,l} = nu sum_m Gammabar^L[i][u][lm] Y_e[lm], for a layer L >= 2
 template <typename T, int LMAX, int CPL>
-__global__ void __launch_bounds__(32 * kGenWarps) gen_wbar_w_kernel(GenRowIO io, int L) {
+__global__ void __launch_bounds__(32 * kGenWarps, 5) gen_wbar_w_kernel(GenRowIO io, int L) {
   pdl_wait();
-  constexpr int S = (LMAX + 1) * (LMAX + 1), LM = LMAX + 1;
-  constexpr int kStage = round16(S * 4);
+  constexpr int S = (LMAX + 1) * (LMAX + 1), LM = LMAX + 1, NP = (CPL + 1) / 2;
+  using Row = GenRow<T, CPL, LM, S>;
+  constexpr int kStage = Row::kY;
   __shared__ __align__(16) unsigned char rings[kGenWarps][kRing * kStage];
   GenLane g;
   if (!gen_lane<CPL>(io, g)) return;
-  float gb[CPL][S];
+  Row row(nullptr, 0, 0, io.Y, g.rb, g.lane);
+  float2 gb[NP][S];
   const float* G = io.Gb[L] + (size_t)g.ia * S * io.C + (g.act ? g.lane : 0);
 #pragma unroll
-  for (int c = 0; c < CPL; ++c)
+  for (int p = 0; p < NP; ++p)
 #pragma unroll
-    for (int a = 0; a < S; ++a) gb[c][a] = io.nu * G[(size_t)a * io.C + 32 * c];
-  T* __restrict__ wLb = reinterpret_cast<T*>(io.wbar[L]) + io.wbcol[L] + g.lane * LM;
+    for (int a = 0; a < S; ++a)
+      gb[p][a] = make_float2(io.nu * G[(size_t)a * io.C + 64 * p], CPL > 1 ? io.nu * G[(size_t)a * io.C + 64 * p + 32] : 0.0f);
+  const int ldwb = io.ldwbar[L];
+  T* __restrict__ wLb = reinterpret_cast<T*>(io.wbar[L]) + io.wbcol[L] + g.lane * LM + (size_t)g.rb * ldwb;
+  const bool amax = io.amax_wbar != nullptr;
   float gmax = 0.0f;
-  auto copy = [&](int e, unsigned char* st) {
-    if (g.lane < S) cp_async4(st + g.lane * 4, io.Y + (size_t)e * S + g.lane);
-  };
-  ring_over<kRing, kStage>(rings[threadIdx.x >> 5], g.rb, g.re, copy, [&](int e, const unsigned char* st) {
+  auto copy = [&](int, unsigned char* st) { row.copy_y(st); };
+  ring_over<kRing, kStage>(rings[threadIdx.x >> 5], g.rb, g.re, copy, [&](int, const unsigned char* st) {
     if (!g.act) return;
-    float y[S];
-    load_y<S>(reinterpret_cast<const float*>(st), y);
+    float2 o[NP][LM];
 #pragma unroll
-    for (int c = 0; c < CPL; ++c) {
-      float o[LM] = {};
+    for (int p = 0; p < NP; ++p)
 #pragma unroll
-      for (int a = 0; a < S; ++a) o[l_of(a)] = fmaf(gb[c][a], y[a], o[l_of(a)]);
+      for (int l = 0; l < LM; ++l) o[p][l] = make_float2(0.0f, 0.0f);
+    // (component by component: few of the harmonics in registers at a time, one block more per SM)
 #pragma unroll
-      for (int l = 0; l < LM; ++l) gmax = fmaxf(gmax, fabsf(o[l]));
-      store_lm<T, LM>(wLb + (size_t)e * io.ldwbar[L] + 32 * c * LM, o);
+    for (int a = 0; a < S; ++a) {
+      const float2 y = *reinterpret_cast<const float2*>(st + 8 * a);
+#pragma unroll
+      for (int p = 0; p < NP; ++p) o[p][l_of(a)] = __ffma2_rn(gb[p][a], y, o[p][l_of(a)]);
     }
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      float oa[LM], ob[LM];
+#pragma unroll
+      for (int l = 0; l < LM; ++l) {
+        oa[l] = o[p][l].x; ob[l] = o[p][l].y;
+        if (amax) gmax = fmaxf(gmax, fmaxf(fabsf(oa[l]), fabsf(ob[l])));
+      }
+      store_lm<T, LM>(wLb + 64 * p * LM, oa);
+      if constexpr (CPL > 1) store_lm<T, LM>(wLb + (64 * p + 32) * LM, ob);
+    }
+    wLb += ldwb;
   });
   record_amax(io.amax_wbar, gmax);
 }
