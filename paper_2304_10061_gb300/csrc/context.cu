@@ -95,9 +95,10 @@ bool is_device_ptr(const void* p) {
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// plain device memory of `device` (a kernel of that device may address it directly)
-bool is_own_device_ptr(const void* p, int device) {
-  if (!p) return false;
+// plain device memory of `device` at a multiple of `align` bytes (a kernel of that device may address it
+// directly)
+bool is_own_device_ptr(const void* p, int device, size_t align) {
+  if (!p || reinterpret_cast<uintptr_t>(p) % align) return false;
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
     cudaGetLastError();
@@ -818,11 +819,11 @@ allegro_status stage_atoms(allegro_ctx* c, int64_t n, const double* pos, const i
     // device inputs are read where they are; others are copied first
     const double* ps = pos;
     const int32_t* ts = types;
-    if (!is_own_device_ptr(pos, c->device)) {
+    if (!is_own_device_ptr(pos, c->device, 8)) {
       CUDA_TRY(c, cudaMemcpyAsync(c->d_pos, pos, (size_t)n * 3 * 8, cudaMemcpyDefault, c->stream));
       ps = c->d_pos;
     }
-    if (!is_own_device_ptr(types, c->device)) {
+    if (!is_own_device_ptr(types, c->device, 4)) {
       CUDA_TRY(c, cudaMemcpyAsync(c->d_types, types, (size_t)n * 4, cudaMemcpyDefault, c->stream));
       ts = c->d_types;
     }
@@ -2318,7 +2319,7 @@ allegro_status allegro_energy_forces(allegro_ctx* c, double* E_total, double* E_
   allegro_status s = evaluate(c, backward);
   if (s != ALLEGRO_OK) return s;
   const size_t n = (size_t)c->n_atoms, B = (size_t)c->nstruct;
-  auto direct = [&](const void* p) { return !p || is_own_device_ptr(p, c->device); };
+  auto direct = [&](const void* p) { return !p || is_own_device_ptr(p, c->device, 8); };
   if (direct(E_total) && direct(E_atom) && direct(F) && direct(virial)) {
     const unsigned blocks = (unsigned)std::min<size_t>((3 * n + 9 * B + 255) / 256, 152 * 8);
     launch(copy_results_kernel, blocks, 256, 0, c->stream, c->d_Eout, c->d_Eatom, c->d_F, c->d_Wout, (long long)B,

@@ -7,8 +7,11 @@ zero (each edge's vector is added once and subtracted once), and the energies of
 are those of a full call.  1e-12 of the sum of magnitudes is 10^4 times float64's rounding unit, above what
 about 10^2 terms per atom accumulate.
 """
+import ctypes
+
 import numpy as np
 import pytest
+import torch
 
 from gpu_util import BF16_F_RMS, FP32_E, FP32_F, FP32_W, assert_same_edges, errors, lib_model
 from oracle.allegro import AllegroOracle
@@ -74,6 +77,28 @@ def test_list_outgrows_its_capacity():
         assert_same_edges(m.get_neighbors(), neighbor_list(s.pos, s.cell, s.pbc, C1.r_c))
         assert np.isfinite(m.energy_forces()["E"].item())
     m.close()
+
+
+@pytest.mark.parametrize("shift", [4, 2])
+def test_device_arrays_off_their_elements_alignment(model, shift):
+    """Device arrays that start between two elements are copied, aligned ones are used in place: the same results."""
+    s = _box(300)
+    n, types = len(s.pos), (s.species % 2).astype(np.int32)
+    L, ctx, st = model._L, model._ctx, lambda v: torch.tensor(np.frombuffer(v.tobytes(), np.uint8).copy(), device="cuda")
+    want_edges = model.neighbors(torch.tensor(s.pos, device="cuda"), torch.tensor(types, device="cuda"), s.cell)
+    want = {k: v.cpu().numpy() for k, v in model.energy_forces().items()}
+    bufs = [torch.zeros(8 * k + 8, dtype=torch.uint8, device="cuda") for k in (3 * n, n, 1, n, 3 * n, 9)]
+    bufs[0][shift:shift + 24 * n] = st(s.pos)
+    bufs[1][shift:shift + 4 * n] = st(types)
+    torch.cuda.synchronize()
+    ptr = [b.data_ptr() + shift for b in bufs]
+    cell, ne = np.ascontiguousarray(s.cell, np.float64), ctypes.c_int64(0)
+    model._check(L.allegro_neighbors(ctx, n, ptr[0], ptr[1], cell.ctypes.data, None, ctypes.byref(ne)))
+    assert ne.value == want_edges
+    model._check(L.allegro_energy_forces(ctx, ptr[2], ptr[3], ptr[4], ptr[5]))
+    for b, key in zip(bufs[2:], ("E", "E_atom", "F", "virial")):
+        raw = b.cpu().numpy()[shift:shift + 8 * want[key].size].copy()
+        np.testing.assert_array_equal(raw.view(np.float64), want[key].ravel())
 
 
 @pytest.mark.parametrize("table", [None, [[4.0, 2.5], [3.0, 3.75]]])
