@@ -768,7 +768,7 @@ allegro_status ensure_ws(allegro_ctx* c, int64_t Ec, int64_t Ac, WS* w) {
     c->ws = nullptr;
     c->ws_edges = c->ws_atoms = 0;
     CUDA_TRY(c, cudaMalloc(&c->ws, bytes));
-    CUDA_TRY(c, cudaMemset(c->ws, 0, bytes));
+    CUDA_TRY(c, cudaMemsetAsync(c->ws, 0, bytes, c->stream));
     c->ws_bytes = bytes;
     c->ws_edges = E2;
     c->ws_atoms = A2;
@@ -1953,8 +1953,12 @@ allegro_status allegro_create(const void* weights_blob, size_t blob_bytes, const
   if (cudaMalloc(&c->d_err, 16) != cudaSuccess || cudaMalloc(&c->d_total, 16) != cudaSuccess ||
       cudaMalloc(&c->d_minmax, 12 * 8) != cudaSuccess || cudaMalloc(&c->d_red_scratch, kStructScratch * sizeof(double)) != cudaSuccess)
     return bail(fail(c, ALLEGRO_E_OOM, "scratch allocation failed"));
-  cudaMemset(c->d_err, 0, 16);
-  cudaMemset(c->d_red_scratch, 0, kStructScratch * sizeof(double));
+  // The context's stream does not wait for the default stream, nor a later one for it: the uploads (on
+  // the default stream) and the clears have ended before the first call.
+  if (cudaMemsetAsync(c->d_err, 0, 16, c->stream) != cudaSuccess ||
+      cudaMemsetAsync(c->d_red_scratch, 0, kStructScratch * sizeof(double), c->stream) != cudaSuccess ||
+      cudaStreamSynchronize(c->stream) != cudaSuccess || cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess)
+    return bail(fail(c, ALLEGRO_E_CUDA, "model upload failed"));
   *out = c;
   return ALLEGRO_OK;
 }

@@ -1,0 +1,80 @@
+"""Host code of the library on a CUDA runtime without a GPU (fake_cudart.c): what its calls queue,
+on which stream, what they leave queued when they return, and what they do with the values that
+kernels leave for the host.  Each test is a program of its own (the fake is preloaded)."""
+import os
+import subprocess
+import sys
+import textwrap
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+PREAMBLE = """
+    import ctypes, sys
+    import numpy as np
+    sys.path.insert(0, {root!r})
+    from paper_2304_10061_gb300 import Allegro, AllegroError
+    from synth import ARCHS, make_weights, weights_to_blob
+
+    fake = ctypes.CDLL({fake!r})
+    for f in (fake.fake_pending, fake.fake_total, fake.fake_pending_all):
+        f.restype = ctypes.c_long
+    fake.fake_pending.argtypes = fake.fake_total.argtypes = [ctypes.c_void_p]
+    HOOK = ctypes.CFUNCTYPE(None, ctypes.c_char_p, ctypes.POINTER(ctypes.c_void_p))
+
+    def param(args, k, ctype=ctypes.c_void_p):
+        return ctype.from_address(args[k]).value
+
+    ARCH = ARCHS["c1"]
+    model = Allegro(weights_to_blob(ARCH, make_weights(ARCH, 0)))
+    N = 64
+    rng = np.random.default_rng(0)
+    cell = np.eye(3) * 8.62
+    pos = rng.uniform(0.0, 8.62, (N, 3))
+    types = (np.arange(N) % 2).astype(np.int32)
+
+    def evaluate():
+        out = [np.zeros(k) for k in (1, N, 3 * N, 9)]
+        model._check(model._L.allegro_energy_forces(model._ctx, *[a.ctypes.data for a in out]))
+        return out
+
+    def status(call):
+        try:
+            call()
+        except AllegroError as e:
+            return e.status
+        return 0
+"""
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    import __graft_entry__ as g
+    from paper_2304_10061_gb300.build import nvcc
+    g.build()
+    so = str(tmp_path_factory.mktemp("fake") / "fake_cudart.so")
+    include = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc()))), "include")
+    subprocess.run(["gcc", "-O1", "-shared", "-fPIC", "-I", include, os.path.join(ROOT, "tests", "fake_cudart.c"), "-o", so],
+                   check=True)
+
+    def run(script):
+        text = textwrap.dedent(PREAMBLE).format(root=ROOT, fake=so) + textwrap.dedent(script)
+        r = subprocess.run([sys.executable, "-c", text], env=dict(os.environ, LD_PRELOAD=so), capture_output=True,
+                           text=True, timeout=300)
+        assert r.returncode == 0, r.stderr[-2000:]
+
+    return run
+
+
+def test_nothing_on_the_default_stream(fake):
+    """The context's stream does not wait for the default stream: uploads on it have ended when
+    allegro_create returns, and no clear is queued on it (a workspace cleared there was cleared
+    while the first kernels wrote it)."""
+    fake("""
+        assert fake.fake_pending(None) == 0, fake.fake_pending(None)
+        before = fake.fake_total(None)
+        model.neighbors(pos, types, cell)
+        evaluate()
+        assert fake.fake_total(None) == before, fake.fake_total(None) - before
+    """)
