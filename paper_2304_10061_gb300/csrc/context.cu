@@ -331,6 +331,20 @@ allegro_status fail(allegro_ctx* c, allegro_status s, const char* fmt, ...) {
   return s;
 }
 
+// A call leaves nothing queued when it returns, whichever way: what it reads (the caller's arrays, its
+// own on the stack) may go after it, and allegro_set_stream orders nothing between two streams.  The
+// calls that wait for their results anyway say so (idle); every other return waits here.
+struct Drain {
+  allegro_ctx* c;
+  bool idle = false;
+  explicit Drain(allegro_ctx* c_) : c(c_) {}
+  ~Drain() {
+    if (idle) return;
+    cudaStreamSynchronize(c->stream);
+    cudaGetLastError();
+  }
+};
+
 #define CUDA_TRY(ctx, call)                                                                        \
   do {                                                                                             \
     cudaError_t e_ = (call);                                                                       \
@@ -2041,6 +2055,7 @@ allegro_status allegro_reserve(allegro_ctx* c, int64_t atom_cap, int64_t edge_ca
                                int64_t chunk_edges) {
   if (!c || atom_cap < 0 || edge_cap < 0 || chunk_edges < 0) return ALLEGRO_E_INVALID;
   cudaSetDevice(c->device);
+  Drain drain(c);
   c->fixed = fixed != 0;
   c->atom_cap = atom_cap;
   c->edge_cap = edge_cap;
@@ -2074,10 +2089,11 @@ static allegro_status build_single(allegro_ctx* c, int64_t n_atoms, const double
   cudaSetDevice(c->device);
   cudaStream_t st = c->stream;
   const int n = (int)n_atoms;
+  const int64_t hoffs[2] = {0, n};
+  Drain drain(c);
   allegro_status s = stage_atoms(c, n, pos, types);
   if (s != ALLEGRO_OK) return s;
   if ((s = ensure_structs(c, 1)) != ALLEGRO_OK) return s;
-  int64_t hoffs[2] = {0, n};
   CUDA_TRY(c, cudaMemcpyAsync(c->d_offs, hoffs, sizeof hoffs, cudaMemcpyHostToDevice, st));
   c->nstruct = 1;
   c->batched = false;
@@ -2206,6 +2222,7 @@ static allegro_status build_single(allegro_ctx* c, int64_t n_atoms, const double
        })) != ALLEGRO_OK)
     return s;
   c->n_centres = g.n_centres;
+  drain.idle = true;
   return ALLEGRO_OK;
 }
 
@@ -2242,11 +2259,13 @@ allegro_status allegro_neighbors_batched(allegro_ctx* c, int32_t n_struct, const
   if (n64 > 1000000000LL) return fail(c, ALLEGRO_E_INVALID, "too many atoms");
   const int n = (int)n64;
   if (n > 0 && (!pos || !types)) return fail(c, ALLEGRO_E_INVALID, "pos and types are required");
+  std::vector<double> hc;
+  std::vector<int> hp((size_t)3 * n_struct, 0), hn((size_t)3 * n_struct, 0);
+  std::vector<double> hinv((size_t)9 * n_struct, 0.0), hspan((size_t)3 * n_struct, 0.0);
+  Drain drain(c);
   allegro_status s = stage_atoms(c, n, pos, types);
   if (s != ALLEGRO_OK) return s;
   if ((s = ensure_structs(c, n_struct)) != ALLEGRO_OK) return s;
-  std::vector<double> hc;
-  std::vector<int> hp((size_t)3 * n_struct, 0), hn((size_t)3 * n_struct, 0);
   if (cells) {
     hc.resize((size_t)9 * n_struct);
     if (is_device_ptr(cells)) CUDA_TRY(c, cudaMemcpy(hc.data(), cells, hc.size() * 8, cudaMemcpyDeviceToHost));
@@ -2261,7 +2280,6 @@ allegro_status allegro_neighbors_batched(allegro_ctx* c, int32_t n_struct, const
   CUDA_TRY(c, cudaMemcpyAsync(c->d_offs, offs.data(), offs.size() * 8, cudaMemcpyHostToDevice, st));
   // image ranges: |S_k| <= ceil(r_c / w_k + span_k), span_k the spread of the
   // structure's fractional coordinates (positions need not be wrapped)
-  std::vector<double> hinv((size_t)9 * n_struct, 0.0), hspan((size_t)3 * n_struct, 0.0);
   if (cells) {
     for (int b = 0; b < n_struct; ++b)
       if (!invert3(&hc[9 * (size_t)b], &hinv[9 * (size_t)b])) return fail(c, ALLEGRO_E_INVALID, "cell %d is singular", b);
@@ -2311,6 +2329,7 @@ allegro_status allegro_neighbors_batched(allegro_ctx* c, int32_t n_struct, const
     return s;
   c->nstruct = n_struct;
   c->batched = true;
+  drain.idle = true;
   return ALLEGRO_OK;
 }
 
@@ -2320,6 +2339,7 @@ allegro_status allegro_energy_forces(allegro_ctx* c, double* E_total, double* E_
   if (!c->have_nb) return fail(c, ALLEGRO_E_STATE, "allegro_neighbors must succeed before energy_forces");
   cudaSetDevice(c->device);
   const bool backward = (F != nullptr) || (virial != nullptr);
+  Drain drain(c);
   allegro_status s = evaluate(c, backward);
   if (s != ALLEGRO_OK) return s;
   const size_t n = (size_t)c->n_atoms, B = (size_t)c->nstruct;
@@ -2337,6 +2357,7 @@ allegro_status allegro_energy_forces(allegro_ctx* c, double* E_total, double* E_
   }
   int err = 0;
   if ((s = read_err(c, &err)) != ALLEGRO_OK) return s;
+  drain.idle = true;
   if (err & kErrTimeout) return fail(c, ALLEGRO_E_TIMEOUT, "a bounded device wait expired; results are invalid");
   if (err & kErrNonFinite) return fail(c, ALLEGRO_E_NONFINITE, "non-finite energy or force");
   return ALLEGRO_OK;
@@ -2375,6 +2396,7 @@ allegro_status allegro_md_verlet(allegro_ctx* c, int64_t n_atoms, double* pos, d
     c->md_steps = n_steps + 1;
   }
   if (n_types > 4096) return fail(c, ALLEGRO_E_INVALID, "md_verlet: too many types");
+  Drain drain(c);
   auto kind = [](const void* p) { return is_device_ptr(p) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice; };
   CUDA_TRY(c, cudaMemcpyAsync(c->d_md_pos, pos, (size_t)n * 24, kind(pos), st));
   CUDA_TRY(c, cudaMemcpyAsync(c->d_md_vel, vel, (size_t)n * 24, kind(vel), st));
@@ -2463,6 +2485,7 @@ allegro_status allegro_md_verlet(allegro_ctx* c, int64_t n_atoms, double* pos, d
   if ((s = copy_out(c, E_pot, c->d_md_E, (size_t)(n_steps + 1) * 8)) != ALLEGRO_OK) return s;
   if ((s = copy_out(c, E_kin, c->d_md_K, (size_t)(n_steps + 1) * 8)) != ALLEGRO_OK) return s;
   if ((s = read_err(c, &err)) != ALLEGRO_OK) return s;
+  drain.idle = true;
   if (err & kErrTimeout) return fail(c, ALLEGRO_E_TIMEOUT, "a bounded device wait expired; results are invalid");
   if (err & kErrNonFinite) return fail(c, ALLEGRO_E_NONFINITE, "non-finite energy or force");
   return ALLEGRO_OK;
@@ -2541,11 +2564,13 @@ allegro_status allegro_get_neighbors(allegro_ctx* c, int32_t* i, int32_t* j, int
   if (cap < c->n_edges) return fail(c, ALLEGRO_E_CAPACITY, "cap %lld < %lld edges", (long long)cap, (long long)c->n_edges);
   cudaSetDevice(c->device);
   const size_t E = (size_t)c->n_edges;
+  Drain drain(c);
   allegro_status s;
   if ((s = copy_out(c, i, c->d_ei, E * 4)) != ALLEGRO_OK) return s;
   if ((s = copy_out(c, j, c->d_ej, E * 4)) != ALLEGRO_OK) return s;
   if ((s = copy_out(c, shift, c->d_eS, E * 12)) != ALLEGRO_OK) return s;
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  drain.idle = true;
   return ALLEGRO_OK;
 }
 

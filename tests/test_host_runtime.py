@@ -35,7 +35,7 @@ PREAMBLE = """
     types = (np.arange(N) % 2).astype(np.int32)
 
     def evaluate():
-        out = [np.zeros(k) for k in (1, N, 3 * N, 9)]
+        out = [np.zeros(k) for k in (model.n_struct, N, 3 * N, 9 * model.n_struct)]
         model._check(model._L.allegro_energy_forces(model._ctx, *[a.ctypes.data for a in out]))
         return out
 
@@ -77,4 +77,31 @@ def test_nothing_on_the_default_stream(fake):
         model.neighbors(pos, types, cell)
         evaluate()
         assert fake.fake_total(None) == before, fake.fake_total(None) - before
+    """)
+
+
+def test_calls_leave_nothing_queued(fake):
+    """Every call has waited for what it queued when it returns, refused ones too: the stream may be
+    changed and the caller's arrays may go."""
+    fake("""
+        def check(want, call):
+            assert status(call) == want
+            assert fake.fake_pending_all() == 0, fake.fake_pending_all()
+
+        flat, nan = np.diag([8.62, 8.62, 0.0]), np.diag([8.62, 8.62, np.nan])
+        offs = np.array([0, 30, N], np.int64)
+        check(0, lambda: model.reserve(1000, 5000))
+        check(1, lambda: model.neighbors(pos, types, flat))
+        check(1, lambda: model.neighbors(pos, types, nan))
+        check(1, lambda: model.neighbors(pos, types, None, [1, 0, 0]))
+        check(1, lambda: model.neighbors_local(10, pos, types, flat))
+        check(1, lambda: model.neighbors_batched(offs, pos, types, np.stack([cell, flat])))
+        check(1, lambda: model.neighbors_batched(offs, pos, types, None, [1] * 6))
+        check(1, lambda: model.md_verlet(pos.copy(), np.zeros((N, 3)), types, [1.0, 1.0], 1.0, 2, flat))
+        check(0, lambda: model.neighbors_batched(offs, pos, types))
+        check(0, evaluate)
+        check(0, lambda: model.neighbors(pos, types, cell))
+        check(0, evaluate)
+        check(0, model.get_neighbors)
+        check(0, lambda: model.md_verlet(pos.copy(), np.zeros((N, 3)), types, [1.0, 1.0], 1.0, 2, cell))
     """)
