@@ -190,6 +190,7 @@ struct allegro_ctx {
   bool rows_on_host = false;
   int64_t bytes_per_edge = 0;              // chunk workspace per edge (0: not computed yet)
   int* h_pin = nullptr;                    // pinned words the waits read {error word, edge count} into
+  bool keep_err = false;                   // MD: the error word of the last evaluation is still to be read
 
   // capacities and policy
   int64_t atom_cap = 0, edge_cap = 0;
@@ -841,7 +842,7 @@ allegro_status stage_atoms(allegro_ctx* c, int64_t n, const double* pos, const i
       CUDA_TRY(c, cudaMemcpyAsync(c->d_types, types, (size_t)n * 4, cudaMemcpyDefault, c->stream));
       ts = c->d_types;
     }
-    CUDA_TRY(c, cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream));
+    if (!c->keep_err) CUDA_TRY(c, cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream));
     launch(stage_atoms_kernel, (unsigned)((n + 255) / 256), 256, 0, c->stream, ts, ps, (int)n, c->d_map, c->nmap, c->d_pos,
                                                                            c->d_species, c->d_err);
     CUDA_TRY(c, cudaGetLastError());
@@ -890,6 +891,13 @@ allegro_status read_err(allegro_ctx* c, int* out, int64_t* n_edges = nullptr) {
   return ALLEGRO_OK;
 }
 
+// What the error word says about the evaluation that ran before it was read.
+allegro_status eval_status(allegro_ctx* c, int err) {
+  if (err & kErrTimeout) return fail(c, ALLEGRO_E_TIMEOUT, "a bounded device wait expired; results are invalid");
+  if (err & kErrNonFinite) return fail(c, ALLEGRO_E_NONFINITE, "non-finite energy or force");
+  return ALLEGRO_OK;
+}
+
 // Edges the list's arrays hold now.
 int64_t edge_room(allegro_ctx* c) {
   const Caps& k = caps_of(c);
@@ -927,6 +935,7 @@ allegro_status fill_rows(allegro_ctx* c, int n, int64_t* n_edges_out, Fill&& fil
     }
     CUDA_TRY(c, cudaGetLastError());
     if ((s = read_err(c, &err, &E)) != ALLEGRO_OK) return s;
+    if ((s = eval_status(c, err)) != ALLEGRO_OK) return s;   // (MD: the evaluation that moved the atoms here)
     if (E < 0) return fail(c, ALLEGRO_E_CAPACITY, "edge count overflows int32");
     if ((s = ensure_edges(c, E)) != ALLEGRO_OK) return s;
     if (room > 0 && E <= room) break;
@@ -2358,9 +2367,7 @@ allegro_status allegro_energy_forces(allegro_ctx* c, double* E_total, double* E_
   int err = 0;
   if ((s = read_err(c, &err)) != ALLEGRO_OK) return s;
   drain.idle = true;
-  if (err & kErrTimeout) return fail(c, ALLEGRO_E_TIMEOUT, "a bounded device wait expired; results are invalid");
-  if (err & kErrNonFinite) return fail(c, ALLEGRO_E_NONFINITE, "non-finite energy or force");
-  return ALLEGRO_OK;
+  return eval_status(c, err);
 }
 
 allegro_status allegro_md_verlet(allegro_ctx* c, int64_t n_atoms, double* pos, double* vel, const int32_t* types,
@@ -2408,6 +2415,13 @@ allegro_status allegro_md_verlet(allegro_ctx* c, int64_t n_atoms, double* pos, d
   allegro_status s = read_err(c, &err);
   if (s != ALLEGRO_OK) return s;
   if (err) return fail(c, ALLEGRO_E_INVALID, "md_verlet: a type has no positive mass");
+  // From here the error word is cleared by the evaluations alone: the list of the next step reads what
+  // the evaluation before it left there (the last one's is read at the end).
+  struct KeepErr {
+    allegro_ctx* c;
+    explicit KeepErr(allegro_ctx* c_) : c(c_) { c->keep_err = true; }
+    ~KeepErr() { c->keep_err = false; }
+  } keep(c);
   // The neighbour list of the current positions: rebuilt by the cell-list
   // search every step, or, with a Verlet skin, filtered from a candidate list
   // built at r_c + skin, rebuilt only once some atom has moved skin/2 since
@@ -2486,9 +2500,7 @@ allegro_status allegro_md_verlet(allegro_ctx* c, int64_t n_atoms, double* pos, d
   if ((s = copy_out(c, E_kin, c->d_md_K, (size_t)(n_steps + 1) * 8)) != ALLEGRO_OK) return s;
   if ((s = read_err(c, &err)) != ALLEGRO_OK) return s;
   drain.idle = true;
-  if (err & kErrTimeout) return fail(c, ALLEGRO_E_TIMEOUT, "a bounded device wait expired; results are invalid");
-  if (err & kErrNonFinite) return fail(c, ALLEGRO_E_NONFINITE, "non-finite energy or force");
-  return ALLEGRO_OK;
+  return eval_status(c, err);
 }
 
 allegro_status allegro_set_autotune(allegro_ctx* c, int32_t enable) {

@@ -105,3 +105,32 @@ def test_calls_leave_nothing_queued(fake):
         check(0, model.get_neighbors)
         check(0, lambda: model.md_verlet(pos.copy(), np.zeros((N, 3)), types, [1.0, 1.0], 1.0, 2, cell))
     """)
+
+
+@pytest.mark.parametrize("skin", [0.0, 1.0])
+@pytest.mark.parametrize("bit,want", [(1, 5), (8, 6)])
+def test_md_reports_every_steps_errors(fake, bit, want, skin):
+    """A device wait that ran out, or a non-finite energy or force, ends the MD run whichever of its
+    evaluations raised it, and is gone in the next call."""
+    fake(f"""
+        BIT, WANT, SKIN = {bit}, {want}, {skin}
+    """ + """
+        seen = [0]
+
+        @HOOK
+        def hook(name, args):
+            if b"struct_reduce_kernel" in name:   # the last kernel of an evaluation; its last parameter is the error word
+                seen[0] += 1
+                if seen[0] == at:
+                    ctypes.c_int.from_address(param(args, 10)).value |= BIT
+
+        fake.fake_on_launch(hook)
+        model.set_md_skin(SKIN)
+        for at in range(1, 6):   # evaluations 1..4 of three steps; 5: none of them
+            seen[0] = 0
+            got = status(lambda: model.md_verlet(pos.copy(), np.zeros((N, 3)), types, [1.0, 1.0], 1.0, 3, cell))
+            assert got == (WANT if at < 5 else 0), (at, got)
+            at = 0
+            assert status(lambda: model.neighbors(pos, types, cell)) == 0
+            assert status(evaluate) == 0
+    """)
