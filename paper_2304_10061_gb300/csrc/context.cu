@@ -909,8 +909,8 @@ int64_t edge_room(allegro_ctx* c) {
 int* col_rank(allegro_ctx* c) { return reinterpret_cast<int*>(c->d_Ee); }
 
 // The second half of every neighbour path, once the counts are scanned into row_ptr (their total in
-// d_err[1]): fill(edge_cap) queues the fill pass (true: it counted and ranked the columns), then come
-// the CSC index and one wait for the error word and the edge count.  When the arrays of an earlier
+// d_err[1]): fill(edge_cap) queues the fill pass in one profile scope (true: it counted and ranked the
+// columns; its 44 bytes per edge are added here), then come the CSC index and one wait for the error word and the edge count.  When the arrays of an earlier
 // list are there all of it is queued before the count is known -- the passes leave a list that does
 // not fit unwritten, and they run again once the arrays have grown -- so a list costs one wait
 // instead of two; the first list waits for the count to size the arrays.
@@ -921,9 +921,10 @@ allegro_status fill_rows(allegro_ctx* c, int n, int64_t* n_edges_out, Fill&& fil
   int err = 0;
   allegro_status s;
   for (bool sized = false;;) {
+    const size_t rec = c->prof.recs.size();   // the profile's records of this pass: fill, nb_csc
     if (room > 0) {
       const bool ranked = fill((int)room);
-      ProfScope ps(c, "nb_csc", 0.0, (double)(sized ? E : c->n_edges) * 16 + (double)n * 16, 0);
+      ProfScope ps(c, "nb_csc", 0.0, (double)n * 16, 0);
       if (!ranked) {
         nb_col_rank(c->d_ej, c->d_row_ptr, n, (int)room, c->d_col_count, col_rank(c), st);
         ++c->launches;
@@ -935,6 +936,11 @@ allegro_status fill_rows(allegro_ctx* c, int n, int64_t* n_edges_out, Fill&& fil
     }
     CUDA_TRY(c, cudaGetLastError());
     if ((s = read_err(c, &err, &E)) != ALLEGRO_OK) return s;
+    // the bytes of the edges, now that their number is known; a pass that left the list unwritten moved none
+    for (size_t k = rec; k < c->prof.recs.size(); ++k) {
+      ProfRec& r = c->prof.recs[k];
+      r.bytes = (E >= 0 && E <= room) ? r.bytes + (double)E * (k == rec ? 44.0 : 16.0) : 0.0;
+    }
     if ((s = eval_status(c, err)) != ALLEGRO_OK) return s;   // (MD: the evaluation that moved the atoms here)
     if (E < 0) return fail(c, ALLEGRO_E_CAPACITY, "edge count overflows int32");
     if ((s = ensure_edges(c, E)) != ALLEGRO_OK) return s;
@@ -2224,7 +2230,7 @@ static allegro_status build_single(allegro_ctx* c, int64_t n_atoms, const double
     c->launches += exclusive_scan_i32(c->d_count, c->d_row_ptr, n, c->d_scan_tmp, false, c->d_err + 1, st);
   }
   if ((s = fill_rows(c, n, n_edges_out, [&](int edge_cap) {
-         ProfScope ps(c, "nb_search_fill", 0.0, (double)c->n_edges * 44 + (double)n * 64);
+         ProfScope ps(c, "nb_search_fill", 0.0, (double)n * 64);
          return nb_search(true, c->d_pos, n, g, c->d_cell_of, c->d_wraps, c->d_cell_start, c->d_sorted, c->d_pos4,
                           c->d_pw, rc2, band, pair_rc2, c->arch.pair_rc2f, c->arch.ns, nullptr, c->d_row_ptr, c->d_ej, c->d_ei, c->d_eS,
                           c->d_ed, c->d_col_count, col_rank(c), edge_cap, c->d_err, st);
@@ -2329,7 +2335,7 @@ allegro_status allegro_neighbors_batched(allegro_ctx* c, int32_t n_struct, const
     c->launches += exclusive_scan_i32(c->d_count, c->d_row_ptr, n, c->d_scan_tmp, false, c->d_err + 1, st);
   }
   if ((s = fill_rows(c, n, n_edges_out, [&](int edge_cap) {
-         ProfScope ps(c, "nb_brute_fill", 0.0, (double)c->n_edges * 44 + (double)n * 64);
+         ProfScope ps(c, "nb_brute_fill", 0.0, (double)n * 64);
          nb_bruteforce_batched(true, c->d_pos, c->d_offs, n_struct, d_cells, c->d_pbc, c->d_nimg, rc2, c->d_species,
                                c->arch.pair_rc2, c->arch.ns, c->d_atom_struct, n, nullptr, c->d_row_ptr, c->d_ej,
                                c->d_ei, c->d_eS, c->d_ed, c->d_col_count, col_rank(c), edge_cap, c->d_err, st);
@@ -2473,7 +2479,7 @@ allegro_status allegro_md_verlet(allegro_ctx* c, int64_t n_atoms, double* pos, d
       c->launches += exclusive_scan_i32(c->d_count, c->d_row_ptr, n, c->d_scan_tmp, false, c->d_err + 1, st);
     }
     return fill_rows(c, n, nullptr, [&](int edge_cap) {
-      ProfScope ps(c, "nb_skin_filter", 0.0, (double)c->n_edges * 44 + (double)n * 64);
+      ProfScope ps(c, "nb_skin_filter", 0.0, (double)n * 64);
       nb_skin_filter(true, c->d_pos, n, c->d_cell9, c->d_sk_row, c->d_sk_j, c->d_sk_S, c->arch.rc * c->arch.rc,
                      c->arch.pair_rc2, c->d_species, c->arch.ns, nullptr, c->d_row_ptr, c->d_ej, c->d_ei, c->d_eS,
                      c->d_ed, c->d_col_count, col_rank(c), edge_cap, st);

@@ -134,3 +134,28 @@ def test_md_reports_every_steps_errors(fake, bit, want, skin):
             assert status(lambda: model.neighbors(pos, types, cell)) == 0
             assert status(evaluate) == 0
     """)
+
+
+def test_profile_counts_the_edges_of_its_own_list(fake):
+    """Bytes of the fill and column passes: those of the list they wrote, whatever list came before,
+    and none for a pass that found its list too long for the arrays."""
+    fake("""
+        @HOOK
+        def hook(name, args):
+            if b"scan_one_kernel" in name and param(args, 4):   # the scan of the row counts leaves the total
+                ctypes.c_int.from_address(param(args, 4)).value = edges
+
+        fake.fake_on_launch(hook)
+        offs = np.array([0, 30, N], np.int64)
+        for build, label in ((lambda: model.neighbors(pos, types, cell), "nb_search_fill"),
+                             (lambda: model.neighbors_batched(offs, pos, types), "nb_brute_fill")):
+            for edges in (1000, 700, 90000, 20, 200000):
+                model.profile(True)
+                assert build() == edges
+                rep, _ = model.profile_report()
+                model.profile(False)
+                assert rep[label]["bytes"] == 44 * edges + 64 * N, (edges, rep[label])
+                assert rep["nb_csc"]["bytes"] == 16 * edges + 16 * N, (edges, rep["nb_csc"])
+            edges = 100
+            build()
+    """)
