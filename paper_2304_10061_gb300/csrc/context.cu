@@ -931,7 +931,7 @@ allegro_status fill_rows(allegro_ctx* c, int n, int64_t* n_edges_out, Fill&& fil
       }
       c->launches += exclusive_scan_i32(c->d_col_count, c->d_col_ptr, n, c->d_scan_tmp, true, nullptr, st);
       nb_place_edges(c->d_ej, col_rank(c), c->d_row_ptr, n, (int)room, c->d_col_ptr, c->d_col_edge, st);
-      nb_sort_columns(c->d_col_ptr, n, c->d_col_edge, st);
+      nb_sort_columns(c->d_col_ptr, n, c->d_col_edge, col_rank(c), st);   // (the ranks have been used)
       c->launches += 2;
     }
     CUDA_TRY(c, cudaGetLastError());
@@ -2197,8 +2197,8 @@ static allegro_status build_single(allegro_ctx* c, int64_t n_atoms, const double
     nb_bin(c->d_pos, n, g, c->d_cell_of, c->d_wrap, c->d_cell_count, c->d_count, st);
     c->launches += exclusive_scan_i32(c->d_cell_count, c->d_cell_start, (int)ncell, c->d_scan_tmp, true, nullptr, st);
     nb_place(c->d_cell_of, c->d_count, n, c->d_cell_start, c->d_sorted, st);
-    nb_sort_cells(c->d_pos, c->d_species, g, (int)ncell, c->d_cell_start, c->d_wrap, c->d_sorted, c->d_pos4, c->d_pw,
-                  c->d_wraps, st);
+    nb_sort_cells(c->d_pos, c->d_species, g, (int)ncell, c->d_cell_start, c->d_wrap, c->d_sorted, c->d_count,
+                  c->d_pos4, c->d_pw, c->d_wraps, st);
   }
   // Error band of the float32 prefilter: bound X on |wrapped coordinate| and
   // |image offset|, per-component error <= 8 ulp(X), squared-distance error

@@ -195,9 +195,9 @@ void nb_bin(const double* pos, int n, const CellGrid& g, int* cell_of, int* wrap
 // sorted[start[seg_of[i]] + rank[i]] = i for i in [0, n)
 void nb_place(const int* seg_of, const int* rank, int n, const int* start, int* sorted, cudaStream_t st);
 // each cell's atoms in index order, and pos4 / pw / wraps: wrapped float32 (with the model species'
-// bits in w) and float64 positions and the wrap counts, all in cell order
+// bits in w) and float64 positions and the wrap counts, all in cell order (tmp: n ints)
 void nb_sort_cells(const double* pos, const int* species, const CellGrid& g, int n_cells, const int* cell_start,
-                   const int* wrap, int* sorted, float4* pos4, double* pw, int4* wraps, cudaStream_t st);
+                   const int* wrap, int* sorted, int* tmp, float4* pos4, double* pw, int4* wraps, cudaStream_t st);
 // pair_rc2 (and pair_rc2f, its float32 rounding): null, or device [ns * ns] squared cutoffs per
 // ordered species pair (each <= rc2, the search radius; `band` is the prefilter band of rc2).  The fill passes also count
 // every edge into its neighbour's column (col_count, zero on entry) and keep its arrival order there
@@ -227,8 +227,8 @@ void nb_col_rank(const int* ej, const int* row_ptr, int n, int edge_cap, int* co
                  cudaStream_t st);
 void nb_place_edges(const int* ej, const int* rank, const int* row_ptr, int n, int edge_cap, const int* col_ptr,
                     int* col_edge, cudaStream_t st);
-// each column's edges in ascending order
-void nb_sort_columns(const int* col_ptr, int n, int* col_edge, cudaStream_t st);
+// each column's edges in ascending order (tmp: as many ints as edges)
+void nb_sort_columns(const int* col_ptr, int n, int* col_edge, int* tmp, cudaStream_t st);
 void nb_struct_span(const double* pos, const int64_t* offs, const double* inv, int nstruct, double* span,
                     cudaStream_t st);
 void nb_minmax_frac(const double* pos, int n, const double* inv, double* d_minmax, cudaStream_t st);

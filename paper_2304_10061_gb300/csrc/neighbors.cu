@@ -308,7 +308,11 @@ void nb_place_edges(const int* ej, const int* rank, const int* row_ptr, int n, i
 // Sort each segment [start[s], start[s+1]) of distinct values: G lanes per segment hold up to 4 G
 // values in registers and each value's rank is the number of smaller ones (a broadcast per value),
 // so a segment takes a few dependent loads instead of an insertion sort's chain through memory.
-// Longer segments (never met at liquid densities) are insertion-sorted by one lane.
+// Longer segments are ranked 8 G values at a time against all of theirs, read from memory, and go
+// through `tmp` (as long as v).  Liquids reach all of these: at the density of water a column holds 27
+// edges at a cutoff of 4 Angstrom, 90 at 6, 214 at 8.  Column passes at 262,144 atoms, us, an insertion
+// sort per thread / by one lane past 4 G values / now: 4 Angstrom 244 / 130 / 130, 6 Angstrom 1,107 /
+// 3,259 / 638, 8 Angstrom 3,427 / 17,382 / 2,157.
 // done(place, value) is called for every element of the segment.
 template <int G, int K, typename Done>
 __device__ __forceinline__ void sort_in_registers(int b, int len, int* __restrict__ v, unsigned mask, Done&& done) {
@@ -337,7 +341,7 @@ __device__ __forceinline__ void sort_in_registers(int b, int len, int* __restric
 }
 
 template <int G, typename Done>
-__device__ __forceinline__ void sort_segment(int b, int len, int* __restrict__ v, Done&& done) {
+__device__ __forceinline__ void sort_segment(int b, int len, int* __restrict__ v, int* __restrict__ tmp, Done&& done) {
   const int lane = threadIdx.x & (G - 1);
   const unsigned mask = ((1u << G) - 1u) << (threadIdx.x & 31 & ~(G - 1));
   if (len <= G) {
@@ -347,28 +351,41 @@ __device__ __forceinline__ void sort_segment(int b, int len, int* __restrict__ v
   } else if (len <= 4 * G) {
     sort_in_registers<G, 4>(b, len, v, mask, done);
   } else {
-    if (lane == 0)
-      for (int p = b + 1; p < b + len; ++p) {
-        const int key = v[p];
-        int y = p - 1;
-        while (y >= b && v[y] > key) {
-          v[y + 1] = v[y];
-          --y;
-        }
-        v[y + 1] = key;
+    constexpr int K = 8;
+    for (int p0 = 0; p0 < len; p0 += K * G) {
+      int x[K], r[K];
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        x[k] = (p0 + k * G + lane < len) ? v[b + p0 + k * G + lane] : 0x7fffffff;
+        r[k] = 0;
       }
+#pragma unroll 4
+      for (int q = 0; q < len; ++q) {
+        const int y = v[b + q];
+#pragma unroll
+        for (int k = 0; k < K; ++k) r[k] += (y < x[k]) ? 1 : 0;
+      }
+#pragma unroll
+      for (int k = 0; k < K; ++k)
+        if (p0 + k * G + lane < len) tmp[b + r[k]] = x[k];
+    }
     __syncwarp(mask);
-    for (int p = lane; p < len; p += G) done(b + p, v[b + p]);
+    for (int p = lane; p < len; p += G) {
+      const int x = tmp[b + p];
+      v[b + p] = x;
+      done(b + p, x);
+    }
   }
 }
 
 // 16 lanes per column (about 25 edges at the density of water and a cutoff of 4 Angstrom)
-__global__ void __launch_bounds__(256) sort_columns_kernel(const int* __restrict__ start, int n, int* __restrict__ v) {
+__global__ void __launch_bounds__(256) sort_columns_kernel(const int* __restrict__ start, int n, int* __restrict__ v,
+                                                           int* __restrict__ tmp) {
   pdl_wait();
   const int s = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 4);
   if (s >= n) return;
   const int b = start[s];
-  sort_segment<16>(b, start[s + 1] - b, v, [](int, int) {});
+  sort_segment<16>(b, start[s + 1] - b, v, tmp, [](int, int) {});
 }
 
 // Arrival order of every edge in its column, as a pass of its own: at large sizes the atomics cost
@@ -390,9 +407,9 @@ void nb_col_rank(const int* ej, const int* row_ptr, int n, int edge_cap, int* co
   launch(col_rank_kernel, blocks, 256, 0, st, ej, row_ptr, n, edge_cap, col_count, col_rank);
 }
 
-void nb_sort_columns(const int* col_ptr, int n, int* col_edge, cudaStream_t st) {
+void nb_sort_columns(const int* col_ptr, int n, int* col_edge, int* tmp, cudaStream_t st) {
   if (n <= 0) return;
-  launch(sort_columns_kernel, (unsigned)(((int64_t)n * 16 + 255) / 256), 256, 0, st, col_ptr, n, col_edge);
+  launch(sort_columns_kernel, (unsigned)(((int64_t)n * 16 + 255) / 256), 256, 0, st, col_ptr, n, col_edge, tmp);
 }
 
 // ---------------------------------------------------------------------------
@@ -527,13 +544,13 @@ __global__ void __launch_bounds__(256) sort_cells_kernel(const double* __restric
                                                          const int* __restrict__ species, CellGrid g, int n_cells,
                                                          const int* __restrict__ cell_start,
                                                          const int* __restrict__ wrap, int* __restrict__ sorted,
-                                                         float4* __restrict__ pos4, double* __restrict__ pw,
+                                                         int* __restrict__ tmp, float4* __restrict__ pos4, double* __restrict__ pw,
                                                          int4* __restrict__ wraps) {
   pdl_wait();
   const int c = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3);
   if (c >= n_cells) return;
   const int b = cell_start[c];
-  sort_segment<8>(b, cell_start[c + 1] - b, sorted, [&](int s, int j) {
+  sort_segment<8>(b, cell_start[c + 1] - b, sorted, tmp, [&](int s, int j) {
     double p[3];
     const int wj[3] = {wrap[3 * (size_t)j], wrap[3 * (size_t)j + 1], wrap[3 * (size_t)j + 2]};
 #pragma unroll
@@ -551,10 +568,10 @@ __global__ void __launch_bounds__(256) sort_cells_kernel(const double* __restric
 }
 
 void nb_sort_cells(const double* pos, const int* species, const CellGrid& g, int n_cells, const int* cell_start,
-                   const int* wrap, int* sorted, float4* pos4, double* pw, int4* wraps, cudaStream_t st) {
+                   const int* wrap, int* sorted, int* tmp, float4* pos4, double* pw, int4* wraps, cudaStream_t st) {
   if (n_cells <= 0) return;
   launch(sort_cells_kernel, (unsigned)(((int64_t)n_cells * 8 + 255) / 256), 256, 0, st, pos, species, g, n_cells, cell_start,
-                                                                                    wrap, sorted, pos4, pw, wraps);
+                                                                                    wrap, sorted, tmp, pos4, pw, wraps);
 }
 
 // Neighbour search.  A float32 prefilter on the wrapped positions decides
