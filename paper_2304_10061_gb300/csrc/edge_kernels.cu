@@ -789,6 +789,11 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// neither infinite nor NaN, from the exponent: isfinite compares on the float64 unit, and four of the
+// ten warps, which it doubles the work of there, set a structure's time (a batch of two structures of
+// 60,000 atoms 626 us, 274 with this; a thread per atom and a tree 306)
+__device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+
 __global__ void __launch_bounds__(kStructThreads) struct_reduce_kernel(
     const int64_t* __restrict__ offs, const double* __restrict__ E_atom, const double* __restrict__ Wat,
     const double* __restrict__ F, bool want_w, int parts, double* __restrict__ part, unsigned* __restrict__ ticket,
@@ -813,8 +818,8 @@ __global__ void __launch_bounds__(kStructThreads) struct_reduce_kernel(
     for (long long i = a0 + lane; i < a1; i += 32) {
       const double x = src[ld * i];
       acc += x;
-      if (q == 0) bad |= !isfinite(x);
-      if (want_w && q >= 1 && q <= 3) bad |= !isfinite(F[3 * i + q - 1]);
+      if (q == 0) bad |= !finite_bits(x);
+      if (want_w && q >= 1 && q <= 3) bad |= !finite_bits(F[3 * i + q - 1]);
     }
     acc = warp_sum(acc);
   }
