@@ -868,7 +868,8 @@ allegro_status ensure_edges(allegro_ctx* c, int64_t E) {
   if (c->fixed && c->edge_cap > 0 && E > c->edge_cap)
     return fail(c, ALLEGRO_E_CAPACITY, "neighbour list needs %lld edges, capacity is %lld", (long long)E,
                 (long long)c->edge_cap);
-  if (E > 2000000000LL) return fail(c, ALLEGRO_E_CAPACITY, "%lld edges exceed the int32 edge index", (long long)E);
+  if (E > 2000000000LL)   // (the scan's sums stop at INT_MAX)
+    return fail(c, ALLEGRO_E_CAPACITY, "%lld edges or more exceed the int32 edge index", (long long)E);
   Caps& k = caps_of(c);
   int64_t need = std::max<int64_t>(std::max<int64_t>(E, c->fixed ? c->edge_cap : 0), 1);
   CUDA_TRY(c, grow(c->d_ej, k.ej, need));
@@ -939,10 +940,9 @@ allegro_status fill_rows(allegro_ctx* c, int n, int64_t* n_edges_out, Fill&& fil
     // the bytes of the edges, now that their number is known; a pass that left the list unwritten moved none
     for (size_t k = rec; k < c->prof.recs.size(); ++k) {
       ProfRec& r = c->prof.recs[k];
-      r.bytes = (E >= 0 && E <= room) ? r.bytes + (double)E * (k == rec ? 44.0 : 16.0) : 0.0;
+      r.bytes = (E <= room) ? r.bytes + (double)E * (k == rec ? 44.0 : 16.0) : 0.0;
     }
     if ((s = eval_status(c, err)) != ALLEGRO_OK) return s;   // (MD: the evaluation that moved the atoms here)
-    if (E < 0) return fail(c, ALLEGRO_E_CAPACITY, "edge count overflows int32");
     if ((s = ensure_edges(c, E)) != ALLEGRO_OK) return s;
     if (room > 0 && E <= room) break;
     if (sized) return fail(c, ALLEGRO_E_CUDA, "internal: the edge count changed between two passes");

@@ -31,14 +31,18 @@ __device__ __forceinline__ int floordiv(int a, int b) {
 // ---------------------------------------------------------------------------
 // exclusive scan of int32 (out has n+1 entries; out[n] = total).  With `clear`
 // the input is zeroed as it is read (the counters the next build adds to).
+// The entries are counts, and their sums stop at INT_MAX: a list of 2^32 edges and some would otherwise
+// show the host a small total, and the fill pass would write its rows at wrapped offsets.
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ int add_sat(int a, int b) { return (int)min((unsigned)a + (unsigned)b, 0x7fffffffu); }
+
 constexpr int kScanBlock = 1024;   // elements per block of the large scan (256 threads x 4)
 
 __device__ __forceinline__ int warp_inclusive(int x, int lane) {
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
+    if (lane >= o) x = add_sat(x, y);
   }
   return x;
 }
@@ -69,8 +73,9 @@ __device__ __forceinline__ int block_scan_tile(int* __restrict__ in, int* __rest
   }
   int s = 0;
 #pragma unroll
-  for (int k = 0; k < PER; ++k) s += v[k];
+  for (int k = 0; k < PER; ++k) s = add_sat(s, v[k]);
   const int x = warp_inclusive(s, lane);
+  const int before = __shfl_up_sync(0xffffffffu, x, 1);
   if (lane == 31) warp_tot[w] = x;
   __syncthreads();
   if (w == 0) {
@@ -78,12 +83,12 @@ __device__ __forceinline__ int block_scan_tile(int* __restrict__ in, int* __rest
     if (lane < kWarps) warp_tot[lane] = wt;
   }
   __syncthreads();
-  int excl = x - s + (w > 0 ? warp_tot[w - 1] : 0);
+  int excl = add_sat(lane > 0 ? before : 0, w > 0 ? warp_tot[w - 1] : 0);
 #pragma unroll
   for (int k = 0; k < PER; k += 4) {
     int4 y;
-    y.x = excl; y.y = y.x + v[k]; y.z = y.y + v[k + 1]; y.w = y.z + v[k + 2];
-    excl = y.w + v[k + 3];
+    y.x = excl; y.y = add_sat(y.x, v[k]); y.z = add_sat(y.y, v[k + 1]); y.w = add_sat(y.z, v[k + 2]);
+    excl = add_sat(y.w, v[k + 3]);
     if (b + k + 3 <= n) {
       *reinterpret_cast<int4*>(out + b + k) = y;
     } else {
@@ -115,7 +120,7 @@ __global__ void scan_add_kernel(int* __restrict__ out, int n, const int* __restr
   for (int k = threadIdx.x; k < kScanBlock; k += blockDim.x) {
     int idx = base + k;
     if (idx <= n) {
-      const int v = out[idx] + add;
+      const int v = add_sat(out[idx], add);
       out[idx] = v;
       if (total && idx == n) *total = v;
     }
