@@ -595,7 +595,10 @@ constexpr int kSearchThreads = 128;
 // 1,553 + 3,298 / 518 + 2,426 (the warp form issues more instructions per candidate).
 constexpr int kSearchWarpAtoms = 65536;
 
-// image q (three signed 10-bit fields) and the exact-test flag of a staged edge
+// image q (three signed 10-bit fields) and the exact-test flag of a staged edge.  Stencils that reach
+// further (a periodic axis thinner than 1/511 of the cutoff) go unpacked: a thread per centre writes
+// every edge itself.
+__host__ __device__ inline bool q_packs(const CellGrid& g) { return g.R[0] < 512 && g.R[1] < 512 && g.R[2] < 512; }
 __device__ __forceinline__ int pack_q(int q0, int q1, int q2, bool exact) {
   return (q0 & 1023) | ((q1 & 1023) << 10) | ((q2 & 1023) << 20) | (exact ? (1 << 30) : 0);
 }
@@ -798,7 +801,7 @@ __global__ void __launch_bounds__(kSearchThreads) search_kernel(
 // image q, whether it took the exact test) in its warp's staging area, then the warp writes the 32 rows
 // one after another with its lanes on consecutive edges of a row, so each store covers consecutive
 // addresses (a row per lane would scatter every store over 32 rows).  Edges past kFillStage in a row
-// are written by their lane directly.
+// are written by their lane directly, and so are all of them when an image does not pack (q_packs).
 constexpr int kFillStage = 32;
 
 template <bool fill>
@@ -825,6 +828,7 @@ __global__ void __launch_bounds__(kSearchThreads) search_thread_kernel(
   int4 wi = make_int4(0, 0, 0, 0);
   double pi[3] = {0.0, 0.0, 0.0}, pwi[3] = {0.0, 0.0, 0.0};
   int k = 0, base = 0, cap = 0;
+  const int nstage = q_packs(g) ? kFillStage : 0;
   if (act) {
     const int ci = cell_of[i];
     int c[3];
@@ -886,7 +890,7 @@ __global__ void __launch_bounds__(kSearchThreads) search_thread_kernel(
                                     prow ? prow[__float_as_int(pj.w)] : rc2, d))
               continue;
             if constexpr (fill) {
-              if (k < kFillStage) {
+              if (k < nstage) {
                 stage[threadIdx.x][k] = make_int2(s, pack_q(q0, q1, q2, exact));
               } else if (k < cap) {
                 // past the staging area: this lane writes the edge itself
@@ -919,7 +923,7 @@ __global__ void __launch_bounds__(kSearchThreads) search_thread_kernel(
     __syncwarp();
     // the warp's rows one after another, lanes on consecutive edges
     const int lane = threadIdx.x & 31, w0 = threadIdx.x & ~31;
-    const int nst = act ? min(min(k, cap), kFillStage) : 0;
+    const int nst = act ? min(min(k, cap), nstage) : 0;
     for (int r = 0; r < 32; ++r) {
       const int nr = __shfl_sync(0xffffffffu, nst, r);
       if (nr == 0) continue;
@@ -971,7 +975,7 @@ bool nb_search(bool fill, const double* pos, int n, const CellGrid& g, const int
                int* ej,               int* ei, int* eS, double* ed, int* col_count, int* col_rank, int edge_cap, int* d_err,
                cudaStream_t st) {
   if (n <= 0) return true;
-  if (n <= kSearchWarpAtoms) {
+  if (n <= kSearchWarpAtoms && q_packs(g)) {
     auto kernel = fill ? search_kernel<true> : search_kernel<false>;
     launch(kernel, (n + kSearchThreads / 32 - 1) / (kSearchThreads / 32), kSearchThreads, 0, st, pos, n, g, cell_of, wraps, cell_start, sorted, pos4, pw, rc2, band, pair_rc2, pair_rc2f, ns, count, row_ptr, ej, ei, eS, ed,
         col_count, col_rank, edge_cap, d_err);
