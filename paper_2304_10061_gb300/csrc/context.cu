@@ -239,7 +239,6 @@ struct allegro_ctx {
   void* d_scan_tmp = nullptr;
   size_t scan_tmp_cap = 0;
   int* d_err = nullptr;
-  int* d_total = nullptr;
   double* d_minmax = nullptr;
   double* d_red_scratch = nullptr;         // partial sums of the per-structure reduction
   Caps caps;
@@ -1732,8 +1731,9 @@ allegro_status run_plan(allegro_ctx* c, const Plan& p, const WS& w, bool backwar
   }
   {
     ProfScope ps(c, "atom_reduce", 0.0, (double)E * (backward ? 60.0 : 4.0) + (double)n * (backward ? 128.0 : 16.0));
-    atom_reduce(n, (int)std::min<int64_t>(c->n_centres, n), c->d_row_ptr, c->d_col_ptr, c->d_col_edge, c->d_Ee, c->d_g, c->d_ed, c->d_species, c->d_sigma,
-                c->d_mu, backward, c->d_Eatom, c->d_F, c->d_Wat, c->d_ei, c->d_ej, c->arch, c->stream);
+    atom_reduce(n, (int)std::min<int64_t>(c->n_centres, n), c->d_row_ptr, c->d_col_ptr, c->d_col_edge, c->d_Ee, c->d_g,
+        c->d_ed, c->d_species, c->d_sigma, c->d_mu, backward, c->d_Eatom, c->d_F, c->d_Wat, c->d_ei, c->d_ej, c->arch,
+        c->stream);
   }
   {
     ProfScope ps(c, "struct_reduce", 0.0, (double)n * (backward ? 104.0 : 8.0));
@@ -1979,7 +1979,7 @@ allegro_status allegro_create(const void* weights_blob, size_t blob_bytes, const
   if (cudaMalloc(&c->d_map, c->nmap * 4) != cudaSuccess ||
       cudaMemcpy(c->d_map, c->species_map.data(), c->nmap * 4, cudaMemcpyHostToDevice) != cudaSuccess)
     return bail(fail(c, ALLEGRO_E_OOM, "species map upload failed"));
-  if (cudaMalloc(&c->d_err, 16) != cudaSuccess || cudaMalloc(&c->d_total, 16) != cudaSuccess ||
+  if (cudaMalloc(&c->d_err, 16) != cudaSuccess ||
       cudaMalloc(&c->d_minmax, 12 * 8) != cudaSuccess || cudaMalloc(&c->d_red_scratch, kStructScratch * sizeof(double)) != cudaSuccess)
     return bail(fail(c, ALLEGRO_E_OOM, "scratch allocation failed"));
   // The context's stream does not wait for the default stream, nor a later one for it: the uploads (on
@@ -2658,7 +2658,7 @@ void allegro_destroy(allegro_ctx* c) {
                   c->d_cell_of, c->d_wrap, c->d_sorted, c->d_pos4, c->d_pw, c->d_atom_struct, c->d_Eatom, c->d_F, c->d_Wat,
                   c->d_ej, c->d_ei, c->d_eS, c->d_ed, c->d_col_edge, c->d_Ee, c->d_g, c->d_cell_count,
                   c->d_cell_start, c->d_col_count, c->d_offs, c->d_cells, c->d_pbc, c->d_nimg, c->d_Eout,
-                  c->d_Wout, c->d_scan_tmp, c->d_err, c->d_total, c->d_minmax, c->d_red_scratch, c->ws,
+                  c->d_Wout, c->d_scan_tmp, c->d_err, c->d_minmax, c->d_red_scratch, c->ws,
                   c->d_md_pos, c->d_md_vel, c->d_md_invm, c->d_md_types, c->d_md_masses, c->d_md_E, c->d_md_K,
                   c->d_md_part, c->d_pair_basis, c->d_pair_rc2, c->d_zbl, c->d_sk_row, c->d_sk_j,
                   c->d_sk_S, c->d_sk_ref, c->d_cell9, c->d_maxd, c->d_amax, c->d_wraps};

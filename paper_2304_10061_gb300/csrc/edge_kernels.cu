@@ -436,7 +436,8 @@ void edge_geom_bwd(int Ec, int e0, const double* ed, const int* ei, const int* e
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const int tiles = (Ec + kGeomBlock - 1) / kGeomBlock;
   const int grid = std::min(tiles, std::max(nsm, 1) * kGeomBwdBlocksPerSM);
-  launch(geom_bwd_kernel<T>, grid, kGeomBlock, smem, st, Ec, e0, ed, ei, ej, species, make_basis(a), zbar0, ldz, W0t, ldW, a.tb[0], ubar, yb, g);
+  launch(geom_bwd_kernel<T>, grid, kGeomBlock, smem, st, Ec, e0, ed, ei, ej, species, make_basis(a), zbar0, ldz, W0t,
+      ldW, a.tb[0], ubar, yb, g);
 }
 template void edge_geom_bwd<float>(int, int, const double*, const int*, const int*, const int*, const Arch&,
                                    const float*, int, const float*, int, const float*, const YbarParts&, float*,
@@ -538,8 +539,8 @@ void mlp_head_bwd(int Ec, int K, const float* xbar, int ld_x, const float* vcons
   constexpr int b4 = 4 * (int)sizeof(T);   // bytes of four activation-type values
   const int vec = al(xbar, 16) && al(vconst, 16) && al(pre, b4) && al(zbar, b4) && al(addx, b4) &&
                   (ld_x % 4 == 0) && (ld_pre % 4 == 0) && (ld_z % 4 == 0) && (!addx || ld_addx % 4 == 0);
-  launch(head_bwd_kernel<T>, (unsigned)((threads + 255) / 256), 256, 0, st, Ec, K, xbar, ld_x, vconst, ei, species, sigma, e0, pre, ld_pre, u, ubar, ubar_init, zbar, ld_z, amax, addx,
-      ld_addx, vec);
+  launch(head_bwd_kernel<T>, (unsigned)((threads + 255) / 256), 256, 0, st, Ec, K, xbar, ld_x, vconst, ei, species,
+      sigma, e0, pre, ld_pre, u, ubar, ubar_init, zbar, ld_z, amax, addx, ld_addx, vec);
 }
 template void mlp_head_bwd<float>(int, int, const float*, int, const float*, const int*, const int*,
                                   const double*, int, const float*, int, const float*, float*, bool, float*, int,
@@ -764,8 +765,9 @@ void atom_reduce(int n, int n_centres, const int* row_ptr, const int* col_ptr, c
   if (n <= 0) return;
   const float2* zbl = reinterpret_cast<const float2*>(a.zbl);
   if (n <= (zbl ? kReduceGroupAtomsZbl : (want_forces ? kReduceGroupAtoms : kReduceGroupAtomsEnergy)))
-    launch(atom_reduce_group_kernel, (n + kReduceAtoms - 1) / kReduceAtoms, 16 * kReduceAtoms, 0, st, n, n_centres, row_ptr, col_ptr, col_edge, Ee, g, ed, species, sigma, mu, want_forces, E_atom, F, Wat, ei, ej,
-        zbl, make_basis(a));
+    launch(atom_reduce_group_kernel, (n + kReduceAtoms - 1) / kReduceAtoms, 16 * kReduceAtoms, 0, st, n, n_centres,
+        row_ptr, col_ptr, col_edge, Ee, g, ed, species, sigma, mu, want_forces, E_atom, F, Wat, ei, ej, zbl,
+        make_basis(a));
   else
     launch(atom_reduce_kernel, (n + 127) / 128, 128, 0, st, n, n_centres, row_ptr, col_ptr, col_edge, Ee, g, ed, species,
                                                         sigma, mu, want_forces, E_atom, F, Wat, ei, ej, zbl,
@@ -852,8 +854,8 @@ void struct_reduce(int nstruct, const int64_t* offs, const double* E_atom, const
   if (nstruct <= 0) return;
   static_assert(kStructScratch > 10 * kStructParts, "partials and the ticket");
   const int parts = nstruct == 1 ? (int)std::min<int64_t>(kStructParts, (n_atoms + kStructAtoms - 1) / kStructAtoms) : 1;
-  launch(struct_reduce_kernel, parts > 1 ? parts : nstruct, kStructThreads, 0, st, offs, E_atom, Wat, F, want_w, std::max(parts, 1), scratch, reinterpret_cast<unsigned*>(scratch + 10 * kStructParts),
-      E_out, W_out, d_err);
+  launch(struct_reduce_kernel, parts > 1 ? parts : nstruct, kStructThreads, 0, st, offs, E_atom, Wat, F, want_w,
+      std::max(parts, 1), scratch, reinterpret_cast<unsigned*>(scratch + 10 * kStructParts), E_out, W_out, d_err);
 }
 
 }  // namespace alg

@@ -39,19 +39,6 @@ __device__ __forceinline__ void st_bf16_row(uint8_t* box, int r, const float (&v
     *reinterpret_cast<uint4*>(box + sw64(r, u)) = x;
   }
 }
-__device__ __forceinline__ void ld_bf16_row(const uint8_t* box, int r, float (&v)[32]) {
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    uint4 x = *reinterpret_cast<const uint4*>(box + sw64(r, u));
-    uint32_t w[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      float2 f = __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&w[t]));
-      v[8 * u + 2 * t] = f.x;
-      v[8 * u + 2 * t + 1] = f.y;
-    }
-  }
-}
 __device__ __forceinline__ void st_f32_row(uint8_t* box, int r, const float (&v)[32]) {
 #pragma unroll
   for (int u = 0; u < 8; ++u)

@@ -80,38 +80,6 @@ __device__ __forceinline__ void load_bf16x32(const bf16* p, float (&v)[32]) {
   }
 }
 
-__device__ __forceinline__ void epi_apply_vec32_bf16(const EpiParams& ep, int m, int n, float (&v)[32]) {
-  if (ep.epi == EPI_FWD_SILU) {
-    if (ep.pre) store_bf16x32(reinterpret_cast<bf16*>(ep.pre) + (size_t)m * ep.ldp + n, v);
-    const float rs = ep.rowscale ? ep.rowscale[m] : 1.0f;
-#pragma unroll
-    for (int j = 0; j < 32; ++j) v[j] = v[j] * epi_sigmoid(v[j]) * rs;
-    store_bf16x32(reinterpret_cast<bf16*>(ep.out) + (size_t)m * ep.ldo + n, v);
-  } else if (ep.epi == EPI_F32) {
-    float4* o = reinterpret_cast<float4*>(reinterpret_cast<float*>(ep.out) + (size_t)m * ep.ldo + n);
-    if (ep.add) {
-      const float4* a = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(ep.add) + (size_t)m * ep.ld_add + n);
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        float4 x = a[k];
-        o[k] = make_float4(v[4 * k] + x.x, v[4 * k + 1] + x.y, v[4 * k + 2] + x.z, v[4 * k + 3] + x.w);
-      }
-    } else {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) o[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
-    }
-  } else {
-    float z[32];
-    load_bf16x32(reinterpret_cast<const bf16*>(ep.pre) + (size_t)m * ep.ldp + n, z);
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      const float s = epi_sigmoid(z[j]);
-      v[j] = v[j] * s * (1.0f + z[j] * (1.0f - s));
-    }
-    store_bf16x32(reinterpret_cast<bf16*>(ep.out) + (size_t)m * ep.ldo + n, v);
-  }
-}
-
 inline EpiParams make_epi(const GemmArgs& g) {
   EpiParams e;
   e.epi = g.epi; e.out = g.out; e.ldo = g.ldo; e.pre = g.pre; e.ldp = g.ldp;

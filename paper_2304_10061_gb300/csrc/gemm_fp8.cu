@@ -206,10 +206,6 @@ __device__ __forceinline__ uint4 f8_convert16(uint4 lo, uint4 hi, float inv) {
   return make_uint4(o[0], o[1], o[2], o[3]);
 }
 
-__device__ __forceinline__ void fence_async_smem_f8() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
 struct F8Params {
   int M, N, K, K1;              // A columns [0, K1) from tmA, [K1, K) from tmA2
   int maps;                     // 1: every epilogue array can be moved by TMA
@@ -560,13 +556,13 @@ __global__ void __launch_bounds__(kF8Threads, 1)
             *reinterpret_cast<uint4*>(a8 + row * 128 + (((4 * h + cc) ^ sw) << 4)) = f8_convert16(lo, hi, invA);
           }
           // the staging reads are ordered before the next TMA write into the half
-          fence_async_smem_f8();
+          fence_async_smem();
           __syncwarp();
           if (lane == 0) mbar_arrive(&sempty[s2]);
         }
         if (!ok) break;
         // the A tile's generic-proxy writes become visible to the tensor core
-        fence_async_smem_f8();
+        fence_async_smem();
         __syncwarp();
         if (lane == 0) mbar_arrive(&afull[s]);
       }

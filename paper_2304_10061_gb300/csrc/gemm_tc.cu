@@ -85,7 +85,6 @@ bool tc_tensor_map_2d(CUtensorMap* tm, CUtensorMapDataType dtype, int esize, con
   return r == CUDA_SUCCESS;
 }
 
-
 bool tc_box_map(CUtensorMap* tm, const void* base, int cols, int rows, int ld, int esize) {
   cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   cuuint64_t strides[1] = {(cuuint64_t)ld * esize};
@@ -164,21 +163,6 @@ static size_t tc_smem_bytes(const TcLayout& L) {
   return (size_t)L.stages * tc_stage_bytes<BN, PAIR>() + (size_t)4 * EPQ * L.epi_slot + 1024 + (PAIR ? kTcMiscPair : kTcMisc);
 }
 
-__device__ __forceinline__ void load_bf16x16(const bf16* p, float (&v)[16]) {
-  const uint4* q = reinterpret_cast<const uint4*>(p);
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    uint4 x = q[k];
-    uint32_t w[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      float2 f = __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&w[t]));
-      v[8 * k + 2 * t] = f.x;
-      v[8 * k + 2 * t + 1] = f.y;
-    }
-  }
-}
-
 // sigma(z) = (1 + tanh(z / 2)) / 2 with the hardware tanh approximation (one
 // transcendental-unit op instead of an exponential and a reciprocal; its
 // relative error, about 2^-11, is below the bf16 rounding of the outputs)
@@ -209,7 +193,6 @@ __device__ __forceinline__ float2 dsilu_factor2(float2 z, float2 sg) {
 __device__ __forceinline__ float2 bf16_word_pair(uint32_t x) {
   return make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u));
 }
-
 
 // Persistent kernel: CTA b handles tiles b, b + gridDim.x, ...  Two TMEM
 // accumulator buffers: the MMA warp fills buffer (t & 1) while the epilogue
@@ -1307,7 +1290,6 @@ bool gemm_tc_bf16(const GemmArgs& g, cudaStream_t st, int* d_err, std::string* w
   }
 }
 
-
 template <int N1, int N2, int E1, int E2>
 static bool launch_chain_pipe(const GemmArgs& g1, const GemmArgs& g2, const bf16* B1, int ldb1, const bf16* B2,
                               int ldb2, cudaStream_t st, int* d_err, std::string* why) {
@@ -1379,7 +1361,6 @@ bool gemm_chain_bf16(const GemmArgs& g1, const GemmArgs& g2, cudaStream_t st, in
   }
   return false;
 }
-
 
 // ---------------------------------------------------------------------------
 // TF32 GEMM on tcgen05 (kind::tf32) for the float32-storage precisions:

@@ -969,21 +969,22 @@ __global__ void __launch_bounds__(kSearchThreads) search_thread_kernel(
   }
 }
 
-bool nb_search(bool fill, const double* pos, int n, const CellGrid& g, const int* cell_of,
-               const int4* wraps, const int* cell_start, const int* sorted, const float4* pos4, const double* pw,
-               double rc2, float band, const double* pair_rc2, const float* pair_rc2f, int ns, int* count, const int* row_ptr,
-               int* ej,               int* ei, int* eS, double* ed, int* col_count, int* col_rank, int edge_cap, int* d_err,
-               cudaStream_t st) {
+bool nb_search(bool fill, const double* pos, int n, const CellGrid& g, const int* cell_of, const int4* wraps,
+               const int* cell_start, const int* sorted, const float4* pos4, const double* pw, double rc2, float band,
+               const double* pair_rc2, const float* pair_rc2f, int ns, int* count, const int* row_ptr, int* ej, int* ei,
+               int* eS, double* ed, int* col_count, int* col_rank, int edge_cap, int* d_err, cudaStream_t st) {
   if (n <= 0) return true;
   if (n <= kSearchWarpAtoms && q_packs(g)) {
     auto kernel = fill ? search_kernel<true> : search_kernel<false>;
-    launch(kernel, (n + kSearchThreads / 32 - 1) / (kSearchThreads / 32), kSearchThreads, 0, st, pos, n, g, cell_of, wraps, cell_start, sorted, pos4, pw, rc2, band, pair_rc2, pair_rc2f, ns, count, row_ptr, ej, ei, eS, ed,
+    launch(kernel, (n + kSearchThreads / 32 - 1) / (kSearchThreads / 32), kSearchThreads, 0, st, pos, n, g, cell_of,
+        wraps, cell_start, sorted, pos4, pw, rc2, band, pair_rc2, pair_rc2f, ns, count, row_ptr, ej, ei, eS, ed,
         col_count, col_rank, edge_cap, d_err);
     return true;
   }
   auto kernel = fill ? search_thread_kernel<true> : search_thread_kernel<false>;
-  launch(kernel, (n + kSearchThreads - 1) / kSearchThreads, kSearchThreads, 0, st, pos, n, g, cell_of, wraps, cell_start, sorted, pos4, pw, rc2, band, pair_rc2, pair_rc2f, ns, count, row_ptr, ej, ei, eS, ed,
-      edge_cap, d_err);
+  launch(kernel, (n + kSearchThreads - 1) / kSearchThreads, kSearchThreads, 0, st, pos, n, g, cell_of, wraps,
+      cell_start, sorted, pos4, pw, rc2, band, pair_rc2, pair_rc2f, ns, count, row_ptr, ej, ei, eS, ed, edge_cap,
+      d_err);
   return false;
 }
 

@@ -282,15 +282,6 @@ struct SbarW {
   static constexpr int NB = CPL * (int)sizeof(T);
   static constexpr int NW = NB / 4;
 };
-template <typename T, int CPL>
-__device__ __forceinline__ void ld_sbar(const void* sbar, int ld, int e, const RowCtx& r,
-                                        uint32_t (&w)[SbarW<T, CPL>::NW]) {
-  if (r.act) ld_words<SbarW<T, CPL>::NB>(reinterpret_cast<const T*>(sbar) + (size_t)e * ld + r.u0, w);
-  else {
-#pragma unroll
-    for (int q = 0; q < SbarW<T, CPL>::NW; ++q) w[q] = 0u;
-  }
-}
 // the same values as CPL separate element loads (raw bits in the low bits of each word)
 template <typename T, int CPL>
 __device__ __forceinline__ void ld_sbar_el(const void* sbar, int ld, int e, const RowCtx& r, uint32_t (&w)[CPL]) {
