@@ -1206,9 +1206,14 @@ allegro_status run_chunk(allegro_ctx* c, const WS& w, int a0, int a1, int e0, in
     if (fused && L == nl) {
       // last latent MLP; its final layer carries the folded edge energy and the start of the adjoint
       if (nlat >= 2) {
-        if ((s = fwd_mlp(c->lat[L - 1], w.Zlat[L - 1], w.ld_Zlat, 0, nlat - 2, in, ld_in, K, nullptr, 0)) !=
-            ALLEGRO_OK)
-          return s;
+        // the layers before the last two, the last of them into H[0] (the pair below goes to H[1], then H[0])
+        for (int k = 0; k < nlat - 2; ++k) {
+          void* out = w.H[(nlat - 3 - k) & 1];
+          if ((s = G(in, ld_in, K, c->lat[L - 1][k], false, EPI_FWD_SILU, out, w.ld_H, a.lat[k], w.Zlat[L - 1][k],
+                     w.ld_Zlat[k])) != ALLEGRO_OK)
+            return s;
+          in = out; ld_in = w.ld_H; K = a.lat[k];
+        }
         GemmArgs g1 = mk(in, ld_in, K, c->lat[L - 1][nlat - 2], false, EPI_FWD_SILU, w.H[1], w.ld_H,
                          a.lat[nlat - 2], w.Zlat[L - 1][nlat - 2], w.ld_Zlat[nlat - 2]);
         GemmArgs g2 = mk(nullptr, 0, a.lat[nlat - 2], c->lat[L - 1][nlat - 1], false, EPI_LAST, w.H[0], w.ld_H,

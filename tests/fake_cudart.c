@@ -2,8 +2,10 @@
  * takes every call the library makes.  Device memory is host memory, copies and clears happen at
  * once, kernels do nothing but call the test's hook (name, arguments).  What a stream still has
  * queued is counted until a call waits for that stream, as on a device: a test can ask what a call
- * left behind, and put values where a kernel would have written them.
+ * left behind, and put values where a kernel would have written them.  Tensor maps (what the TMA
+ * copies of a kernel may touch) are refused when they leave their allocation or TMA's alignments.
  */
+#include <cuda.h>
 #include <cuda_runtime_api.h>
 #include <stdint.h>
 #include <stdlib.h>
@@ -121,12 +123,34 @@ cudaError_t cudaGetDeviceCount(int* n) { *n = 1; return cudaSuccess; }
 cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
 cudaError_t cudaSetDevice(int d) { (void)d; return cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int* v, enum cudaDeviceAttr a, int d) { (void)a; (void)d; *v = 152; return cudaSuccess; }
-cudaError_t cudaGetDeviceProperties(struct cudaDeviceProp* p, int d) { (void)d; memset(p, 0, sizeof *p); return cudaSuccess; }
+cudaError_t cudaGetDeviceProperties(struct cudaDeviceProp* p, int d) {
+  (void)d;
+  memset(p, 0, sizeof *p);
+  p->major = 10;
+  p->minor = 3;
+  return cudaSuccess;
+}
+static CUresult encode(CUtensorMap* tm, CUtensorMapDataType type, cuuint32_t rank, void* base, const cuuint64_t* dim,
+                       const cuuint64_t* stride, const cuuint32_t* box, const cuuint32_t* step,
+                       CUtensorMapInterleave il, CUtensorMapSwizzle sw, CUtensorMapL2promotion l2,
+                       CUtensorMapFloatOOBfill fill) {
+  (void)step; (void)il; (void)sw; (void)l2; (void)fill;
+  const size_t es = type == CU_TENSOR_MAP_DATA_TYPE_UINT8 ? 1 : (type == CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 ? 2 : 4);
+  const char* p = (const char*)base;
+  memset(tm, 0, sizeof *tm);
+  if (rank != 2 || !dim[0] || !dim[1] || dim[0] * es > stride[0] || (uintptr_t)p % 16 || stride[0] % 16 ||
+      box[0] * es % 16 || box[0] > 256 || box[1] > 256)
+    return CUDA_ERROR_INVALID_VALUE;
+  for (int k = 0; k < g_nalloc; ++k)
+    if (p >= g_alloc[k].p && p + (dim[1] - 1) * stride[0] + dim[0] * es <= g_alloc[k].p + g_alloc[k].n) return CUDA_SUCCESS;
+  return CUDA_ERROR_INVALID_VALUE;
+}
 cudaError_t cudaGetDriverEntryPointByVersion(const char* n, void** f, unsigned v, unsigned long long fl,
                                              enum cudaDriverEntryPointQueryResult* r) {
-  (void)n; (void)v; (void)fl; (void)r;
-  *f = 0;
-  return cudaErrorNotSupported;
+  (void)v; (void)fl;
+  *f = strcmp(n, "cuTensorMapEncodeTiled") ? 0 : (void*)encode;
+  *r = *f ? cudaDriverEntryPointSuccess : cudaDriverEntryPointSymbolNotFound;
+  return cudaSuccess;
 }
 cudaError_t cudaGetSymbolAddress(void** p, const void* s) { (void)p; (void)s; return cudaErrorNotSupported; }
 cudaError_t cudaGetLastError(void) { return cudaSuccess; }

@@ -159,3 +159,32 @@ def test_profile_counts_the_edges_of_its_own_list(fake):
             edges = 100
             build()
     """)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "tf32", "bf16", "fp8"])
+def test_every_array_a_gemm_names_is_there(fake, precision):
+    """MLPs of 1 to 5 layers: each tensor map of an evaluation (operands, outputs, pre-activations) lies in an
+    allocation.  (BF16 latent MLPs of three layers and more wrote a layer at address zero.)"""
+    fake(f"""
+        PRECISION = {precision!r}
+    """ + """
+        from synth import Arch
+
+        @HOOK
+        def hook(name, args):
+            if b"scan_one_kernel" in name and param(args, 4):
+                ctypes.c_int.from_address(param(args, 4)).value = 3000
+
+        fake.fake_on_launch(hook)
+        for layers, lmax, channels in ((1, 1, 16), (1, 2, 64), (2, 1, 32), (2, 2, 64), (2, 2, 32), (3, 2, 64), (2, 3, 16)):
+            for depth in range(1, 6):
+                for widths in ((64, 128, 256, 32, 96), (40, 24, 192, 256, 16), (256, 512, 64, 320, 128)):
+                    if max(widths[:depth]) > 256 and PRECISION == "bf16" and channels * (lmax + 1) % 64:
+                        continue   # (refused)
+                    arch = Arch(n_species=2, lmax=lmax, n_layers=layers, channels=channels, two_body=widths[:depth],
+                                latent=widths[:depth][::-1], edge=(8,))
+                    model = Allegro(weights_to_blob(arch, make_weights(arch, 0)), precision=PRECISION)
+                    assert model.neighbors(pos, types, cell) == 3000
+                    evaluate()
+                    model.close()
+    """)
